@@ -14,6 +14,7 @@
 #include "ucn_kernels.cuh"
 #include "ucn_lanes.cuh"
 #include "ucn_pair.cuh"
+#include "ucn_rows.cuh"
 
 using namespace ucn;
 
@@ -120,6 +121,58 @@ Layout make_layout(int model, int nodes, int max_obs, int tsize, bool reg_mats, 
   return L;
 }
 
+template <class M>
+static Layout rows_layout_of(int nodes, int max_obs, int csize) {
+  typedef Rec<M, 2> R;
+  Layout L;
+  std::memset(&L, 0, sizeof(L));
+  const bool quad = IsQuad<M>::value;
+  const int mo = std::max(max_obs, 1);
+  L.MS = quad ? mo : M14::MS;
+  L.MB = quad ? max_obs : 6;
+  const int ms = pad4(L.MS);
+  L.MD = quad ? 4 * ms : pad4(M14::MD);
+  L.oS = R::END;
+  L.oNus = L.oS + ms;
+  L.oMd = L.oNus + ms;
+  const int nt = L.oMd + L.MD;
+  L.oA = L.oB = L.oH = -1;
+  L.csize = csize;
+  L.chunk = (nodes + csize - 1) / csize;
+  const int recs = L.chunk + (csize > 1 ? 2 : 0);
+  L.S = recs;
+  L.NS = nt + ((4 - nt) % 32 + 32) % 32;   // 4 mod 32: a warp's 8 nodes x 4 rows in distinct banks
+  L.DS = R::DEND | 1;
+  L.tbytes = round_up((long long)recs * L.NS * 4, 16);
+  L.oC = round_up(L.tbytes + (long long)recs * L.DS * 8, 16);
+  L.bytes = round_up(L.oC + 8LL * CB<M>::END, 16);
+  L.oPH = -1;
+  return L;
+}
+
+// The fewest CTAs whose nodes fit their threads: a CTA of 61 nodes takes 1.25 us
+// per ADMM iteration, one of 91 (384 threads, 168 registers) 1.79 us, and 121
+// nodes as a cluster of two 1.75 us (GB300, 20 obstacles) -- a split costs two
+// cluster barriers per iteration, half a microsecond, so it is made only where
+// one CTA cannot hold the instance.
+bool rows_layout(int model, int precision, int nodes, int max_obs, int group, int tpn, int optin, Layout* out) {
+  if (precision != UCN_PREC_FP32_REFINE) return false;
+  const bool quad12 = model == UCN_MODEL_QUAD12;
+  if (quad12 ? tpn != 4 : (tpn != 1 || (model != UCN_MODEL_QUAT13 && model != UCN_MODEL_MARS14))) return false;
+  const long long fixed = (long long)sizeof(InstShared) + sizeof(RowCluster) + (group > 1 ? (long long)sizeof(GroupShared) : 0) + 64;
+  for (int csize = 1; csize <= (group > 1 ? 1 : 4); csize *= 2) {
+    const int cap = (csize == 1 && quad12 ? ROWS_WIDE_THREADS : ROWS_THREADS) / 4;
+    if ((nodes + csize - 1) / csize > cap) continue;
+    const Layout L = quad12 ? rows_layout_of<Quad12>(nodes, max_obs, csize)
+                     : model == UCN_MODEL_QUAT13 ? rows_layout_of<Quat13>(nodes, max_obs, csize)
+                                                 : rows_layout_of<Mars14>(nodes, max_obs, csize);
+    if (L.bytes + fixed > optin) continue;
+    *out = L;
+    return true;
+  }
+  return false;
+}
+
 }  // namespace ucn
 
 struct ucn_problem {
@@ -137,6 +190,8 @@ struct ucn_problem {
   int tpn;               // threads per node of the fused solve
   int last_launches = 0; // kernel launches of the last fused solve
   int optin;             // shared memory per CTA the device allows
+  bool rows;             // the row kernel serves this problem at its default threads per node, on
+  Layout Lr;             // this layout
   unsigned char* warm_ones;   // batch flags, all 1: every instance starts from the given state
 };
 
@@ -365,6 +420,8 @@ ucn_status ucn_problem_create(const ucn_problem_desc* d, ucn_problem** out) {
     p->L = make_layout(d->model, Nmax + 1, p->max_obs, tsize, false, p->tpn);
   }
   p->optin = optin;
+  p->rows = rows_layout(d->model, d->precision, Nmax + 1, p->max_obs, group, default_tpn(d->model, Nmax + 1, d->precision),
+                        optin, &p->Lr);
   p->threads = (int)round_up(Nmax + 1, 32);
   p->smem_bytes = p->smem ? p->L.bytes : 0;
   if (group > 1 && !p->smem) {
@@ -464,6 +521,9 @@ static LaunchCfg cfg_of(ucn_problem* p, void* stream) {
   c.threads = p->threads; c.blocks = p->batch; c.stream = as_stream(stream); c.group = p->gcsize;
   c.nodes = p->Nmax + 1; c.tpn = p->tpn;
   c.launched = &p->last_launches;
+  if (p->rows && p->tpn == default_tpn(p->model, p->Nmax + 1, p->precision)) {
+    c.L = &p->Lr; c.smem = true; c.smem_bytes = p->Lr.bytes;
+  }
   p->last_launches = 1;   // one launch unless the launcher splits the batch
   return c;
 }

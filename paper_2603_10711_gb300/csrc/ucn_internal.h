@@ -24,6 +24,13 @@ int fault_alloc_at();
 // (defined in ucn_api.cu).
 Layout make_layout(int model, int nodes, int max_obs, int tsize, bool reg_mats, int tpn);
 
+// The row kernel's layout (ucn_rows.cuh) of an instance of `nodes` nodes, for the
+// problems it serves: FP32, a 16- or 17-row model at its default threads per
+// node (12-state quadrotor 4, the others 1), 96 nodes per CTA (64 for the
+// others) and up to four CTAs per instance (one for scenario groups), within
+// the device's shared memory per CTA.  False where it does not.
+bool rows_layout(int model, int precision, int nodes, int max_obs, int group, int tpn, int optin, Layout* out);
+
 // Everything one kernel launch needs besides its buffers.
 struct LaunchCfg {
   const void* P;        // ProblemDev*

@@ -87,7 +87,7 @@ __device__ __forceinline__ void deliver_result(const ProblemDev& P, int b, const
 // array.  The mirror arrays (whose length depends on the obstacle count) follow
 // at the runtime offsets Layout::oS / oNus / oMd, then the matrices A, B, H^-1
 // at Layout::oA / oB / oH -- absent from the record when they live in registers.
-template <class M>
+template <class M, int LAY = 1>
 struct Rec {
   static constexpr int NX = M::NX, NU = M::NU, NN = NX + NU;
   static constexpr int C = 0;
@@ -96,6 +96,23 @@ struct Rec {
   static constexpr int U = Nux + NX, Uh = U + NU, Nuu = Uh + NU, Ex1 = Nuu + NU, Ex2 = Ex1 + NX, END = Ex2 + NX;
   // wide record (FP64, or double-float on the FP32 path): nominal state,
   // nominal control, candidate state (exchange)
+  static constexpr int Xbar = 0, Ubar = NX, Xc = NX + NU, DEND = 2 * NX + NU;
+};
+
+// Layout 2, the row kernel's (ucn_rows.cuh; four lanes per node): every array of
+// the record starts at a multiple of four, so that lane q of a node finds its
+// row 4 m + q at a compile-time distance from its own base, and the arrays over
+// the whole of xi = (x, u) are contiguous (U = X + NX and so on): row e of xi
+// is element e of all of them.  Ga (models with vector sets): the mirror sets'
+// part of the Step-1 right-hand side.
+__host__ __device__ constexpr int pad4(int n) { return (n + 3) / 4 * 4; }
+template <class M>
+struct Rec<M, 2> {
+  static constexpr int NX = M::NX, NU = M::NU, NN = NX + NU, PX = pad4(NX), PN = pad4(NN);
+  static constexpr int C = 0, Z = PX, Lam = 2 * PX, Mu = 3 * PX, Ex1 = 4 * PX, Ex2 = 5 * PX;
+  static constexpr int X = 6 * PX, U = X + NX, Xh = X + PN, Uh = Xh + NX, Nux = Xh + PN, Nuu = Nux + NX;
+  static constexpr int Xlo = Nux + PN, Ulo = Xlo + NX, Xhi = Xlo + PN, Uhi = Xhi + NX, Ga = Xhi + PN;
+  static constexpr int END = Ga + (NX == 14 ? PN : 0);
   static constexpr int Xbar = 0, Ubar = NX, Xc = NX + NU, DEND = 2 * NX + NU;
 };
 
@@ -115,8 +132,13 @@ struct CB {
 //  shared memory: node i's record at t + i*NS (NS odd: conflict-free banks),
 //                 FP64 record at d + i*DS (DS odd);
 //  global slice:  element k of node i at t[k*S + i] (coalesced SoA).
+// Layout 2 (row kernel): as in shared memory, NS = 4 mod 32 (a warp reads 8
+// nodes x 4 consecutive rows: 32 distinct banks); an instance may be split over
+// the CTAs of a cluster, `chunk` consecutive nodes each, with one more record
+// on either side for the neighbours' boundary nodes.
 struct Layout {
   int S, NS, DS;           // SoA stride (nodes); AoS record strides (elements)
+  int chunk, csize;        // row kernel: nodes per CTA, CTAs per instance (0, 0: another kernel's layout)
   int MS, MD, MB;          // mirror scalars / mirror data per node; exported mirror blocks
   int oS, oNus, oMd;       // runtime offsets of the mirror arrays in the record
   int oA, oB, oH;          // matrices in the record (-1 when register-resident)
@@ -128,13 +150,14 @@ struct Layout {
 
 // Per-thread view of its node.  W is the wide type of the precision (FP64,
 // or double-float for the FP32 path).
-template <class T, bool AOS>
+template <class T, int AOS>
 struct Node {
   typedef typename WideOf<T>::type W;
   T* t;          // T region base
   W* d;          // wide region base
   W* c;          // CB block of the instance (FP32 path)
   int S, NS, DS, i, N;
+  // (layout 2: t and d point at the record node 0 of the instance would have)
   __device__ __forceinline__ T& at(int off, int k) const { return AOS ? t[i * NS + off + k] : t[(long long)(off + k) * S + i]; }
   __device__ __forceinline__ T& nb(int off, int k, int j) const { return AOS ? t[j * NS + off + k] : t[(long long)(off + k) * S + j]; }
   __device__ __forceinline__ W& dat(int off, int k) const { return AOS ? d[i * DS + off + k] : d[(long long)(off + k) * S + i]; }
@@ -171,6 +194,14 @@ template <class M> struct LaneModel {
 // in distinct banks.
 template <class T> struct ObsStride { static constexpr int value = sizeof(T) == 4 ? 5 : 4; };
 
+// Component c (normal 0..2, bound 3) of obstacle j of a node.  Layout 2: the
+// obstacles of one lane (j mod 4) four apart, component by component.
+template <class T, int AOS>
+__device__ __forceinline__ T& obs_at(const Node<T, AOS>& nd, const Layout& L, int j, int c) {
+  if constexpr (AOS == 2) return nd.at(L.oMd, (j >> 2) * 16 + c * 4 + (j & 3));
+  else return nd.at(L.oMd, ObsStride<T>::value * j + c);
+}
+
 // Row strides of A and B in the record: odd (NX | 1, NU | 1) for the FP32 lane
 // layout, so that lanes reading different rows, or different columns, of their
 // node's matrix fall in distinct banks; unpadded otherwise.
@@ -193,7 +224,7 @@ template <> struct APattern<Mars7> {
   }
 };
 
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 struct SmemMats {
   __host__ __device__ static constexpr int akind(int, int) { return 2; }
   Node<T, AOS> nd;
@@ -227,7 +258,7 @@ struct RegMatsS : RegMats<M, T> {
 };
 // OWNJ: the matrices are the kernel's own Jacobians (their structure holds);
 // a caller's A (ucn_admm_solve) is taken as dense.
-template <class M, class T, bool AOS, bool OWNJ = false>
+template <class M, class T, int AOS, bool OWNJ = false>
 using MatsFor = typename std::conditional<AOS && SmallModel<M>::value,
                                           typename std::conditional<OWNJ, RegMatsS<M, T>, RegMats<M, T>>::type,
                                           SmemMats<M, T, AOS>>::type;
@@ -249,11 +280,11 @@ __device__ __forceinline__ void acc_AA(T& acc, const MS& MT, int k, int r, int c
   else acc += MT.A(k, r) * MT.A(k, c);
 }
 
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 __device__ __forceinline__ void init_mats(SmemMats<M, T, AOS>& m, const Node<T, AOS>& nd, const Layout& L) {
   m.nd = nd; m.oA = L.oA; m.oB = L.oB; m.oH = L.oH;
 }
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 __device__ __forceinline__ void init_mats(RegMats<M, T>& m, const Node<T, AOS>& nd, const Layout& L) {}
 
 // Per-node constants of one SCP iteration, held in registers across the ADMM
@@ -591,7 +622,7 @@ __device__ __forceinline__ void reduce_residuals(InstShared& sh, DF rp, DF rdl, 
 // ------------------------------------------------------------------ per-node pieces
 // The CB block of the instance (FP32 path): every thread of the CTA converts
 // a share of the entries; the caller synchronises before the first use.
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 __device__ void stage_consts(const Node<T, AOS>& nd, const ProblemDev& P, int b) {
   if constexpr (IsDF<T>::value) {
     typedef CB<M> C;
@@ -618,28 +649,28 @@ __device__ void stage_consts(const Node<T, AOS>& nd, const ProblemDev& P, int b)
 }
 
 // Nominal of node i from packed global trajectories.
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 __device__ void load_nominal(const Node<T, AOS>& nd, const Layout& L, const double* xg, const double* ug,
                              long long xo, long long uo) {
   typedef typename Node<T, AOS>::W W;
-  for (int j = 0; j < M::NX; ++j) nd.dat(Rec<M>::Xbar, j) = wide_from_double<W>(xg[(xo + nd.i) * M::NX + j]);
+  for (int j = 0; j < M::NX; ++j) nd.dat(Rec<M, AOS>::Xbar, j) = wide_from_double<W>(xg[(xo + nd.i) * M::NX + j]);
   if (nd.i < nd.N)
-    for (int j = 0; j < M::NU; ++j) nd.dat(Rec<M>::Ubar, j) = wide_from_double<W>(ug[(uo + nd.i) * M::NU + j]);
+    for (int j = 0; j < M::NU; ++j) nd.dat(Rec<M, AOS>::Ubar, j) = wide_from_double<W>(ug[(uo + nd.i) * M::NU + j]);
 }
 
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 __device__ __forceinline__ void read_nominal(const Node<T, AOS>& nd, bool hasU, typename Node<T, AOS>::W* xb,
                                              typename Node<T, AOS>::W* ub) {
   typedef typename Node<T, AOS>::W W;
 #pragma unroll
-  for (int j = 0; j < M::NX; ++j) xb[j] = nd.dat(Rec<M>::Xbar, j);
+  for (int j = 0; j < M::NX; ++j) xb[j] = nd.dat(Rec<M, AOS>::Xbar, j);
 #pragma unroll
-  for (int j = 0; j < M::NU; ++j) ub[j] = hasU ? nd.dat(Rec<M>::Ubar, j) : W();
+  for (int j = 0; j < M::NU; ++j) ub[j] = hasU ? nd.dat(Rec<M, AOS>::Ubar, j) : W();
 }
 
 // One RK4 step of the instance's model in the wide type: FP64 from the problem
 // arrays, or double-float from the CB block.
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 __device__ __forceinline__ void rk4_wide(const Node<T, AOS>& nd, const ProblemDev& P, int b,
                                          const typename Node<T, AOS>::W* x, const typename Node<T, AOS>::W* u,
                                          typename Node<T, AOS>::W* xn) {
@@ -659,7 +690,7 @@ __device__ __forceinline__ double wide_abs(double a) { return fabs(a); }
 __device__ __forceinline__ DF wide_abs(DF a) { return a.hi < 0.0f ? df_neg(a) : a; }
 
 // A_i, B_i by forward-mode differentiation of the RK4 map (Eq. (2b)), in T.
-template <class M, class T, bool AOS, class MS>
+template <class M, class T, int AOS, class MS>
 __device__ __forceinline__ void node_jacobians(const Node<T, AOS>& nd, const MS& MT, const T* prm, const Step3<T>& hs) {
   constexpr int NX = M::NX, NU = M::NU;
   typename Node<T, AOS>::W xb[NX], ub[NU];
@@ -734,10 +765,14 @@ __device__ __forceinline__ void node_jacobians(const Node<T, AOS>& nd, const MS&
   }
 }
 
+template <class M, class T, int AOS>
+__device__ void node_mirror_data(const Node<T, AOS>& nd, const Layout& L, const ProblemDev& P, int b,
+                                 const typename Node<T, AOS>::W* xb, const typename Node<T, AOS>::W* ub);
+
 // QP data of node i at the nominal: cost gradient in deviations, the
 // trust-region boxes of Eq. (2c) (with the boundary conditions of Eq. (1c)
 // as degenerate boxes at nodes 0 and N), and the mirror-set data.
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 __device__ void node_setup(const Node<T, AOS>& nd, const Layout& L, const ProblemDev& P, const Inst<T>& I, int b,
                            double radius, T re, T rg, NodeConst<M, T>& K) {
   constexpr int NX = M::NX, NU = M::NU;
@@ -767,8 +802,8 @@ __device__ void node_setup(const Node<T, AOS>& nd, const Layout& L, const Proble
       T hi = fminf(wide_diff<T>(cb[C::Xhi + j], xb[j]), rad);
       if (i == 0) lo = hi = wide_diff<T>(cb[C::Xinit + j], xb[j]);
       else if (term && P.tmask[b * NX + j]) lo = hi = wide_diff<T>(cb[C::Xtgt + j], xb[j]);
-      nd.at(Rec<M>::Xlo, j) = lo;
-      nd.at(Rec<M>::Xhi, j) = hi;
+      nd.at(Rec<M, AOS>::Xlo, j) = lo;
+      nd.at(Rec<M, AOS>::Xhi, j) = hi;
     }
     for (int j = 0; j < NU; ++j) { K.q[NX + j] = T(0); K.hd[NX + j] = T(1); }
     if (!term) {
@@ -776,8 +811,8 @@ __device__ void node_setup(const Node<T, AOS>& nd, const Layout& L, const Proble
         const DF w = cb[C::Rd + j];
         K.q[NX + j] = I.run_cost ? df_to_float(df_mul(df_sub(ub[j], cb[C::Uref + j]), w)) : T(0);
         K.hd[NX + j] = df_to_float(w) + rg;
-        nd.at(Rec<M>::Ulo, j) = fmaxf(wide_diff<T>(cb[C::Ulo + j], ub[j]), -rad);
-        nd.at(Rec<M>::Uhi, j) = fminf(wide_diff<T>(cb[C::Uhi + j], ub[j]), rad);
+        nd.at(Rec<M, AOS>::Ulo, j) = fmaxf(wide_diff<T>(cb[C::Ulo + j], ub[j]), -rad);
+        nd.at(Rec<M, AOS>::Uhi, j) = fminf(wide_diff<T>(cb[C::Uhi + j], ub[j]), rad);
       }
     }
   } else {
@@ -789,19 +824,27 @@ __device__ void node_setup(const Node<T, AOS>& nd, const Layout& L, const Proble
     double hi = fmin(P.xhi[b * NX + j], xb[j] + radius) - xb[j];
     if (i == 0) lo = hi = P.xinit[b * NX + j] - xb[j];
     else if (term && P.tmask[b * NX + j]) lo = hi = P.xtarget[b * NX + j] - xb[j];
-    nd.at(Rec<M>::Xlo, j) = (T)lo;
-    nd.at(Rec<M>::Xhi, j) = (T)hi;
+    nd.at(Rec<M, AOS>::Xlo, j) = (T)lo;
+    nd.at(Rec<M, AOS>::Xhi, j) = (T)hi;
   }
   for (int j = 0; j < NU; ++j) { K.q[NX + j] = T(0); K.hd[NX + j] = T(1); }
   if (!term) {
     for (int j = 0; j < NU; ++j) {
       K.q[NX + j] = (T)(P.Rd[b * NU + j] * (ub[j] - P.uref[b * NU + j]));
       K.hd[NX + j] = (T)P.Rd[b * NU + j] + rg;
-      nd.at(Rec<M>::Ulo, j) = (T)(fmax(P.ulo[b * NU + j], ub[j] - radius) - ub[j]);
-      nd.at(Rec<M>::Uhi, j) = (T)(fmin(P.uhi[b * NU + j], ub[j] + radius) - ub[j]);
+      nd.at(Rec<M, AOS>::Ulo, j) = (T)(fmax(P.ulo[b * NU + j], ub[j] - radius) - ub[j]);
+      nd.at(Rec<M, AOS>::Uhi, j) = (T)(fmin(P.uhi[b * NU + j], ub[j] + radius) - ub[j]);
     }
   }
   }
+  node_mirror_data<M, T, AOS>(nd, L, P, b, xb, ub);
+}
+
+// The mirror-set data of node i at its nominal (xb, ub).
+template <class M, class T, int AOS>
+__device__ void node_mirror_data(const Node<T, AOS>& nd, const Layout& L, const ProblemDev& P, int b,
+                                 const typename Node<T, AOS>::W* xb, const typename Node<T, AOS>::W* ub) {
+  const bool term = (nd.i == nd.N);
   if constexpr (IsQuad<M>::value) {
     // Obstacle j linearised about the nominal position: n = (p - c)/|p - c|,
     // keep n^T p >= n^T c + r; in deviations n^T dp >= n^T (c - pbar) + r.
@@ -816,10 +859,10 @@ __device__ void node_setup(const Node<T, AOS>& nd, const Layout& L, const Proble
       const T inn = T(1) / nn;
       const T n0 = nv[0] * inn, n1 = nv[1] * inn, n2 = nv[2] * inn;
       const T bd = -(n0 * dp[0] + n1 * dp[1] + n2 * dp[2]) + (T)P.obs_r[(long long)b * P.max_obs + j];
-      nd.at(L.oMd, ObsStride<T>::value * j + 0) = (T)n0;
-      nd.at(L.oMd, ObsStride<T>::value * j + 1) = (T)n1;
-      nd.at(L.oMd, ObsStride<T>::value * j + 2) = (T)n2;
-      nd.at(L.oMd, ObsStride<T>::value * j + 3) = (T)bd;
+      obs_at(nd, L, j, 0) = (T)n0;
+      obs_at(nd, L, j, 1) = (T)n1;
+      obs_at(nd, L, j, 2) = (T)n2;
+      obs_at(nd, L, j, 3) = (T)bd;
     }
   } else {
     // nominal position / thrust in T, the offsets of the cone and ball projections
@@ -857,7 +900,7 @@ __device__ __forceinline__ bool factor_invert_packed(const MS& MT);
 // diagonal holds 1/L_jj).  Returns false on a non-positive pivot.  Node N,
 // which has no control, is factored at the same size with an identity
 // control block and no coupling, so its state block is H_N exactly.
-template <class M, class T, bool AOS, int n, class MS>
+template <class M, class T, int AOS, int n, class MS>
 __device__ __forceinline__ bool node_factor(const Node<T, AOS>& nd, const MS& MT, const Layout& L, const Inst<T>& I,
                                             const NodeConst<M, T>& K, T rd, T rg) {
   constexpr int NX = M::NX;
@@ -881,7 +924,7 @@ __device__ __forceinline__ bool node_factor(const Node<T, AOS>& nd, const MS& MT
           if (r < 3 && c < 3) {
             T acc = T(0);
             #pragma unroll
-            for (int j = 0; j < I.nobs; ++j) acc += nd.at(L.oMd, ObsStride<T>::value * j + r) * nd.at(L.oMd, ObsStride<T>::value * j + c);
+            for (int j = 0; j < I.nobs; ++j) acc += obs_at(nd, L, j, r) * obs_at(nd, L, j, c);
             h += rg * acc;
           }
         } else {
@@ -992,7 +1035,7 @@ __device__ __forceinline__ void sym_solve(const MS& MT, const T* g, T* xi) {
 
 // H xi without forming H (A, B, the cost diagonals, the rho terms and the
 // mirror Gram terms), for the refinement residual g - H xi.
-template <class M, class T, bool AOS, int n, class MS>
+template <class M, class T, int AOS, int n, class MS>
 __device__ __forceinline__ void apply_H(const Node<T, AOS>& nd, const MS& MT, const Layout& L, const Inst<T>& I,
                                         const NodeConst<M, T>& K, T rd, T rg, const T* xi, T* out) {
   constexpr int NX = M::NX, NU = M::NU;
@@ -1032,7 +1075,7 @@ __device__ __forceinline__ void apply_H(const Node<T, AOS>& nd, const MS& MT, co
   }
   if constexpr (IsQuad<M>::value) {
     for (int j = 0; j < I.nobs; ++j) {
-      const T n0 = nd.at(L.oMd, ObsStride<T>::value * j), n1 = nd.at(L.oMd, ObsStride<T>::value * j + 1), n2 = nd.at(L.oMd, ObsStride<T>::value * j + 2);
+      const T n0 = obs_at(nd, L, j, 0), n1 = obs_at(nd, L, j, 1), n2 = obs_at(nd, L, j, 2);
       const T y = rg * (n0 * xi[0] + n1 * xi[1] + n2 * xi[2]);
       out[0] += n0 * y; out[1] += n1 * y; out[2] += n2 * y;
     }
@@ -1062,9 +1105,9 @@ __device__ __forceinline__ void apply_H(const Node<T, AOS>& nd, const MS& MT, co
 // the node record before it and written back after it (the register-resident
 // FP32 kernels of small models, where the structure of A leaves room);
 // otherwise references into the record.
-template <class M, class T, bool AOS, bool REG>
+template <class M, class T, int AOS, bool REG>
 struct NodeState;
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 struct NodeState<M, T, AOS, true> {
   mutable T zv[M::NX], lamv[M::NX], muv[M::NX], nuxv[M::NX], nuuv[M::NU];
   __device__ __forceinline__ T& z(int j) const { return zv[j]; }
@@ -1075,47 +1118,47 @@ struct NodeState<M, T, AOS, true> {
   __device__ __forceinline__ void load(const Node<T, AOS>& nd) {
 #pragma unroll
     for (int j = 0; j < M::NX; ++j) {
-      zv[j] = nd.at(Rec<M>::Z, j); lamv[j] = nd.at(Rec<M>::Lam, j); muv[j] = nd.at(Rec<M>::Mu, j);
-      nuxv[j] = nd.at(Rec<M>::Nux, j);
+      zv[j] = nd.at(Rec<M, AOS>::Z, j); lamv[j] = nd.at(Rec<M, AOS>::Lam, j); muv[j] = nd.at(Rec<M, AOS>::Mu, j);
+      nuxv[j] = nd.at(Rec<M, AOS>::Nux, j);
     }
 #pragma unroll
-    for (int j = 0; j < M::NU; ++j) nuuv[j] = nd.at(Rec<M>::Nuu, j);
+    for (int j = 0; j < M::NU; ++j) nuuv[j] = nd.at(Rec<M, AOS>::Nuu, j);
   }
   __device__ __forceinline__ void store(const Node<T, AOS>& nd) const {
 #pragma unroll
     for (int j = 0; j < M::NX; ++j) {
-      nd.at(Rec<M>::Z, j) = zv[j]; nd.at(Rec<M>::Lam, j) = lamv[j]; nd.at(Rec<M>::Mu, j) = muv[j];
-      nd.at(Rec<M>::Nux, j) = nuxv[j];
+      nd.at(Rec<M, AOS>::Z, j) = zv[j]; nd.at(Rec<M, AOS>::Lam, j) = lamv[j]; nd.at(Rec<M, AOS>::Mu, j) = muv[j];
+      nd.at(Rec<M, AOS>::Nux, j) = nuxv[j];
     }
 #pragma unroll
-    for (int j = 0; j < M::NU; ++j) nd.at(Rec<M>::Nuu, j) = nuuv[j];
+    for (int j = 0; j < M::NU; ++j) nd.at(Rec<M, AOS>::Nuu, j) = nuuv[j];
   }
 };
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 struct NodeState<M, T, AOS, false> {
   Node<T, AOS> nd;
-  __device__ __forceinline__ T& z(int j) const { return nd.at(Rec<M>::Z, j); }
-  __device__ __forceinline__ T& lam(int j) const { return nd.at(Rec<M>::Lam, j); }
-  __device__ __forceinline__ T& mu(int j) const { return nd.at(Rec<M>::Mu, j); }
-  __device__ __forceinline__ T& nux(int j) const { return nd.at(Rec<M>::Nux, j); }
-  __device__ __forceinline__ T& nuu(int j) const { return nd.at(Rec<M>::Nuu, j); }
+  __device__ __forceinline__ T& z(int j) const { return nd.at(Rec<M, AOS>::Z, j); }
+  __device__ __forceinline__ T& lam(int j) const { return nd.at(Rec<M, AOS>::Lam, j); }
+  __device__ __forceinline__ T& mu(int j) const { return nd.at(Rec<M, AOS>::Mu, j); }
+  __device__ __forceinline__ T& nux(int j) const { return nd.at(Rec<M, AOS>::Nux, j); }
+  __device__ __forceinline__ T& nuu(int j) const { return nd.at(Rec<M, AOS>::Nuu, j); }
   __device__ __forceinline__ void load(const Node<T, AOS>& n) { nd = n; }
   __device__ __forceinline__ void store(const Node<T, AOS>&) const {}
 };
 // REGS: the kernel variant leaves registers for the state (the 3-CTAs-per-SM
 // variant of the one-thread kernel does not).
-template <class M, class T, bool AOS, bool REGS = true>
+template <class M, class T, int AOS, bool REGS = true>
 using NodeStateFor = NodeState<M, T, AOS, REGS && AOS && SmallModel<M>::value && std::is_same<T, float>::value>;
 
 // Right-hand side g_i of Step 1 (stationarity of Eq. (3) in (x_i, u_i)).
-template <class M, class T, bool AOS, int n, class MS, class NS>
+template <class M, class T, int AOS, int n, class MS, class NS>
 __device__ __forceinline__ void node_rhs(const Node<T, AOS>& nd, const MS& MT, const Layout& L, const Inst<T>& I,
                                          const NodeConst<M, T>& K, const NS& S, T re, T rd, T rg, T* g) {
   constexpr int NX = M::NX, NU = M::NU;
   const int i = nd.i;
 #pragma unroll
   for (int j = 0; j < NX; ++j) {
-    T v = -K.q[j] + rg * nd.at(Rec<M>::Xh, j) - S.nux(j);
+    T v = -K.q[j] + rg * nd.at(Rec<M, AOS>::Xh, j) - S.nux(j);
     if (i > 0) v += re * S.z(j) - S.lam(j);
     g[j] = v;
   }
@@ -1124,7 +1167,7 @@ __device__ __forceinline__ void node_rhs(const Node<T, AOS>& nd, const MS& MT, c
     // w_i = mu_{i+1} + rho_dyn (z_{i+1} - c_i); node i+1 publishes mu + rho_dyn z
     T w[NX];
 #pragma unroll
-    for (int k = 0; k < NX; ++k) w[k] = nd.nb(Rec<M>::Ex2, k, i + 1) - rd * nd.at(Rec<M>::C, k);
+    for (int k = 0; k < NX; ++k) w[k] = nd.nb(Rec<M, AOS>::Ex2, k, i + 1) - rd * nd.at(Rec<M, AOS>::C, k);
 #pragma unroll
     for (int j = 0; j < NX; ++j) {
       T acc = T(0);
@@ -1137,7 +1180,7 @@ __device__ __forceinline__ void node_rhs(const Node<T, AOS>& nd, const MS& MT, c
       T acc = T(0);
 #pragma unroll
       for (int k = 0; k < NX; ++k) acc += MT.B(k, j) * w[k];
-      g[NX + j] = -K.q[NX + j] + acc + rg * nd.at(Rec<M>::Uh, j) - S.nuu(j);
+      g[NX + j] = -K.q[NX + j] + acc + rg * nd.at(Rec<M, AOS>::Uh, j) - S.nuu(j);
     }
    } else {
 #pragma unroll
@@ -1147,9 +1190,9 @@ __device__ __forceinline__ void node_rhs(const Node<T, AOS>& nd, const MS& MT, c
   if constexpr (IsQuad<M>::value) {
     for (int j = 0; j < I.nobs; ++j) {
       const T a = rg * nd.at(L.oS, j) - nd.at(L.oNus, j);
-      g[0] += nd.at(L.oMd, ObsStride<T>::value * j) * a;
-      g[1] += nd.at(L.oMd, ObsStride<T>::value * j + 1) * a;
-      g[2] += nd.at(L.oMd, ObsStride<T>::value * j + 2) * a;
+      g[0] += obs_at(nd, L, j, 0) * a;
+      g[1] += obs_at(nd, L, j, 1) * a;
+      g[2] += obs_at(nd, L, j, 2) * a;
     }
   } else {
     constexpr int RC = IsMars14<M>::value ? 1 : 0;
@@ -1180,14 +1223,14 @@ __device__ __forceinline__ void node_rhs(const Node<T, AOS>& nd, const MS& MT, c
 // sets; `sv` accumulates rho_geo G^T (s_new - s_old) for the dual residual,
 // `rp` the squared primal residual |G xi - s|^2.  Initialisation (reseed)
 // mode projects G xi alone and leaves the duals untouched.
-template <class M, class T, bool AOS, int n>
+template <class M, class T, int AOS, int n>
 __device__ __forceinline__ void node_mirrors(const Node<T, AOS>& nd, const Layout& L, const Inst<T>& I,
                                              T rg, T irg, const T* xi, bool reseed, bool want_res, T* sv, typename WideOf<T>::type& rp) {
   constexpr int NX = M::NX;
   if constexpr (IsQuad<M>::value) {
     for (int j = 0; j < I.nobs; ++j) {
-      const T n0 = nd.at(L.oMd, ObsStride<T>::value * j), n1 = nd.at(L.oMd, ObsStride<T>::value * j + 1), n2 = nd.at(L.oMd, ObsStride<T>::value * j + 2);
-      const T bd = nd.at(L.oMd, ObsStride<T>::value * j + 3);
+      const T n0 = obs_at(nd, L, j, 0), n1 = obs_at(nd, L, j, 1), n2 = obs_at(nd, L, j, 2);
+      const T bd = obs_at(nd, L, j, 3);
       const T y = n0 * xi[0] + n1 * xi[1] + n2 * xi[2];
       if (reseed) { nd.at(L.oS, j) = maxv(bd, y); continue; }
       const T so = nd.at(L.oS, j);
@@ -1300,14 +1343,14 @@ __device__ __forceinline__ void node_mirrors(const Node<T, AOS>& nd, const Layou
 }
 
 // Mirror initialisation / re-seeding from (x-hat, u-hat) in deviations.
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 __device__ void node_reseed(const Node<T, AOS>& nd, const Layout& L, const Inst<T>& I) {
   constexpr int NX = M::NX, NU = M::NU;
   T xi[NX + NU], sv[NX + NU];
   typename WideOf<T>::type rp{};
-  for (int j = 0; j < NX; ++j) xi[j] = nd.at(Rec<M>::Xh, j);
+  for (int j = 0; j < NX; ++j) xi[j] = nd.at(Rec<M, AOS>::Xh, j);
   if (nd.i < nd.N) {
-    for (int j = 0; j < NU; ++j) xi[NX + j] = nd.at(Rec<M>::Uh, j);
+    for (int j = 0; j < NU; ++j) xi[NX + j] = nd.at(Rec<M, AOS>::Uh, j);
     node_mirrors<M, T, AOS, NX + NU>(nd, L, I, T(1), T(1), xi, true, false, sv, rp);
   } else {
     node_mirrors<M, T, AOS, NX>(nd, L, I, T(1), T(1), xi, true, false, sv, rp);
@@ -1327,7 +1370,7 @@ __device__ void node_reseed(const Node<T, AOS>& nd, const Layout& L, const Inst<
 // group all-reduce combines them, and each CTA sets u-hat_0 to the projection
 // onto {equal u_0} intersected with every box, i.e. the average clamped to the
 // common box, before its Step 4.
-template <class M, class T, bool AOS, bool REFINE, bool LAST, bool GROUP, class MS, class NS>
+template <class M, class T, int AOS, bool REFINE, bool LAST, bool GROUP, class MS, class NS>
 __device__ __forceinline__ void admm_iteration(const Node<T, AOS>& nd, const MS& MT, const Layout& L, const Inst<T>& I,
                                                const NodeConst<M, T>& K, bool active, T re, T rd, T rg,
                                                T irg, T ired, typename WideOf<T>::type& rp,
@@ -1360,19 +1403,19 @@ __device__ __forceinline__ void admm_iteration(const Node<T, AOS>& nd, const MS&
         // linearised propagation d_dyn,i = A x + B u + c_i, published to node i+1
 #pragma unroll
         for (int r = 0; r < NX; ++r) {
-          T acc = nd.at(Rec<M>::C, r);
+          T acc = nd.at(Rec<M, AOS>::C, r);
 #pragma unroll
           for (int c = 0; c < NX; ++c) acc_A(acc, MT, r, c, x[c]);
 #pragma unroll
           for (int c = 0; c < NU; ++c) acc += MT.B(r, c) * x[NX + c];
-          nd.at(Rec<M>::Ex1, r) = acc;
+          nd.at(Rec<M, AOS>::Ex1, r) = acc;
         }
       }
 #pragma unroll
-      for (int j = 0; j < NX; ++j) nd.at(Rec<M>::X, j) = x[j];
+      for (int j = 0; j < NX; ++j) nd.at(Rec<M, AOS>::X, j) = x[j];
       if (i < N) {
 #pragma unroll
-        for (int j = 0; j < NU; ++j) nd.at(Rec<M>::U, j) = x[NX + j];
+        for (int j = 0; j < NU; ++j) nd.at(Rec<M, AOS>::U, j) = x[NX + j];
       }
     }
     // Steps 2 and 3 use disjoint variables (z, lambda, mu | x-hat, u-hat, nu,
@@ -1391,9 +1434,9 @@ __device__ __forceinline__ void admm_iteration(const Node<T, AOS>& nd, const MS&
 #pragma unroll
       for (int j = 0; j < NX; ++j) {
         const T nux = S.nux(j);
-        const T xh = clampv(x[j] + nux * irg, nd.at(Rec<M>::Xlo, j), nd.at(Rec<M>::Xhi, j));
-        if (last) { sv[j] += rg * (xh - nd.at(Rec<M>::Xh, j)); acc_sq_diff(rp, x[j], xh); }
-        nd.at(Rec<M>::Xh, j) = xh;
+        const T xh = clampv(x[j] + nux * irg, nd.at(Rec<M, AOS>::Xlo, j), nd.at(Rec<M, AOS>::Xhi, j));
+        if (last) { sv[j] += rg * (xh - nd.at(Rec<M, AOS>::Xh, j)); acc_sq_diff(rp, x[j], xh); }
+        nd.at(Rec<M, AOS>::Xh, j) = xh;
         S.nux(j) = nux + rg * (x[j] - xh);
       }
       if (i < N) {
@@ -1402,17 +1445,17 @@ __device__ __forceinline__ void admm_iteration(const Node<T, AOS>& nd, const MS&
           const T nuu = S.nuu(j);
           if constexpr (GROUP) {
             if (i == 0) {   // sum of arguments | max of lower bounds | max of -upper bounds
-              const double ub = wide_to_double(nd.dat(Rec<M>::Ubar, j));
+              const double ub = wide_to_double(nd.dat(Rec<M, AOS>::Ubar, j));
               double* m = G->mine[X.epoch & 1];
               m[j] = ub + (double)(x[NX + j] + nuu * irg);
-              m[NU + j] = ub + (double)nd.at(Rec<M>::Ulo, j);
-              m[2 * NU + j] = -(ub + (double)nd.at(Rec<M>::Uhi, j));
+              m[NU + j] = ub + (double)nd.at(Rec<M, AOS>::Ulo, j);
+              m[2 * NU + j] = -(ub + (double)nd.at(Rec<M, AOS>::Uhi, j));
               continue;
             }
           }
-          const T uh = clampv(x[NX + j] + nuu * irg, nd.at(Rec<M>::Ulo, j), nd.at(Rec<M>::Uhi, j));
-          if (last) { sv[NX + j] += rg * (uh - nd.at(Rec<M>::Uh, j)); acc_sq_diff(rp, x[NX + j], uh); }
-          nd.at(Rec<M>::Uh, j) = uh;
+          const T uh = clampv(x[NX + j] + nuu * irg, nd.at(Rec<M, AOS>::Ulo, j), nd.at(Rec<M, AOS>::Uhi, j));
+          if (last) { sv[NX + j] += rg * (uh - nd.at(Rec<M, AOS>::Uh, j)); acc_sq_diff(rp, x[NX + j], uh); }
+          nd.at(Rec<M, AOS>::Uh, j) = uh;
           S.nuu(j) = nuu + rg * (x[NX + j] - uh);
         }
       }
@@ -1424,7 +1467,7 @@ __device__ __forceinline__ void admm_iteration(const Node<T, AOS>& nd, const MS&
       if (i >= 1) {
 #pragma unroll
         for (int j = 0; j < NX; ++j) {
-          const T dd = nd.nb(Rec<M>::Ex1, j, i - 1);
+          const T dd = nd.nb(Rec<M, AOS>::Ex1, j, i - 1);
           const T zo = S.z(j);
           const T lam = S.lam(j), mu = S.mu(j);
           const T z = (re * x[j] + lam + rd * dd - mu) * ired;
@@ -1448,10 +1491,10 @@ __device__ __forceinline__ void admm_iteration(const Node<T, AOS>& nd, const MS&
         for (int j = 0; j < NU; ++j) {
           const double v = fmin(fmax(tot[j] / (double)P.group, tot[NU + j]), -tot[2 * NU + j]);
           G->u0[j] = v;
-          const T uh = (T)(v - wide_to_double(nd.dat(Rec<M>::Ubar, j)));
+          const T uh = (T)(v - wide_to_double(nd.dat(Rec<M, AOS>::Ubar, j)));
           const T nuu = S.nuu(j);
-          if (last) { sv[NX + j] += rg * (uh - nd.at(Rec<M>::Uh, j)); acc_sq_diff(rp, x[NX + j], uh); }
-          nd.at(Rec<M>::Uh, j) = uh;
+          if (last) { sv[NX + j] += rg * (uh - nd.at(Rec<M, AOS>::Uh, j)); acc_sq_diff(rp, x[NX + j], uh); }
+          nd.at(Rec<M, AOS>::Uh, j) = uh;
           S.nuu(j) = nuu + rg * (x[NX + j] - uh);
         }
       }
@@ -1461,7 +1504,7 @@ __device__ __forceinline__ void admm_iteration(const Node<T, AOS>& nd, const MS&
       __syncthreads();
       if (active && i >= 1) {
 #pragma unroll
-        for (int j = 0; j < NX; ++j) nd.at(Rec<M>::Ex1, j) = rd * dz[j];
+        for (int j = 0; j < NX; ++j) nd.at(Rec<M, AOS>::Ex1, j) = rd * dz[j];
       }
       __syncthreads();
       if (active) {
@@ -1471,14 +1514,14 @@ __device__ __forceinline__ void admm_iteration(const Node<T, AOS>& nd, const MS&
             T acc = T(0);
 #pragma unroll
             for (int k = 0; k < NX; ++k)
-              if (MS::akind(k, j)) acc_A(acc, MT, k, j, nd.nb(Rec<M>::Ex1, k, i + 1));
+              if (MS::akind(k, j)) acc_A(acc, MT, k, j, nd.nb(Rec<M, AOS>::Ex1, k, i + 1));
             sv[j] += acc;
           }
 #pragma unroll
           for (int j = 0; j < NU; ++j) {
             T acc = T(0);
 #pragma unroll
-            for (int k = 0; k < NX; ++k) acc += MT.B(k, j) * nd.nb(Rec<M>::Ex1, k, i + 1);
+            for (int k = 0; k < NX; ++k) acc += MT.B(k, j) * nd.nb(Rec<M, AOS>::Ex1, k, i + 1);
             sv[NX + j] += acc;
           }
         }
@@ -1489,7 +1532,7 @@ __device__ __forceinline__ void admm_iteration(const Node<T, AOS>& nd, const MS&
     }
     if (active && i >= 1) {
 #pragma unroll
-      for (int j = 0; j < NX; ++j) nd.at(Rec<M>::Ex2, j) = S.mu(j) + rd * S.z(j);
+      for (int j = 0; j < NX; ++j) nd.at(Rec<M, AOS>::Ex2, j) = S.mu(j) + rd * S.z(j);
     }
     __syncthreads();
   }
@@ -1497,7 +1540,7 @@ __device__ __forceinline__ void admm_iteration(const Node<T, AOS>& nd, const MS&
 
 // `iters` iterations of Steps 1-4; the primal and dual residuals of the last
 // one are returned, squared, in res[0..1].
-template <class M, class T, bool AOS, bool REFINE, bool GROUP = false, bool REGS = true, class MS>
+template <class M, class T, int AOS, bool REFINE, bool GROUP = false, bool REGS = true, class MS>
 __device__ __forceinline__ void admm_iterations(const Node<T, AOS>& nd, const MS& MT, const Layout& L, const Inst<T>& I,
                                 const NodeConst<M, T>& K, bool active, T re, T rd, T rg, int iters,
                                 InstShared& sh, double* res, GroupShared* G, GroupX& X, const ProblemDev& P) {
@@ -1514,29 +1557,29 @@ __device__ __forceinline__ void admm_iterations(const Node<T, AOS>& nd, const MS
 }
 
 // Publish mu_i + rho_dyn z_i before the first Step 1.
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 __device__ __forceinline__ void publish_ex2(const Node<T, AOS>& nd, const Layout& L, bool active, T rd) {
   if (active && nd.i >= 1)
-    for (int j = 0; j < M::NX; ++j) nd.at(Rec<M>::Ex2, j) = nd.at(Rec<M>::Mu, j) + rd * nd.at(Rec<M>::Z, j);
+    for (int j = 0; j < M::NX; ++j) nd.at(Rec<M, AOS>::Ex2, j) = nd.at(Rec<M, AOS>::Mu, j) + rd * nd.at(Rec<M, AOS>::Z, j);
 }
 
 // Cold start: x = x-hat = z = nominal, u = u-hat = nominal, zero duals.
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 __device__ void node_cold_start(const Node<T, AOS>& nd, const Layout& L) {
   for (int j = 0; j < M::NX; ++j) {
-    nd.at(Rec<M>::X, j) = T(0); nd.at(Rec<M>::Z, j) = T(0); nd.at(Rec<M>::Lam, j) = T(0); nd.at(Rec<M>::Mu, j) = T(0);
-    nd.at(Rec<M>::Xh, j) = T(0); nd.at(Rec<M>::Nux, j) = T(0);
+    nd.at(Rec<M, AOS>::X, j) = T(0); nd.at(Rec<M, AOS>::Z, j) = T(0); nd.at(Rec<M, AOS>::Lam, j) = T(0); nd.at(Rec<M, AOS>::Mu, j) = T(0);
+    nd.at(Rec<M, AOS>::Xh, j) = T(0); nd.at(Rec<M, AOS>::Nux, j) = T(0);
   }
-  for (int j = 0; j < M::NU; ++j) { nd.at(Rec<M>::U, j) = T(0); nd.at(Rec<M>::Uh, j) = T(0); nd.at(Rec<M>::Nuu, j) = T(0); }
+  for (int j = 0; j < M::NU; ++j) { nd.at(Rec<M, AOS>::U, j) = T(0); nd.at(Rec<M, AOS>::Uh, j) = T(0); nd.at(Rec<M, AOS>::Nuu, j) = T(0); }
   for (int j = 0; j < L.MS; ++j) { nd.at(L.oS, j) = T(0); nd.at(L.oNus, j) = T(0); }
 }
 
 // The ADMM state a solve starts from: cold (x = x-hat = z = nominal, zero
 // duals), or -- warm[b] -- the absolute state in state_abs (a kept state of an
 // earlier solve), taken relative to this solve's nominal.
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 __device__ void node_import(const Node<T, AOS>& nd, const Layout& L, const ProblemDev& P, int b, const double* in);
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 __device__ __forceinline__ void node_start(const Node<T, AOS>& nd, const Layout& L, const ProblemDev& P, int b) {
   if (P.warm && P.warm[b]) node_import<M, T, AOS>(nd, L, P, b, P.state_abs + P.soff[b]);
   else node_cold_start<M, T, AOS>(nd, L);
@@ -1544,7 +1587,7 @@ __device__ __forceinline__ void node_start(const Node<T, AOS>& nd, const Layout&
 
 // ------------------------------------------------------------------ absolute state in/out
 // Flat per-instance order: x, u, z, lam, mu, xh, uh, nux, nuu, s[(N+1)][MB][3], nus[...].
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 __device__ void node_export(const Node<T, AOS>& nd, const Layout& L, const ProblemDev& P, int b, double* out) {
   constexpr int NX = M::NX, NU = M::NU;
   const int i = nd.i, N = nd.N;
@@ -1556,20 +1599,20 @@ __device__ void node_export(const Node<T, AOS>& nd, const Layout& L, const Probl
   double* pnuu = pnux + nX;   double* ps = pnuu + nU;
   double* pnus = ps + (long long)(N + 1) * L.MB * 3;
   for (int j = 0; j < NX; ++j) {
-    const double xb = wide_to_double(nd.dat(Rec<M>::Xbar, j));
-    px[i * NX + j] = xb + (double)nd.at(Rec<M>::X, j);
-    pz[i * NX + j] = (i >= 1) ? xb + (double)nd.at(Rec<M>::Z, j) : 0.0;
-    plam[i * NX + j] = (i >= 1) ? (double)nd.at(Rec<M>::Lam, j) : 0.0;
-    pmu[i * NX + j] = (i >= 1) ? (double)nd.at(Rec<M>::Mu, j) : 0.0;
-    pxh[i * NX + j] = xb + (double)nd.at(Rec<M>::Xh, j);
-    pnux[i * NX + j] = (double)nd.at(Rec<M>::Nux, j);
+    const double xb = wide_to_double(nd.dat(Rec<M, AOS>::Xbar, j));
+    px[i * NX + j] = xb + (double)nd.at(Rec<M, AOS>::X, j);
+    pz[i * NX + j] = (i >= 1) ? xb + (double)nd.at(Rec<M, AOS>::Z, j) : 0.0;
+    plam[i * NX + j] = (i >= 1) ? (double)nd.at(Rec<M, AOS>::Lam, j) : 0.0;
+    pmu[i * NX + j] = (i >= 1) ? (double)nd.at(Rec<M, AOS>::Mu, j) : 0.0;
+    pxh[i * NX + j] = xb + (double)nd.at(Rec<M, AOS>::Xh, j);
+    pnux[i * NX + j] = (double)nd.at(Rec<M, AOS>::Nux, j);
   }
   if (i < N)
     for (int j = 0; j < NU; ++j) {
-      const double ub = wide_to_double(nd.dat(Rec<M>::Ubar, j));
-      pu[i * NU + j] = ub + (double)nd.at(Rec<M>::U, j);
-      puh[i * NU + j] = ub + (double)nd.at(Rec<M>::Uh, j);
-      pnuu[i * NU + j] = (double)nd.at(Rec<M>::Nuu, j);
+      const double ub = wide_to_double(nd.dat(Rec<M, AOS>::Ubar, j));
+      pu[i * NU + j] = ub + (double)nd.at(Rec<M, AOS>::U, j);
+      puh[i * NU + j] = ub + (double)nd.at(Rec<M, AOS>::Uh, j);
+      pnuu[i * NU + j] = (double)nd.at(Rec<M, AOS>::Nuu, j);
     }
   double* si = ps + (long long)i * L.MB * 3;
   double* ni = pnus + (long long)i * L.MB * 3;
@@ -1577,7 +1620,7 @@ __device__ void node_export(const Node<T, AOS>& nd, const Layout& L, const Probl
   if constexpr (IsQuad<M>::value) {
     for (int j = 0; j < nobs_of(P, b); ++j) {
       double np = 0.0;
-      for (int k = 0; k < 3; ++k) np += (double)nd.at(L.oMd, ObsStride<T>::value * j + k) * wide_to_double(nd.dat(Rec<M>::Xbar, k));
+      for (int k = 0; k < 3; ++k) np += (double)obs_at(nd, L, j, k) * wide_to_double(nd.dat(Rec<M, AOS>::Xbar, k));
       si[3 * j] = (double)nd.at(L.oS, j) + np;
       ni[3 * j] = (double)nd.at(L.oNus, j);
     }
@@ -1585,45 +1628,45 @@ __device__ void node_export(const Node<T, AOS>& nd, const Layout& L, const Probl
     // blocks as the problem's sets: glide cone, tilt, body rate, thrust ball, thrust lower bound, gimbal
     const double* st = &P.sets[b * UCN_SET_PARAMS];
     if (st[2] > 0.0)
-      for (int k = 0; k < 3; ++k) { si[k] = (double)nd.at(L.oS, k) + wide_to_double(nd.dat(Rec<M>::Xbar, 1 + k)); ni[k] = (double)nd.at(L.oNus, k); }
+      for (int k = 0; k < 3; ++k) { si[k] = (double)nd.at(L.oS, k) + wide_to_double(nd.dat(Rec<M, AOS>::Xbar, 1 + k)); ni[k] = (double)nd.at(L.oNus, k); }
     if (st[4] > 0.0)
       for (int k = 0; k < 2; ++k) {
-        si[3 + k] = (double)nd.at(L.oS, M14::S_TILT + k) + wide_to_double(nd.dat(Rec<M>::Xbar, 9 + k));
+        si[3 + k] = (double)nd.at(L.oS, M14::S_TILT + k) + wide_to_double(nd.dat(Rec<M, AOS>::Xbar, 9 + k));
         ni[3 + k] = (double)nd.at(L.oNus, M14::S_TILT + k);
       }
     if (st[5] > 0.0)
       for (int k = 0; k < 3; ++k) {
-        si[6 + k] = (double)nd.at(L.oS, M14::S_W + k) + wide_to_double(nd.dat(Rec<M>::Xbar, 11 + k));
+        si[6 + k] = (double)nd.at(L.oS, M14::S_W + k) + wide_to_double(nd.dat(Rec<M, AOS>::Xbar, 11 + k));
         ni[6 + k] = (double)nd.at(L.oNus, M14::S_W + k);
       }
     if (i < N && st[1] > 0.0)
-      for (int k = 0; k < 3; ++k) { si[9 + k] = (double)nd.at(L.oS, 3 + k) + wide_to_double(nd.dat(Rec<M>::Ubar, k)); ni[9 + k] = (double)nd.at(L.oNus, 3 + k); }
+      for (int k = 0; k < 3; ++k) { si[9 + k] = (double)nd.at(L.oS, 3 + k) + wide_to_double(nd.dat(Rec<M, AOS>::Ubar, k)); ni[9 + k] = (double)nd.at(L.oNus, 3 + k); }
     if (i < N && st[0] > 0.0) {
       double np = 0.0;
-      for (int k = 0; k < 3; ++k) np += (double)nd.at(L.oMd, k) * wide_to_double(nd.dat(Rec<M>::Ubar, k));
+      for (int k = 0; k < 3; ++k) np += (double)nd.at(L.oMd, k) * wide_to_double(nd.dat(Rec<M, AOS>::Ubar, k));
       si[12] = (double)nd.at(L.oS, 6) + np;
       ni[12] = (double)nd.at(L.oNus, 6);
     }
     if (i < N && st[3] > 0.0)
       for (int k = 0; k < 3; ++k) {
-        si[15 + k] = (double)nd.at(L.oS, M14::S_GIM + k) + wide_to_double(nd.dat(Rec<M>::Ubar, k));
+        si[15 + k] = (double)nd.at(L.oS, M14::S_GIM + k) + wide_to_double(nd.dat(Rec<M, AOS>::Ubar, k));
         ni[15 + k] = (double)nd.at(L.oNus, M14::S_GIM + k);
       }
   } else {
     if (P.sets[b * UCN_SET_PARAMS + 2] > 0.0)
-      for (int k = 0; k < 3; ++k) { si[k] = (double)nd.at(L.oS, k) + wide_to_double(nd.dat(Rec<M>::Xbar, k)); ni[k] = (double)nd.at(L.oNus, k); }
+      for (int k = 0; k < 3; ++k) { si[k] = (double)nd.at(L.oS, k) + wide_to_double(nd.dat(Rec<M, AOS>::Xbar, k)); ni[k] = (double)nd.at(L.oNus, k); }
     if (i < N && P.sets[b * UCN_SET_PARAMS + 1] > 0.0)
-      for (int k = 0; k < 3; ++k) { si[3 + k] = (double)nd.at(L.oS, 3 + k) + wide_to_double(nd.dat(Rec<M>::Ubar, k)); ni[3 + k] = (double)nd.at(L.oNus, 3 + k); }
+      for (int k = 0; k < 3; ++k) { si[3 + k] = (double)nd.at(L.oS, 3 + k) + wide_to_double(nd.dat(Rec<M, AOS>::Ubar, k)); ni[3 + k] = (double)nd.at(L.oNus, 3 + k); }
     if (i < N && P.sets[b * UCN_SET_PARAMS + 0] > 0.0) {
       double np = 0.0;
-      for (int k = 0; k < 3; ++k) np += (double)nd.at(L.oMd, k) * wide_to_double(nd.dat(Rec<M>::Ubar, k));
+      for (int k = 0; k < 3; ++k) np += (double)nd.at(L.oMd, k) * wide_to_double(nd.dat(Rec<M, AOS>::Ubar, k));
       si[6] = (double)nd.at(L.oS, 6) + np;
       ni[6] = (double)nd.at(L.oNus, 6);
     }
   }
 }
 
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 __device__ void node_import(const Node<T, AOS>& nd, const Layout& L, const ProblemDev& P, int b, const double* in) {
   constexpr int NX = M::NX, NU = M::NU;
   const int i = nd.i, N = nd.N;
@@ -1635,19 +1678,19 @@ __device__ void node_import(const Node<T, AOS>& nd, const Layout& L, const Probl
   const double* pnuu = pnux + nX; const double* ps = pnuu + nU;
   const double* pnus = ps + (long long)(N + 1) * L.MB * 3;
   for (int j = 0; j < NX; ++j) {
-    const double xb = wide_to_double(nd.dat(Rec<M>::Xbar, j));
-    nd.at(Rec<M>::X, j) = (T)(px[i * NX + j] - xb);
-    nd.at(Rec<M>::Z, j) = (i >= 1) ? (T)(pz[i * NX + j] - xb) : T(0);
-    nd.at(Rec<M>::Lam, j) = (T)plam[i * NX + j];
-    nd.at(Rec<M>::Mu, j) = (T)pmu[i * NX + j];
-    nd.at(Rec<M>::Xh, j) = (T)(pxh[i * NX + j] - xb);
-    nd.at(Rec<M>::Nux, j) = (T)pnux[i * NX + j];
+    const double xb = wide_to_double(nd.dat(Rec<M, AOS>::Xbar, j));
+    nd.at(Rec<M, AOS>::X, j) = (T)(px[i * NX + j] - xb);
+    nd.at(Rec<M, AOS>::Z, j) = (i >= 1) ? (T)(pz[i * NX + j] - xb) : T(0);
+    nd.at(Rec<M, AOS>::Lam, j) = (T)plam[i * NX + j];
+    nd.at(Rec<M, AOS>::Mu, j) = (T)pmu[i * NX + j];
+    nd.at(Rec<M, AOS>::Xh, j) = (T)(pxh[i * NX + j] - xb);
+    nd.at(Rec<M, AOS>::Nux, j) = (T)pnux[i * NX + j];
   }
   for (int j = 0; j < NU; ++j) {
-    const double ub = (i < N) ? wide_to_double(nd.dat(Rec<M>::Ubar, j)) : 0.0;
-    nd.at(Rec<M>::U, j) = (i < N) ? (T)(pu[i * NU + j] - ub) : T(0);
-    nd.at(Rec<M>::Uh, j) = (i < N) ? (T)(puh[i * NU + j] - ub) : T(0);
-    nd.at(Rec<M>::Nuu, j) = (i < N) ? (T)pnuu[i * NU + j] : T(0);
+    const double ub = (i < N) ? wide_to_double(nd.dat(Rec<M, AOS>::Ubar, j)) : 0.0;
+    nd.at(Rec<M, AOS>::U, j) = (i < N) ? (T)(pu[i * NU + j] - ub) : T(0);
+    nd.at(Rec<M, AOS>::Uh, j) = (i < N) ? (T)(puh[i * NU + j] - ub) : T(0);
+    nd.at(Rec<M, AOS>::Nuu, j) = (i < N) ? (T)pnuu[i * NU + j] : T(0);
   }
   for (int j = 0; j < L.MS; ++j) { nd.at(L.oS, j) = T(0); nd.at(L.oNus, j) = T(0); }
   const double* si = ps + (long long)i * L.MB * 3;
@@ -1655,38 +1698,38 @@ __device__ void node_import(const Node<T, AOS>& nd, const Layout& L, const Probl
   if constexpr (IsQuad<M>::value) {
     for (int j = 0; j < nobs_of(P, b); ++j) {
       double np = 0.0;
-      for (int k = 0; k < 3; ++k) np += (double)nd.at(L.oMd, ObsStride<T>::value * j + k) * wide_to_double(nd.dat(Rec<M>::Xbar, k));
+      for (int k = 0; k < 3; ++k) np += (double)obs_at(nd, L, j, k) * wide_to_double(nd.dat(Rec<M, AOS>::Xbar, k));
       nd.at(L.oS, j) = (T)(si[3 * j] - np);
       nd.at(L.oNus, j) = (T)ni[3 * j];
     }
   } else if constexpr (IsMars14<M>::value) {
     // blocks as exported: glide cone, tilt, body rate, thrust ball, thrust lower bound, gimbal
-    for (int k = 0; k < 3; ++k) { nd.at(L.oS, k) = (T)(si[k] - wide_to_double(nd.dat(Rec<M>::Xbar, 1 + k))); nd.at(L.oNus, k) = (T)ni[k]; }
+    for (int k = 0; k < 3; ++k) { nd.at(L.oS, k) = (T)(si[k] - wide_to_double(nd.dat(Rec<M, AOS>::Xbar, 1 + k))); nd.at(L.oNus, k) = (T)ni[k]; }
     for (int k = 0; k < 2; ++k) {
-      nd.at(L.oS, M14::S_TILT + k) = (T)(si[3 + k] - wide_to_double(nd.dat(Rec<M>::Xbar, 9 + k)));
+      nd.at(L.oS, M14::S_TILT + k) = (T)(si[3 + k] - wide_to_double(nd.dat(Rec<M, AOS>::Xbar, 9 + k)));
       nd.at(L.oNus, M14::S_TILT + k) = (T)ni[3 + k];
     }
     for (int k = 0; k < 3; ++k) {
-      nd.at(L.oS, M14::S_W + k) = (T)(si[6 + k] - wide_to_double(nd.dat(Rec<M>::Xbar, 11 + k)));
+      nd.at(L.oS, M14::S_W + k) = (T)(si[6 + k] - wide_to_double(nd.dat(Rec<M, AOS>::Xbar, 11 + k)));
       nd.at(L.oNus, M14::S_W + k) = (T)ni[6 + k];
     }
     if (i < N) {
-      for (int k = 0; k < 3; ++k) { nd.at(L.oS, 3 + k) = (T)(si[9 + k] - wide_to_double(nd.dat(Rec<M>::Ubar, k))); nd.at(L.oNus, 3 + k) = (T)ni[9 + k]; }
+      for (int k = 0; k < 3; ++k) { nd.at(L.oS, 3 + k) = (T)(si[9 + k] - wide_to_double(nd.dat(Rec<M, AOS>::Ubar, k))); nd.at(L.oNus, 3 + k) = (T)ni[9 + k]; }
       double np = 0.0;
-      for (int k = 0; k < 3; ++k) np += (double)nd.at(L.oMd, k) * wide_to_double(nd.dat(Rec<M>::Ubar, k));
+      for (int k = 0; k < 3; ++k) np += (double)nd.at(L.oMd, k) * wide_to_double(nd.dat(Rec<M, AOS>::Ubar, k));
       nd.at(L.oS, 6) = (T)(si[12] - np);
       nd.at(L.oNus, 6) = (T)ni[12];
       for (int k = 0; k < 3; ++k) {
-        nd.at(L.oS, M14::S_GIM + k) = (T)(si[15 + k] - wide_to_double(nd.dat(Rec<M>::Ubar, k)));
+        nd.at(L.oS, M14::S_GIM + k) = (T)(si[15 + k] - wide_to_double(nd.dat(Rec<M, AOS>::Ubar, k)));
         nd.at(L.oNus, M14::S_GIM + k) = (T)ni[15 + k];
       }
     }
   } else {
-    for (int k = 0; k < 3; ++k) { nd.at(L.oS, k) = (T)(si[k] - wide_to_double(nd.dat(Rec<M>::Xbar, k))); nd.at(L.oNus, k) = (T)ni[k]; }
+    for (int k = 0; k < 3; ++k) { nd.at(L.oS, k) = (T)(si[k] - wide_to_double(nd.dat(Rec<M, AOS>::Xbar, k))); nd.at(L.oNus, k) = (T)ni[k]; }
     if (i < N) {
-      for (int k = 0; k < 3; ++k) { nd.at(L.oS, 3 + k) = (T)(si[3 + k] - wide_to_double(nd.dat(Rec<M>::Ubar, k))); nd.at(L.oNus, 3 + k) = (T)ni[3 + k]; }
+      for (int k = 0; k < 3; ++k) { nd.at(L.oS, 3 + k) = (T)(si[3 + k] - wide_to_double(nd.dat(Rec<M, AOS>::Ubar, k))); nd.at(L.oNus, 3 + k) = (T)ni[3 + k]; }
       double np = 0.0;
-      for (int k = 0; k < 3; ++k) np += (double)nd.at(L.oMd, k) * wide_to_double(nd.dat(Rec<M>::Ubar, k));
+      for (int k = 0; k < 3; ++k) np += (double)nd.at(L.oMd, k) * wide_to_double(nd.dat(Rec<M, AOS>::Ubar, k));
       nd.at(L.oS, 6) = (T)(si[6] - np);
       nd.at(L.oNus, 6) = (T)ni[6];
     }
@@ -1695,27 +1738,27 @@ __device__ void node_import(const Node<T, AOS>& nd, const Layout& L, const Probl
 
 // After an accepted step the nominal moves by (dxh, duh): express the mirror
 // variables in deviations from the new nominal (same absolute values).
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 __device__ void node_rebase_mirrors(const Node<T, AOS>& nd, const Layout& L, const ProblemDev& P, int b) {
   if constexpr (IsQuad<M>::value) {
     for (int j = 0; j < nobs_of(P, b); ++j) {
       T y = T(0);
-      for (int k = 0; k < 3; ++k) y += nd.at(L.oMd, ObsStride<T>::value * j + k) * nd.at(Rec<M>::Xh, k);
+      for (int k = 0; k < 3; ++k) y += obs_at(nd, L, j, k) * nd.at(Rec<M, AOS>::Xh, k);
       nd.at(L.oS, j) -= y;
     }
   } else {
     constexpr int RC = IsMars14<M>::value ? 1 : 0;
-    for (int k = 0; k < 3; ++k) nd.at(L.oS, k) -= nd.at(Rec<M>::Xh, RC + k);
+    for (int k = 0; k < 3; ++k) nd.at(L.oS, k) -= nd.at(Rec<M, AOS>::Xh, RC + k);
     if constexpr (IsMars14<M>::value) {
-      for (int k = 0; k < 2; ++k) nd.at(L.oS, M14::S_TILT + k) -= nd.at(Rec<M>::Xh, 9 + k);
-      for (int k = 0; k < 3; ++k) nd.at(L.oS, M14::S_W + k) -= nd.at(Rec<M>::Xh, 11 + k);
+      for (int k = 0; k < 2; ++k) nd.at(L.oS, M14::S_TILT + k) -= nd.at(Rec<M, AOS>::Xh, 9 + k);
+      for (int k = 0; k < 3; ++k) nd.at(L.oS, M14::S_W + k) -= nd.at(Rec<M, AOS>::Xh, 11 + k);
     }
     if (nd.i < nd.N) {
       T y = T(0);
-      for (int k = 0; k < 3; ++k) { nd.at(L.oS, 3 + k) -= nd.at(Rec<M>::Uh, k); y += nd.at(L.oMd, k) * nd.at(Rec<M>::Uh, k); }
+      for (int k = 0; k < 3; ++k) { nd.at(L.oS, 3 + k) -= nd.at(Rec<M, AOS>::Uh, k); y += nd.at(L.oMd, k) * nd.at(Rec<M, AOS>::Uh, k); }
       nd.at(L.oS, 6) -= y;
       if constexpr (IsMars14<M>::value)
-        for (int k = 0; k < 3; ++k) nd.at(L.oS, M14::S_GIM + k) -= nd.at(Rec<M>::Uh, k);
+        for (int k = 0; k < 3; ++k) nd.at(L.oS, M14::S_GIM + k) -= nd.at(Rec<M, AOS>::Uh, k);
     }
   }
 }
@@ -1783,7 +1826,7 @@ __global__ void __launch_bounds__(MAX_THREADS) admm_kernel(ProblemDev P, Layout 
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ InstShared sh;
   const int b = blockIdx.x;
-  constexpr bool AOS = SMEM;
+  constexpr int AOS = SMEM;
   Node<T, AOS> nd = make_node<T, SMEM>(P, L, smem, b);
   MatsFor<M, T, AOS> MT;
   init_mats<M, T, AOS>(MT, nd, L);
@@ -1806,9 +1849,9 @@ __global__ void __launch_bounds__(MAX_THREADS) admm_kernel(ProblemDev P, Layout 
     }
     for (int r = 0; r < NX; ++r) {
       double acc = dg[g * NX + r];
-      for (int c = 0; c < NX; ++c) acc += Ag[g * NX * NX + r * NX + c] * wide_to_double(nd.dat(Rec<M>::Xbar, c));
-      for (int c = 0; c < NU; ++c) acc += Bg[g * NX * NU + r * NU + c] * wide_to_double(nd.dat(Rec<M>::Ubar, c));
-      nd.at(Rec<M>::C, r) = (T)(acc - wide_to_double(nd.dnb(Rec<M>::Xbar, r, i + 1)));
+      for (int c = 0; c < NX; ++c) acc += Ag[g * NX * NX + r * NX + c] * wide_to_double(nd.dat(Rec<M, AOS>::Xbar, c));
+      for (int c = 0; c < NU; ++c) acc += Bg[g * NX * NU + r * NU + c] * wide_to_double(nd.dat(Rec<M, AOS>::Ubar, c));
+      nd.at(Rec<M, AOS>::C, r) = (T)(acc - wide_to_double(nd.dnb(Rec<M, AOS>::Xbar, r, i + 1)));
     }
   }
   const T re = (T)P.rho_eq, rd = (T)P.rho_dyn, rg = (T)P.rho_geo;
@@ -1833,9 +1876,9 @@ __global__ void __launch_bounds__(MAX_THREADS) admm_kernel(ProblemDev P, Layout 
   if (!sh.fail) admm_iterations<M, T, AOS, REFINE>(nd, MT, L, I, K, active, re, rd, rg, iters, sh, r2, nullptr, X, P);
   if (active) {
     node_export<M, T, AOS>(nd, L, P, b, P.state_abs + P.soff[b]);
-    for (int j = 0; j < NX; ++j) xhat[(xo + i) * NX + j] = wide_to_double(nd.dat(Rec<M>::Xbar, j)) + (double)nd.at(Rec<M>::Xh, j);
+    for (int j = 0; j < NX; ++j) xhat[(xo + i) * NX + j] = wide_to_double(nd.dat(Rec<M, AOS>::Xbar, j)) + (double)nd.at(Rec<M, AOS>::Xh, j);
     if (i < N)
-      for (int j = 0; j < NU; ++j) uhat[(uo + i) * NU + j] = wide_to_double(nd.dat(Rec<M>::Ubar, j)) + (double)nd.at(Rec<M>::Uh, j);
+      for (int j = 0; j < NU; ++j) uhat[(uo + i) * NU + j] = wide_to_double(nd.dat(Rec<M, AOS>::Ubar, j)) + (double)nd.at(Rec<M, AOS>::Uh, j);
   }
   if (threadIdx.x == 0) {
     res[2 * b] = sqrt(r2[0]);
@@ -1846,7 +1889,7 @@ __global__ void __launch_bounds__(MAX_THREADS) admm_kernel(ProblemDev P, Layout 
 
 // Nonlinear cost l(x_i,u_i) (or phi(x_N)) of node i in the wide type (FP64
 // from the problem arrays, or double-float from the CB block).
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 __device__ __forceinline__ typename Node<T, AOS>::W node_cost(const Node<T, AOS>& nd, const ProblemDev& P,
                                                               const Inst<T>& I, int b, int i, int N,
                                                               const typename Node<T, AOS>::W* x,
@@ -1934,7 +1977,7 @@ __device__ void flag_bad_inputs(const ProblemDev& P, int b, const double* x0, co
 }
 
 // Start of a solve: c_i = RK4(xbar_i, ubar_i) - xbar_{i+1} and J(nominal) in sh.Jn.
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 __device__ void scp_start(const Node<T, AOS>& nd, const ProblemDev& P, const Inst<T>& I, int b, bool act,
                           InstShared& sh) {
   typedef typename Node<T, AOS>::W W;
@@ -1950,8 +1993,8 @@ __device__ void scp_start(const Node<T, AOS>& nd, const ProblemDev& P, const Ins
       W fn[NX];
       rk4_wide<M, T, AOS>(nd, P, b, xb, ub, fn);
       for (int j = 0; j < NX; ++j) {
-        const W e = fn[j] - nd.dnb(Rec<M>::Xbar, j, i + 1);
-        nd.at(Rec<M>::C, j) = wide_to<T>(e);
+        const W e = fn[j] - nd.dnb(Rec<M, AOS>::Xbar, j, i + 1);
+        nd.at(Rec<M, AOS>::C, j) = wide_to<T>(e);
         ac[1] = ac[1] + wide_abs(e);
       }
     }
@@ -1968,7 +2011,7 @@ __device__ void scp_start(const Node<T, AOS>& nd, const ProblemDev& P, const Ins
 // The candidate (x-hat, u-hat) of an SCP iteration: its trajectory (xc, uc),
 // defects fc_i = RK4(xc_i, uc_i) - xc_{i+1}, and CTA totals in v: cost, l1
 // defect, l1 defect of the linear model | max defect, max step.
-template <class M, class T, bool AOS, bool GROUP, class MS>
+template <class M, class T, int AOS, bool GROUP, class MS>
 __device__ void scp_candidate(const Node<T, AOS>& nd, const MS& MT, const ProblemDev& P, const Inst<T>& I, int b,
                               bool act, const GroupShared* G, InstShared& sh, typename Node<T, AOS>::W* xc,
                               typename Node<T, AOS>::W* uc, typename Node<T, AOS>::W* fc, double* v) {
@@ -1976,8 +2019,8 @@ __device__ void scp_candidate(const Node<T, AOS>& nd, const MS& MT, const Proble
   constexpr int NX = M::NX, NU = M::NU;
   const int i = nd.i, N = nd.N;
   if (act) {
-    for (int j = 0; j < NX; ++j) { xc[j] = wide_add(nd.dat(Rec<M>::Xbar, j), nd.at(Rec<M>::Xh, j)); nd.dat(Rec<M>::Xc, j) = xc[j]; }
-    for (int j = 0; j < NU; ++j) uc[j] = (i < N) ? wide_add(nd.dat(Rec<M>::Ubar, j), nd.at(Rec<M>::Uh, j)) : W();
+    for (int j = 0; j < NX; ++j) { xc[j] = wide_add(nd.dat(Rec<M, AOS>::Xbar, j), nd.at(Rec<M, AOS>::Xh, j)); nd.dat(Rec<M, AOS>::Xc, j) = xc[j]; }
+    for (int j = 0; j < NU; ++j) uc[j] = (i < N) ? wide_add(nd.dat(Rec<M, AOS>::Ubar, j), nd.at(Rec<M, AOS>::Uh, j)) : W();
     if constexpr (GROUP) {
       // the shared first control exactly (bitwise equal across the group)
       if (i == 0)
@@ -1990,21 +2033,21 @@ __device__ void scp_candidate(const Node<T, AOS>& nd, const MS& MT, const Proble
   T st = T(0), lin1 = T(0);
   if (act) {
     vs[0] = node_cost<M, T, AOS>(nd, P, I, b, i, N, xc, uc);
-    for (int j = 0; j < NX; ++j) st = maxv(st, absv(nd.at(Rec<M>::Xh, j)));
+    for (int j = 0; j < NX; ++j) st = maxv(st, absv(nd.at(Rec<M, AOS>::Xh, j)));
     if (i < N) {
-      for (int j = 0; j < NU; ++j) st = maxv(st, absv(nd.at(Rec<M>::Uh, j)));
+      for (int j = 0; j < NU; ++j) st = maxv(st, absv(nd.at(Rec<M, AOS>::Uh, j)));
       rk4_wide<M, T, AOS>(nd, P, b, xc, uc, fc);
 #pragma unroll
       for (int r = 0; r < NX; ++r) {
-        fc[r] = fc[r] - nd.dnb(Rec<M>::Xc, r, i + 1);
+        fc[r] = fc[r] - nd.dnb(Rec<M, AOS>::Xc, r, i + 1);
         vs[1] = vs[1] + wide_abs(fc[r]);
         dinf = maxv(dinf, wide_abs_round(fc[r]));
-        T lin = nd.at(Rec<M>::C, r) - nd.nb(Rec<M>::Xh, r, i + 1);
+        T lin = nd.at(Rec<M, AOS>::C, r) - nd.nb(Rec<M, AOS>::Xh, r, i + 1);
 #pragma unroll
         for (int c = 0; c < NX; ++c)
-          if (MS::akind(r, c)) acc_A(lin, MT, r, c, nd.at(Rec<M>::Xh, c));
+          if (MS::akind(r, c)) acc_A(lin, MT, r, c, nd.at(Rec<M, AOS>::Xh, c));
 #pragma unroll
-        for (int c = 0; c < NU; ++c) lin += MT.B(r, c) * nd.at(Rec<M>::Uh, c);
+        for (int c = 0; c < NU; ++c) lin += MT.B(r, c) * nd.at(Rec<M, AOS>::Uh, c);
         lin1 += absv(lin);
       }
     }
@@ -2021,7 +2064,7 @@ __device__ void scp_candidate(const Node<T, AOS>& nd, const MS& MT, const Proble
 
 // Accepted: the candidate becomes the nominal, its defect becomes c_i, and the
 // deviations are re-based on it.
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 __device__ void scp_move_nominal(const Node<T, AOS>& nd, const Layout& L, const ProblemDev& P, int b,
                                  const typename Node<T, AOS>::W* xc, const typename Node<T, AOS>::W* uc,
                                  const typename Node<T, AOS>::W* fc) {
@@ -2029,26 +2072,26 @@ __device__ void scp_move_nominal(const Node<T, AOS>& nd, const Layout& L, const 
   const int i = nd.i, N = nd.N;
   node_rebase_mirrors<M, T, AOS>(nd, L, P, b);
   for (int j = 0; j < NX; ++j) {
-    const T xh = nd.at(Rec<M>::Xh, j);
-    nd.dat(Rec<M>::Xbar, j) = xc[j];
-    nd.at(Rec<M>::X, j) -= xh;
-    if (i >= 1) nd.at(Rec<M>::Z, j) -= xh;
-    nd.at(Rec<M>::Xh, j) = T(0);
-    if (i < N) nd.at(Rec<M>::C, j) = wide_to<T>(fc[j]);
+    const T xh = nd.at(Rec<M, AOS>::Xh, j);
+    nd.dat(Rec<M, AOS>::Xbar, j) = xc[j];
+    nd.at(Rec<M, AOS>::X, j) -= xh;
+    if (i >= 1) nd.at(Rec<M, AOS>::Z, j) -= xh;
+    nd.at(Rec<M, AOS>::Xh, j) = T(0);
+    if (i < N) nd.at(Rec<M, AOS>::C, j) = wide_to<T>(fc[j]);
   }
   if (i < N)
     for (int j = 0; j < NU; ++j) {
-      const T uh = nd.at(Rec<M>::Uh, j);
-      nd.dat(Rec<M>::Ubar, j) = uc[j];
-      nd.at(Rec<M>::U, j) -= uh;
-      nd.at(Rec<M>::Uh, j) = T(0);
+      const T uh = nd.at(Rec<M, AOS>::Uh, j);
+      nd.dat(Rec<M, AOS>::Ubar, j) = uc[j];
+      nd.at(Rec<M, AOS>::U, j) -= uh;
+      nd.at(Rec<M, AOS>::Uh, j) = T(0);
     }
 }
 
 // End of a solve: the returned (last accepted) trajectory, its cost, l1 and
 // max defect (w[0..2], CTA totals; the defects by FP64 RK4 steps and FP64
 // sums: once per launch) and the exported ADMM state.
-template <class M, class T, bool AOS>
+template <class M, class T, int AOS>
 __device__ void scp_finish(const Node<T, AOS>& nd, const Layout& L, const ProblemDev& P, const Inst<T>& I, int b,
                            bool act, long long xo, long long uo, double* xout, double* uout, InstShared& sh,
                            double* w) {
@@ -2078,7 +2121,7 @@ __device__ void scp_finish(const Node<T, AOS>& nd, const Layout& L, const Proble
       double fn[NX];
       rk4<M, double>(P.params + b * 8, P.dt[b], xd, ud, fn);
       for (int j = 0; j < NX; ++j) {
-        const double e = fabs(fn[j] - wide_to_double(nd.dnb(Rec<M>::Xbar, j, i + 1)));
+        const double e = fabs(fn[j] - wide_to_double(nd.dnb(Rec<M, AOS>::Xbar, j, i + 1)));
         w[1] += e;
         w[2] = fmax(w[2], e);
       }
@@ -2169,7 +2212,7 @@ __device__ __forceinline__ void scp_body(const ProblemDev& P, const Layout& L, c
     X.k = (int)blockIdx.x % P.group;
     if (threadIdx.x == 0) G->gfail = 0;
   }
-  constexpr bool AOS = SMEM;
+  constexpr int AOS = SMEM;
   Node<T, AOS> nd = make_node<T, SMEM>(P, L, smem, b);
   MatsFor<M, T, AOS, true> MT;
   init_mats<M, T, AOS>(MT, nd, L);

@@ -104,7 +104,7 @@ struct LaneH<M, T, TPN, false> {
 };
 
 // A_i, B_i (Eq. (2b)): the NN forward-mode directions split over the lanes.
-template <class M, class T, bool AOS, int TPN, class MS>
+template <class M, class T, int AOS, int TPN, class MS>
 __device__ __forceinline__ void lanes_jacobians(const Node<T, AOS>& nd, const MS& MT, const T* prm, const Step3<T>& hs,
                                                 int q) {
   constexpr int NX = M::NX, NU = M::NU;
@@ -148,7 +148,7 @@ __device__ __forceinline__ void lanes_jacobians(const Node<T, AOS>& nd, const MS
 // The lane's rows of the cost gradient (q_i, r_i) in deviations and of the
 // diagonal of H_i without its A/B and mirror Gram terms (the same numbers as
 // node_setup's NodeConst, for the own rows only).
-template <class M, class T, bool AOS, int TPN>
+template <class M, class T, int AOS, int TPN>
 __device__ __forceinline__ void lanes_consts(const Node<T, AOS>& nd, const ProblemDev& P, int b, int q, T re, T rg,
                                              T* kq, T* khd) {
   using LR = LaneRows<M, TPN>;
@@ -205,7 +205,7 @@ __device__ __forceinline__ void lanes_consts(const Node<T, AOS>& nd, const Probl
 // One iteration of Steps 1-4 over the CTA's instance, lane-parallel.  Every
 // thread of the CTA calls it (inactive nodes with zero data: the shuffles
 // need whole warps).  Quadrotor mirror sets (linearised obstacles) only.
-template <class M, class T, bool AOS, bool REFINE, bool LAST, bool GROUP, int TPN, class MS, class HR>
+template <class M, class T, int AOS, bool REFINE, bool LAST, bool GROUP, int TPN, class MS, class HR>
 __device__ __forceinline__ void admm_iteration_lanes(const Node<T, AOS>& nd, const MS& MT, const HR& H, const Layout& L,
                                                      const Inst<T>& I, const T* kq, const T* khd, bool active, int q,
                                                      T re, T rd, T rg, T irg, T ired, typename WideOf<T>::type& rp,
@@ -238,7 +238,7 @@ __device__ __forceinline__ void admm_iteration_lanes(const Node<T, AOS>& nd, con
           v += acc;
         }
         if (m == 0 && j < 3)
-          for (int o = 0; o < I.nobs; ++o) v += nd.at(L.oMd, ObsStride<T>::value * o + j) * (rg * nd.at(L.oS, o) - nd.at(L.oNus, o));
+          for (int o = 0; o < I.nobs; ++o) v += obs_at(nd, L, o, j) * (rg * nd.at(L.oS, o) - nd.at(L.oNus, o));
       }
       g[m] = v;
     }
@@ -294,8 +294,8 @@ __device__ __forceinline__ void admm_iteration_lanes(const Node<T, AOS>& nd, con
         }
         if (active && m == 0 && j < 3)
           for (int o = 0; o < I.nobs; ++o) {
-            const T n0 = nd.at(L.oMd, ObsStride<T>::value * o), n1 = nd.at(L.oMd, ObsStride<T>::value * o + 1), n2 = nd.at(L.oMd, ObsStride<T>::value * o + 2);
-            hx += nd.at(L.oMd, ObsStride<T>::value * o + j) * (rg * (n0 * xf[0] + n1 * xf[1] + n2 * xf[2]));
+            const T n0 = obs_at(nd, L, o, 0), n1 = obs_at(nd, L, o, 1), n2 = obs_at(nd, L, o, 2);
+            hx += obs_at(nd, L, o, j) * (rg * (n0 * xf[0] + n1 * xf[1] + n2 * xf[2]));
           }
         res[m] = g[m] - hx;
       }
@@ -393,8 +393,8 @@ __device__ __forceinline__ void admm_iteration_lanes(const Node<T, AOS>& nd, con
     }
     // linearised obstacles (mirror half-spaces on the position), split over the lanes
     for (int o = q; o < I.nobs; o += TPN) {
-      const T n0 = nd.at(L.oMd, ObsStride<T>::value * o), n1 = nd.at(L.oMd, ObsStride<T>::value * o + 1), n2 = nd.at(L.oMd, ObsStride<T>::value * o + 2);
-      const T bd = nd.at(L.oMd, ObsStride<T>::value * o + 3);
+      const T n0 = obs_at(nd, L, o, 0), n1 = obs_at(nd, L, o, 1), n2 = obs_at(nd, L, o, 2);
+      const T bd = obs_at(nd, L, o, 3);
       const T y = n0 * xf[0] + n1 * xf[1] + n2 * xf[2];
       const T so = nd.at(L.oS, o);
       const T s = maxv(bd, y + nd.at(L.oNus, o) * irg);
@@ -501,7 +501,7 @@ __device__ __forceinline__ void admm_iteration_lanes(const Node<T, AOS>& nd, con
   __syncthreads();
 }
 
-template <class M, class T, bool AOS, bool REFINE, bool GROUP, int TPN, class MS, class HR>
+template <class M, class T, int AOS, bool REFINE, bool GROUP, int TPN, class MS, class HR>
 __device__ __forceinline__ void admm_iterations_lanes(const Node<T, AOS>& nd, const MS& MT, const HR& H, const Layout& L,
                                                       const Inst<T>& I, const T* kq, const T* khd, bool active, int q,
                                                       T re, T rd, T rg, int iters, InstShared& sh, double* res,
@@ -544,7 +544,7 @@ __device__ __forceinline__ void scp_lanes_body(const ProblemDev& P, const Layout
     X.k = (int)blockIdx.x % P.group;
     if (threadIdx.x == 0) G->gfail = 0;
   }
-  constexpr bool AOS = SMEM;
+  constexpr int AOS = SMEM;
   const int q = (int)threadIdx.x % TPN;
   Node<T, AOS> nd = make_node_at<T, SMEM>(P, L, smem, b, (int)threadIdx.x / TPN);
   SmemMats<M, T, AOS> MT;

@@ -4,6 +4,7 @@
 #include "ucn_kernels.cuh"
 #include "ucn_lanes.cuh"
 #include "ucn_pair.cuh"
+#include "ucn_rows.cuh"
 
 namespace ucn {
 
@@ -199,19 +200,112 @@ cudaError_t launch_scpp_v(const LaunchCfg& c, const double* x0, const double* u0
   return cudaGetLastError();
 }
 
+// The row kernel (ucn_rows.cuh), one kernel per function, each in its own
+// translation unit (declared here, defined by UCN_DEFINE_ROWS_*).  The 17-row
+// models' FP32 solves run on nothing else (four CTAs of 64 nodes hold the
+// longest horizon); the 12-state quadrotor's do on four threads per node (128
+// nodes at most), and keep the one-thread kernel beyond and on request.
+template <class M, class T>
+constexpr bool row_kernel_only = RowModel<M>::value && std::is_same<T, float>::value && !std::is_same<M, Quad12>::value;
+typedef void (*RowScpKernel)(ProblemDev, Layout, const double*, const double*, double*, double*, ucn_scp_stats*, int*);
+typedef void (*RowAdmmKernel)(ProblemDev, Layout, const double*, const double*, const double*, const double*,
+                              const double*, const double*, int, int, double*, double*, double*, int*);
+template <class M, bool GROUP, bool CL, int MAXT> RowScpKernel rows_scp_kernel();
+template <class M, bool CL, int MAXT> RowAdmmKernel rows_admm_kernel();
+
+// Launch of a row kernel: one CTA per instance, or a cluster of L.csize CTAs.
+template <class K, class... Args>
+cudaError_t launch_rows_k(K k, const LaunchCfg& c, const Layout& L, int threads, unsigned cluster, Args... args) {
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem_bytes);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(c.blocks * L.csize), 1, 1);
+  cfg.blockDim = dim3((unsigned)threads, 1, 1);
+  cfg.dynamicSmemBytes = (size_t)c.smem_bytes;
+  cfg.stream = c.stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cluster;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, *(const ProblemDev*)c.P, L, args...);
+}
+
+// The register class of a launch of `threads`-thread CTAs: the 168-register one
+// where the 255-register one cannot run it, or keeps fewer CTAs per SM resident
+// while there are CTAs to fill the difference.
+template <class K>
+cudaError_t rows_pick(const LaunchCfg& c, int threads, K wide, K narrow, K* out) {
+  *out = narrow;
+  if (threads > ROWS_THREADS) return cudaSuccess;
+  *out = wide;
+  int bw = 0, bn = 0, dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  for (auto k : {wide, narrow})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem_bytes);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bw, wide, threads, c.smem_bytes);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bn, narrow, threads, c.smem_bytes);
+  if (e != cudaSuccess) return e;
+  if (bn > bw && c.blocks > sms * bw) *out = narrow;
+  return cudaSuccess;
+}
+
+template <class M>
+cudaError_t launch_scp_rows(const LaunchCfg& c, const double* x0, const double* u0, double* xo, double* uo,
+                            ucn_scp_stats* st, int* status) {
+  const Layout& L = *(const Layout*)c.L;
+  const int threads = (4 * L.chunk + 31) / 32 * 32;
+  if (L.csize > 1)
+    return launch_rows_k(rows_scp_kernel<M, false, true, ROWS_THREADS>(), c, L, threads, (unsigned)L.csize, x0, u0, xo,
+                         uo, st, status);
+  RowScpKernel k = rows_scp_kernel<M, false, false, ROWS_THREADS>();
+  if constexpr (std::is_same<M, Quad12>::value) {
+    const cudaError_t e = rows_pick(c, threads, k, rows_scp_kernel<M, false, false, ROWS_WIDE_THREADS>(), &k);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_rows_k(k, c, L, threads, 1u, x0, u0, xo, uo, st, status);
+}
+
+template <class M>
+cudaError_t launch_admm_rows(const LaunchCfg& c, const double* xbar, const double* ubar, const double* A,
+                             const double* B, const double* d, const double* radius, int iters, int warm,
+                             double* xhat, double* uhat, double* res, int* status) {
+  const Layout& L = *(const Layout*)c.L;
+  const int threads = (4 * L.chunk + 31) / 32 * 32;
+  RowAdmmKernel k = rows_admm_kernel<M, false, ROWS_THREADS>();
+  if (L.csize > 1) {
+    k = rows_admm_kernel<M, true, ROWS_THREADS>();
+  } else if constexpr (std::is_same<M, Quad12>::value) {
+    const cudaError_t e = rows_pick(c, threads, k, rows_admm_kernel<M, false, ROWS_WIDE_THREADS>(), &k);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_rows_k(k, c, L, threads, (unsigned)L.csize, xbar, ubar, A, B, d, radius, iters, warm, xhat, uhat, res,
+                       status);
+}
+
 template <class M, class T, bool R>
 cudaError_t launch_scp_t(const LaunchCfg& c, const double* x0, const double* u0, double* xo, double* uo,
                          ucn_scp_stats* st, int* status) {
+  if constexpr (row_kernel_only<M, T>) {
+    return launch_scp_rows<M>(c, x0, u0, xo, uo, st, status);
+  } else {
+  if constexpr (RowModel<M>::value && std::is_same<T, float>::value) {
+    if (((const Layout*)c.L)->csize > 0) return launch_scp_rows<M>(c, x0, u0, xo, uo, st, status);
+  }
   if constexpr (std::is_same<M, Mars7>::value && std::is_same<T, float>::value && R) {
     if (c.tpn == 2) return launch_scpp_v<M, R>(c, x0, u0, xo, uo, st, status);
   }
-  if constexpr (LaneModel<M>::value) {
+  if constexpr (LaneModel<M>::value && std::is_same<T, double>::value) {
     if (c.tpn == 4)
       return c.smem ? launch_scpl_v<M, T, true, R>(c, x0, u0, xo, uo, st, status)
                     : launch_scpl_v<M, T, false, R>(c, x0, u0, xo, uo, st, status);
   }
   return c.smem ? launch_scp_v<M, T, true, R>(c, x0, u0, xo, uo, st, status)
                 : launch_scp_v<M, T, false, R>(c, x0, u0, xo, uo, st, status);
+  }
 }
 
 // The group kernels of the lane layout, one per register class (each in its
@@ -256,7 +350,14 @@ cudaError_t launch_scp_group_t(const LaunchCfg& c, const double* x0, const doubl
   ScpKernelPtr<M, T, R> k = scp_kernel<M, T, true, R, true>;
   cudaError_t e = cudaSuccess;
   if (c.tpn == 4) {
-    e = pick_group_lanes<M, T, R>(c, threads, &k);
+    // four threads per node: FP32 records that fit the lane layout fit the row kernel's
+    if constexpr (std::is_same<T, float>::value) {
+      if (L.csize != 1) return cudaErrorInvalidConfiguration;
+      e = rows_pick(c, threads, rows_scp_kernel<M, true, false, ROWS_THREADS>(),
+                    rows_scp_kernel<M, true, false, ROWS_WIDE_THREADS>(), &k);
+    } else {
+      e = pick_group_lanes<M, T, R>(c, threads, &k);
+    }
     if (e != cudaSuccess) return e;
   }
   e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem_bytes);
@@ -304,8 +405,16 @@ template <class M, class T, bool R>
 cudaError_t launch_admm_t(const LaunchCfg& c, const double* xbar, const double* ubar, const double* A,
                           const double* B, const double* d, const double* radius, int iters, int warm,
                           double* xhat, double* uhat, double* res, int* status) {
+  if constexpr (row_kernel_only<M, T>) {
+    return launch_admm_rows<M>(c, xbar, ubar, A, B, d, radius, iters, warm, xhat, uhat, res, status);
+  } else {
+  if constexpr (RowModel<M>::value && std::is_same<T, float>::value) {
+    if (((const Layout*)c.L)->csize > 0)
+      return launch_admm_rows<M>(c, xbar, ubar, A, B, d, radius, iters, warm, xhat, uhat, res, status);
+  }
   return c.smem ? launch_admm_v<M, T, true, R>(c, xbar, ubar, A, B, d, radius, iters, warm, xhat, uhat, res, status)
                 : launch_admm_v<M, T, false, R>(c, xbar, ubar, A, B, d, radius, iters, warm, xhat, uhat, res, status);
+  }
 }
 
 template <class M, class T>
@@ -379,6 +488,18 @@ cudaError_t launch_linearize_t(const void* Pv, const int* node_inst, long long t
 // The 3-CTAs-per-SM variant of the one-thread kernel in its own translation unit.
 #define UCN_INSTANTIATE_SCP3(MODEL, T, SMEM, REFINE) template struct ucn::Scp3Variant<ucn::MODEL, T, SMEM, REFINE>;
 #define UCN_EXTERN_SCP3(MODEL, T, SMEM, REFINE) extern template struct ucn::Scp3Variant<ucn::MODEL, T, SMEM, REFINE>;
+
+// Row-kernel variants, each in its own translation unit.
+#define UCN_DEFINE_ROWS_SCP(MODEL, GROUP, CL, MAXT, REG)                                                   \
+  namespace ucn {                                                                                          \
+  template <>                                                                                              \
+  RowScpKernel rows_scp_kernel<MODEL, GROUP, CL, MAXT>() { return scp_rows_kernel<MODEL, GROUP, CL, MAXT, REG>; } \
+  }
+#define UCN_DEFINE_ROWS_ADMM(MODEL, CL, MAXT, REG)                                                         \
+  namespace ucn {                                                                                          \
+  template <>                                                                                              \
+  RowAdmmKernel rows_admm_kernel<MODEL, CL, MAXT>() { return admm_rows_kernel<MODEL, CL, MAXT, REG>; }     \
+  }
 
 // Pair-kernel variant in its own translation unit.
 #define UCN_SCPP_V(MODEL, REFINE)                                                                          \

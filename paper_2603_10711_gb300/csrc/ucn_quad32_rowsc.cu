@@ -1,0 +1,4 @@
+// Row kernel, FP32: the fused solve, an instance over a cluster.
+#include "ucn_launch.cuh"
+
+UCN_DEFINE_ROWS_SCP(Quad12, false, true, ROWS_THREADS, true)

@@ -1,0 +1,4 @@
+// Row kernel, FP32: the fused solve, 168 registers per thread.
+#include "ucn_launch.cuh"
+
+UCN_DEFINE_ROWS_SCP(Quad12, false, false, ROWS_WIDE_THREADS, false)

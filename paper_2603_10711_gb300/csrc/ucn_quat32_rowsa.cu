@@ -1,0 +1,5 @@
+// Row kernel, FP32: the stand-alone ADMM call.
+#include "ucn_launch.cuh"
+
+UCN_DEFINE_ROWS_ADMM(Quat13, false, ROWS_THREADS, false)
+UCN_DEFINE_ROWS_ADMM(Quat13, true, ROWS_THREADS, false)

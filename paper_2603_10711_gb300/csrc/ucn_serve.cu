@@ -86,6 +86,8 @@ struct ucn_server {
   Layout L;
   bool smem;
   long long smem_bytes;
+  bool rows = false;     // pump launches run the row kernel, on this layout (the request loop does not)
+  Layout Lr;
   int threads;
   int tpn;               // threads per node of the fused solve
   int* status_d;         // per-slot status of the fused solve
@@ -369,6 +371,7 @@ ucn_status ucn_serve_create(const ucn_serve_config* c, ucn_server** out) {
     s->L = make_layout(c->model, s->Nmax + 1, s->max_obs, tsize, false, s->tpn);
   }
   s->smem_bytes = s->smem ? s->L.bytes : 0;
+  s->rows = rows_layout(c->model, c->precision, s->Nmax + 1, s->max_obs, 1, s->tpn, optin, &s->Lr);
   s->threads = (s->Nmax + 1 + 31) / 32 * 32;
   s->R = c->kept > 0 ? c->kept : 2 * S;
   s->rl = rec_layout(NX, NU, MO, (int)Xn, (int)Un);
@@ -598,6 +601,7 @@ ucn_status ucn_serve_pump(ucn_server* s, int* launched) {
     c.P = &P; c.L = &s->L; c.smem = s->smem; c.smem_bytes = s->smem_bytes;
     c.threads = s->threads; c.blocks = n; c.stream = st; c.group = 1;
     c.nodes = s->cfg.max_horizon + 1; c.tpn = s->tpn;
+    if (s->rows) { c.L = &s->Lr; c.smem = true; c.smem_bytes = s->Lr.bytes; }
     auto fn = launchers_for(s->cfg.model, s->cfg.precision).scp;
     e = fn(c, s->D.x0, s->D.u0, s->D.xo, s->D.uo, s->D.stats, s->status_d);
   }
