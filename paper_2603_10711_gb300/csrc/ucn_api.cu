@@ -236,7 +236,9 @@ __global__ void mpc_shift_kernel(ProblemDev P, const double* x, const double* u,
     double xi[NX], ui[NU];
     for (int j = 0; j < NX; ++j) xi[j] = P.xinit[lead * NX + j];
     for (int j = 0; j < NU; ++j) ui[j] = u[P.uoff[lead] * NU + j];
-    rk4<M, double>(P.params + lead * 8, P.dt[lead], xi, ui, x0n);
+    double prm[PRM];
+    for (int j = 0; j < PRM; ++j) prm[j] = derived_param<M>(P.params + lead * 8, j);
+    rk4<M, double>(prm, P.dt[lead], xi, ui, x0n);
   }
   __syncthreads();
   for (int i = threadIdx.x; i <= N; i += blockDim.x) {

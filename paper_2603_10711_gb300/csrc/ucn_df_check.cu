@@ -42,8 +42,8 @@ __global__ void df_rk4_kernel(const double* x, const double* u, const double* pr
   const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
   constexpr int NX = M::NX, NU = M::NU;
-  DF p[8], xs[NX], us[NU], xn[NX];
-  for (int j = 0; j < 8; ++j) p[j] = df_from(prm[j]);
+  DF p[PRM], xs[NX], us[NU], xn[NX];
+  for (int j = 0; j < PRM; ++j) p[j] = df_from(derived_param<M>(prm, j));
   for (int j = 0; j < NX; ++j) xs[j] = df_from(x[k * NX + j]);
   for (int j = 0; j < NU; ++j) us[j] = df_from(u[k * NU + j]);
   rk4h<M, DF, DF, DF>(p, df_from(h), df_from(0.5 * h), df_from(h / 6.0), xs, us, xn);

@@ -125,7 +125,7 @@ struct CB {
   static constexpr int NX = M::NX, NU = M::NU;
   static constexpr int Xlo = 0, Xhi = NX, Xref = 2 * NX, Xinit = 3 * NX, Xtgt = 4 * NX, Qd = 5 * NX, QNd = 6 * NX,
                        QN = 7 * NX, Ulo = 8 * NX, Uhi = Ulo + NU, Uref = Uhi + NU, Rd = Uref + NU, Prm = Rd + NU,
-                       Step = Prm + 8, END = Step + 3;
+                       Step = Prm + PRM, END = Step + 3;
 };
 
 // Where the per-node records of one instance live.
@@ -156,6 +156,7 @@ struct Node {
   T* t;          // T region base
   W* d;          // wide region base
   W* c;          // CB block of the instance (FP32 path)
+  const double* prm;   // the model's constants in FP64 (InstShared)
   int S, NS, DS, i, N;
   // (layout 2: t and d point at the record node 0 of the instance would have)
   __device__ __forceinline__ T& at(int off, int k) const { return AOS ? t[i * NS + off + k] : t[(long long)(off + k) * S + i]; }
@@ -306,7 +307,6 @@ struct Inst {
   bool gim, tilt, wball;    // Mars 6-DOF: gimbal cone, tilt ball, body-rate ball
   T tg, cg, sg, rtilt, wmax;
   bool run_cost, term_quad; // nonzero running weights / terminal quadratic weights
-  T prm[8];                 // model constants in T (Jacobian passes)
 };
 
 // Obstacles of instance b, clamped to [0, max_obs]: ucn_problem_create checks
@@ -352,7 +352,6 @@ __device__ __forceinline__ Inst<T> make_inst(const ProblemDev& P, int b) {
   I.half = f & 1u; I.ball = f & 2u; I.cone = f & 4u;
   I.gim = f & 8u; I.tilt = f & 16u; I.wball = f & 32u;
   I.run_cost = f & 64u; I.term_quad = f & 128u;
-  for (int k = 0; k < 8; ++k) I.prm[k] = (T)P.params[b * 8 + k];
   return I;
 }
 
@@ -364,9 +363,24 @@ struct InstShared {
   double rho[3];            // rho_eq, rho_dyn, rho_geo of the SCP iteration
   float rhof[3];            // the same in FP32 (no conversion per thread)
   double out[8];
+  double prm[PRM];          // the model's constants (derived_param)
+  float prmf[PRM];          // the same in FP32
   int fail;
   int accept, stop, status;
 };
+
+// The instance's model constants, by the CTA's first PRM threads (the caller
+// synchronises), and the arithmetic type's copy.
+template <class M>
+__device__ __forceinline__ void stage_params(InstShared& sh, const ProblemDev& P, int b) {
+  if (threadIdx.x < PRM) {
+    const double v = derived_param<M>(P.params + b * 8, (int)threadIdx.x);
+    sh.prm[threadIdx.x] = v;
+    sh.prmf[threadIdx.x] = (float)v;
+  }
+}
+template <class T> __device__ __forceinline__ const T* prm_of(const InstShared& sh) { return sh.prm; }
+template <> __device__ __forceinline__ const float* prm_of<float>(const InstShared& sh) { return sh.prmf; }
 
 // Per-CTA state of a scenario group's exchanges (one CTA per scenario).
 struct GroupShared {
@@ -641,7 +655,7 @@ __device__ void stage_consts(const Node<T, AOS>& nd, const ProblemDev& P, int b)
       else if (e < C::Uref) v = P.uhi[b * NU + e - C::Uhi];
       else if (e < C::Rd) v = P.uref[b * NU + e - C::Uref];
       else if (e < C::Prm) v = P.Rd[b * NU + e - C::Rd];
-      else if (e < C::Step) v = P.params[b * 8 + e - C::Prm];
+      else if (e < C::Step) v = derived_param<M>(P.params + b * 8, e - C::Prm);
       else v = P.dt[b] * (e == C::Step ? 1.0 : e == C::Step + 1 ? 0.5 : 1.0 / 6.0);
       nd.c[e] = df_from(v);
     }
@@ -678,7 +692,7 @@ __device__ __forceinline__ void rk4_wide(const Node<T, AOS>& nd, const ProblemDe
     typedef CB<M> C;
     rk4h<M, DF, DF, DF>(nd.c + C::Prm, nd.c[C::Step], nd.c[C::Step + 1], nd.c[C::Step + 2], x, u, xn);
   } else {
-    rk4<M, double>(P.params + b * 8, P.dt[b], x, u, xn);
+    rk4<M, double>(nd.prm, P.dt[b], x, u, xn);
   }
 }
 
@@ -1793,12 +1807,14 @@ __global__ void __launch_bounds__(128) linearize_kernel(ProblemDev P, const int*
   double x[NX], u[NU];
   for (int j = 0; j < NX; ++j) x[j] = xbar[xr * NX + j];
   for (int j = 0; j < NU; ++j) u[j] = ubar[g * NU + j];
-  const double* prm = P.params + b * 8;
+  double prm[PRM];
+  T prmt[PRM];
+  for (int k = 0; k < PRM; ++k) { prm[k] = derived_param<M>(P.params + b * 8, k); prmt[k] = (T)prm[k]; }
   const double h = P.dt[b];
   double Ad[NX * NX], Bd[NX * NU];
   for (int dir = 0; dir < NX + NU; ++dir) {
     T col[NX];
-    rk4_jvp<M, T>(prm, step_of<T>(h), x, u, dir, col);
+    rk4_jvp<M, T>(prmt, step_of<T>(h), x, u, dir, col);
     for (int r = 0; r < NX; ++r) {
       if (dir < NX) Ad[r * NX + dir] = (double)col[r];
       else Bd[r * NU + dir - NX] = (double)col[r];
@@ -2119,7 +2135,7 @@ __device__ void scp_finish(const Node<T, AOS>& nd, const Layout& L, const Proble
       // (once per launch): the reported defect and the defect_tol status are
       // FP64 quantities of exactly the doubles returned
       double fn[NX];
-      rk4<M, double>(P.params + b * 8, P.dt[b], xd, ud, fn);
+      rk4<M, double>(nd.prm, P.dt[b], xd, ud, fn);
       for (int j = 0; j < NX; ++j) {
         const double e = fabs(fn[j] - wide_to_double(nd.dnb(Rec<M, AOS>::Xbar, j, i + 1)));
         w[1] += e;
@@ -2229,6 +2245,8 @@ __device__ __forceinline__ void scp_body(const ProblemDev& P, const Layout& L, c
     split_barrier_init(sh.xbar, blockDim.x);
   }
   X.bar = sh.xbar;
+  nd.prm = sh.prm;
+  stage_params<M>(sh, P, b);
   stage_consts<M, T, AOS>(nd, P, b);
   if (active) load_nominal<M, T, AOS>(nd, L, x0, u0, xo, uo);
   __syncthreads();
@@ -2255,7 +2273,7 @@ __device__ __forceinline__ void scp_body(const ProblemDev& P, const Layout& L, c
     const T re = rho_of<T>(sh, 0), rd = rho_of<T>(sh, 1), rg = rho_of<T>(sh, 2);
     const double radius = sh.radius;
     if (active) {
-      if (i < N) node_jacobians<M, T, AOS>(nd, MT, I.prm, hs);
+      if (i < N) node_jacobians<M, T, AOS>(nd, MT, prm_of<T>(sh), hs);
       node_setup<M, T, AOS>(nd, L, P, I, b, radius, re, rg, K);
       const bool ok = node_factor<M, T, AOS, NN>(nd, MT, L, I, K, rd, rg);
       if (!ok) atomicOr(&sh.fail, 1);

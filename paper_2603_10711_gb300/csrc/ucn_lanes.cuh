@@ -575,6 +575,8 @@ __device__ __forceinline__ void scp_lanes_body(const ProblemDev& P, const Layout
     split_barrier_init(sh.xbar, blockDim.x);
   }
   X.bar = sh.xbar;
+  nd.prm = ndd.prm = sh.prm;
+  stage_params<M>(sh, P, b);
   stage_consts<M, T, AOS>(ndd, P, b);
   if (dact) load_nominal<M, T, AOS>(ndd, L, x0, u0, xo, uo);
   __syncthreads();
@@ -600,7 +602,7 @@ __device__ __forceinline__ void scp_lanes_body(const ProblemDev& P, const Layout
     __syncthreads();
     const T re = rho_of<T>(sh, 0), rd = rho_of<T>(sh, 1), rg = rho_of<T>(sh, 2);
     const double radius = sh.radius;
-    if (active && i < N) lanes_jacobians<M, T, AOS, TPN>(nd, MT, I.prm, hs, q);
+    if (active && i < N) lanes_jacobians<M, T, AOS, TPN>(nd, MT, prm_of<T>(sh), hs, q);
     if (active) lanes_consts<M, T, AOS, TPN>(nd, P, b, q, re, rg, kq, khd);
     __syncthreads();
     if (dact) {
@@ -667,7 +669,7 @@ __device__ __forceinline__ void scp_lanes_body(const ProblemDev& P, const Layout
 
 // CTAs of up to 512 threads; the compiler chooses the registers (128 at most).
 template <class M, class T, bool SMEM, bool REFINE, bool GROUP, int TPN>
-__global__ void __launch_bounds__(LANES_MAX_THREADS) scp_kernel_lanes(ProblemDev P, Layout L, const double* x0,
+__global__ void __launch_bounds__(LANES_MAX_THREADS, 1) scp_kernel_lanes(ProblemDev P, Layout L, const double* x0,
                                                                       const double* u0, double* xout, double* uout,
                                                                       ucn_scp_stats* stats, int* status_out) {
   scp_lanes_body<M, T, SMEM, REFINE, GROUP, TPN>(P, L, x0, u0, xout, uout, stats, status_out, cta_instance<GROUP>(P));

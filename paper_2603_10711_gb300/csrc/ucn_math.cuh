@@ -115,11 +115,7 @@ template <class T, int K> __device__ __forceinline__ DualN<T, K> operator/(DualN
   return r;
 }
 
-__device__ __forceinline__ float sin_(float a) { return sinf(a); }
-__device__ __forceinline__ float cos_(float a) { return cosf(a); }
 __device__ __forceinline__ float sqrt_(float a) { return sqrtf(a); }
-__device__ __forceinline__ double sin_(double a) { return sin(a); }
-__device__ __forceinline__ double cos_(double a) { return cos(a); }
 __device__ __forceinline__ double sqrt_(double a) { return sqrt(a); }
 // 1 / sqrt(a) of a Cholesky pivot: FP64 correctly rounded; FP32 by the hardware
 // reciprocal square root and one Newton-Raphson step y (3 - a y^2) / 2 (within
@@ -130,13 +126,8 @@ __device__ __forceinline__ float inv_sqrt_(float a) {
   const float y = rsqrtf(a);
   return y * fmaf(-0.5f * a * y, y, 1.5f);
 }
-// Double-float: the root by one corrected step; sine and cosine (the 12-state
-// quadrotor's Euler angles only) through FP64.
+// Double-float: the root by one corrected step.
 __device__ __forceinline__ DF sqrt_(DF a) { return df_sqrt(a); }
-__device__ __forceinline__ DF sin_(DF a) { return df_from(sin(df_to_double(a))); }
-__device__ __forceinline__ DF cos_(DF a) { return df_from(cos(df_to_double(a))); }
-template <class T> __device__ __forceinline__ Dual<T> sin_(Dual<T> a) { return {sin_(a.v), cos_(a.v) * a.d}; }
-template <class T> __device__ __forceinline__ Dual<T> cos_(Dual<T> a) { return {cos_(a.v), -sin_(a.v) * a.d}; }
 template <class T> __device__ __forceinline__ Dual<T> sqrt_(Dual<T> a) {
   T s = sqrt_(a.v);
   return {s, s > T(0) ? a.d / (T(2) * s) : T(0)};
@@ -158,22 +149,6 @@ template <int K> __device__ __forceinline__ DualN<float, K> operator/(float a, D
   for (int q = 0; q < K; ++q) r.d[q] = -r.v * b.d[q] * rr;
   return r;
 }
-template <class T, int K> __device__ __forceinline__ DualN<T, K> sin_(DualN<T, K> a) {
-  const T c = cos_(a.v);
-  DualN<T, K> r;
-  r.v = sin_(a.v);
-#pragma unroll
-  for (int q = 0; q < K; ++q) r.d[q] = c * a.d[q];
-  return r;
-}
-template <class T, int K> __device__ __forceinline__ DualN<T, K> cos_(DualN<T, K> a) {
-  const T sn = sin_(a.v);
-  DualN<T, K> r;
-  r.v = cos_(a.v);
-#pragma unroll
-  for (int q = 0; q < K; ++q) r.d[q] = -sn * a.d[q];
-  return r;
-}
 template <class T, int K> __device__ __forceinline__ DualN<T, K> sqrt_(DualN<T, K> a) {
   DualN<T, K> r;
   r.v = sqrt_(a.v);
@@ -182,44 +157,95 @@ template <class T, int K> __device__ __forceinline__ DualN<T, K> sqrt_(DualN<T, 
   return r;
 }
 
+// Sine and cosine together: one range reduction for the two.
+__device__ __forceinline__ void sincos_(float a, float& s, float& c) { sincosf(a, &s, &c); }
+__device__ __forceinline__ void sincos_(double a, double& s, double& c) { sincos(a, &s, &c); }
+__device__ __forceinline__ void sincos_(DF a, DF& s, DF& c) { df_sincos(a, s, c); }
+template <class T> __device__ __forceinline__ void sincos_(Dual<T> a, Dual<T>& s, Dual<T>& c) {
+  T sv, cv;
+  sincos_(a.v, sv, cv);
+  s = {sv, cv * a.d};
+  c = {cv, -sv * a.d};
+}
+template <class T, int K> __device__ __forceinline__ void sincos_(DualN<T, K> a, DualN<T, K>& s, DualN<T, K>& c) {
+  sincos_(a.v, s.v, c.v);
+#pragma unroll
+  for (int q = 0; q < K; ++q) {
+    s.d[q] = c.v * a.d[q];
+    c.d[q] = -s.v * a.d[q];
+  }
+}
+
 // ------------------------------------------------------------------ models
+// A model's constants as the dynamics read them: PRM values, the problem's
+// eight (model_params) and quotients of them, formed once per instance in FP64
+// (derived_param) and rounded to the arithmetic's type -- a division costs ~25
+// dependent FP64 instructions, or ~40 FP32 ones in double-float, and the RK4
+// map evaluated nine of them at every stage of every tangent.
+constexpr int PRM = 16;
+
+// What an RK4 step holds constant: the control enters through a few combined
+// quantities (Held), formed once per step; f is the dynamics given them.
+
 // Quadrotor, 12 states (position, velocity, ZYX Euler angles phi/theta/psi,
 // body rates), 4 rotor thrusts in a "+" layout.
-// prm: m, Jx, Jy, Jz, arm, km (yaw moment per unit thrust), drag, g.
+// prm: m, Jx, Jy, Jz, arm, km (yaw moment per unit thrust), drag, g | 1/m, 1/Jx,
+// 1/Jy, 1/Jz, drag/m, (Jz-Jy)/Jx, (Jx-Jz)/Jy, (Jy-Jx)/Jz.
+__host__ __device__ inline double rigid_param(const double* p, int k, int m, int jx) {
+  const double Jx = p[jx], Jy = p[jx + 1], Jz = p[jx + 2];
+  switch (k) {
+    case 8: return 1.0 / p[m];
+    case 9: return 1.0 / Jx;
+    case 10: return 1.0 / Jy;
+    case 11: return 1.0 / Jz;
+    case 13: return (Jz - Jy) / Jx;
+    case 14: return (Jx - Jz) / Jy;
+    default: return (Jy - Jx) / Jz;
+  }
+}
 struct Quad12 {
   static constexpr int NX = 12, NU = 4;
+  __host__ __device__ static double derived(const double* p, int k) {
+    return k == 12 ? p[6] / p[0] : rigid_param(p, k, 0, 1);
+  }
+  template <class S> struct Held { S Fm, ax, ay, az; };
   template <class S, class P>
-  __device__ static void f(const P* prm, const S* x, const S* u, S* xd) {
+  __device__ static __forceinline__ Held<S> hold(const P* prm, const S* u) {
     typedef typename BaseOf<S>::type R;
-    const R m = (R)prm[0], Jx = (R)prm[1], Jy = (R)prm[2], Jz = (R)prm[3];
-    const R arm = (R)prm[4], km = (R)prm[5], cd = (R)prm[6], g = (R)prm[7];
-    const S sph = sin_(x[6]), cph = cos_(x[6]);
-    const S sth = sin_(x[7]), cth = cos_(x[7]);
-    const S sps = sin_(x[8]), cps = cos_(x[8]);
-    const S F = u[0] + u[1] + u[2] + u[3];
+    const R arm = (R)prm[4], km = (R)prm[5];
+    Held<S> H;
+    H.Fm = (u[0] + u[1] + u[2] + u[3]) * (R)prm[8];
+    H.ax = (arm * (R)prm[9]) * (u[1] - u[3]);
+    H.ay = (arm * (R)prm[10]) * (u[2] - u[0]);
+    H.az = (km * (R)prm[11]) * (u[0] - u[1] + u[2] - u[3]);
+    return H;
+  }
+  template <class S, class P>
+  __device__ static __forceinline__ void f(const P* prm, const S* x, const Held<S>& H, S* xd) {
+    typedef typename BaseOf<S>::type R;
+    const R g = (R)prm[7], cdm = (R)prm[12];
+    S sph, cph, sth, cth, sps, cps;
+    sincos_(x[6], sph, cph);
+    sincos_(x[7], sth, cth);
+    sincos_(x[8], sps, cps);
     // third column of R = Rz(psi) Ry(theta) Rx(phi): the body thrust axis in the world frame
-    const S a0 = cph * sth * cps + sph * sps;
-    const S a1 = cph * sth * sps - sph * cps;
-    const S a2 = cph * cth;
+    const S cs = cph * sth;
     xd[0] = x[3];
     xd[1] = x[4];
     xd[2] = x[5];
-    xd[3] = a0 * F / m - (cd / m) * x[3];
-    xd[4] = a1 * F / m - (cd / m) * x[4];
-    xd[5] = a2 * F / m - g - (cd / m) * x[5];
+    xd[3] = (cs * cps + sph * sps) * H.Fm - cdm * x[3];
+    xd[4] = (cs * sps - sph * cps) * H.Fm - cdm * x[4];
+    xd[5] = (cph * cth) * H.Fm - g - cdm * x[5];
     const S wx = x[9], wy = x[10], wz = x[11];
-    const S tth = sth / cth;
     // Euler-angle rates from body rates (ZYX kinematics)
-    xd[6] = wx + sph * tth * wy + cph * tth * wz;
+    const S w = (sph * wy + cph * wz) / cth;
+    xd[6] = wx + sth * w;
     xd[7] = cph * wy - sph * wz;
-    xd[8] = (sph * wy + cph * wz) / cth;
+    xd[8] = w;
     // rigid-body rotation: J w' = tau - w x (J w)
-    const S tx = arm * (u[1] - u[3]);
-    const S ty = arm * (u[2] - u[0]);
-    const S tz = km * (u[0] - u[1] + u[2] - u[3]);
-    xd[9] = (tx - (Jz - Jy) * wy * wz) / Jx;
-    xd[10] = (ty - (Jx - Jz) * wz * wx) / Jy;
-    xd[11] = (tz - (Jy - Jx) * wx * wy) / Jz;
+    xd[9] = H.ax - (R)prm[13] * (wy * wz);
+    xd[10] = H.ay - (R)prm[14] * (wz * wx);
+    xd[11] = H.az - (R)prm[15] * (wx * wy);
   }
 };
 
@@ -228,32 +254,42 @@ struct Quad12 {
 // body torques (Sec. IV-A1).  prm as Quad12 (arm and km unused).
 struct Quat13 {
   static constexpr int NX = 13, NU = 4;
+  __host__ __device__ static double derived(const double* p, int k) { return Quad12::derived(p, k); }
+  template <class S> struct Held { S Tm, ax, ay, az; };
   template <class S, class P>
-  __device__ static void f(const P* prm, const S* x, const S* u, S* xd) {
+  __device__ static __forceinline__ Held<S> hold(const P* prm, const S* u) {
     typedef typename BaseOf<S>::type R;
-    const R m = (R)prm[0], Jx = (R)prm[1], Jy = (R)prm[2], Jz = (R)prm[3];
-    const R cd = (R)prm[6], g = (R)prm[7];
+    Held<S> H;
+    H.Tm = u[0] * (R)prm[8];
+    H.ax = u[1] * (R)prm[9];
+    H.ay = u[2] * (R)prm[10];
+    H.az = u[3] * (R)prm[11];
+    return H;
+  }
+  template <class S, class P>
+  __device__ static __forceinline__ void f(const P* prm, const S* x, const Held<S>& H, S* xd) {
+    typedef typename BaseOf<S>::type R;
+    const R g = (R)prm[7], cdm = (R)prm[12];
     const S qw = x[6], qx = x[7], qy = x[8], qz = x[9];
     const S wx = x[10], wy = x[11], wz = x[12];
     // body z axis in the world frame, R(q) e3 (quadratic form, exact for unit q)
     const S a0 = R(2) * (qx * qz + qw * qy);
     const S a1 = R(2) * (qy * qz - qw * qx);
     const S a2 = qw * qw - qx * qx - qy * qy + qz * qz;
-    const S Tm = u[0] / m;
     xd[0] = x[3];
     xd[1] = x[4];
     xd[2] = x[5];
-    xd[3] = a0 * Tm - (cd / m) * x[3];
-    xd[4] = a1 * Tm - (cd / m) * x[4];
-    xd[5] = a2 * Tm - g - (cd / m) * x[5];
+    xd[3] = a0 * H.Tm - cdm * x[3];
+    xd[4] = a1 * H.Tm - cdm * x[4];
+    xd[5] = a2 * H.Tm - g - cdm * x[5];
     // q' = q (x) (0, w) / 2
     xd[6] = R(0.5) * (-(qx * wx) - qy * wy - qz * wz);
     xd[7] = R(0.5) * (qw * wx + qy * wz - qz * wy);
     xd[8] = R(0.5) * (qw * wy - qx * wz + qz * wx);
     xd[9] = R(0.5) * (qw * wz + qx * wy - qy * wx);
-    xd[10] = (u[1] - (Jz - Jy) * wy * wz) / Jx;
-    xd[11] = (u[2] - (Jx - Jz) * wz * wx) / Jy;
-    xd[12] = (u[3] - (Jy - Jx) * wx * wy) / Jz;
+    xd[10] = H.ax - (R)prm[13] * (wy * wz);
+    xd[11] = H.ay - (R)prm[14] * (wz * wx);
+    xd[12] = H.az - (R)prm[15] * (wx * wy);
   }
 };
 
@@ -262,31 +298,27 @@ struct Quat13 {
 // unit thrust), non-dimensional units.
 struct Mars7 {
   static constexpr int NX = 7, NU = 3;
-  // The mass rate -alpha |T|, which depends on the control alone: constant over
-  // an RK4 step (the control is held), so rk4h forms it once per step.
+  __host__ __device__ static double derived(const double*, int) { return 0.0; }
+  // the mass rate -alpha |T| depends on the control alone
+  template <class S> struct Held { S u0, u1, u2, mdot; };
   template <class S, class P>
-  __device__ static S mass_rate(const P* prm, const S* u) {
+  __device__ static __forceinline__ Held<S> hold(const P* prm, const S* u) {
     typedef typename BaseOf<S>::type R;
-    const R alpha = (R)prm[1];
     const S Tn = sqrt_(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-    return -(alpha * Tn);
+    return {u[0], u[1], u[2], -((R)prm[1] * Tn)};
   }
   template <class S, class P>
-  __device__ static void f_held(const P* prm, const S* x, const S* u, const S& mdot, S* xd) {
+  __device__ static __forceinline__ void f(const P* prm, const S* x, const Held<S>& H, S* xd) {
     typedef typename BaseOf<S>::type R;
     const R g = (R)prm[0];
     const S im = R(1) / x[6];   // one division per evaluation (GB300's FP64 divide is costly)
     xd[0] = x[3];
     xd[1] = x[4];
     xd[2] = x[5];
-    xd[3] = u[0] * im - g;
-    xd[4] = u[1] * im;
-    xd[5] = u[2] * im;
-    xd[6] = mdot;
-  }
-  template <class S, class P>
-  __device__ static void f(const P* prm, const S* x, const S* u, S* xd) {
-    f_held(prm, x, u, mass_rate(prm, u), xd);
+    xd[3] = H.u0 * im - g;
+    xd[4] = H.u1 * im;
+    xd[5] = H.u2 * im;
+    xd[6] = H.mdot;
   }
 };
 
@@ -294,79 +326,86 @@ struct Mars7 {
 // (Up-East-North), velocity, quaternion body-to-world scalar first, body rates;
 // control = thrust in the body frame (body x = thrust axis).  prm: alpha (mass
 // flow per unit thrust), g (along -Up), Jx, Jy, Jz, l (the thrust acts at
-// -l e_x in the body).  Non-dimensional units.
+// -l e_x in the body) | l/Jy at 10, l/Jz at 11, the inertia quotients at 13..15.
+// Non-dimensional units.
 struct Mars14 {
   static constexpr int NX = 14, NU = 3;
+  __host__ __device__ static double derived(const double* p, int k) {
+    return k == 10 ? p[5] / p[3] : k == 11 ? p[5] / p[4] : k >= 13 ? rigid_param(p, k, 0, 2) : 0.0;
+  }
+  template <class S> struct Held { S u0, u1, u2, mdot, ay, az; };
   template <class S, class P>
-  __device__ static void f(const P* prm, const S* x, const S* u, S* xd) {
+  __device__ static __forceinline__ Held<S> hold(const P* prm, const S* u) {
     typedef typename BaseOf<S>::type R;
-    const R alpha = (R)prm[0], g = (R)prm[1], Jx = (R)prm[2], Jy = (R)prm[3], Jz = (R)prm[4], l = (R)prm[5];
+    const S Tn = sqrt_(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+    return {u[0], u[1], u[2], -((R)prm[0] * Tn), (R)prm[10] * u[2], (R)prm[11] * u[1]};
+  }
+  template <class S, class P>
+  __device__ static __forceinline__ void f(const P* prm, const S* x, const Held<S>& H, S* xd) {
+    typedef typename BaseOf<S>::type R;
+    const R g = (R)prm[1];
     const S qw = x[7], qx = x[8], qy = x[9], qz = x[10];
     const S wx = x[11], wy = x[12], wz = x[13];
-    const S Tn = sqrt_(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
     const S im = R(1) / x[0];
     // rotation body -> world (quadratic form), applied to the body thrust
     const S c00 = qw * qw + qx * qx - qy * qy - qz * qz, c01 = R(2) * (qx * qy - qw * qz), c02 = R(2) * (qx * qz + qw * qy);
     const S c10 = R(2) * (qx * qy + qw * qz), c11 = qw * qw - qx * qx + qy * qy - qz * qz, c12 = R(2) * (qy * qz - qw * qx);
     const S c20 = R(2) * (qx * qz - qw * qy), c21 = R(2) * (qy * qz + qw * qx), c22 = qw * qw - qx * qx - qy * qy + qz * qz;
-    xd[0] = -(alpha * Tn);
+    xd[0] = H.mdot;
     xd[1] = x[4];
     xd[2] = x[5];
     xd[3] = x[6];
-    xd[4] = (c00 * u[0] + c01 * u[1] + c02 * u[2]) * im - g;
-    xd[5] = (c10 * u[0] + c11 * u[1] + c12 * u[2]) * im;
-    xd[6] = (c20 * u[0] + c21 * u[1] + c22 * u[2]) * im;
+    xd[4] = (c00 * H.u0 + c01 * H.u1 + c02 * H.u2) * im - g;
+    xd[5] = (c10 * H.u0 + c11 * H.u1 + c12 * H.u2) * im;
+    xd[6] = (c20 * H.u0 + c21 * H.u1 + c22 * H.u2) * im;
     xd[7] = R(0.5) * (-(qx * wx) - qy * wy - qz * wz);
     xd[8] = R(0.5) * (qw * wx + qy * wz - qz * wy);
     xd[9] = R(0.5) * (qw * wy - qx * wz + qz * wx);
     xd[10] = R(0.5) * (qw * wz + qx * wy - qy * wx);
     // J w' = r_T x T - w x (J w), r_T = (-l, 0, 0): r_T x T = (0, l T_z, -l T_y)
-    xd[11] = (-((Jz - Jy) * wy * wz)) / Jx;
-    xd[12] = (l * u[2] - (Jx - Jz) * wz * wx) / Jy;
-    xd[13] = (-(l * u[1]) - (Jy - Jx) * wx * wy) / Jz;
+    xd[11] = -((R)prm[13] * (wy * wz));
+    xd[12] = H.ay - (R)prm[14] * (wz * wx);
+    xd[13] = -H.az - (R)prm[15] * (wx * wy);
   }
 };
+
+// Entry k of a model's constants from the problem's eight.
+template <class M>
+__host__ __device__ inline double derived_param(const double* p, int k) {
+  return k < 8 ? p[k] : M::derived(p, k);
+}
 
 // a + b c in the type of a and c (one fused pass for double-float).
 template <class S, class R> __device__ __forceinline__ S fma_(S a, R b, S c) { return a + b * c; }
 __device__ __forceinline__ DF fma_(DF a, DF b, DF c) { return df_fma(a, b, c); }
 
-// f with the control held over an RK4 step, as a callable x -> x-dot.  For
-// the 3-DOF Mars model the control-only part (the mass rate) is formed once,
-// at construction, instead of at each of the four stages: the same numbers.
-template <class M, class S, class P>
-struct HeldControl {
-  const P* prm;
-  const S* u;
-  __device__ __forceinline__ HeldControl(const P* p, const S* uu) : prm(p), u(uu) {}
-  __device__ __forceinline__ void operator()(const S* x, S* xd) const { M::f(prm, x, u, xd); }
-};
-template <class S, class P>
-struct HeldControl<Mars7, S, P> {
-  const P* prm;
-  const S* u;
-  S mdot;
-  __device__ __forceinline__ HeldControl(const P* p, const S* uu) : prm(p), u(uu), mdot(Mars7::mass_rate(p, uu)) {}
-  __device__ __forceinline__ void operator()(const S* x, S* xd) const { Mars7::f_held(prm, x, u, mdot, xd); }
-};
-
 // Classical fourth-order Runge-Kutta step (Eq. (1b)) with the step h and its
-// multiples h/2, h/6 given in the base type R of S.
+// multiples h/2, h/6 given in the base type R of S.  The four stages are one
+// loop: unrolled, a step of the larger models is 30 to 180 KB of code that runs
+// once per SCP iteration, and the instruction fetch is what it waits for.  The
+// 3-DOF Mars model's step is small; rolled, its kernels spill in the ADMM loop.
 template <class M, class S, class P, class R>
 __device__ __forceinline__ void rk4h(const P* prm, R h, R hh, R h6, const S* x, const S* u, S* xn) {
   constexpr int NX = M::NX;
   S k[NX], t[NX], acc[NX];
-  const HeldControl<M, S, P> F(prm, u);
-  F(x, k);
+  const typename M::template Held<S> H = M::template hold<S, P>(prm, u);
 #pragma unroll
-  for (int j = 0; j < NX; ++j) { acc[j] = k[j]; t[j] = fma_(x[j], hh, k[j]); }
-  F(t, k);
+  for (int j = 0; j < NX; ++j) t[j] = x[j];
+#pragma unroll (M::NX == 7 ? 4 : 1)
+  for (int s = 0; s < 4; ++s) {
+    M::template f<S, P>(prm, t, H, k);
+    if (s == 3) break;
+    const R w = s == 2 ? h : hh;
+    if (s == 0) {
 #pragma unroll
-  for (int j = 0; j < NX; ++j) { acc[j] = fma_(acc[j], R(2), k[j]); t[j] = fma_(x[j], hh, k[j]); }
-  F(t, k);
+      for (int j = 0; j < NX; ++j) acc[j] = k[j];
+    } else {
 #pragma unroll
-  for (int j = 0; j < NX; ++j) { acc[j] = fma_(acc[j], R(2), k[j]); t[j] = fma_(x[j], h, k[j]); }
-  F(t, k);
+      for (int j = 0; j < NX; ++j) acc[j] = fma_(acc[j], R(2), k[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < NX; ++j) t[j] = fma_(x[j], w, k[j]);
+  }
 #pragma unroll
   for (int j = 0; j < NX; ++j) xn[j] = fma_(x[j], h6, acc[j] + k[j]);
 }

@@ -623,6 +623,8 @@ __global__ void __launch_bounds__(PAIR_MAX_THREADS, 2) scp_kernel_pair(ProblemDe
     split_barrier_init(sh.xbar, blockDim.x);
   }
   X.bar = sh.xbar;
+  nd.prm = ndd.prm = sh.prm;
+  stage_params<M>(sh, P, b);
   stage_consts<M, float, true>(ndd, P, b);
   if (dact) load_nominal<M, float, true>(ndd, L, x0, u0, xo, uo);
   __syncthreads();
@@ -648,7 +650,7 @@ __global__ void __launch_bounds__(PAIR_MAX_THREADS, 2) scp_kernel_pair(ProblemDe
     __syncthreads();
     const float re = sh.rhof[0], rd = sh.rhof[1], rg = sh.rhof[2];
     const double radius = sh.radius;
-    pair_jacobians<M>(nd, PM, I.prm, hs, q, has_u);
+    pair_jacobians<M>(nd, PM, sh.prmf, hs, q, has_u);
     if (dact) {
       node_setup<M, float, true>(ndd, L, P, I, b, radius, re, rg, Kd);
       node_reseed<M, float, true>(ndd, L, I);

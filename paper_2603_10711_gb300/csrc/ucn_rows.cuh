@@ -649,7 +649,7 @@ __device__ __forceinline__ void rows_put_column(RowMats<M>& A, const float* col,
     A.g[m][k][1] = on ? float2{got[2], got[3]} : float2{0.0f, 0.0f};
   }
 }
-template <class M>
+template <class M, int K>
 __device__ __forceinline__ void rows_jacobians(const RowPos& p, const Node<float, 2>& nd, RowMats<M>& A,
                                                const float* prm, const Step3<float>& hs) {
   constexpr int NX = M::NX, NU = M::NU, RX = RowMats<M>::RX;
@@ -658,12 +658,20 @@ __device__ __forceinline__ void rows_jacobians(const RowPos& p, const Node<float
   for (int j = 0; j < NX; ++j) xt[j] = df_to_float(nd.dat(Rec<M>::Xbar, j));
 #pragma unroll
   for (int j = 0; j < NU; ++j) ut[j] = p.hasU ? df_to_float(nd.dat(Rec<M>::Ubar, j)) : 1.0f;
+  // one pass of code for all columns (what the set-up phases wait for is
+  // instruction fetch): the columns move up a group per pass, so that the
+  // register indexes stay fixed
+#pragma unroll 1
+  for (int k = 0; k < 4; k += K) {
+    float cols[K][NX];
+    if constexpr (K == 2) rk4_jvpn<M, float, 2>(prm, hs, xt, ut, p.q + 4 * k, 4, cols);
+    else rk4_jvp<M, float>(prm, hs, xt, ut, p.q + 4 * k, cols[0]);
 #pragma unroll
-  for (int k = 0; k < 4; k += 2) {
-    float cols[2][NX];
-    rk4_jvpn<M, float, 2>(prm, hs, xt, ut, p.q + 4 * k, 4, cols);
-    rows_put_column<M>(A, cols[0], k, p.q, p.hasU);
-    rows_put_column<M>(A, cols[1], k + 1, p.q, p.hasU);
+    for (int m = 0; m < RX; ++m)
+#pragma unroll
+      for (int c = 0; c + K < 4; ++c) { A.g[m][c][0] = A.g[m][c + K][0]; A.g[m][c][1] = A.g[m][c + K][1]; }
+#pragma unroll
+    for (int c = 0; c < K; ++c) rows_put_column<M>(A, cols[c], 4 - K + c, p.q, p.hasU);
   }
   if constexpr (RowMats<M>::EX) {   // column 16: the same pass in all four lanes
     float col[NX];
@@ -804,7 +812,7 @@ __device__ __forceinline__ float rows_obstacle_setup(const RowPos& p, const Node
 template <class M>
 __device__ __forceinline__ bool rows_factor(const RowPos& p, RowMats<M>& A, const RowConst<M>& K, const Inst<float>& I,
                                             float rd, float rg) {
-  constexpr int NX = M::NX;
+  constexpr int RX = RowMats<M>::RX;
   constexpr bool EX = RowMats<M>::EX, QUAD = IsQuad<M>::value;
   const int q = p.q;
   float h[4][16], hx[4], rx[17];   // own rows, their column 16, row 16
@@ -816,28 +824,48 @@ __device__ __forceinline__ bool rows_factor(const RowPos& p, RowMats<M>& A, cons
   }
 #pragma unroll
   for (int c = 0; c < 17; ++c) rx[c] = 0.0f;
+  // sum over the rows of G of their outer products: a group of four rows (one
+  // per lane) per pass, the groups moving up in between
+#pragma unroll 1
+  for (int k0 = 0; k0 < RX; ++k0) {
 #pragma unroll
-  for (int k = 0; k < NX; ++k) {   // sum over rows k of G of their outer products
-    const int o = k & 3, m0 = k >> 2;
-    float row[17];
+    for (int o = 0; o < 4; ++o) {
+      float row[17];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      row[4 * c + (0 ^ o)] = rows_from(A.g[m0][c][0].x, o);
-      row[4 * c + (1 ^ o)] = rows_from(A.g[m0][c][0].y, o);
-      row[4 * c + (2 ^ o)] = rows_from(A.g[m0][c][1].x, o);
-      row[4 * c + (3 ^ o)] = rows_from(A.g[m0][c][1].y, o);
+      for (int c = 0; c < 4; ++c) {
+        row[4 * c + (0 ^ o)] = rows_from(A.g[0][c][0].x, o);
+        row[4 * c + (1 ^ o)] = rows_from(A.g[0][c][0].y, o);
+        row[4 * c + (2 ^ o)] = rows_from(A.g[0][c][1].x, o);
+        row[4 * c + (3 ^ o)] = rows_from(A.g[0][c][1].y, o);
+      }
+      if constexpr (EX) row[16] = rows_from(A.gx[0], o);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const float f = sel4(row[4 * m], row[4 * m + 1], row[4 * m + 2], row[4 * m + 3], q);
+#pragma unroll
+        for (int c = 0; c < 16; ++c) h[m][c] += f * row[c];
+        if constexpr (EX) hx[m] += f * row[16];
+      }
+      if constexpr (EX) {
+#pragma unroll
+        for (int c = 0; c < 17; ++c) rx[c] += row[16] * row[c];
+      }
     }
-    if constexpr (EX) row[16] = rows_from(A.gx[m0], o);
+    // (after RX passes the rows are back in place)
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      const float f = sel4(row[4 * m], row[4 * m + 1], row[4 * m + 2], row[4 * m + 3], q);
+    for (int c = 0; c < 4; ++c)
 #pragma unroll
-      for (int c = 0; c < 16; ++c) h[m][c] += f * row[c];
-      if constexpr (EX) hx[m] += f * row[16];
-    }
+      for (int s = 0; s < 2; ++s) {
+        const float2 t = A.g[0][c][s];
+#pragma unroll
+        for (int m = 0; m + 1 < RX; ++m) A.g[m][c][s] = A.g[m + 1][c][s];
+        A.g[RX - 1][c][s] = t;
+      }
     if constexpr (EX) {
+      const float t = A.gx[0];
 #pragma unroll
-      for (int c = 0; c < 17; ++c) rx[c] += row[16] * row[c];
+      for (int m = 0; m + 1 < RX; ++m) A.gx[m] = A.gx[m + 1];
+      A.gx[RX - 1] = t;
     }
   }
 #pragma unroll
@@ -863,37 +891,71 @@ __device__ __forceinline__ bool rows_factor(const RowPos& p, RowMats<M>& A, cons
     h[3][14] += w * n14; h[3][15] += w * n15; hx[3] += w * K.nx;
     rx[14] += rg * K.nx * n14; rx[15] += rg * K.nx * n15; rx[16] += rg * K.nx * K.nx;
   }
+  // Gauss-Jordan, four pivots (one per lane) per pass; rows and columns rotate by
+  // four in between, back in place after the fourth pass
   bool ok = true;
+#pragma unroll 1
+  for (int k0 = 0; k0 < 4; ++k0) {
 #pragma unroll
-  for (int k = 0; k < (EX ? 17 : 16); ++k) {
-    float row[17], piv;
-    if (k < 16) {
-      const int o = k & 3, m0 = k >> 2;
+    for (int o = 0; o < 4; ++o) {
+      float row[17];
 #pragma unroll
-      for (int c = 0; c < 16; ++c) row[c] = rows_from(h[m0][c], o);
-      if constexpr (EX) row[16] = rows_from(hx[m0], o);
-    } else {
+      for (int c = 0; c < 16; ++c) row[c] = rows_from(h[0][c], o);
+      if constexpr (EX) row[16] = rows_from(hx[0], o);
+      if (!(row[o] > 0.0f)) { ok = false; row[o] = 1.0f; }
+      const float d = __frcp_rn(row[o]);
 #pragma unroll
-      for (int c = 0; c < 17; ++c) row[c] = rx[c];
+      for (int c = 0; c < (EX ? 17 : 16); ++c) row[c] *= d;
+      row[o] = d;
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const float f = h[m][o];
+        const bool mine = m == 0 && q == o;
+#pragma unroll
+        for (int c = 0; c < 16; ++c) h[m][c] = mine ? row[c] : (c == o ? -f * d : h[m][c] - f * row[c]);
+        if constexpr (EX) hx[m] = mine ? row[16] : hx[m] - f * row[16];
+      }
+      if constexpr (EX) {
+        const float f = rx[o];
+#pragma unroll
+        for (int c = 0; c < 17; ++c) rx[c] = c == o ? -f * d : rx[c] - f * row[c];
+      }
     }
-    piv = row[k];
-    if (!(piv > 0.0f)) { ok = false; piv = 1.0f; }
-    const float d = __frcp_rn(piv);
+    float h0[16];
 #pragma unroll
-    for (int c = 0; c < (EX ? 17 : 16); ++c) row[c] *= d;
-    row[k] = d;
+    for (int c = 0; c < 16; ++c) h0[c] = h[0][(c + 4) & 15];
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      float t[16];
+#pragma unroll
+      for (int c = 0; c < 16; ++c) t[c] = h[m + 1][(c + 4) & 15];
+#pragma unroll
+      for (int c = 0; c < 16; ++c) h[m][c] = t[c];
+    }
+#pragma unroll
+    for (int c = 0; c < 16; ++c) h[3][c] = h0[c];
+    if constexpr (EX) {
+      const float x0 = hx[0];
+      hx[0] = hx[1]; hx[1] = hx[2]; hx[2] = hx[3]; hx[3] = x0;
+      float t[16];
+#pragma unroll
+      for (int c = 0; c < 16; ++c) t[c] = rx[(c + 4) & 15];
+#pragma unroll
+      for (int c = 0; c < 16; ++c) rx[c] = t[c];
+    }
+  }
+  if constexpr (EX) {   // the last pivot, row 16
+    if (!(rx[16] > 0.0f)) { ok = false; rx[16] = 1.0f; }
+    const float d = __frcp_rn(rx[16]);
+#pragma unroll
+    for (int c = 0; c < 16; ++c) rx[c] *= d;
+    rx[16] = d;
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
-      const float f = k < 16 ? h[m][k & 15] : hx[m];
-      const bool mine = k < 16 && m == (k >> 2) && q == (k & 3);
+      const float f = hx[m];
 #pragma unroll
-      for (int c = 0; c < 16; ++c) h[m][c] = mine ? row[c] : (c == k ? -f * d : h[m][c] - f * row[c]);
-      if constexpr (EX) hx[m] = mine ? row[16] : (k == 16 ? -f * d : hx[m] - f * row[16]);
-    }
-    if constexpr (EX) {
-      const float f = rx[k];
-#pragma unroll
-      for (int c = 0; c < 17; ++c) rx[c] = k == 16 ? row[c] : (c == k ? -f * d : rx[c] - f * row[c]);
+      for (int c = 0; c < 16; ++c) h[m][c] -= f * rx[c];
+      hx[m] = -f * d;
     }
   }
   // columns into slot order (exchange by the bits of q); threads without a node: zero
@@ -1124,6 +1186,8 @@ __device__ __forceinline__ void scp_rows_body(const ProblemDev& P, const Layout&
   X.bar = sh.xbar;
   // the records start at zero: rows beyond a model's are read, never set
   for (int e = threadIdx.x; e < (L.chunk + (CL ? 2 : 0)) * L.NS; e += blockDim.x) ((float*)smem)[e] = 0.0f;
+  nd.prm = ndd.prm = sh.prm;
+  stage_params<M>(sh, P, b);
   stage_consts<M, float, 2>(ndd, P, b);
   if (dact) load_nominal<M, float, 2>(ndd, L, x0, u0, xo, uo);
   if constexpr (CL) {   // the halo's nominal: the next CTA's first node
@@ -1162,7 +1226,7 @@ __device__ __forceinline__ void scp_rows_body(const ProblemDev& P, const Layout&
     }
     __syncthreads();
     const float re = sh.rhof[0], rd = sh.rhof[1], rg = sh.rhof[2];
-    rows_jacobians<M>(p, nd, A, I.prm, hs);
+    rows_jacobians<M, REG ? 2 : 1>(p, nd, A, sh.prmf, hs);
     const float mg = rows_prepare<M, CL>(p, nd, ndd, dact, L, P, I, b, (float)sh.radius, re, rd, rg, A, K, sh);
     if constexpr (CL) {   // a failed factorisation anywhere stops the instance
       if (sh.fail && threadIdx.x < ncta) st_cluster(&sh.fail, threadIdx.x, 1);
@@ -1278,6 +1342,8 @@ __global__ void __launch_bounds__(MAXT, 1) admm_rows_kernel(ProblemDev P, Layout
   const Inst<float> I = make_inst<M, float>(P, b);
   if (threadIdx.x == 0) { sh.fail = 0; split_barrier_init(sh.xbar, blockDim.x); }
   for (int e = threadIdx.x; e < (L.chunk + (CL ? 2 : 0)) * L.NS; e += blockDim.x) ((float*)smem)[e] = 0.0f;
+  nd.prm = ndd.prm = sh.prm;
+  stage_params<M>(sh, P, b);
   stage_consts<M, float, 2>(ndd, P, b);
   if (dact) load_nominal<M, float, 2>(ndd, L, xbar, ubar, xo, uo);
   __syncthreads();
