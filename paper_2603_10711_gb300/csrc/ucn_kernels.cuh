@@ -358,7 +358,8 @@ __device__ __forceinline__ Inst<T> make_inst(const ProblemDev& P, int b) {
 // Per-instance scalars in shared memory.
 struct InstShared {
   unsigned long long xbar[2];   // split barrier of the ADMM exchange + failure flag
-  double red[32][6];
+  double red[22][6];        // block reductions (CTAs of up to 16 warps); scenario groups also
+                            // receive their peers' values here during an ADMM call (GroupX::in)
   double Jn, radius;
   double rho[3];            // rho_eq, rho_dyn, rho_geo of the SCP iteration
   float rhof[3];            // the same in FP32 (no conversion per thread)
@@ -385,7 +386,8 @@ template <> __device__ __forceinline__ const float* prm_of<float>(const InstShar
 // Per-CTA state of a scenario group's exchanges (one CTA per scenario).
 struct GroupShared {
   double mine[2][16];   // this CTA's contribution to the current exchange (double-buffered)
-  double u0[4];         // the consensus u-hat_0 of the latest iteration, absolute
+  double box[8];        // the scenarios' common box of u_0: max lower, -(min upper), absolute
+  double u0[4];         // the consensus u-hat_0 of the latest iteration, absolute (wide type)
   int gfail;            // sticky: a wait for another scenario of the group gave up
 };
 
@@ -393,6 +395,12 @@ struct GroupShared {
 struct GroupX {
   unsigned epoch;       // exchanges done
   int g, k;             // group index, scenario index within the group
+  unsigned pub;         // consensus exchanges done within one cluster
+  // one cluster per group: the scenarios' Step-3 arguments of u_0 (in the wide
+  // type's 8 bytes), pushed by their CTAs, [2][16][4] double-buffered -- in
+  // InstShared::red, which no reduction uses during an ADMM call (cluster
+  // barriers lie between a CTA's last reduction and its peers' next push)
+  double* in;
   unsigned long long* bar;   // the CTA's split barrier (mbarrier) and its failure flag
   unsigned ph;               // completed phases of the split barrier
 };
@@ -481,6 +489,21 @@ __device__ void group_allreduce_cluster(GroupShared* G, GroupX& X, int ns, doubl
 // scenario can be at most one exchange ahead of another.  A wait that gives up
 // marks the group failed and stops waiting for the rest of the launch (status
 // ETIMEOUT), so the kernel always ends.
+__device__ __forceinline__ bool group_wait(const ProblemDev& P, GroupShared* G, const unsigned* f, unsigned want) {
+  if (G->gfail) return false;
+  // relaxed polling, one acquire once the counter is seen (an acquire per poll
+  // would also cost the SM its L1 lines); the clock is read every 256 polls
+  unsigned long long t0 = 0;
+  for (unsigned spins = 1; ld_relaxed_gpu(f) < want; ++spins) {
+    if ((spins & 255u) == 0u) {
+      const unsigned long long now = globaltimer_ns();
+      if (t0 == 0) t0 = now;
+      else if (now - t0 > P.gwait_ns) { G->gfail = 1; return false; }
+    }
+  }
+  (void)ld_acquire_gpu(f);
+  return true;
+}
 template <int NV>
 __device__ void group_allreduce_flat(const ProblemDev& P, GroupShared* G, GroupX& X, int ns, double* out) {
   static_assert(NV <= 16, "exchange slots hold 16 values");
@@ -498,23 +521,7 @@ __device__ void group_allreduce_flat(const ProblemDev& P, GroupShared* G, GroupX
 #pragma unroll
     for (int j = 0; j < NV; ++j) pv[j] = j < ns ? 0.0 : -INFINITY;
     for (int r = lane; r < K; r += 32) {
-      const unsigned* f = &P.gflag[base + r];
-      bool ok = !G->gfail;
-      if (ok) {
-        // relaxed polling, one acquire once the counter is seen (an acquire per
-        // poll would also cost the SM its L1 lines); the clock is read every
-        // 256 polls
-        unsigned long long t0 = 0;
-        for (unsigned spins = 1; ld_relaxed_gpu(f) < X.epoch + 1; ++spins) {
-          if ((spins & 255u) == 0u) {
-            const unsigned long long now = globaltimer_ns();
-            if (t0 == 0) t0 = now;
-            else if (now - t0 > P.gwait_ns) { ok = false; G->gfail = 1; break; }
-          }
-        }
-        if (ok) (void)ld_acquire_gpu(f);
-      }
-      if (!ok) continue;
+      if (!group_wait(P, G, &P.gflag[base + r], X.epoch + 1)) continue;
       const double* src = P.gx + ((base + r) * 2 + par) * 16;
       double v[NV];
 #pragma unroll
@@ -539,6 +546,128 @@ template <int NV>
 __device__ __forceinline__ void group_allreduce(const ProblemDev& P, GroupShared* G, GroupX& X, int ns, double* out) {
   if (P.gclusters <= 1) group_allreduce_cluster<NV>(G, X, ns, out);
   else group_allreduce_flat<NV>(P, G, X, ns, out);
+}
+
+// The first-control consensus of an ADMM iteration.  Warp 0 of every CTA
+// publishes its scenario's Step-3 arguments as soon as Step 1 is done (lane l
+// holds that of control l mod 4), and collects the group's sums after Step 2:
+// the exchange has Steps 2 and 3 to travel.  The boxes are constant over an
+// ADMM call and are intersected before it (GroupShared::box).  Values are of the
+// wide type W -- double-float on the FP32 path, whose sum of a 64-scenario group
+// is FP32 work: as FP64 all-reduce of twelve values (sums and both bounds) the
+// exchange took 9 us per iteration of a 16-scenario group, the iteration itself
+// 1.6 us.  Every CTA of a group gets the same bits: one order of summation, of
+// an addition that commutes.
+//
+// One cluster per group: each CTA writes its values into all its peers' shared
+// memory before the iteration's cluster barrier.  Several: through its global
+// slot and counter, as group_allreduce_flat.
+__device__ __forceinline__ double wide_shfl_xor(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ DF wide_shfl_xor(DF a, int o) {
+  return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
+}
+__device__ __forceinline__ double wide_shfl(double a, int l) { return __shfl_sync(0xffffffffu, a, l); }
+__device__ __forceinline__ DF wide_shfl(DF a, int l) {
+  return {__shfl_sync(0xffffffffu, a.hi, l), __shfl_sync(0xffffffffu, a.lo, l)};
+}
+__device__ __forceinline__ double wide_bits(double a) { return a; }
+__device__ __forceinline__ double wide_bits(DF a) { return __hiloint2double(__float_as_int(a.lo), __float_as_int(a.hi)); }
+template <class W> __device__ __forceinline__ W wide_of_bits(double a);
+template <> __device__ __forceinline__ double wide_of_bits<double>(double a) { return a; }
+template <> __device__ __forceinline__ DF wide_of_bits<DF>(double a) {
+  return {__int_as_float(__double2loint(a)), __int_as_float(__double2hiint(a))};
+}
+template <class W>
+__device__ __forceinline__ void group_publish(const ProblemDev& P, GroupShared* G, const GroupX& X, W v) {
+  const int lane = threadIdx.x, j = lane & 3;
+  const double bits = wide_bits(v);
+  if (P.gclusters <= 1) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int r = (lane >> 2) + 8 * h;
+      if (r < P.group) st_cluster(X.in + ((X.pub & 1) * 16 + X.k) * 4 + j, (unsigned)r, bits);
+    }
+  } else {
+    double* slot = P.gx + (((long long)X.g * P.group + X.k) * 2 + (X.epoch & 1)) * 16;
+    if (lane < 4) {
+      __stcg(slot + j, bits);
+      __threadfence();
+    }
+    __syncwarp();
+    if (lane == 0) st_release_gpu(&P.gflag[(long long)X.g * P.group + X.k], X.epoch + 1);
+  }
+}
+template <class W>
+__device__ __forceinline__ W group_collect(const ProblemDev& P, GroupShared* G, const GroupX& X) {
+  const int lane = threadIdx.x, j = lane & 3, K = P.group;
+  W a = W();
+  if (P.gclusters <= 1) {
+    const double* in = X.in + (X.pub & 1) * 64;
+    if ((lane >> 2) < K) a = wide_of_bits<W>(in[4 * (lane >> 2) + j]);
+    if ((lane >> 2) + 8 < K) a = a + wide_of_bits<W>(in[4 * (lane >> 2) + 32 + j]);
+#pragma unroll
+    for (int o = 4; o <= 16; o <<= 1) a = a + wide_shfl_xor(a, o);
+    return a;
+  }
+  const long long base = (long long)X.g * K;
+  W s[4] = {W(), W(), W(), W()};
+  for (int r = lane; r < K; r += 32) {
+    if (!group_wait(P, G, &P.gflag[base + r], X.epoch + 1)) continue;
+    const double* src = P.gx + ((base + r) * 2 + (X.epoch & 1)) * 16;
+    double v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = __ldcg(src + i);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s[i] = s[i] + wide_of_bits<W>(v[i]);
+  }
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s[i] = s[i] + wide_shfl_xor(s[i], o);
+  const W lo = (j & 1) ? s[1] : s[0], hi = (j & 1) ? s[3] : s[2];
+  return (j & 2) ? hi : lo;
+}
+// Both are done (every thread's sequence state).
+__device__ __forceinline__ void group_advance(const ProblemDev& P, GroupX& X) {
+  if (P.gclusters <= 1) X.pub++;
+  else X.epoch++;
+}
+// The average of the K arguments of control j, clamped to the common box.
+__device__ __forceinline__ double group_mean(const GroupShared* G, double sum, int K, int j) {
+  return fmin(fmax(sum / (double)K, G->box[j]), -G->box[4 + j]);
+}
+__device__ __forceinline__ bool df_less(DF a, DF b) { return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo); }
+__device__ __forceinline__ DF group_mean(const GroupShared* G, DF sum, int K, int j) {
+  DF v = df_div(sum, df_from((float)K));
+  const DF lo = wide_of_bits<DF>(G->box[j]), hi = wide_of_bits<DF>(G->box[4 + j]);
+  if (df_less(v, lo)) v = lo;
+  if (df_less(hi, v)) v = hi;
+  return v;
+}
+// The common box of u_0 and whether any scenario's factorisation failed, before
+// an ADMM call; lo, hi: absolute, this scenario's, by the thread(s) of node 0
+// for the controls j they hold (put in G->mine beforehand, entries 1 + j and 5 + j).
+template <class W>
+__device__ __forceinline__ void group_box_put(GroupShared* G, const GroupX& X, int j, W lo, W hi) {
+  double* m = G->mine[X.epoch & 1];
+  m[1 + j] = wide_to_double(lo);
+  m[5 + j] = -wide_to_double(hi);
+}
+template <class W>
+__device__ __forceinline__ void group_begin(const ProblemDev& P, GroupShared* G, GroupX& X, InstShared& sh) {
+  if (threadIdx.x == 0) G->mine[X.epoch & 1][0] = (double)sh.fail;
+  double a[9];
+  group_allreduce<9>(P, G, X, 0, a);
+  if (threadIdx.x == 0) {
+    sh.fail = a[0] != 0.0;
+    for (int j = 0; j < 4; ++j) {
+      const double hi = -a[5 + j];
+      G->box[j] = wide_bits(wide_from_double<W>(a[1 + j]));
+      // (the FP64 form keeps the negated bound, as it was exchanged)
+      G->box[4 + j] = std::is_same<W, double>::value ? a[5 + j] : wide_bits(wide_from_double<W>(hi));
+    }
+  }
+  __syncthreads();
 }
 
 // The end of a group kernel: no CTA of a one-cluster group may exit while
@@ -1356,6 +1485,17 @@ __device__ __forceinline__ void node_mirrors(const Node<T, AOS>& nd, const Layou
   }
 }
 
+// The barrier between Steps 1 and 2 of a scenario group: the cluster's (the
+// peers' arguments have arrived with it) or, across clusters, the CTA's.
+__device__ __forceinline__ void group_arrive(const ProblemDev& P, GroupX& X) {
+  if (P.gclusters <= 1) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  else split_barrier_arrive(X.bar);
+}
+__device__ __forceinline__ void group_arrived(const ProblemDev& P, GroupX& X) {
+  if (P.gclusters <= 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  else split_barrier_wait(X.bar, X.ph);
+}
+
 // Mirror initialisation / re-seeding from (x-hat, u-hat) in deviations.
 template <class M, class T, int AOS>
 __device__ void node_reseed(const Node<T, AOS>& nd, const Layout& L, const Inst<T>& I) {
@@ -1437,8 +1577,21 @@ __device__ __forceinline__ void admm_iteration(const Node<T, AOS>& nd, const MS&
     // between the arrival on the split barrier (Ex1 published) and the wait
     // for the left neighbour's Ex1 that Step 2 needs: a warp that is ahead
     // projects instead of idling at a barrier.
-    if constexpr (GROUP) __syncthreads();   // groups: their exchange follows Step 2 on a plain barrier
-    else split_barrier_arrive(X.bar);
+    if constexpr (GROUP) {
+      if (threadIdx.x < 32) {   // node 0 is lane 0; lane l hands over control l mod 4
+        typedef typename Node<T, AOS>::W W;
+        W own = W();
+#pragma unroll
+        for (int j = 0; j < NU; ++j) {
+          W v = W();
+          if (i == 0) v = wide_add(nd.dat(Rec<M, AOS>::Ubar, j), x[NX + j] + S.nuu(j) * irg);
+          v = wide_shfl(v, 0);
+          if (((int)threadIdx.x & 3) == j) own = v;
+        }
+        group_publish<W>(P, G, X, own);
+      }
+      group_arrive(P, X);
+    } else split_barrier_arrive(X.bar);
     T dz[NX];
     T sv[NN];
 #pragma unroll
@@ -1458,14 +1611,7 @@ __device__ __forceinline__ void admm_iteration(const Node<T, AOS>& nd, const MS&
         for (int j = 0; j < NU; ++j) {
           const T nuu = S.nuu(j);
           if constexpr (GROUP) {
-            if (i == 0) {   // sum of arguments | max of lower bounds | max of -upper bounds
-              const double ub = wide_to_double(nd.dat(Rec<M, AOS>::Ubar, j));
-              double* m = G->mine[X.epoch & 1];
-              m[j] = ub + (double)(x[NX + j] + nuu * irg);
-              m[NU + j] = ub + (double)nd.at(Rec<M, AOS>::Ulo, j);
-              m[2 * NU + j] = -(ub + (double)nd.at(Rec<M, AOS>::Uhi, j));
-              continue;
-            }
+            if (i == 0) continue;   // the consensus sets it
           }
           const T uh = clampv(x[NX + j] + nuu * irg, nd.at(Rec<M, AOS>::Ulo, j), nd.at(Rec<M, AOS>::Uhi, j));
           if (last) { sv[NX + j] += rg * (uh - nd.at(Rec<M, AOS>::Uh, j)); acc_sq_diff(rp, x[NX + j], uh); }
@@ -1475,7 +1621,8 @@ __device__ __forceinline__ void admm_iteration(const Node<T, AOS>& nd, const MS&
       }
       node_mirrors<M, T, AOS, NN>(nd, L, I, rg, irg, x, false, last, sv, rp);   // control sets: i < N only
     }
-    if constexpr (!GROUP) split_barrier_wait(X.bar, X.ph);
+    if constexpr (GROUP) group_arrived(P, X);
+    else split_barrier_wait(X.bar, X.ph);
     if (active) {
       // ---- Step 2: dynamic consensus, Eq. (5), then its duals (Step 4)
       if (i >= 1) {
@@ -1498,14 +1645,20 @@ __device__ __forceinline__ void admm_iteration(const Node<T, AOS>& nd, const MS&
       }
     }
     if constexpr (GROUP) {
-      double tot[3 * NU];
-      group_allreduce<3 * NU>(P, G, X, NU, tot);
+      typedef typename Node<T, AOS>::W W;
+      W tot[NU];
+      if (threadIdx.x < 32) {
+        const W sum = group_collect<W>(P, G, X);
+#pragma unroll
+        for (int j = 0; j < NU; ++j) tot[j] = wide_shfl(sum, j);
+      }
+      group_advance(P, X);
       if (active && i == 0 && i < N) {
 #pragma unroll
         for (int j = 0; j < NU; ++j) {
-          const double v = fmin(fmax(tot[j] / (double)P.group, tot[NU + j]), -tot[2 * NU + j]);
-          G->u0[j] = v;
-          const T uh = (T)(v - wide_to_double(nd.dat(Rec<M, AOS>::Ubar, j)));
+          const W v = group_mean(G, tot[j], P.group, j);
+          G->u0[j] = wide_bits(v);
+          const T uh = wide_diff<T>(v, nd.dat(Rec<M, AOS>::Ubar, j));
           const T nuu = S.nuu(j);
           if (last) { sv[NX + j] += rg * (uh - nd.at(Rec<M, AOS>::Uh, j)); acc_sq_diff(rp, x[NX + j], uh); }
           nd.at(Rec<M, AOS>::Uh, j) = uh;
@@ -1888,7 +2041,7 @@ __global__ void __launch_bounds__(MAX_THREADS) admm_kernel(ProblemDev P, Layout 
   }
   __syncthreads();
   double r2[2] = {0.0, 0.0};
-  GroupX X{0u, 0, 0, sh.xbar, 0u};
+  GroupX X{0u, 0, 0, 0u, nullptr, sh.xbar, 0u};
   if (!sh.fail) admm_iterations<M, T, AOS, REFINE>(nd, MT, L, I, K, active, re, rd, rg, iters, sh, r2, nullptr, X, P);
   if (active) {
     node_export<M, T, AOS>(nd, L, P, b, P.state_abs + P.soff[b]);
@@ -2040,7 +2193,7 @@ __device__ void scp_candidate(const Node<T, AOS>& nd, const MS& MT, const Proble
     if constexpr (GROUP) {
       // the shared first control exactly (bitwise equal across the group)
       if (i == 0)
-        for (int j = 0; j < NU; ++j) uc[j] = wide_from_double<W>(G->u0[j]);
+        for (int j = 0; j < NU; ++j) uc[j] = wide_of_bits<W>(G->u0[j]);
     }
   }
   __syncthreads();
@@ -2245,6 +2398,7 @@ __device__ __forceinline__ void scp_body(const ProblemDev& P, const Layout& L, c
     split_barrier_init(sh.xbar, blockDim.x);
   }
   X.bar = sh.xbar;
+  X.in = &sh.red[0][0];
   nd.prm = sh.prm;
   stage_params<M>(sh, P, b);
   stage_consts<M, T, AOS>(nd, P, b);
@@ -2283,11 +2437,11 @@ __device__ __forceinline__ void scp_body(const ProblemDev& P, const Layout& L, c
     __syncthreads();
     if constexpr (GROUP) {
       // a failed factorisation in any scenario stops the whole group
-      if (threadIdx.x == 0) G->mine[X.epoch & 1][0] = (double)sh.fail;
-      double f[1];
-      group_allreduce<1>(P, G, X, 0, f);
-      if (threadIdx.x == 0) sh.fail = f[0] != 0.0;
-      __syncthreads();
+      if (i == 0)
+        for (int j = 0; j < NU; ++j)
+          group_box_put<W>(G, X, j, wide_add(nd.dat(Rec<M, AOS>::Ubar, j), nd.at(Rec<M, AOS>::Ulo, j)),
+                           wide_add(nd.dat(Rec<M, AOS>::Ubar, j), nd.at(Rec<M, AOS>::Uhi, j)));
+      group_begin<W>(P, G, X, sh);
     }
     if (sh.fail) { if (threadIdx.x == 0) sh.status = ST_NUMERIC; iters_run++; break; }
     admm_iterations<M, T, AOS, REFINE, GROUP, REGS>(nd, MT, L, I, K, active, re, rd, rg, P.admm_iters, sh, res, G, X, P);

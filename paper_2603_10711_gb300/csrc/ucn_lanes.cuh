@@ -347,8 +347,16 @@ __device__ __forceinline__ void admm_iteration_lanes(const Node<T, AOS>& nd, con
   // Step 3 before Step 2 (disjoint variables, both read only this iteration's
   // xi): between the arrival on the split barrier and the wait for the left
   // neighbour's Ex1
-  if constexpr (GROUP) __syncthreads();   // groups: their exchange follows Step 2 on a plain barrier
-  else split_barrier_arrive(X.bar);
+  if constexpr (GROUP) {
+    if (threadIdx.x < 32) {   // node 0 is the first four lanes; lane l hands over control l mod 4
+      typedef typename Node<T, AOS>::W W;
+      W a = i == 0 ? nd.dat(Rec<M>::Ubar, q) : W();
+      const T nuu = i == 0 ? nd.at(Rec<M>::Nuu, q) : T(0);
+      a = wide_shfl(wide_add(a, xo[RX] + nuu * irg), (int)threadIdx.x & 3);
+      group_publish<W>(P, G, X, a);
+    }
+    group_arrive(P, X);
+  } else split_barrier_arrive(X.bar);
   T dz[RX];
   T sv[R];
 #pragma unroll
@@ -373,14 +381,7 @@ __device__ __forceinline__ void admm_iteration_lanes(const Node<T, AOS>& nd, con
         const int j = q + TPN * m;
         const T nuu = nd.at(Rec<M>::Nuu, j);
         if constexpr (GROUP) {
-          if (i == 0) {   // sum of arguments | max of lower bounds | max of -upper bounds
-            const double ub = wide_to_double(nd.dat(Rec<M>::Ubar, j));
-            double* mm = G->mine[X.epoch & 1];
-            mm[j] = ub + (double)(xo[RX + m] + nuu * irg);
-            mm[NU + j] = ub + (double)nd.at(Rec<M>::Ulo, j);
-            mm[2 * NU + j] = -(ub + (double)nd.at(Rec<M>::Uhi, j));
-            continue;
-          }
+          if (i == 0) continue;   // the consensus sets it
         }
         const T uh = clampv(xo[RX + m] + nuu * irg, nd.at(Rec<M>::Ulo, j), nd.at(Rec<M>::Uhi, j));
         if (LAST) {
@@ -407,7 +408,8 @@ __device__ __forceinline__ void admm_iteration_lanes(const Node<T, AOS>& nd, con
       }
     }
   }
-  if constexpr (!GROUP) split_barrier_wait(X.bar, X.ph);
+  if constexpr (GROUP) group_arrived(P, X);
+  else split_barrier_wait(X.bar, X.ph);
   if (active) {
     // ---- Step 2: dynamic consensus, Eq. (5), then its duals (Step 4)
     if (i >= 1) {
@@ -430,28 +432,23 @@ __device__ __forceinline__ void admm_iteration_lanes(const Node<T, AOS>& nd, con
     }
   }
   if constexpr (GROUP) {
-    double tot[3 * NU];
-#pragma unroll
-    for (int j = 0; j < 3 * NU; ++j) tot[j] = 0.0;
-    group_allreduce<3 * NU>(P, G, X, NU, tot);
-#pragma unroll
-    for (int j = 0; j < 3 * NU; ++j) tot[j] = __shfl_sync(WARP_ALL, tot[j], 0, TPN);
-    if (active && i == 0 && i < N) {
-#pragma unroll
-      for (int m = 0; m < RU; ++m) {
-        const int j = q + TPN * m;
-        const double v = fmin(fmax(tot[j] / (double)P.group, tot[NU + j]), -tot[2 * NU + j]);
-        G->u0[j] = v;
-        const T uh = (T)(v - wide_to_double(nd.dat(Rec<M>::Ubar, j)));
-        const T nuu = nd.at(Rec<M>::Nuu, j);
+    typedef typename Node<T, AOS>::W W;
+    if (threadIdx.x < 32) {
+      const W sum = group_collect<W>(P, G, X);
+      if (active && i == 0 && i < N) {
+        const W v = group_mean(G, sum, P.group, q);
+        G->u0[q] = wide_bits(v);
+        const T uh = wide_diff<T>(v, nd.dat(Rec<M>::Ubar, q));
+        const T nuu = nd.at(Rec<M>::Nuu, q);
         if (LAST) {
-          sv[RX + m] += rg * (uh - nd.at(Rec<M>::Uh, j));
-          acc_sq_diff(rp, xo[RX + m], uh);
+          sv[RX] += rg * (uh - nd.at(Rec<M>::Uh, q));
+          acc_sq_diff(rp, xo[RX], uh);
         }
-        nd.at(Rec<M>::Uh, j) = uh;
-        nd.at(Rec<M>::Nuu, j) = nuu + rg * (xo[RX + m] - uh);
+        nd.at(Rec<M>::Uh, q) = uh;
+        nd.at(Rec<M>::Nuu, q) = nuu + rg * (xo[RX] - uh);
       }
     }
+    group_advance(P, X);
   }
   if constexpr (LAST) {
     // the obstacle terms of the dual residual belong to the position rows
@@ -534,7 +531,7 @@ __device__ __forceinline__ void scp_lanes_body(const ProblemDev& P, const Layout
                                                int* status_out, const int b) {
   using LR = LaneRows<M, TPN>;
   constexpr int NX = M::NX, NU = M::NU, NN = NX + NU, R = LR::R;
-  static_assert(!GROUP || NU <= 4, "GroupShared holds nu <= 4");
+  static_assert(!GROUP || NU == 4, "GroupShared holds nu = 4, one control per lane");
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ InstShared sh;
   GroupShared* G = group_slot<GROUP>();
@@ -575,6 +572,7 @@ __device__ __forceinline__ void scp_lanes_body(const ProblemDev& P, const Layout
     split_barrier_init(sh.xbar, blockDim.x);
   }
   X.bar = sh.xbar;
+  X.in = &sh.red[0][0];
   nd.prm = ndd.prm = sh.prm;
   stage_params<M>(sh, P, b);
   stage_consts<M, T, AOS>(ndd, P, b);
@@ -615,11 +613,10 @@ __device__ __forceinline__ void scp_lanes_body(const ProblemDev& P, const Layout
     __syncthreads();
     H.load(MT, q, active);
     if constexpr (GROUP) {
-      if (threadIdx.x == 0) G->mine[X.epoch & 1][0] = (double)sh.fail;
-      double f[1];
-      group_allreduce<1>(P, G, X, 0, f);
-      if (threadIdx.x == 0) sh.fail = f[0] != 0.0;
-      __syncthreads();
+      if (i == 0 && active)
+        group_box_put<W>(G, X, q, wide_add(nd.dat(Rec<M>::Ubar, q), nd.at(Rec<M>::Ulo, q)),
+                         wide_add(nd.dat(Rec<M>::Ubar, q), nd.at(Rec<M>::Uhi, q)));
+      group_begin<W>(P, G, X, sh);
     }
     if (sh.fail) { if (threadIdx.x == 0) sh.status = ST_NUMERIC; iters_run++; break; }
     admm_iterations_lanes<M, T, AOS, REFINE, GROUP, TPN>(nd, MT, H, L, I, kq, khd, active, q, re, rd, rg, P.admm_iters,

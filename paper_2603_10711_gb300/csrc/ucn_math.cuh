@@ -573,6 +573,26 @@ __device__ __forceinline__ double ld_cluster(const double* local, unsigned rank)
   return v;
 }
 
+// Stores to the same shared-memory location of another CTA of the cluster.
+__device__ __forceinline__ unsigned cluster_addr(const void* local, unsigned rank) {
+  unsigned r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(local)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void st_cluster(const float* local, unsigned rank, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr(local, rank)), "f"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster(const double* local, unsigned rank, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(cluster_addr(local, rank)), "d"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster(const int* local, unsigned rank, int v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(local, rank)), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster(const DF* local, unsigned rank, DF v) {
+  st_cluster(&local->hi, rank, v.hi);
+  st_cluster(&local->lo, rank, v.lo);
+}
+
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));

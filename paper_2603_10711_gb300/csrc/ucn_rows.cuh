@@ -67,25 +67,6 @@ __device__ __forceinline__ float sel4(float a, float b, float c, float d, int q)
   return (q & 2) ? hi : lo;
 }
 
-// Stores to the same shared-memory location of another CTA of the cluster.
-__device__ __forceinline__ unsigned cluster_addr(const void* local, unsigned rank) {
-  unsigned r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(local)), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void st_cluster(const float* local, unsigned rank, float v) {
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr(local, rank)), "f"(v) : "memory");
-}
-__device__ __forceinline__ void st_cluster(const double* local, unsigned rank, double v) {
-  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(cluster_addr(local, rank)), "d"(v) : "memory");
-}
-__device__ __forceinline__ void st_cluster(const int* local, unsigned rank, int v) {
-  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(local, rank)), "r"(v) : "memory");
-}
-__device__ __forceinline__ void st_cluster(const DF* local, unsigned rank, DF v) {
-  st_cluster(&local->hi, rank, v.hi);
-  st_cluster(&local->lo, rank, v.lo);
-}
 __device__ __forceinline__ unsigned cluster_rank() {
   unsigned r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -410,7 +391,7 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
                                                float rg, float irg, float ired, DF& rp, DF& rdl, GroupShared* G,
                                                GroupX& X, const ProblemDev& P, const Node<float, 2>& nd) {
   typedef Rec<M, 2> R;
-  constexpr int NU = M::NU, RX = RowMats<M>::RX, RE = RowConst<M>::R;
+  constexpr int RX = RowMats<M>::RX, RE = RowConst<M>::R;
   constexpr bool EX = RowMats<M>::EX, QUAD = IsQuad<M>::value;
   float* tp = p.tp;
   const int q = p.q;
@@ -477,8 +458,14 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
   }
   // Step 3 before Step 2, between the arrival (Ex1 published) and the wait
   if constexpr (CL) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-  else if constexpr (GROUP) __syncthreads();
-  else split_barrier_arrive(X.bar);
+  else if constexpr (GROUP) {
+    if (threadIdx.x < 32) {   // node 0 is the first four lanes; lane l hands over control l mod 4
+      DF a = p.i == 0 ? nd.dat(R::Ubar, q) : DF();
+      a = wide_shfl(df_add(a, xo[3] + S.nu(3) * irg), (int)threadIdx.x & 3);
+      group_publish<DF>(P, G, X, a);
+    }
+    group_arrive(P, X);
+  } else split_barrier_arrive(X.bar);
   float sv[RE], dz[RX], svr[3] = {0.0f, 0.0f, 0.0f};
   if (LAST) {
 #pragma unroll
@@ -489,16 +476,7 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
   for (int m = 0; m < RE; ++m) {
     const float nu = S.nu(m), arg = xo[m] + nu * irg;
     if constexpr (GROUP) {
-      if (m == 3 && p.i == 0) {   // sum of arguments | max of lower bounds | max of -upper bounds
-        if (p.active) {
-          const double ub = wide_to_double(nd.dat(Rec<M>::Ubar, q));
-          double* mm = G->mine[X.epoch & 1];
-          mm[q] = ub + (double)arg;
-          mm[NU + q] = ub + (double)S.lo(m);
-          mm[2 * NU + q] = -(ub + (double)S.hi(m));
-        }
-        continue;
-      }
+      if (m == 3 && p.i == 0) continue;   // the consensus sets it
     }
     const float xh = clampv(arg, S.lo(m), S.hi(m));
     if (LAST) {
@@ -511,7 +489,8 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
   if constexpr (QUAD) mg = rows_obstacles<M, LAST>(p, L, I.nobs, xo, rg, irg, sv, rp);
   else rows_sets<M, LAST, false>(p, L, I, rg, irg, R::X, svr, rp);
   if constexpr (CL) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-  else if constexpr (!GROUP) split_barrier_wait(X.bar, X.ph);
+  else if constexpr (GROUP) group_arrived(P, X);
+  else split_barrier_wait(X.bar, X.ph);
   // ---- Step 2: dynamic consensus, Eq. (5), then its duals (Step 4)
 #pragma unroll
   for (int m = 0; m < RX; ++m) dz[m] = 0.0f;
@@ -536,24 +515,18 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
       }
   }
   if constexpr (GROUP) {
-    double tot[3 * NU];
-#pragma unroll
-    for (int j = 0; j < 3 * NU; ++j) tot[j] = 0.0;
-    group_allreduce<3 * NU>(P, G, X, NU, tot);
-#pragma unroll
-    for (int j = 0; j < 3 * NU; ++j) tot[j] = __shfl_sync(ROWS_ALL, tot[j], 0, 4);
-    if (p.i == 0 && p.active) {
-#pragma unroll
-      for (int j = 0; j < NU; ++j)
-        if (j == q) {
-          const double v = fmin(fmax(tot[j] / (double)P.group, tot[NU + j]), -tot[2 * NU + j]);
-          G->u0[j] = v;
-          const float uh = (float)(v - wide_to_double(nd.dat(Rec<M>::Ubar, j)));
-          const float nu = S.nu(3);
-          if (LAST) { sv[3] += rg * (uh - S.hat(3)); acc_sq_diff(rp, xo[3], uh); }
-          S.set_box(3, uh, nu + rg * (xo[3] - uh), true);
-        }
+    if (threadIdx.x < 32) {
+      const DF sum = group_collect<DF>(P, G, X);
+      if (p.i == 0 && p.active) {
+        const DF v = group_mean(G, sum, P.group, q);
+        G->u0[q] = wide_bits(v);
+        const float uh = wide_diff<float>(v, nd.dat(R::Ubar, q));
+        const float nu = S.nu(3);
+        if (LAST) { sv[3] += rg * (uh - S.hat(3)); acc_sq_diff(rp, xo[3], uh); }
+        S.set_box(3, uh, nu + rg * (xo[3] - uh), true);
+      }
     }
+    group_advance(P, X);
   }
   if constexpr (LAST) {
     // dual residual needs rho_dyn (z_{i+1,new} - z_{i+1,old}) from the right neighbour
@@ -1113,7 +1086,7 @@ __device__ __forceinline__ void rows_candidate(const RowPos& p, const Node<float
     for (int j = 0; j < NU; ++j) uc[j] = i < N ? df_add(nd.dat(R::Ubar, j), nd.at(R::Uh, j)) : DF();
     if constexpr (GROUP) {
       if (i == 0)
-        for (int j = 0; j < NU; ++j) uc[j] = df_from(G->u0[j]);
+        for (int j = 0; j < NU; ++j) uc[j] = wide_of_bits<DF>(G->u0[j]);
     }
   }
   if constexpr (CL) {
@@ -1184,6 +1157,7 @@ __device__ __forceinline__ void scp_rows_body(const ProblemDev& P, const Layout&
     split_barrier_init(sh.xbar, blockDim.x);
   }
   X.bar = sh.xbar;
+  X.in = &sh.red[0][0];
   // the records start at zero: rows beyond a model's are read, never set
   for (int e = threadIdx.x; e < (L.chunk + (CL ? 2 : 0)) * L.NS; e += blockDim.x) ((float*)smem)[e] = 0.0f;
   nd.prm = ndd.prm = sh.prm;
@@ -1233,11 +1207,11 @@ __device__ __forceinline__ void scp_rows_body(const ProblemDev& P, const Layout&
       cluster_sync();
     }
     if constexpr (GROUP) {
-      if (threadIdx.x == 0) G->mine[X.epoch & 1][0] = (double)sh.fail;
-      double f[1];
-      group_allreduce<1>(P, G, X, 0, f);
-      if (threadIdx.x == 0) sh.fail = f[0] != 0.0;
-      __syncthreads();
+      if (p.i == 0 && p.active) {
+        const DF ub = nd.dat(Rec<M, 2>::Ubar, p.q);
+        group_box_put<DF>(G, X, p.q, df_add(ub, p.tp[Rec<M, 2>::Xlo + 12]), df_add(ub, p.tp[Rec<M, 2>::Xhi + 12]));
+      }
+      group_begin<DF>(P, G, X, sh);
     }
     if (sh.fail) { if (threadIdx.x == 0) sh.status = ST_NUMERIC; iters_run++; break; }
     rows_admm<M, GROUP, CL, REG>(p, A, K, L, I, mg, re, rd, rg, P.admm_iters, sh, res, G, X, P, nd);
@@ -1380,7 +1354,7 @@ __global__ void __launch_bounds__(MAXT, 1) admm_rows_kernel(ProblemDev P, Layout
     cluster_sync();
   }
   double r2[2] = {0.0, 0.0};
-  GroupX X{0u, 0, 0, sh.xbar, 0u};
+  GroupX X{0u, 0, 0, 0u, nullptr, sh.xbar, 0u};
   if (!sh.fail) rows_admm<M, false, CL, REG>(p, A, K, L, I, mg, re, rd, rg, iters, sh, r2, nullptr, X, P, nd);
   __syncthreads();
   if (dact) {
