@@ -187,9 +187,9 @@ ucn_status ucn_problem_set_lanes(ucn_problem* prob, int lanes_per_node);
 int ucn_problem_lanes(const ucn_problem* prob);
 
 /* Kernel launches made by the last ucn_scp_solve / ucn_scp_solve_warm /
- * ucn_admm_solve call on this problem: 1, or 2 when the fused
- * solve ran a first round on its three-CTAs-per-SM variant (see
- * ucn_scp_solve); 0 before the first call, -1 for NULL.  (Not in the paper;
+ * ucn_admm_solve call on this problem: 1; 2 when the fused
+ * solve ran a first round on its three-CTAs-per-SM variant; up to 3 for an
+ * uneven FP32 batch, one per CTA shape (see ucn_scp_solve); 0 before the first call, -1 for NULL.  (Not in the paper;
  * for launch accounting.) */
 int ucn_problem_last_launches(const ucn_problem* prob);
 
@@ -234,7 +234,11 @@ ucn_status ucn_state_export(ucn_problem* prob, double* state_d, void* stream);
  * instance by persistent kernel launches that each run whole solves: per SCP
  * iteration the RK4 linearisation, assembly + factorisation, admm_iters ADMM
  * iterations, and the rollout / defect / trust-region acceptance test, all on
- * the device, one CTA per instance.  One launch; for batches of the 3-DOF Mars
+ * the device, one CTA per instance (or, FP32 and 16- or 17-row models beyond
+ * 96 or 64 nodes, a thread-block cluster of two or four).  One launch; FP32
+ * batches of those models whose instances need different CTA shapes take one
+ * launch per shape, side by side on streams of the problem forked from and
+ * joined to `stream`; for batches of the 3-DOF Mars
  * model in FP32 that are not a whole number of resident rounds, a first launch
  * runs one round on a three-CTAs-per-SM variant of the same kernel and a second
  * the rest (same results per instance).  In: initial guesses x0_d, u0_d.  Out:

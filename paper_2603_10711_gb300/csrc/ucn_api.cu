@@ -175,6 +175,8 @@ bool rows_layout(int model, int precision, int nodes, int max_obs, int group, in
 
 }  // namespace ucn
 
+constexpr int MAX_ROW_PARTS = 3;
+
 struct ucn_problem {
   int model, nx, nu, batch, max_obs, Nmax, precision;
   long long total_x, total_u, state_size;
@@ -190,8 +192,14 @@ struct ucn_problem {
   int tpn;               // threads per node of the fused solve
   int last_launches = 0; // kernel launches of the last fused solve
   int optin;             // shared memory per CTA the device allows
-  bool rows;             // the row kernel serves this problem at its default threads per node, on
-  Layout Lr;             // this layout
+  // The row kernel serves this problem at its default threads per node, in parts
+  // of the CTA order: instances of the same CTA shape (see rows_parts), each part
+  // a launch of its own layout, the second and later ones on streams of their own.
+  struct RowsPart { Layout L; int first, count; };
+  std::vector<RowsPart> parts;
+  std::vector<int> horizon;
+  cudaStream_t aux[MAX_ROW_PARTS - 1] = {};
+  cudaEvent_t fork = nullptr, join[MAX_ROW_PARTS - 1] = {};
   unsigned char* warm_ones;   // batch flags, all 1: every instance starts from the given state
 };
 
@@ -216,6 +224,50 @@ ucn_status dev_copy(ucn_problem* p, int& nalloc, int fault_at, const V* host, si
 }
 
 cudaStream_t as_stream(void* s) { return (cudaStream_t)s; }
+
+// The row kernel's parts of a batch: its instances by the CTA shape their own
+// length needs -- one CTA of 64 nodes, of 96 (12-state quadrotor), clusters of
+// two, of four -- longest first, the given order kept within each.  One layout
+// for the longest would give every instance the largest shape: 1023 quadrotors
+// of 40..120 nodes took 57.9 ms as clusters of two throughout, 36.9 ms in parts
+// (64 nodes: 1.14 us per ADMM iteration on one SM; 91: 2.0; 121: 1.6 on two).
+// At most MAX_ROW_PARTS: shorter shapes join the next longer one beyond that.
+void rows_parts(ucn_problem* p, std::vector<int>& order) {
+  p->parts.clear();
+  const int tpn = default_tpn(p->model, p->Nmax + 1, p->precision);
+  Layout L;
+  if (!rows_layout(p->model, p->precision, p->Nmax + 1, p->max_obs, p->group, tpn, p->optin, &L)) return;
+  if (p->group > 1) {
+    p->parts.push_back({L, 0, p->batch});
+    return;
+  }
+  // shape of an instance: CTAs, and of one CTA which register class
+  auto shape = [&](int b) {
+    const int nodes = p->horizon[b] + 1;
+    Layout l;
+    rows_layout(p->model, p->precision, nodes, p->max_obs, 1, tpn, p->optin, &l);
+    return 2 * l.csize + (l.csize == 1 && l.chunk > ROWS_THREADS / 4 ? 1 : 0);
+  };
+  std::vector<int> s(p->batch), all;
+  for (int b = 0; b < p->batch; ++b) s[b] = shape(b);
+  all = s;
+  std::sort(all.begin(), all.end(), [](int x, int y) { return x > y; });
+  all.erase(std::unique(all.begin(), all.end()), all.end());
+  if (all.size() > MAX_ROW_PARTS) {   // join the shortest shapes
+    for (int& v : s) v = std::max(v, all[MAX_ROW_PARTS - 1]);
+    all.resize(MAX_ROW_PARTS);
+  }
+  std::vector<int> out;
+  for (int v : all) {
+    const int first = (int)out.size();
+    int nodes = 0;
+    for (int b : order)
+      if (s[b] == v) { out.push_back(b); nodes = std::max(nodes, p->horizon[b] + 1); }
+    rows_layout(p->model, p->precision, nodes, p->max_obs, 1, tpn, p->optin, &L);
+    p->parts.push_back({L, first, (int)out.size() - first});
+  }
+  order = out;
+}
 
 }  // namespace
 
@@ -269,6 +321,11 @@ void ucn_problem_destroy(ucn_problem* p) {
   if (!p) return;
   cudaDeviceSynchronize();
   for (void* a : p->allocs) cudaFree(a);
+  for (cudaStream_t s : p->aux)
+    if (s) cudaStreamDestroy(s);
+  for (cudaEvent_t e : p->join)
+    if (e) cudaEventDestroy(e);
+  if (p->fork) cudaEventDestroy(p->fork);
   delete p;
 }
 
@@ -311,6 +368,9 @@ ucn_status ucn_problem_create(const ucn_problem_desc* d, ucn_problem** out) {
   if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return fail(UCN_ECUDA, "no CUDA device"); }
   ucn_problem* p = new ucn_problem();
   p->model = d->model; p->nx = NX; p->nu = NU; p->batch = d->batch; p->max_obs = obst ? d->max_obs : 0;
+  int optin = 0;
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  p->optin = optin;
   p->Nmax = Nmax; p->precision = d->precision; p->group = group;
   p->tpn = default_tpn(d->model, Nmax + 1, d->precision);
   const int B = d->batch;
@@ -368,6 +428,8 @@ ucn_status ucn_problem_create(const ucn_problem_desc* d, ucn_problem** out) {
       w[b] = (d->horizon[b] + 1.0) * (1.0 + ((obst && d->max_obs > 0) ? d->n_obs[b] / 8.0 : 0.0));
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return w[x] > w[y]; });
   }
+  p->horizon.assign(d->horizon, d->horizon + B);
+  rows_parts(p, order);
   int* ord = nullptr;
   COPY(ord, order.data(), B);
   const std::vector<double> fac = rho_schedule(d->rho_final, d->rho_geo, d->scp_iters);
@@ -412,8 +474,6 @@ ucn_status ucn_problem_create(const ucn_problem_desc* d, ucn_problem** out) {
   // their matrices in registers), else a structure-of-arrays slice of global memory
   const int tsize = d->precision == UCN_PREC_FP64 ? 8 : 4;
   const bool small = d->model == UCN_MODEL_MARS7;   // SmallModel<Mars7> (registers hold A, B, H^-1)
-  int optin = 0;
-  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   const long long static_sh = (long long)sizeof(InstShared) + (group > 1 ? (long long)sizeof(GroupShared) : 0) + 64;
   p->L = make_layout(d->model, Nmax + 1, p->max_obs, tsize, small, p->tpn);
   p->smem = p->L.bytes + static_sh <= optin;
@@ -421,9 +481,6 @@ ucn_status ucn_problem_create(const ucn_problem_desc* d, ucn_problem** out) {
     if (!tpn_allowed(p->tpn, d->model, Nmax + 1, d->precision, false)) p->tpn = 1;
     p->L = make_layout(d->model, Nmax + 1, p->max_obs, tsize, false, p->tpn);
   }
-  p->optin = optin;
-  p->rows = rows_layout(d->model, d->precision, Nmax + 1, p->max_obs, group, default_tpn(d->model, Nmax + 1, d->precision),
-                        optin, &p->Lr);
   p->threads = (int)round_up(Nmax + 1, 32);
   p->smem_bytes = p->smem ? p->L.bytes : 0;
   if (group > 1 && !p->smem) {
@@ -465,6 +522,18 @@ ucn_status ucn_problem_create(const ucn_problem_desc* d, ucn_problem** out) {
     p->allocs.push_back(ws);
     P.ws = ws;
   }
+  if (p->parts.size() > 1) {
+    cudaError_t e = cudaEventCreateWithFlags(&p->fork, cudaEventDisableTiming);
+    for (size_t k = 0; k + 1 < p->parts.size() && e == cudaSuccess; ++k) {
+      e = cudaStreamCreateWithFlags(&p->aux[k], cudaStreamNonBlocking);
+      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->join[k], cudaEventDisableTiming);
+    }
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      ucn_problem_destroy(p);
+      return fail(UCN_ECUDA, "streams of the batch's parts: %s", cudaGetErrorString(e));
+    }
+  }
   *out = p;
   return UCN_OK;
 }
@@ -484,6 +553,7 @@ ucn_status ucn_problem_set_order(ucn_problem* p, const int* order) {
   } else {
     for (int b = 0; b < p->batch; ++b) o[b] = b;
   }
+  rows_parts(p, o);
   const cudaError_t e = cudaMemcpy(p->order_d, o.data(), sizeof(int) * p->batch, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return fail(UCN_ECUDA, "order copy: %s", cudaGetErrorString(e));
   return UCN_OK;
@@ -517,18 +587,56 @@ long long ucn_total_x(const ucn_problem* p) { return p ? p->total_x : -1; }
 long long ucn_total_u(const ucn_problem* p) { return p ? p->total_u : -1; }
 long long ucn_state_size(const ucn_problem* p) { return p ? p->state_size : -1; }
 
+// Whether the fused solve and the ADMM call run the row kernel.
+static bool rows_on(const ucn_problem* p) {
+  return !p->parts.empty() && p->tpn == default_tpn(p->model, p->Nmax + 1, p->precision);
+}
+
 static LaunchCfg cfg_of(ucn_problem* p, void* stream) {
   LaunchCfg c;
   c.P = &p->dev; c.L = &p->L; c.smem = p->smem; c.smem_bytes = p->smem_bytes;
   c.threads = p->threads; c.blocks = p->batch; c.stream = as_stream(stream); c.group = p->gcsize;
   c.nodes = p->Nmax + 1; c.tpn = p->tpn;
   c.launched = &p->last_launches;
-  if (p->rows && p->tpn == default_tpn(p->model, p->Nmax + 1, p->precision)) {
-    c.L = &p->Lr; c.smem = true; c.smem_bytes = p->Lr.bytes;
+  if (rows_on(p)) {   // (a batch of several parts goes through launch_parts)
+    c.L = &p->parts[0].L; c.smem = true; c.smem_bytes = p->parts[0].L.bytes;
   }
   p->last_launches = 1;   // one launch unless the launcher splits the batch
   return c;
 }
+
+// A launch of the whole batch (`launch`), or of each of its parts: the first on
+// the caller's stream, the others on the problem's own, forked from it and
+// joined to it by events (so that a capture of the caller's stream holds them),
+// so that a part's CTAs fill the SMs that an earlier part's last ones leave.
+extern "C++" {
+template <class F>
+static cudaError_t launch_parts(ucn_problem* p, LaunchCfg c, F launch) {
+  if (!rows_on(p) || p->parts.size() == 1) return launch(c);
+  cudaStream_t s = c.stream;
+  cudaError_t e = cudaEventRecord(p->fork, s);
+  const ProblemDev base = *(const ProblemDev*)c.P;
+  for (size_t k = 0; k < p->parts.size() && e == cudaSuccess; ++k) {
+    const ucn_problem::RowsPart& q = p->parts[k];
+    ProblemDev P = base;
+    P.order = base.order + q.first;
+    c.P = &P;
+    c.L = &q.L; c.smem_bytes = q.L.bytes; c.blocks = q.count;
+    if (k > 0) {
+      c.stream = p->aux[k - 1];
+      e = cudaStreamWaitEvent(c.stream, p->fork, 0);
+    }
+    if (e == cudaSuccess) e = launch(c);
+    if (k > 0) {   // joined whatever the launch said: the caller's stream never runs ahead
+      cudaError_t j = cudaEventRecord(p->join[k - 1], c.stream);
+      if (j == cudaSuccess) j = cudaStreamWaitEvent(s, p->join[k - 1], 0);
+      if (e == cudaSuccess) e = j;
+    }
+  }
+  p->last_launches = (int)p->parts.size();
+  return e;
+}
+}  // extern "C++"
 
 ucn_status ucn_linearize(ucn_problem* p, const double* xbar_d, const double* ubar_d, double* A_d, double* B_d,
                          double* d_d, void* stream) {
@@ -550,7 +658,9 @@ ucn_status ucn_admm_solve(ucn_problem* p, const double* xbar_d, const double* ub
   if (p->group > 1) return fail(UCN_EINVAL, "the scenario consensus runs inside ucn_scp_solve only");
   const LaunchCfg c = cfg_of(p, stream);
   auto fn = launchers_for(p->model, p->precision).admm;
-  const cudaError_t e = fn(c, xbar_d, ubar_d, A_d, B_d, d_d, radius_d, iters, warm ? 1 : 0, xhat_d, uhat_d, res_d, status_d);
+  const cudaError_t e = launch_parts(p, c, [&](const LaunchCfg& k) {
+    return fn(k, xbar_d, ubar_d, A_d, B_d, d_d, radius_d, iters, warm ? 1 : 0, xhat_d, uhat_d, res_d, status_d);
+  });
   if (e != cudaSuccess) return fail(UCN_ECUDA, "admm launch: %s", cudaGetErrorString(e));
   return UCN_OK;
 }
@@ -583,7 +693,9 @@ ucn_status ucn_scp_solve(ucn_problem* p, const double* x0_d, const double* u0_d,
     return UCN_OK;
   }
   auto fn = launchers_for(p->model, p->precision).scp;
-  const cudaError_t e = fn(c, x0_d, u0_d, x_out_d, u_out_d, stats_d, status_d);
+  const cudaError_t e = launch_parts(p, c, [&](const LaunchCfg& k) {
+    return fn(k, x0_d, u0_d, x_out_d, u_out_d, stats_d, status_d);
+  });
   if (e != cudaSuccess) return fail(UCN_ECUDA, "scp launch: %s", cudaGetErrorString(e));
   return UCN_OK;
 }
@@ -604,7 +716,9 @@ ucn_status ucn_scp_solve_warm(ucn_problem* p, const double* x0_d, const double* 
   LaunchCfg c = cfg_of(p, stream);
   c.P = &Pw;
   auto fn = launchers_for(p->model, p->precision).scp;
-  const cudaError_t e = fn(c, x0_d, u0_d, x_out_d, u_out_d, stats_d, status_d);
+  const cudaError_t e = launch_parts(p, c, [&](const LaunchCfg& k) {
+    return fn(k, x0_d, u0_d, x_out_d, u_out_d, stats_d, status_d);
+  });
   if (e != cudaSuccess) return fail(UCN_ECUDA, "scp launch: %s", cudaGetErrorString(e));
   return UCN_OK;
 }
