@@ -1946,45 +1946,6 @@ __device__ __forceinline__ Node<T, SMEM> make_node(const ProblemDev& P, const La
   return nd;
 }
 
-// Linearisation of every node of every instance (one thread per control node).
-template <class M, class T>
-__global__ void __launch_bounds__(128) linearize_kernel(ProblemDev P, const int* node_inst, long long total_u,
-                                                        const double* xbar, const double* ubar,
-                                                        double* A, double* B, double* d) {
-  constexpr int NX = M::NX, NU = M::NU;
-  const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= total_u) return;
-  const int b = node_inst[g];
-  const long long i = g - P.uoff[b];
-  const long long xr = P.xoff[b] + i;
-  double x[NX], u[NU];
-  for (int j = 0; j < NX; ++j) x[j] = xbar[xr * NX + j];
-  for (int j = 0; j < NU; ++j) u[j] = ubar[g * NU + j];
-  double prm[PRM];
-  T prmt[PRM];
-  for (int k = 0; k < PRM; ++k) { prm[k] = derived_param<M>(P.params + b * 8, k); prmt[k] = (T)prm[k]; }
-  const double h = P.dt[b];
-  double Ad[NX * NX], Bd[NX * NU];
-  for (int dir = 0; dir < NX + NU; ++dir) {
-    T col[NX];
-    rk4_jvp<M, T>(prmt, step_of<T>(h), x, u, dir, col);
-    for (int r = 0; r < NX; ++r) {
-      if (dir < NX) Ad[r * NX + dir] = (double)col[r];
-      else Bd[r * NU + dir - NX] = (double)col[r];
-    }
-  }
-  double xn[NX];
-  rk4<M, double>(prm, h, x, u, xn);
-  for (int r = 0; r < NX; ++r) {
-    double acc = xn[r];
-    for (int c = 0; c < NX; ++c) acc -= Ad[r * NX + c] * x[c];
-    for (int c = 0; c < NU; ++c) acc -= Bd[r * NU + c] * u[c];
-    d[g * NX + r] = acc;
-  }
-  for (int e = 0; e < NX * NX; ++e) A[g * NX * NX + e] = Ad[e];
-  for (int e = 0; e < NX * NU; ++e) B[g * NX * NU + e] = Bd[e];
-}
-
 // Standalone ADMM call on caller-supplied linearisations (one CTA per instance).
 template <class M, class T, bool SMEM, bool REFINE>
 __global__ void __launch_bounds__(MAX_THREADS) admm_kernel(ProblemDev P, Layout L, const double* xbar, const double* ubar,

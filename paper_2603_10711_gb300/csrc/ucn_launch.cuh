@@ -3,6 +3,7 @@
 #include "ucn_internal.h"
 #include "ucn_kernels.cuh"
 #include "ucn_lanes.cuh"
+#include "ucn_linearize.cuh"
 #include "ucn_pair.cuh"
 #include "ucn_rows.cuh"
 

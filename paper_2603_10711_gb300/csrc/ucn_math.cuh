@@ -27,8 +27,8 @@ template <class T> __device__ __forceinline__ Dual<T> operator+(Dual<T> a, Dual<
 template <class T> __device__ __forceinline__ Dual<T> operator-(Dual<T> a, Dual<T> b) { return {a.v - b.v, a.d - b.d}; }
 template <class T> __device__ __forceinline__ Dual<T> operator-(Dual<T> a) { return {-a.v, -a.d}; }
 template <class T> __device__ __forceinline__ Dual<T> operator*(Dual<T> a, Dual<T> b) { return {a.v * b.v, a.d * b.v + a.v * b.d}; }
-// FP32 duals divide through one correctly rounded reciprocal (the Jacobian
-// passes' latency is the chain of divisions); FP64 keeps the IEEE quotient.
+// Duals divide through one reciprocal (the Jacobian passes' latency is the chain
+// of divisions), correctly rounded in FP32.
 __device__ __forceinline__ Dual<float> operator/(Dual<float> a, Dual<float> b) {
   const float r = __frcp_rn(b.v), q = a.v * r;
   return {q, (a.d - q * b.d) * r};
@@ -38,8 +38,8 @@ __device__ __forceinline__ Dual<float> operator/(float a, Dual<float> b) {
   return {q, -q * b.d * r};
 }
 template <class T> __device__ __forceinline__ Dual<T> operator/(Dual<T> a, Dual<T> b) {
-  T q = a.v / b.v;
-  return {q, (a.d - q * b.d) / b.v};
+  const T r = T(1) / b.v, q = a.v * r;
+  return {q, (a.d - q * b.d) * r};
 }
 template <class T> __device__ __forceinline__ Dual<T> operator+(Dual<T> a, T b) { return {a.v + b, a.d}; }
 template <class T> __device__ __forceinline__ Dual<T> operator+(T b, Dual<T> a) { return {a.v + b, a.d}; }
@@ -49,8 +49,8 @@ template <class T> __device__ __forceinline__ Dual<T> operator*(Dual<T> a, T b) 
 template <class T> __device__ __forceinline__ Dual<T> operator*(T b, Dual<T> a) { return {a.v * b, a.d * b}; }
 template <class T> __device__ __forceinline__ Dual<T> operator/(Dual<T> a, T b) { return {a.v / b, a.d / b}; }
 template <class T> __device__ __forceinline__ Dual<T> operator/(T a, Dual<T> b) {
-  T q = a / b.v;
-  return {q, -q * b.d / b.v};
+  const T r = T(1) / b.v, q = a * r;
+  return {q, -q * b.d * r};
 }
 
 // K tangent directions on one value (the Jacobian passes of the FP32 path): the
@@ -132,7 +132,23 @@ template <class T> __device__ __forceinline__ Dual<T> sqrt_(Dual<T> a) {
   T s = sqrt_(a.v);
   return {s, s > T(0) ? a.d / (T(2) * s) : T(0)};
 }
-// DualN<float> as Dual<float> per tangent (one reciprocal per division)
+// DualN as Dual per tangent (one reciprocal per division)
+template <int K> __device__ __forceinline__ DualN<double, K> operator/(DualN<double, K> a, DualN<double, K> b) {
+  const double rr = 1.0 / b.v;
+  DualN<double, K> r;
+  r.v = a.v * rr;
+#pragma unroll
+  for (int q = 0; q < K; ++q) r.d[q] = (a.d[q] - r.v * b.d[q]) * rr;
+  return r;
+}
+template <int K> __device__ __forceinline__ DualN<double, K> operator/(double a, DualN<double, K> b) {
+  const double rr = 1.0 / b.v;
+  DualN<double, K> r;
+  r.v = a * rr;
+#pragma unroll
+  for (int q = 0; q < K; ++q) r.d[q] = -r.v * b.d[q] * rr;
+  return r;
+}
 template <int K> __device__ __forceinline__ DualN<float, K> operator/(DualN<float, K> a, DualN<float, K> b) {
   const float rr = __frcp_rn(b.v);
   DualN<float, K> r;
