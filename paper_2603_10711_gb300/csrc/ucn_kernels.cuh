@@ -362,7 +362,9 @@ struct InstShared {
                             // receive their peers' values here during an ADMM call (GroupX::in)
   double Jn, radius;
   double rho[3];            // rho_eq, rho_dyn, rho_geo of the SCP iteration
-  float rhof[3];            // the same in FP32 (no conversion per thread)
+  float rhof[4];            // the same, and the trust radius, in FP32 (no conversion per thread:
+                            // those are instructions of the FP64 pipe)
+  unsigned tmask;           // terminal selection, bit per state
   double out[8];
   double prm[PRM];          // the model's constants (derived_param)
   float prmf[PRM];          // the same in FP32
@@ -370,10 +372,15 @@ struct InstShared {
   int accept, stop, status;
 };
 
-// The instance's model constants, by the CTA's first PRM threads (the caller
-// synchronises), and the arithmetic type's copy.
+// The instance's model constants and terminal selection, by the CTA's first PRM
+// threads (the caller synchronises), and the arithmetic type's copy.
 template <class M>
 __device__ __forceinline__ void stage_params(InstShared& sh, const ProblemDev& P, int b) {
+  if (threadIdx.x == 0) {
+    unsigned m = 0;
+    for (int j = 0; j < M::NX; ++j) m |= P.tmask[b * M::NX + j] ? 1u << j : 0u;
+    sh.tmask = m;
+  }
   if (threadIdx.x < PRM) {
     const double v = derived_param<M>(P.params + b * 8, (int)threadIdx.x);
     sh.prm[threadIdx.x] = v;
@@ -687,6 +694,8 @@ __device__ __forceinline__ GroupShared* group_slot() {
   }
 }
 
+template <class T> __device__ __forceinline__ T radius_of(const InstShared& sh) { return sh.radius; }
+template <> __device__ __forceinline__ float radius_of<float>(const InstShared& sh) { return sh.rhof[3]; }
 template <class T> __device__ __forceinline__ T rho_of(const InstShared& sh, int r) { return (T)sh.rho[r]; }
 template <> __device__ __forceinline__ float rho_of<float>(const InstShared& sh, int r) { return sh.rhof[r]; }
 
@@ -917,7 +926,7 @@ __device__ void node_mirror_data(const Node<T, AOS>& nd, const Layout& L, const 
 // as degenerate boxes at nodes 0 and N), and the mirror-set data.
 template <class M, class T, int AOS>
 __device__ void node_setup(const Node<T, AOS>& nd, const Layout& L, const ProblemDev& P, const Inst<T>& I, int b,
-                           double radius, T re, T rg, NodeConst<M, T>& K) {
+                           T rad, unsigned tmask, T re, T rg, NodeConst<M, T>& K) {
   constexpr int NX = M::NX, NU = M::NU;
   const int i = nd.i, N = nd.N;
   typename Node<T, AOS>::W xb[NX], ub[NU];
@@ -927,7 +936,6 @@ __device__ void node_setup(const Node<T, AOS>& nd, const Layout& L, const Proble
     // the same quantities from the CB block in double-float, rounded to T
     typedef CB<M> C;
     const DF* cb = nd.c;
-    const T rad = (T)radius;
     // running nodes of a problem without running state cost (the Mars batch):
     // zero gradient and weight without the double-float product
     const bool cost = term || I.run_cost;
@@ -944,7 +952,7 @@ __device__ void node_setup(const Node<T, AOS>& nd, const Layout& L, const Proble
       T lo = fmaxf(wide_diff<T>(cb[C::Xlo + j], xb[j]), -rad);
       T hi = fminf(wide_diff<T>(cb[C::Xhi + j], xb[j]), rad);
       if (i == 0) lo = hi = wide_diff<T>(cb[C::Xinit + j], xb[j]);
-      else if (term && P.tmask[b * NX + j]) lo = hi = wide_diff<T>(cb[C::Xtgt + j], xb[j]);
+      else if (term && (tmask >> j & 1u)) lo = hi = wide_diff<T>(cb[C::Xtgt + j], xb[j]);
       nd.at(Rec<M, AOS>::Xlo, j) = lo;
       nd.at(Rec<M, AOS>::Xhi, j) = hi;
     }
@@ -963,10 +971,10 @@ __device__ void node_setup(const Node<T, AOS>& nd, const Layout& L, const Proble
     const double w = term ? P.QNd[b * NX + j] : P.Qd[b * NX + j];
     K.q[j] = (T)(w * (xb[j] - P.xref[b * NX + j]) + (term ? P.qN[b * NX + j] : 0.0));
     K.hd[j] = (T)w + rg + (i > 0 ? re : T(0));
-    double lo = fmax(P.xlo[b * NX + j], xb[j] - radius) - xb[j];
-    double hi = fmin(P.xhi[b * NX + j], xb[j] + radius) - xb[j];
+    double lo = fmax(P.xlo[b * NX + j], xb[j] - rad) - xb[j];
+    double hi = fmin(P.xhi[b * NX + j], xb[j] + rad) - xb[j];
     if (i == 0) lo = hi = P.xinit[b * NX + j] - xb[j];
-    else if (term && P.tmask[b * NX + j]) lo = hi = P.xtarget[b * NX + j] - xb[j];
+    else if (term && (tmask >> j & 1u)) lo = hi = P.xtarget[b * NX + j] - xb[j];
     nd.at(Rec<M, AOS>::Xlo, j) = (T)lo;
     nd.at(Rec<M, AOS>::Xhi, j) = (T)hi;
   }
@@ -975,8 +983,8 @@ __device__ void node_setup(const Node<T, AOS>& nd, const Layout& L, const Proble
     for (int j = 0; j < NU; ++j) {
       K.q[NX + j] = (T)(P.Rd[b * NU + j] * (ub[j] - P.uref[b * NU + j]));
       K.hd[NX + j] = (T)P.Rd[b * NU + j] + rg;
-      nd.at(Rec<M, AOS>::Ulo, j) = (T)(fmax(P.ulo[b * NU + j], ub[j] - radius) - ub[j]);
-      nd.at(Rec<M, AOS>::Uhi, j) = (T)(fmin(P.uhi[b * NU + j], ub[j] + radius) - ub[j]);
+      nd.at(Rec<M, AOS>::Ulo, j) = (T)(fmax(P.ulo[b * NU + j], ub[j] - rad) - ub[j]);
+      nd.at(Rec<M, AOS>::Uhi, j) = (T)(fmin(P.uhi[b * NU + j], ub[j] + rad) - ub[j]);
     }
   }
   }
@@ -1964,6 +1972,7 @@ __global__ void __launch_bounds__(MAX_THREADS) admm_kernel(ProblemDev P, Layout 
   const bool active = i <= N;
   const long long xo = P.xoff[b], uo = P.uoff[b];
   if (threadIdx.x == 0) { sh.fail = 0; split_barrier_init(sh.xbar, blockDim.x); }
+  stage_params<M>(sh, P, b);
   stage_consts<M, T, AOS>(nd, P, b);
   if (active) load_nominal<M, T, AOS>(nd, L, xbar, ubar, xo, uo);
   __syncthreads();
@@ -1988,7 +1997,7 @@ __global__ void __launch_bounds__(MAX_THREADS) admm_kernel(ProblemDev P, Layout 
   const Inst<T> I = make_inst<M, T>(P, b);
   NodeConst<M, T> K;
   if (active) {
-    node_setup<M, T, AOS>(nd, L, P, I, b, radius[b], re, rg, K);
+    node_setup<M, T, AOS>(nd, L, P, I, b, (T)radius[b], sh.tmask, re, rg, K);
     const bool ok = node_factor<M, T, AOS, NX + NU>(nd, MT, L, I, K, rd, rg);
     if (!ok) atomicOr(&sh.fail, 1);
     const double* sa = P.state_abs + P.soff[b];
@@ -2383,13 +2392,14 @@ __device__ __forceinline__ void scp_body(const ProblemDev& P, const Layout& L, c
       else if (P.rho_final > 0.0 && Kscp > 1) f = pow(P.rho_final / P.rho_geo, (double)ks / (double)(Kscp - 1));
       sh.rho[0] = P.rho_eq * f; sh.rho[1] = P.rho_dyn * f; sh.rho[2] = P.rho_geo * f;
       for (int r = 0; r < 3; ++r) sh.rhof[r] = (float)sh.rho[r];
+      sh.rhof[3] = (float)sh.radius;
     }
     __syncthreads();
     const T re = rho_of<T>(sh, 0), rd = rho_of<T>(sh, 1), rg = rho_of<T>(sh, 2);
-    const double radius = sh.radius;
+    const T radius = radius_of<T>(sh);
     if (active) {
       if (i < N) node_jacobians<M, T, AOS>(nd, MT, prm_of<T>(sh), hs);
-      node_setup<M, T, AOS>(nd, L, P, I, b, radius, re, rg, K);
+      node_setup<M, T, AOS>(nd, L, P, I, b, radius, sh.tmask, re, rg, K);
       const bool ok = node_factor<M, T, AOS, NN>(nd, MT, L, I, K, rd, rg);
       if (!ok) atomicOr(&sh.fail, 1);
       node_reseed<M, T, AOS>(nd, L, I);

@@ -596,15 +596,16 @@ __device__ __forceinline__ void scp_lanes_body(const ProblemDev& P, const Layout
       else if (P.rho_final > 0.0 && Kscp > 1) f = pow(P.rho_final / P.rho_geo, (double)ks / (double)(Kscp - 1));
       sh.rho[0] = P.rho_eq * f; sh.rho[1] = P.rho_dyn * f; sh.rho[2] = P.rho_geo * f;
       for (int r = 0; r < 3; ++r) sh.rhof[r] = (float)sh.rho[r];
+      sh.rhof[3] = (float)sh.radius;
     }
     __syncthreads();
     const T re = rho_of<T>(sh, 0), rd = rho_of<T>(sh, 1), rg = rho_of<T>(sh, 2);
-    const double radius = sh.radius;
+    const T radius = radius_of<T>(sh);
     if (active && i < N) lanes_jacobians<M, T, AOS, TPN>(nd, MT, prm_of<T>(sh), hs, q);
     if (active) lanes_consts<M, T, AOS, TPN>(nd, P, b, q, re, rg, kq, khd);
     __syncthreads();
     if (dact) {
-      node_setup<M, T, AOS>(ndd, L, P, I, b, radius, re, rg, K);
+      node_setup<M, T, AOS>(ndd, L, P, I, b, radius, sh.tmask, re, rg, K);
       const bool ok = node_factor<M, T, AOS, NN>(ndd, MTd, L, I, K, rd, rg);
       if (!ok) atomicOr(&sh.fail, 1);
       node_reseed<M, T, AOS>(ndd, L, I);

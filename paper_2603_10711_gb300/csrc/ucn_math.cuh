@@ -399,7 +399,8 @@ __device__ __forceinline__ DF fma_(DF a, DF b, DF c) { return df_fma(a, b, c); }
 // multiples h/2, h/6 given in the base type R of S.  The four stages are one
 // loop: unrolled, a step of the larger models is 30 to 180 KB of code that runs
 // once per SCP iteration, and the instruction fetch is what it waits for.  The
-// 3-DOF Mars model's step is small; rolled, its kernels spill in the ADMM loop.
+// 3-DOF Mars model's step is small outside double-float; rolled, its kernels
+// spill in the ADMM loop.
 template <class M, class S, class P, class R>
 __device__ __forceinline__ void rk4h(const P* prm, R h, R hh, R h6, const S* x, const S* u, S* xn) {
   constexpr int NX = M::NX;
@@ -407,7 +408,7 @@ __device__ __forceinline__ void rk4h(const P* prm, R h, R hh, R h6, const S* x, 
   const typename M::template Held<S> H = M::template hold<S, P>(prm, u);
 #pragma unroll
   for (int j = 0; j < NX; ++j) t[j] = x[j];
-#pragma unroll (M::NX == 7 ? 4 : 1)
+#pragma unroll (M::NX == 7 && !std::is_same<S, DF>::value ? 4 : 1)
   for (int s = 0; s < 4; ++s) {
     M::template f<S, P>(prm, t, H, k);
     if (s == 3) break;
@@ -484,8 +485,10 @@ __device__ __forceinline__ void rk4_jvpn(const P* prm, const Step3<T>& hs, const
 }
 
 // ------------------------------------------------------------------ projections
-// Ball {|y| <= R}: vector scaling.  FP32: the test on squares and the scale
-// from one reciprocal square root (no square root, no division).
+// Ball {|y| <= R}: vector scaling, the test on squares: a node inside its set
+// -- the most, so that whole warps skip -- takes no square root and no division
+// (in FP64 some 55 instructions of a 1/64-rate pipe).  FP32: the scale from one
+// reciprocal square root.
 template <class T>
 __device__ __forceinline__ void proj_ball3(T* y, T R) {
   if constexpr (std::is_same<T, float>::value) {
@@ -495,53 +498,32 @@ __device__ __forceinline__ void proj_ball3(T* y, T R) {
       y[0] *= s; y[1] *= s; y[2] *= s;
     }
   } else {
-    const T n = sqrt_(y[0] * y[0] + y[1] * y[1] + y[2] * y[2]);
-    if (n > R) {
-      const T s = R / n;
+    const T n2 = y[0] * y[0] + y[1] * y[1] + y[2] * y[2];
+    if (n2 > R * R) {
+      const T s = R / sqrt_(n2);
       y[0] *= s; y[1] *= s; y[2] *= s;
     }
   }
 }
 
-// Lorentz cone {(t, y1, y2) : |y| <= tau t}: inside -> unchanged; inside the
-// polar cone (tau |y| <= -t) -> 0; otherwise onto the boundary ray.
-template <class T>
-__device__ __forceinline__ void proj_cone3(T* v, T tau) {
-  const T t = v[0];
-  const T s = sqrt_(v[1] * v[1] + v[2] * v[2]);
-  if (s <= tau * t) return;
-  if (tau * s <= -t) { v[0] = v[1] = v[2] = T(0); return; }
-  const T ca = T(1) / sqrt_(T(1) + tau * tau), sa = tau * ca;
-  const T c = t * ca + s * sa;
-  v[0] = c * ca;
-  const T r = c * sa / s;
-  v[1] *= r;
-  v[2] *= r;
-}
-
-// The same cone projection with cos / sin of the half-angle precomputed.
-// FP32: the two tests on squares (tau >= 0) and one reciprocal square root.
+// Lorentz cone {(t, y1, y2) : |y| <= tau t}, tau >= 0: inside -> unchanged;
+// inside the polar cone (tau |y| <= -t) -> 0; otherwise onto the boundary ray.
+// Both tests on squares; ca, sa the cosine and sine of the half-angle.
 template <class T>
 __device__ __forceinline__ void proj_cone3c(T* v, T tau, T ca, T sa) {
+  const T t = v[0], s2 = v[1] * v[1] + v[2] * v[2], t2 = t * t, tau2 = tau * tau;
+  if (t >= T(0) && s2 <= tau2 * t2) return;                                     // inside
+  if (t <= T(0) && tau2 * s2 <= t2) { v[0] = v[1] = v[2] = T(0); return; }      // polar cone
+  T s, r;   // s2 > 0 here
   if constexpr (std::is_same<T, float>::value) {
-    const float t = v[0], s2 = v[1] * v[1] + v[2] * v[2], t2 = t * t, tau2 = tau * tau;
-    if (t >= 0.0f && s2 <= tau2 * t2) return;                              // inside
-    if (t <= 0.0f && tau2 * s2 <= t2) { v[0] = v[1] = v[2] = 0.0f; return; }   // polar cone
-    const float rs = rsqrtf(s2), s = s2 * rs;                               // s2 > 0 here
-    const float c = t * ca + s * sa;
-    v[0] = c * ca;
-    const float r = c * sa * rs;
-    v[1] *= r;
-    v[2] *= r;
-    return;
+    const float rs = rsqrtf(s2);
+    s = s2 * rs;
+    r = (t * ca + s * sa) * sa * rs;
+  } else {
+    s = sqrt_(s2);
+    r = (t * ca + s * sa) * sa / s;
   }
-  const T t = v[0];
-  const T s = sqrt_(v[1] * v[1] + v[2] * v[2]);
-  if (s <= tau * t) return;
-  if (tau * s <= -t) { v[0] = v[1] = v[2] = T(0); return; }
-  const T c = t * ca + s * sa;
-  v[0] = c * ca;
-  const T r = c * sa / s;
+  v[0] = (t * ca + s * sa) * ca;
   v[1] *= r;
   v[2] *= r;
 }

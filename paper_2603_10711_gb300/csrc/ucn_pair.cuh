@@ -646,13 +646,14 @@ __global__ void __launch_bounds__(PAIR_MAX_THREADS, 2) scp_kernel_pair(ProblemDe
       else if (P.rho_final > 0.0 && Kscp > 1) f = pow(P.rho_final / P.rho_geo, (double)ks / (double)(Kscp - 1));
       sh.rho[0] = P.rho_eq * f; sh.rho[1] = P.rho_dyn * f; sh.rho[2] = P.rho_geo * f;
       for (int r = 0; r < 3; ++r) sh.rhof[r] = (float)sh.rho[r];
+      sh.rhof[3] = (float)sh.radius;
     }
     __syncthreads();
     const float re = sh.rhof[0], rd = sh.rhof[1], rg = sh.rhof[2];
-    const double radius = sh.radius;
+    const float radius = radius_of<float>(sh);
     pair_jacobians<M>(nd, PM, sh.prmf, hs, q, has_u);
     if (dact) {
-      node_setup<M, float, true>(ndd, L, P, I, b, radius, re, rg, Kd);
+      node_setup<M, float, true>(ndd, L, P, I, b, radius, sh.tmask, re, rg, Kd);
       node_reseed<M, float, true>(ndd, L, I);
       publish_ex2<M, float, true>(ndd, L, true, rd);
     }

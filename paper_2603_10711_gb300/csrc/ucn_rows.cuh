@@ -686,8 +686,9 @@ __device__ __forceinline__ void rows_load_G(const RowPos& p, RowMats<M>& A, cons
 
 // The lane's cost gradient, diagonal of H and boxes (Eq. (2c)), as node_setup.
 template <class M>
-__device__ __forceinline__ void rows_setup(const RowPos& p, const Node<float, 2>& nd, const ProblemDev& P,
-                                           const Inst<float>& I, int b, float rad, float re, float rg, RowConst<M>& K) {
+__device__ __forceinline__ void rows_setup(const RowPos& p, const Node<float, 2>& nd,
+                                           const Inst<float>& I, float rad, unsigned tmask, float re, float rg,
+                                           RowConst<M>& K) {
   typedef CB<M> C;
   typedef Rec<M, 2> R;
   constexpr int NX = M::NX, RE = RowConst<M>::R;
@@ -713,7 +714,7 @@ __device__ __forceinline__ void rows_setup(const RowPos& p, const Node<float, 2>
       lo = fmaxf(wide_diff<float>(cb[C::Xlo + e], xb), -rad);
       hi = fminf(wide_diff<float>(cb[C::Xhi + e], xb), rad);
       if (p.i == 0) lo = hi = wide_diff<float>(cb[C::Xinit + e], xb);
-      else if (term && P.tmask[b * NX + e]) lo = hi = wide_diff<float>(cb[C::Xtgt + e], xb);
+      else if (term && (tmask >> e & 1u)) lo = hi = wide_diff<float>(cb[C::Xtgt + e], xb);
     } else if (p.hasU) {   // node N's control rows: an identity block of H, a box at 0
       const int j = e - NX;
       const DF ub = nd.dat(Rec<M>::Ubar, j), w = cb[C::Rd + j];
@@ -958,7 +959,7 @@ __device__ __forceinline__ float rows_prepare(const RowPos& p, const Node<float,
   typedef Rec<M, 2> R;
   constexpr int RX = RowMats<M>::RX;
   float mg = 0.0f;
-  rows_setup<M>(p, nd, P, I, b, rad, re, rg, K);
+  rows_setup<M>(p, nd, I, rad, sh.tmask, re, rg, K);
   if constexpr (IsQuad<M>::value) {
     mg = rows_obstacle_setup<M>(p, nd, L, P, b, I.nobs, rg, kept, K);
   } else {
@@ -1197,11 +1198,12 @@ __device__ __forceinline__ void scp_rows_body(const ProblemDev& P, const Layout&
       else if (P.rho_final > 0.0 && Kscp > 1) f = pow(P.rho_final / P.rho_geo, (double)ks / (double)(Kscp - 1));
       sh.rho[0] = P.rho_eq * f; sh.rho[1] = P.rho_dyn * f; sh.rho[2] = P.rho_geo * f;
       for (int r = 0; r < 3; ++r) sh.rhof[r] = (float)sh.rho[r];
+      sh.rhof[3] = (float)sh.radius;
     }
     __syncthreads();
     const float re = sh.rhof[0], rd = sh.rhof[1], rg = sh.rhof[2];
     rows_jacobians<M, REG ? 2 : 1>(p, nd, A, sh.prmf, hs);
-    const float mg = rows_prepare<M, CL>(p, nd, ndd, dact, L, P, I, b, (float)sh.radius, re, rd, rg, A, K, sh);
+    const float mg = rows_prepare<M, CL>(p, nd, ndd, dact, L, P, I, b, sh.rhof[3], re, rd, rg, A, K, sh);
     if constexpr (CL) {   // a failed factorisation anywhere stops the instance
       if (sh.fail && threadIdx.x < ncta) st_cluster(&sh.fail, threadIdx.x, 1);
       cluster_sync();
