@@ -14,6 +14,7 @@
 #include "ucn_kernels.cuh"
 #include "ucn_lanes.cuh"
 #include "ucn_pair.cuh"
+#include "ucn_fan.cuh"
 #include "ucn_rows.cuh"
 
 using namespace ucn;
@@ -122,7 +123,7 @@ Layout make_layout(int model, int nodes, int max_obs, int tsize, bool reg_mats, 
 }
 
 template <class M>
-static Layout rows_layout_of(int nodes, int max_obs, int csize) {
+static Layout rows_layout_of(int nodes, int max_obs, int csize, int lanes) {
   typedef Rec<M, 2> R;
   Layout L;
   std::memset(&L, 0, sizeof(L));
@@ -135,17 +136,21 @@ static Layout rows_layout_of(int nodes, int max_obs, int csize) {
   L.oS = R::END;
   L.oNus = L.oS + ms;
   L.oMd = L.oNus + ms;
-  const int nt = L.oMd + L.MD;
+  // (fan kernel: float copies of the obstacles beside them)
+  const int nt = L.oMd + L.MD + (lanes == 4 ? 0 : 2 * ms);
   L.oA = L.oB = L.oH = -1;
+  const int ts = lanes == 4 ? 4 : 8;   // FP32 rows, FP64 fan
   L.csize = csize;
+  L.lanes = lanes;
   L.chunk = (nodes + csize - 1) / csize;
   const int recs = L.chunk + (csize > 1 ? 2 : 0);
   L.S = recs;
   L.NS = nt + ((4 - nt) % 32 + 32) % 32;   // 4 mod 32: a warp's 8 nodes x 4 rows in distinct banks
   L.DS = R::DEND | 1;
-  L.tbytes = round_up((long long)recs * L.NS * 4, 16);
+  L.tbytes = round_up((long long)recs * L.NS * ts, 16);
   L.oC = round_up(L.tbytes + (long long)recs * L.DS * 8, 16);
-  L.bytes = round_up(L.oC + 8LL * CB<M>::END, 16);
+  L.oX = round_up(L.oC + (lanes == 4 ? 8LL * CB<M>::END : 0), 16);
+  L.bytes = L.oX + (lanes == 4 ? 0 : 8LL * FAN_STAGE * (round_up((long long)L.chunk * lanes, 32) / lanes));
   L.oPH = -1;
   return L;
 }
@@ -155,17 +160,43 @@ static Layout rows_layout_of(int nodes, int max_obs, int csize) {
 // nodes as a cluster of two 1.75 us (GB300, 20 obstacles) -- a split costs two
 // cluster barriers per iteration, half a microsecond, so it is made only where
 // one CTA cannot hold the instance.
-bool rows_layout(int model, int precision, int nodes, int max_obs, int group, int tpn, int optin, Layout* out) {
-  if (precision != UCN_PREC_FP32_REFINE) return false;
+//
+// FP64: the fan kernel for batches of at most one instance per SM -- 32 lanes per
+// node and 16 CTAs for one or two instances, 16 lanes and eight CTAs while the
+// SMs have room for them, else 8 lanes and 16 nodes per CTA.  More instances fill
+// the SMs' FP64 pipes with one CTA each, and four lanes per node do less work:
+// us per ADMM iteration, fan / lane kernel (GB300): one instance of 51 nodes 3.9
+// / 15.1, 40 of 31 nodes 7.2 / 11.1, 152 of 26 nodes 10.2 / 11.1, but 304 of
+// them 19.8 / 16.4 and 608 of 41 nodes 68 / 48.
+bool rows_layout(int model, int precision, int nodes, int max_obs, int group, int tpn, int batch, int optin, Layout* out) {
+  if (precision != UCN_PREC_FP32_REFINE) {
+    if (model != UCN_MODEL_QUAD12 || tpn != 4 || group > 1) return false;
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      return false;
+    if (batch > sms) return false;
+    const int lanes = batch <= 2 ? 32 : (long long)batch * 8 <= sms ? 16 : 8, cap = lanes == 32 ? 4 : lanes == 16 ? 8 : 16;
+    const int most = lanes == 32 ? 16 : 8;
+    for (int csize = lanes == 32 ? 2 : 1; csize <= most; csize *= 2) {
+      const int chunk = (nodes + csize - 1) / csize;
+      if (chunk > cap && (csize < most || chunk * lanes > FAN_THREADS)) continue;
+      const Layout L = rows_layout_of<Quad12>(nodes, max_obs, csize, lanes);
+      if (L.bytes + (long long)sizeof(InstShared) + (long long)sizeof(RowCluster) + 64 > optin) continue;
+      *out = L;
+      return true;
+    }
+    return false;
+  }
   const bool quad12 = model == UCN_MODEL_QUAD12;
   if (quad12 ? tpn != 4 : (tpn != 1 || (model != UCN_MODEL_QUAT13 && model != UCN_MODEL_MARS14))) return false;
   const long long fixed = (long long)sizeof(InstShared) + sizeof(RowCluster) + (group > 1 ? (long long)sizeof(GroupShared) : 0) + 64;
   for (int csize = 1; csize <= (group > 1 ? 1 : 4); csize *= 2) {
     const int cap = (csize == 1 && quad12 ? ROWS_WIDE_THREADS : ROWS_THREADS) / 4;
     if ((nodes + csize - 1) / csize > cap) continue;
-    const Layout L = quad12 ? rows_layout_of<Quad12>(nodes, max_obs, csize)
-                     : model == UCN_MODEL_QUAT13 ? rows_layout_of<Quat13>(nodes, max_obs, csize)
-                                                 : rows_layout_of<Mars14>(nodes, max_obs, csize);
+    const Layout L = quad12 ? rows_layout_of<Quad12>(nodes, max_obs, csize, 4)
+                     : model == UCN_MODEL_QUAT13 ? rows_layout_of<Quat13>(nodes, max_obs, csize, 4)
+                                                 : rows_layout_of<Mars14>(nodes, max_obs, csize, 4);
     if (L.bytes + fixed > optin) continue;
     *out = L;
     return true;
@@ -236,7 +267,7 @@ void rows_parts(ucn_problem* p, std::vector<int>& order) {
   p->parts.clear();
   const int tpn = default_tpn(p->model, p->Nmax + 1, p->precision);
   Layout L;
-  if (!rows_layout(p->model, p->precision, p->Nmax + 1, p->max_obs, p->group, tpn, p->optin, &L)) return;
+  if (!rows_layout(p->model, p->precision, p->Nmax + 1, p->max_obs, p->group, tpn, p->batch, p->optin, &L)) return;
   if (p->group > 1) {
     p->parts.push_back({L, 0, p->batch});
     return;
@@ -245,8 +276,8 @@ void rows_parts(ucn_problem* p, std::vector<int>& order) {
   auto shape = [&](int b) {
     const int nodes = p->horizon[b] + 1;
     Layout l;
-    rows_layout(p->model, p->precision, nodes, p->max_obs, 1, tpn, p->optin, &l);
-    return 2 * l.csize + (l.csize == 1 && l.chunk > ROWS_THREADS / 4 ? 1 : 0);
+    rows_layout(p->model, p->precision, nodes, p->max_obs, 1, tpn, p->batch, p->optin, &l);
+    return 2 * l.csize + (l.csize == 1 && l.lanes == 4 && l.chunk > ROWS_THREADS / 4 ? 1 : 0);
   };
   std::vector<int> s(p->batch), all;
   for (int b = 0; b < p->batch; ++b) s[b] = shape(b);
@@ -263,7 +294,7 @@ void rows_parts(ucn_problem* p, std::vector<int>& order) {
     int nodes = 0;
     for (int b : order)
       if (s[b] == v) { out.push_back(b); nodes = std::max(nodes, p->horizon[b] + 1); }
-    rows_layout(p->model, p->precision, nodes, p->max_obs, 1, tpn, p->optin, &L);
+    rows_layout(p->model, p->precision, nodes, p->max_obs, 1, tpn, p->batch, p->optin, &L);
     p->parts.push_back({L, first, (int)out.size() - first});
   }
   order = out;
@@ -587,18 +618,18 @@ long long ucn_total_x(const ucn_problem* p) { return p ? p->total_x : -1; }
 long long ucn_total_u(const ucn_problem* p) { return p ? p->total_u : -1; }
 long long ucn_state_size(const ucn_problem* p) { return p ? p->state_size : -1; }
 
-// Whether the fused solve and the ADMM call run the row kernel.
-static bool rows_on(const ucn_problem* p) {
-  return !p->parts.empty() && p->tpn == default_tpn(p->model, p->Nmax + 1, p->precision);
+// Whether the fused solve (or the ADMM call: FP32) runs the row or fan kernel.
+static bool rows_on(const ucn_problem* p, bool admm) {
+  return !p->parts.empty() && !(admm && p->precision == UCN_PREC_FP64) && p->tpn == default_tpn(p->model, p->Nmax + 1, p->precision);
 }
 
-static LaunchCfg cfg_of(ucn_problem* p, void* stream) {
+static LaunchCfg cfg_of(ucn_problem* p, void* stream, bool admm = false) {
   LaunchCfg c;
   c.P = &p->dev; c.L = &p->L; c.smem = p->smem; c.smem_bytes = p->smem_bytes;
   c.threads = p->threads; c.blocks = p->batch; c.stream = as_stream(stream); c.group = p->gcsize;
   c.nodes = p->Nmax + 1; c.tpn = p->tpn;
   c.launched = &p->last_launches;
-  if (rows_on(p)) {   // (a batch of several parts goes through launch_parts)
+  if (rows_on(p, admm)) {   // (a batch of several parts goes through launch_parts)
     c.L = &p->parts[0].L; c.smem = true; c.smem_bytes = p->parts[0].L.bytes;
   }
   p->last_launches = 1;   // one launch unless the launcher splits the batch
@@ -611,8 +642,8 @@ static LaunchCfg cfg_of(ucn_problem* p, void* stream) {
 // so that a part's CTAs fill the SMs that an earlier part's last ones leave.
 extern "C++" {
 template <class F>
-static cudaError_t launch_parts(ucn_problem* p, LaunchCfg c, F launch) {
-  if (!rows_on(p) || p->parts.size() == 1) return launch(c);
+static cudaError_t launch_parts(ucn_problem* p, LaunchCfg c, bool admm, F launch) {
+  if (!rows_on(p, admm) || p->parts.size() == 1) return launch(c);
   cudaStream_t s = c.stream;
   cudaError_t e = cudaEventRecord(p->fork, s);
   const ProblemDev base = *(const ProblemDev*)c.P;
@@ -656,9 +687,9 @@ ucn_status ucn_admm_solve(ucn_problem* p, const double* xbar_d, const double* ub
     return fail(UCN_EINVAL, "null argument");
   if (iters < 1) return fail(UCN_EINVAL, "iters must be >= 1");
   if (p->group > 1) return fail(UCN_EINVAL, "the scenario consensus runs inside ucn_scp_solve only");
-  const LaunchCfg c = cfg_of(p, stream);
+  const LaunchCfg c = cfg_of(p, stream, true);
   auto fn = launchers_for(p->model, p->precision).admm;
-  const cudaError_t e = launch_parts(p, c, [&](const LaunchCfg& k) {
+  const cudaError_t e = launch_parts(p, c, true, [&](const LaunchCfg& k) {
     return fn(k, xbar_d, ubar_d, A_d, B_d, d_d, radius_d, iters, warm ? 1 : 0, xhat_d, uhat_d, res_d, status_d);
   });
   if (e != cudaSuccess) return fail(UCN_ECUDA, "admm launch: %s", cudaGetErrorString(e));
@@ -693,7 +724,7 @@ ucn_status ucn_scp_solve(ucn_problem* p, const double* x0_d, const double* u0_d,
     return UCN_OK;
   }
   auto fn = launchers_for(p->model, p->precision).scp;
-  const cudaError_t e = launch_parts(p, c, [&](const LaunchCfg& k) {
+  const cudaError_t e = launch_parts(p, c, false, [&](const LaunchCfg& k) {
     return fn(k, x0_d, u0_d, x_out_d, u_out_d, stats_d, status_d);
   });
   if (e != cudaSuccess) return fail(UCN_ECUDA, "scp launch: %s", cudaGetErrorString(e));
@@ -716,7 +747,7 @@ ucn_status ucn_scp_solve_warm(ucn_problem* p, const double* x0_d, const double* 
   LaunchCfg c = cfg_of(p, stream);
   c.P = &Pw;
   auto fn = launchers_for(p->model, p->precision).scp;
-  const cudaError_t e = launch_parts(p, c, [&](const LaunchCfg& k) {
+  const cudaError_t e = launch_parts(p, c, false, [&](const LaunchCfg& k) {
     return fn(k, x0_d, u0_d, x_out_d, u_out_d, stats_d, status_d);
   });
   if (e != cudaSuccess) return fail(UCN_ECUDA, "scp launch: %s", cudaGetErrorString(e));

@@ -29,7 +29,9 @@ Layout make_layout(int model, int nodes, int max_obs, int tsize, bool reg_mats, 
 // node (12-state quadrotor 4, the others 1), 96 nodes per CTA (64 for the
 // others) and up to four CTAs per instance (one for scenario groups), within
 // the device's shared memory per CTA.  False where it does not.
-bool rows_layout(int model, int precision, int nodes, int max_obs, int group, int tpn, int optin, Layout* out);
+// FP64: the fan kernel's (ucn_fan.cuh) for the 12-state quadrotor at its default
+// threads per node, without scenario groups; `batch` instances share the device.
+bool rows_layout(int model, int precision, int nodes, int max_obs, int group, int tpn, int batch, int optin, Layout* out);
 
 // Everything one kernel launch needs besides its buffers.
 struct LaunchCfg {

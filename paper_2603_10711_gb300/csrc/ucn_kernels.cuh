@@ -138,13 +138,15 @@ struct CB {
 // on either side for the neighbours' boundary nodes.
 struct Layout {
   int S, NS, DS;           // SoA stride (nodes); AoS record strides (elements)
-  int chunk, csize;        // row kernel: nodes per CTA, CTAs per instance (0, 0: another kernel's layout)
+  int chunk, csize, lanes; // row and fan kernels: nodes per CTA, CTAs per instance, lanes per node (0: another
+                           // kernel's layout)
   int MS, MD, MB;          // mirror scalars / mirror data per node; exported mirror blocks
   int oS, oNus, oMd;       // runtime offsets of the mirror arrays in the record
   int oA, oB, oH;          // matrices in the record (-1 when register-resident)
   long long tbytes;        // bytes of the T region (16-byte multiple)
   long long bytes;         // bytes per instance
   long long oC;            // byte offset of the CB block (FP32 path; -1 without)
+  long long oX;            // byte offset of the fan kernel's staging
   long long oPH;           // byte offset of the pair kernel's per-lane H^-1 records (-1 without)
 };
 

@@ -6,6 +6,7 @@
 #include "ucn_linearize.cuh"
 #include "ucn_pair.cuh"
 #include "ucn_rows.cuh"
+#include "ucn_fan.cuh"
 
 namespace ucn {
 
@@ -218,6 +219,7 @@ template <class M, bool CL, int MAXT> RowAdmmKernel rows_admm_kernel();
 template <class K, class... Args>
 cudaError_t launch_rows_k(K k, const LaunchCfg& c, const Layout& L, int threads, unsigned cluster, Args... args) {
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem_bytes);
+  if (e == cudaSuccess && cluster > 8) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(c.blocks * L.csize), 1, 1);
@@ -287,6 +289,23 @@ cudaError_t launch_admm_rows(const LaunchCfg& c, const double* xbar, const doubl
                        status);
 }
 
+// The fan kernel (FP64, 12-state quadrotor), F lanes per node, alone or over a
+// cluster.
+template <int F, bool CL> RowScpKernel fan_scp_kernel();
+template <> RowScpKernel fan_scp_kernel<8, false>();
+template <> RowScpKernel fan_scp_kernel<8, true>();
+template <> RowScpKernel fan_scp_kernel<16, false>();
+template <> RowScpKernel fan_scp_kernel<16, true>();
+template <> RowScpKernel fan_scp_kernel<32, true>();
+inline cudaError_t launch_scp_fan(const LaunchCfg& c, const double* x0, const double* u0, double* xo, double* uo,
+                                  ucn_scp_stats* st, int* status) {
+  const Layout& L = *(const Layout*)c.L;
+  RowScpKernel k = L.lanes == 32 ? fan_scp_kernel<32, true>()
+                   : L.lanes == 16 ? (L.csize > 1 ? fan_scp_kernel<16, true>() : fan_scp_kernel<16, false>())
+                                 : (L.csize > 1 ? fan_scp_kernel<8, true>() : fan_scp_kernel<8, false>());
+  return launch_rows_k(k, c, L, (L.lanes * L.chunk + 31) / 32 * 32, (unsigned)L.csize, x0, u0, xo, uo, st, status);
+}
+
 template <class M, class T, bool R>
 cudaError_t launch_scp_t(const LaunchCfg& c, const double* x0, const double* u0, double* xo, double* uo,
                          ucn_scp_stats* st, int* status) {
@@ -295,6 +314,9 @@ cudaError_t launch_scp_t(const LaunchCfg& c, const double* x0, const double* u0,
   } else {
   if constexpr (RowModel<M>::value && std::is_same<T, float>::value) {
     if (((const Layout*)c.L)->csize > 0) return launch_scp_rows<M>(c, x0, u0, xo, uo, st, status);
+  }
+  if constexpr (std::is_same<M, Quad12>::value && std::is_same<T, double>::value) {
+    if (((const Layout*)c.L)->csize > 0) return launch_scp_fan(c, x0, u0, xo, uo, st, status);
   }
   if constexpr (std::is_same<M, Mars7>::value && std::is_same<T, float>::value && R) {
     if (c.tpn == 2) return launch_scpp_v<M, R>(c, x0, u0, xo, uo, st, status);
@@ -500,6 +522,12 @@ cudaError_t launch_linearize_t(const void* Pv, const int* node_inst, long long t
   namespace ucn {                                                                                          \
   template <>                                                                                              \
   RowAdmmKernel rows_admm_kernel<MODEL, CL, MAXT>() { return admm_rows_kernel<MODEL, CL, MAXT, REG>; }     \
+  }
+
+#define UCN_DEFINE_FAN(F, CL)                                                                              \
+  namespace ucn {                                                                                          \
+  template <>                                                                                              \
+  RowScpKernel fan_scp_kernel<F, CL>() { return scp_fan_kernel<F, CL>; }                                   \
   }
 
 // Pair-kernel variant in its own translation unit.

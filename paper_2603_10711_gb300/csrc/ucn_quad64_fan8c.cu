@@ -1,0 +1,4 @@
+// Fan kernel, FP64 12-state quadrotor: 8 lanes per node, an instance over a cluster.
+#include "ucn_launch.cuh"
+
+UCN_DEFINE_FAN(8, true)

@@ -994,7 +994,7 @@ __device__ __forceinline__ float rows_prepare(const RowPos& p, const Node<float,
 
 // ------------------------------------------------------------------ the fused solve
 struct RowCluster {
-  double x[2][8][6];   // totals of the CTAs of an instance (double-buffered)
+  double x[2][16][6];   // totals of the CTAs of an instance (double-buffered)
   unsigned par;
 };
 
@@ -1068,63 +1068,118 @@ __device__ __forceinline__ void rows_linear_model(const RowPos& p, const RowMats
   }
 }
 
-// scp_candidate for the row kernel: the rollout one thread per node, the linear
-// model by rows.
-template <class M, bool GROUP, bool CL>
-__device__ __forceinline__ void rows_candidate(const RowPos& p, const Node<float, 2>& nd, bool dact, const RowMats<M>& A,
-                                               const Layout& L, const ProblemDev& P, const Inst<float>& I, int b,
-                                               const GroupShared* G, InstShared& sh, DF* xc, DF* uc, DF* fc, double* v) {
+// scp_candidate with several lanes per node: the rollout one thread per node, the
+// linear model by rows.
+template <class E>
+__device__ __forceinline__ void split_candidate(const typename E::Pos& p, const Node<typename E::T, 2>& nd, bool dact,
+                                                const typename E::Mats& A, const Layout& L, const ProblemDev& P,
+                                                const Inst<typename E::T>& I, int b, const GroupShared* G,
+                                                InstShared& sh, typename WideOf<typename E::T>::type* xc,
+                                                typename WideOf<typename E::T>::type* uc,
+                                                typename WideOf<typename E::T>::type* fc, double* v) {
+  typedef typename E::M M;
+  typedef typename E::T T;
+  typedef typename WideOf<T>::type W;
   typedef Rec<M, 2> R;
-  constexpr int NX = M::NX, NU = M::NU, RX = RowMats<M>::RX;
+  constexpr int NX = M::NX, NU = M::NU;
   const int i = nd.i, N = nd.N;
   if (dact) {
     for (int j = 0; j < NX; ++j) {
-      xc[j] = df_add(nd.dat(R::Xbar, j), nd.at(R::Xh, j));
+      xc[j] = wide_add(nd.dat(R::Xbar, j), nd.at(R::Xh, j));
       nd.dat(R::Xc, j) = xc[j];
-      if constexpr (CL)
+      if constexpr (E::CL)
         if (threadIdx.x == 0 && p.rank > 0) st_cluster(nd.d + (i + L.chunk) * L.DS + R::Xc + j, p.rank - 1, xc[j]);
     }
-    for (int j = 0; j < NU; ++j) uc[j] = i < N ? df_add(nd.dat(R::Ubar, j), nd.at(R::Uh, j)) : DF();
-    if constexpr (GROUP) {
+    for (int j = 0; j < NU; ++j) uc[j] = i < N ? wide_add(nd.dat(R::Ubar, j), nd.at(R::Uh, j)) : W();
+    if constexpr (E::GROUP) {
       if (i == 0)
-        for (int j = 0; j < NU; ++j) uc[j] = wide_of_bits<DF>(G->u0[j]);
+        for (int j = 0; j < NU; ++j) uc[j] = wide_of_bits<W>(G->u0[j]);
     }
   }
-  if constexpr (CL) {
-    if (p.first) {
-#pragma unroll
-      for (int m = 0; m < RX; ++m)
-        if (rows_is_x<M>(m, p.q)) st_cluster(p.halo1 + R::Xh + 4 * m, p.rank - 1, p.tp[R::Xh + 4 * m]);
-    }
+  if constexpr (E::CL) {
+    E::push_hat(p);
     cluster_sync();
   } else {
     __syncthreads();
   }
-  float lin1 = 0.0f, st = 0.0f;
-  rows_linear_model<M>(p, A, lin1, st);
-  DF vs[3];
-  float dinf = 0.0f;
+  T lin1 = T(0), st = T(0);
+  E::linear_model(p, A, L, lin1, st);
+  W vs[3] = {W(), W(), W()};
+  decltype(wide_abs_round(W())) dinf = 0;
   if (dact) {
-    vs[0] = node_cost<M, float, 2>(nd, P, I, b, i, N, xc, uc);
+    vs[0] = node_cost<M, T, 2>(nd, P, I, b, i, N, xc, uc);
     if (i < N) {
-      rk4_wide<M, float, 2>(nd, P, b, xc, uc, fc);
+      rk4_wide<M, T, 2>(nd, P, b, xc, uc, fc);
 #pragma unroll
       for (int r = 0; r < NX; ++r) {
-        fc[r] = df_sub(fc[r], nd.dnb(R::Xc, r, i + 1));
-        vs[1] = df_add(vs[1], wide_abs(fc[r]));
-        dinf = fmaxf(dinf, wide_abs_round(fc[r]));
+        fc[r] = fc[r] - nd.dnb(R::Xc, r, i + 1);
+        vs[1] = vs[1] + wide_abs(fc[r]);
+        dinf = maxv(dinf, wide_abs_round(fc[r]));
       }
     }
   }
-  vs[2] = df_from(lin1);
-  float mx[2] = {dinf, st};
-  block_reduce_df(sh, vs, 3, mx, 2, v);
+  if constexpr (IsDF<T>::value) {
+    vs[2] = df_from(lin1);
+    float mx[2] = {dinf, st};
+    block_reduce_df(sh, vs, 3, mx, 2, v);
+  } else {
+    v[0] = vs[0]; v[1] = vs[1]; v[2] = lin1; v[3] = dinf; v[4] = st;
+    block_reduce(sh, v, 3, 5);
+  }
 }
 
-template <class M, bool GROUP, bool CL, bool REG>
-__device__ __forceinline__ void scp_rows_body(const ProblemDev& P, const Layout& L, const double* x0, const double* u0,
+// The row kernel as an engine of the split solve.
+template <class M_, bool GROUP_, bool CL_, bool REG>
+struct RowEngine {
+  typedef M_ M;
+  typedef float T;
+  static constexpr bool GROUP = GROUP_, CL = CL_;
+  typedef RowPos Pos;
+  typedef RowMats<M> Mats;
+  typedef RowConst<M> Const;
+  __device__ static __forceinline__ Pos place(const ProblemDev& P, const Layout& L, unsigned char* smem, int b,
+                                              Node<float, 2>& nd, Node<float, 2>& ndd, bool& dact) {
+    return rows_place<M, CL>(P, L, smem, b, nd, ndd, dact);
+  }
+  __device__ static __forceinline__ void jacobians(const Pos& p, const Node<float, 2>& nd, Mats& A, const float* prm,
+                                                   const Step3<float>& hs, const Layout&) {
+    rows_jacobians<M, REG ? 2 : 1>(p, nd, A, prm, hs);
+  }
+  __device__ static __forceinline__ float prepare(const Pos& p, const Node<float, 2>& nd, const Node<float, 2>& ndd,
+                                                  bool dact, const Layout& L, const ProblemDev& P, const Inst<float>& I,
+                                                  int b, float rad, float re, float rd, float rg, Mats& A, Const& K,
+                                                  InstShared& sh) {
+    return rows_prepare<M, CL>(p, nd, ndd, dact, L, P, I, b, rad, re, rd, rg, A, K, sh);
+  }
+  __device__ static __forceinline__ void admm(const Pos& p, const Mats& A, const Const& K, const Layout& L,
+                                              const Inst<float>& I, float mg, float re, float rd, float rg, int iters,
+                                              InstShared& sh, double* res, GroupShared* G, GroupX& X,
+                                              const ProblemDev& P, const Node<float, 2>& nd) {
+    rows_admm<M, GROUP, CL, REG>(p, A, K, L, I, mg, re, rd, rg, iters, sh, res, G, X, P, nd);
+  }
+  // the first node's candidate, for the linear model of the previous CTA's last node
+  __device__ static __forceinline__ void push_hat(const Pos& p) {
+    typedef Rec<M, 2> R;
+    if (p.first) {
+#pragma unroll
+      for (int m = 0; m < RowMats<M>::RX; ++m)
+        if (rows_is_x<M>(m, p.q)) st_cluster(p.halo1 + R::Xh + 4 * m, p.rank - 1, p.tp[R::Xh + 4 * m]);
+    }
+  }
+  __device__ static __forceinline__ void linear_model(const Pos& p, const Mats& A, const Layout&, float& lin1, float& st) {
+    rows_linear_model<M>(p, A, lin1, st);
+  }
+};
+
+// The fused solve (scp_body) by an engine E that puts several lanes on a node.
+template <class E>
+__device__ __forceinline__ void scp_split_body(const ProblemDev& P, const Layout& L, const double* x0, const double* u0,
                                               double* xout, double* uout, ucn_scp_stats* stats, int* status_out,
                                               const int b) {
+  typedef typename E::M M;
+  typedef typename E::T T;
+  typedef typename WideOf<T>::type W;
+  constexpr bool GROUP = E::GROUP, CL = E::CL;
   static_assert(!(GROUP && CL), "a scenario group's cluster holds one CTA per scenario");
   constexpr int NX = M::NX, NU = M::NU;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -1143,16 +1198,16 @@ __device__ __forceinline__ void scp_rows_body(const ProblemDev& P, const Layout&
     X.k = (int)blockIdx.x % P.group;
     if (threadIdx.x == 0) G->gfail = 0;
   }
-  Node<float, 2> nd, ndd;
+  Node<T, 2> nd, ndd;
   bool dact;
-  const RowPos p = rows_place<M, CL>(P, L, smem, b, nd, ndd, dact);
+  const typename E::Pos p = E::place(P, L, smem, b, nd, ndd, dact);
   const bool lead = p.rank == 0;
-  RowMats<M> A;
-  RowConst<M> K;
+  typename E::Mats A;
+  typename E::Const K;
   const long long xo = P.xoff[b], uo = P.uoff[b];
-  const Step3<float> hs = step_of<float>(P.dt[b]);
+  const Step3<T> hs = step_of<T>(P.dt[b]);
   const unsigned long long t0 = globaltimer_ns();
-  const Inst<float> I = make_inst<M, float>(P, b);
+  const Inst<T> I = make_inst<M, T>(P, b);
   if (threadIdx.x == 0) {
     sh.fail = 0; sh.status = ST_OK; sh.radius = P.tr_init; sh.stop = 0;
     split_barrier_init(sh.xbar, blockDim.x);
@@ -1160,22 +1215,22 @@ __device__ __forceinline__ void scp_rows_body(const ProblemDev& P, const Layout&
   X.bar = sh.xbar;
   X.in = &sh.red[0][0];
   // the records start at zero: rows beyond a model's are read, never set
-  for (int e = threadIdx.x; e < (L.chunk + (CL ? 2 : 0)) * L.NS; e += blockDim.x) ((float*)smem)[e] = 0.0f;
+  for (int e = threadIdx.x; e < (L.chunk + (CL ? 2 : 0)) * L.NS; e += blockDim.x) ((T*)smem)[e] = T(0);
   nd.prm = ndd.prm = sh.prm;
   stage_params<M>(sh, P, b);
-  stage_consts<M, float, 2>(ndd, P, b);
-  if (dact) load_nominal<M, float, 2>(ndd, L, x0, u0, xo, uo);
+  stage_consts<M, T, 2>(ndd, P, b);
+  if (dact) load_nominal<M, T, 2>(ndd, L, x0, u0, xo, uo);
   if constexpr (CL) {   // the halo's nominal: the next CTA's first node
     const int ih = ndd.i;
     if ((int)threadIdx.x == L.chunk && ih <= p.N)
-      for (int j = 0; j < NX; ++j) ndd.dat(Rec<M, 2>::Xbar, j) = df_from(x0[(xo + ih) * NX + j]);
+      for (int j = 0; j < NX; ++j) ndd.dat(Rec<M, 2>::Xbar, j) = wide_from_double<W>(x0[(xo + ih) * NX + j]);
     cluster_sync();
   } else {
     __syncthreads();
   }
   flag_bad_inputs<M>(P, b, x0, u0, xo, uo, sh);
-  scp_start<M, float, 2>(ndd, P, I, b, dact, sh);
-  if (dact) node_start<M, float, 2>(ndd, L, P, b);
+  scp_start<M, T, 2>(ndd, P, I, b, dact, sh);
+  if (dact) node_start<M, T, 2>(ndd, L, P, b);
   __syncthreads();
   double Jn0[1];
   if constexpr (CL) {   // J(nominal) over the instance (scp_start left this CTA's share)
@@ -1201,26 +1256,26 @@ __device__ __forceinline__ void scp_rows_body(const ProblemDev& P, const Layout&
       sh.rhof[3] = (float)sh.radius;
     }
     __syncthreads();
-    const float re = sh.rhof[0], rd = sh.rhof[1], rg = sh.rhof[2];
-    rows_jacobians<M, REG ? 2 : 1>(p, nd, A, sh.prmf, hs);
-    const float mg = rows_prepare<M, CL>(p, nd, ndd, dact, L, P, I, b, sh.rhof[3], re, rd, rg, A, K, sh);
+    const T re = rho_of<T>(sh, 0), rd = rho_of<T>(sh, 1), rg = rho_of<T>(sh, 2);
+    E::jacobians(p, nd, A, prm_of<T>(sh), hs, L);
+    const T mg = E::prepare(p, nd, ndd, dact, L, P, I, b, radius_of<T>(sh), re, rd, rg, A, K, sh);
     if constexpr (CL) {   // a failed factorisation anywhere stops the instance
       if (sh.fail && threadIdx.x < ncta) st_cluster(&sh.fail, threadIdx.x, 1);
       cluster_sync();
     }
     if constexpr (GROUP) {
       if (p.i == 0 && p.active) {
-        const DF ub = nd.dat(Rec<M, 2>::Ubar, p.q);
-        group_box_put<DF>(G, X, p.q, df_add(ub, p.tp[Rec<M, 2>::Xlo + 12]), df_add(ub, p.tp[Rec<M, 2>::Xhi + 12]));
+        const W ub = nd.dat(Rec<M, 2>::Ubar, p.q);
+        group_box_put<W>(G, X, p.q, wide_add(ub, p.tp[Rec<M, 2>::Xlo + 12]), wide_add(ub, p.tp[Rec<M, 2>::Xhi + 12]));
       }
-      group_begin<DF>(P, G, X, sh);
+      group_begin<W>(P, G, X, sh);
     }
     if (sh.fail) { if (threadIdx.x == 0) sh.status = ST_NUMERIC; iters_run++; break; }
-    rows_admm<M, GROUP, CL, REG>(p, A, K, L, I, mg, re, rd, rg, P.admm_iters, sh, res, G, X, P, nd);
+    E::admm(p, A, K, L, I, mg, re, rd, rg, P.admm_iters, sh, res, G, X, P, nd);
     ++iters_run;
-    DF xc[NX], uc[NU], fc[NX];
+    W xc[NX], uc[NU], fc[NX];
     double v[6] = {0, 0, 0, 0, 0, 0};
-    rows_candidate<M, GROUP, CL>(p, ndd, dact, A, L, P, I, b, G, sh, xc, uc, fc, v);
+    split_candidate<E>(p, ndd, dact, A, L, P, I, b, G, sh, xc, uc, fc, v);
     bool timed_out = false;
     if (threadIdx.x == 0) timed_out = globaltimer_ns() - t0 > P.timeout_ns;
     if constexpr (CL) {   // rank 0's clock decides (thread 0 of each CTA writes all the shares)
@@ -1250,7 +1305,7 @@ __device__ __forceinline__ void scp_rows_body(const ProblemDev& P, const Layout&
     if (sh.accept) {
       ++accepted;
       if (k < 64) mask |= (1ull << k);
-      if (dact) scp_move_nominal<M, float, 2>(ndd, L, P, b, xc, uc, fc);
+      if (dact) scp_move_nominal<M, T, 2>(ndd, L, P, b, xc, uc, fc);
       if constexpr (CL) {
         if ((int)threadIdx.x == L.chunk && ndd.i <= p.N)
           for (int j = 0; j < NX; ++j) ndd.dat(Rec<M, 2>::Xbar, j) = ndd.dat(Rec<M, 2>::Xc, j);
@@ -1260,7 +1315,7 @@ __device__ __forceinline__ void scp_rows_body(const ProblemDev& P, const Layout&
     if (sh.stop) break;
   }
   double w[6] = {0, 0, 0, 0, 0, 0};
-  scp_finish<M, float, 2>(ndd, L, P, I, b, dact, xo, uo, xout, uout, sh, w);
+  scp_finish<M, T, 2>(ndd, L, P, I, b, dact, xo, uo, xout, uout, sh, w);
   if constexpr (CL) {
     // cost, l1 defect, the two residual norms | max defect
     double t[6] = {w[0], w[1], res[0], res[1], w[2], sh.xbar[1] ? 1.0 : 0.0};
@@ -1286,7 +1341,7 @@ __global__ void __launch_bounds__(MAXT, 1) scp_rows_kernel(ProblemDev P, Layout 
                                                            int* status_out) {
   const int k = CL ? (int)blockIdx.x / L.csize : (int)blockIdx.x;
   const int b = (GROUP || !P.order) ? k : P.order[k];
-  scp_rows_body<M, GROUP, CL, REG>(P, L, x0, u0, xout, uout, stats, status_out, b);
+  scp_split_body<RowEngine<M, GROUP, CL, REG>>(P, L, x0, u0, xout, uout, stats, status_out, b);
 }
 
 // The stand-alone ADMM call (admm_kernel) on the row mapping: the caller's A, B
