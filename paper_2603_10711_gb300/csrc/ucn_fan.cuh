@@ -20,9 +20,9 @@
 // ~88 for two (F = 16) or ~140 for four (F = 8), against ~275 for eight with four
 // lanes per node: the more lanes the shorter, the fewer the less work in all.
 // Measured (GB300, four lanes per node -> this): one quadrotor of 50 nodes, 15 x
-// 200 iterations, 52.2 -> 13.6 ms (15.1 -> 4.1 us per ADMM iteration, 445 ->
+// 200 iterations, 52.2 -> 13.3 ms (15.1 -> 3.9 us per ADMM iteration, 445 ->
 // 90 us per SCP iteration outside it); 149 of 40..120 nodes, 10 x 200, 102.5 ->
-// 94.6 ms.  What bounds it: the FP64 pipes at F = 8 (70% busy, counters), else
+// 92.7 ms.  What bounds it: the FP64 pipes at F = 8 (70% busy, counters), else
 // the iteration's chain of FP64 latencies (64 cycles each) and exchanges.
 #pragma once
 #include "ucn_rows.cuh"
@@ -43,6 +43,7 @@ struct FanPos {
   int NS;
   double *t, *st;          // the node's record and staging
   double *halo0, *halo1;   // records before the first and after the last node
+  RowHalo* hb;             // arrival of the neighbours' boundary values
 };
 // Rows per lane, and lanes that share a row (F = 32: two, half of its columns each).
 template <int F>
@@ -172,7 +173,8 @@ __device__ __forceinline__ double fan_obstacles(const FanPos& p, const Layout& L
 template <int F, bool LAST, bool CL>
 __device__ __forceinline__ void fan_iteration(const FanPos& p, const FanMats<F>& A, const FanConst<F>& K, const Layout& L,
                                               int nobs, bool full, double& mg, double re, double rd, double rg,
-                                              double irg, double ired, double& rp, double& rdl, GroupX& X) {
+                                              double irg, double ired, bool head, RowHaloPhase& hp, double& rp,
+                                              double& rdl, GroupX& X) {
   typedef Rec<Quad12, 2> R;
   constexpr int NX = 12, RW = FanRows<F>::R;
   double* t = p.t;
@@ -180,6 +182,8 @@ __device__ __forceinline__ void fan_iteration(const FanPos& p, const FanMats<F>&
   const int q = p.q;
   double xo[RW];
   // ---- Step 1
+  if constexpr (CL)
+    if (!head) halo_wait<8 * NX>(p.hb, hp, 1, p.last, p.lane == 0);
 #pragma unroll
   for (int m = 0; m < RW; ++m) {
     const int e = q + F * m;
@@ -209,12 +213,11 @@ __device__ __forceinline__ void fan_iteration(const FanPos& p, const FanMats<F>&
       const double d = t[R::C + e] + gx;
       t[R::Ex1 + e] = d;
       if constexpr (CL)
-        if (p.last && p.owner) st_cluster(p.halo0 + R::Ex1 + e, p.rank + 1, d);
+        if (p.last && p.owner) st_async(p.halo0 + R::Ex1 + e, p.rank + 1, d, &p.hb->bar[0]);
     }
     if (LAST && p.active) t[R::X + e] = xo[m];
   }
-  if constexpr (CL) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-  else split_barrier_arrive(X.bar);
+  split_barrier_arrive(X.bar);
   // ---- Step 3 (before Step 2: see admm_iteration) and Step 4 for nu_x, nu_u
   double sv[RW], dz[RW];
 #pragma unroll
@@ -233,8 +236,8 @@ __device__ __forceinline__ void fan_iteration(const FanPos& p, const FanMats<F>&
     }
   }
   mg = fan_obstacles<F, LAST>(p, L, nobs, K.gr, vx, rg, irg, full, sv, rp);
-  if constexpr (CL) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-  else split_barrier_wait(X.bar, X.ph);
+  split_barrier_wait(X.bar, X.ph);
+  if constexpr (CL) halo_wait<8 * NX>(p.hb, hp, 0, p.first, p.lane == 0);
   // ---- Step 2: dynamic consensus, Eq. (5), then its duals (Step 4)
   if (p.later) {
 #pragma unroll
@@ -256,8 +259,8 @@ __device__ __forceinline__ void fan_iteration(const FanPos& p, const FanMats<F>&
         t[R::Lam + e] = lam + re * (xo[m] - z);
         t[R::Mu + e] = mun;
         t[R::Ex2 + e] = ex;
-        if constexpr (CL)
-          if (p.first && p.owner) st_cluster(p.halo1 + R::Ex2 + e, p.rank - 1, ex);
+        if constexpr (CL && !LAST)
+          if (p.first && p.owner) st_async(p.halo1 + R::Ex2 + e, p.rank - 1, ex, &p.hb->bar[1]);
       }
     }
   }
@@ -290,8 +293,7 @@ __device__ __forceinline__ void fan_iteration(const FanPos& p, const FanMats<F>&
       if (p.active && p.owner && (q + F * m < NX || p.hasU)) acc_sq(rdl, sv[m] + gz);
     }
   }
-  if constexpr (CL) cluster_sync();
-  else __syncthreads();
+  __syncthreads();
 }
 
 // The lane's consts and boxes (as node_setup), obstacles (as node_mirror_data and
@@ -536,12 +538,13 @@ struct FanEngine {
   __device__ static __forceinline__ void admm(const Pos& p, const Mats& A, const Const& K, const Layout& L,
                                               const Inst<double>& I, double mg, double re, double rd, double rg,
                                               int iters, InstShared& sh, double* res, GroupShared*, GroupX& X,
-                                              const ProblemDev&, const Node<double, 2>&) {
+                                              const ProblemDev&, const Node<double, 2>&, RowHaloPhase& hp) {
     const double irg = 1.0 / rg, ired = 1.0 / (re + rd);
     double rp = 0.0, rdl = 0.0;
     for (int it = 0; it + 1 < iters; ++it)
-      fan_iteration<F, false, CL>(p, A, K, L, I.nobs, it + 2 == iters, mg, re, rd, rg, irg, ired, rp, rdl, X);
-    fan_iteration<F, true, CL>(p, A, K, L, I.nobs, true, mg, re, rd, rg, irg, ired, rp, rdl, X);
+      fan_iteration<F, false, CL>(p, A, K, L, I.nobs, it + 2 == iters, mg, re, rd, rg, irg, ired, it == 0, hp, rp,
+                                  rdl, X);
+    fan_iteration<F, true, CL>(p, A, K, L, I.nobs, true, mg, re, rd, rg, irg, ired, iters == 1, hp, rp, rdl, X);
     reduce_residuals(sh, rp, rdl, res);
   }
   __device__ static __forceinline__ void push_hat(const Pos& p) {

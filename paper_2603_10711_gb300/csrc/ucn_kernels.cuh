@@ -395,7 +395,9 @@ template <> __device__ __forceinline__ const float* prm_of<float>(const InstShar
 // Per-CTA state of a scenario group's exchanges (one CTA per scenario).
 struct GroupShared {
   double mine[2][16];   // this CTA's contribution to the current exchange (double-buffered)
+  double inv;           // 1 / K (wide type)
   double box[8];        // the scenarios' common box of u_0: max lower, -(min upper), absolute
+  unsigned long long bar[2];   // one cluster per group: arrival of the peers' arguments, by parity
   double u0[4];         // the consensus u-hat_0 of the latest iteration, absolute (wide type)
   int gfail;            // sticky: a wait for another scenario of the group gave up
 };
@@ -557,6 +559,16 @@ __device__ __forceinline__ void group_allreduce(const ProblemDev& P, GroupShared
   else group_allreduce_flat<NV>(P, G, X, ns, out);
 }
 
+// Start of a group kernel, by thread 0 (a cluster barrier follows before the first exchange).
+__device__ __forceinline__ void group_init(const ProblemDev& P, GroupShared* G) {
+  G->gfail = 0;
+  if (P.gclusters <= 1)
+    for (int k = 0; k < 2; ++k) {
+      tx_init(&G->bar[k]);
+      tx_arm(&G->bar[k], (unsigned)P.group * 32u);
+    }
+}
+
 // The first-control consensus of an ADMM iteration.  Warp 0 of every CTA
 // publishes its scenario's Step-3 arguments as soon as Step 1 is done (lane l
 // holds that of control l mod 4), and collects the group's sums after Step 2:
@@ -568,9 +580,11 @@ __device__ __forceinline__ void group_allreduce(const ProblemDev& P, GroupShared
 // 1.6 us.  Every CTA of a group gets the same bits: one order of summation, of
 // an addition that commutes.
 //
-// One cluster per group: each CTA writes its values into all its peers' shared
-// memory before the iteration's cluster barrier.  Several: through its global
-// slot and counter, as group_allreduce_flat.
+// One cluster per group: each CTA stores its values into all its peers' shared
+// memory, which count the bytes on an mbarrier that warp 0 waits on -- no barrier
+// across the cluster (with a cluster barrier per iteration 16 groups of 16 took
+// 6.04 us per iteration, so 5.37; 64 groups 15.1, so 13.6).  Several:
+// through its global slot and counter, as group_allreduce_flat.
 __device__ __forceinline__ double wide_shfl_xor(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
 __device__ __forceinline__ DF wide_shfl_xor(DF a, int o) {
   return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
@@ -594,7 +608,7 @@ __device__ __forceinline__ void group_publish(const ProblemDev& P, GroupShared* 
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int r = (lane >> 2) + 8 * h;
-      if (r < P.group) st_cluster(X.in + ((X.pub & 1) * 16 + X.k) * 4 + j, (unsigned)r, bits);
+      if (r < P.group) st_async(X.in + ((X.pub & 1) * 16 + X.k) * 4 + j, (unsigned)r, bits, &G->bar[X.pub & 1]);
     }
   } else {
     double* slot = P.gx + (((long long)X.g * P.group + X.k) * 2 + (X.epoch & 1)) * 16;
@@ -612,6 +626,9 @@ __device__ __forceinline__ W group_collect(const ProblemDev& P, GroupShared* G, 
   W a = W();
   if (P.gclusters <= 1) {
     const double* in = X.in + (X.pub & 1) * 64;
+    if (!G->gfail && !tx_wait(&G->bar[X.pub & 1], (X.pub >> 1) & 1)) G->gfail = 1;
+    __syncwarp();
+    if (lane == 0) tx_arm(&G->bar[X.pub & 1], (unsigned)K * 32u);   // the exchange after next
     if ((lane >> 2) < K) a = wide_of_bits<W>(in[4 * (lane >> 2) + j]);
     if ((lane >> 2) + 8 < K) a = a + wide_of_bits<W>(in[4 * (lane >> 2) + 32 + j]);
 #pragma unroll
@@ -642,12 +659,12 @@ __device__ __forceinline__ void group_advance(const ProblemDev& P, GroupX& X) {
   else X.epoch++;
 }
 // The average of the K arguments of control j, clamped to the common box.
-__device__ __forceinline__ double group_mean(const GroupShared* G, double sum, int K, int j) {
-  return fmin(fmax(sum / (double)K, G->box[j]), -G->box[4 + j]);
+__device__ __forceinline__ double group_mean(const GroupShared* G, double sum, int j) {
+  return fmin(fmax(sum * G->inv, G->box[j]), -G->box[4 + j]);
 }
 __device__ __forceinline__ bool df_less(DF a, DF b) { return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo); }
-__device__ __forceinline__ DF group_mean(const GroupShared* G, DF sum, int K, int j) {
-  DF v = df_div(sum, df_from((float)K));
+__device__ __forceinline__ DF group_mean(const GroupShared* G, DF sum, int j) {
+  DF v = df_mul(sum, wide_of_bits<DF>(G->inv));
   const DF lo = wide_of_bits<DF>(G->box[j]), hi = wide_of_bits<DF>(G->box[4 + j]);
   if (df_less(v, lo)) v = lo;
   if (df_less(hi, v)) v = hi;
@@ -669,6 +686,7 @@ __device__ __forceinline__ void group_begin(const ProblemDev& P, GroupShared* G,
   group_allreduce<9>(P, G, X, 0, a);
   if (threadIdx.x == 0) {
     sh.fail = a[0] != 0.0;
+    G->inv = wide_bits(wide_from_double<W>(1.0 / (double)P.group));
     for (int j = 0; j < 4; ++j) {
       const double hi = -a[5 + j];
       G->box[j] = wide_bits(wide_from_double<W>(a[1 + j]));
@@ -1495,17 +1513,6 @@ __device__ __forceinline__ void node_mirrors(const Node<T, AOS>& nd, const Layou
   }
 }
 
-// The barrier between Steps 1 and 2 of a scenario group: the cluster's (the
-// peers' arguments have arrived with it) or, across clusters, the CTA's.
-__device__ __forceinline__ void group_arrive(const ProblemDev& P, GroupX& X) {
-  if (P.gclusters <= 1) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-  else split_barrier_arrive(X.bar);
-}
-__device__ __forceinline__ void group_arrived(const ProblemDev& P, GroupX& X) {
-  if (P.gclusters <= 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-  else split_barrier_wait(X.bar, X.ph);
-}
-
 // Mirror initialisation / re-seeding from (x-hat, u-hat) in deviations.
 template <class M, class T, int AOS>
 __device__ void node_reseed(const Node<T, AOS>& nd, const Layout& L, const Inst<T>& I) {
@@ -1600,8 +1607,8 @@ __device__ __forceinline__ void admm_iteration(const Node<T, AOS>& nd, const MS&
         }
         group_publish<W>(P, G, X, own);
       }
-      group_arrive(P, X);
-    } else split_barrier_arrive(X.bar);
+    }
+    split_barrier_arrive(X.bar);
     T dz[NX];
     T sv[NN];
 #pragma unroll
@@ -1631,8 +1638,7 @@ __device__ __forceinline__ void admm_iteration(const Node<T, AOS>& nd, const MS&
       }
       node_mirrors<M, T, AOS, NN>(nd, L, I, rg, irg, x, false, last, sv, rp);   // control sets: i < N only
     }
-    if constexpr (GROUP) group_arrived(P, X);
-    else split_barrier_wait(X.bar, X.ph);
+    split_barrier_wait(X.bar, X.ph);
     if (active) {
       // ---- Step 2: dynamic consensus, Eq. (5), then its duals (Step 4)
       if (i >= 1) {
@@ -1666,7 +1672,7 @@ __device__ __forceinline__ void admm_iteration(const Node<T, AOS>& nd, const MS&
       if (active && i == 0 && i < N) {
 #pragma unroll
         for (int j = 0; j < NU; ++j) {
-          const W v = group_mean(G, tot[j], P.group, j);
+          const W v = group_mean(G, tot[j], j);
           G->u0[j] = wide_bits(v);
           const T uh = wide_diff<T>(v, nd.dat(Rec<M, AOS>::Ubar, j));
           const T nuu = S.nuu(j);
@@ -2351,7 +2357,7 @@ __device__ __forceinline__ void scp_body(const ProblemDev& P, const Layout& L, c
   if constexpr (GROUP) {
     X.g = (int)blockIdx.x / P.group;
     X.k = (int)blockIdx.x % P.group;
-    if (threadIdx.x == 0) G->gfail = 0;
+    if (threadIdx.x == 0) group_init(P, G);
   }
   constexpr int AOS = SMEM;
   Node<T, AOS> nd = make_node<T, SMEM>(P, L, smem, b);

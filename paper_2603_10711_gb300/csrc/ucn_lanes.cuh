@@ -8,6 +8,8 @@
 // warps per scheduler and is latency-bound.  The per-SCP-iteration work
 // (assembly and factorisation, the wide rollout, acceptance) maps one thread
 // to one node again; the Jacobian directions are split over the lanes.
+// Serves the FP64 solves of more than one instance per SM, FP64 scenario groups
+// and the request loop; the others have the row and the fan kernel.
 #pragma once
 #include "ucn_kernels.cuh"
 
@@ -355,8 +357,8 @@ __device__ __forceinline__ void admm_iteration_lanes(const Node<T, AOS>& nd, con
       a = wide_shfl(wide_add(a, xo[RX] + nuu * irg), (int)threadIdx.x & 3);
       group_publish<W>(P, G, X, a);
     }
-    group_arrive(P, X);
-  } else split_barrier_arrive(X.bar);
+  }
+  split_barrier_arrive(X.bar);
   T dz[RX];
   T sv[R];
 #pragma unroll
@@ -408,8 +410,7 @@ __device__ __forceinline__ void admm_iteration_lanes(const Node<T, AOS>& nd, con
       }
     }
   }
-  if constexpr (GROUP) group_arrived(P, X);
-  else split_barrier_wait(X.bar, X.ph);
+  split_barrier_wait(X.bar, X.ph);
   if (active) {
     // ---- Step 2: dynamic consensus, Eq. (5), then its duals (Step 4)
     if (i >= 1) {
@@ -436,7 +437,7 @@ __device__ __forceinline__ void admm_iteration_lanes(const Node<T, AOS>& nd, con
     if (threadIdx.x < 32) {
       const W sum = group_collect<W>(P, G, X);
       if (active && i == 0 && i < N) {
-        const W v = group_mean(G, sum, P.group, q);
+        const W v = group_mean(G, sum, q);
         G->u0[q] = wide_bits(v);
         const T uh = wide_diff<T>(v, nd.dat(Rec<M>::Ubar, q));
         const T nuu = nd.at(Rec<M>::Nuu, q);
@@ -539,7 +540,7 @@ __device__ __forceinline__ void scp_lanes_body(const ProblemDev& P, const Layout
   if constexpr (GROUP) {
     X.g = (int)blockIdx.x / P.group;
     X.k = (int)blockIdx.x % P.group;
-    if (threadIdx.x == 0) G->gfail = 0;
+    if (threadIdx.x == 0) group_init(P, G);
   }
   constexpr int AOS = SMEM;
   const int q = (int)threadIdx.x % TPN;

@@ -528,6 +528,22 @@ __device__ __forceinline__ void proj_cone3c(T* v, T tau, T ca, T sa) {
   v[2] *= r;
 }
 
+// The FP32 forms of both by selection instead of branches (the same numbers).
+__device__ __forceinline__ void proj_ball3s(float* y, float R) {
+  const float n2 = y[0] * y[0] + y[1] * y[1] + y[2] * y[2];
+  const float s = n2 > R * R ? R * rsqrtf(n2) : 1.0f;
+  y[0] *= s; y[1] *= s; y[2] *= s;
+}
+__device__ __forceinline__ void proj_cone3s(float* v, float tau, float ca, float sa) {
+  const float t = v[0], s2 = v[1] * v[1] + v[2] * v[2], t2 = t * t, tau2 = tau * tau;
+  const bool in = t >= 0.0f && s2 <= tau2 * t2, polar = t <= 0.0f && tau2 * s2 <= t2;
+  const float rs = rsqrtf(s2), c = t * ca + s2 * rs * sa;   // (not used where s2 = 0: in or polar)
+  v[0] = in ? t : polar ? 0.0f : c * ca;
+  const float r = in ? 1.0f : polar ? 0.0f : c * sa * rs;
+  v[1] *= r;
+  v[2] *= r;
+}
+
 template <class T> __device__ __forceinline__ T clampv(T v, T lo, T hi) { return fmin(fmax(v, lo), hi); }
 // max / |.| in the type of the arguments (never promoted to FP64 for floats)
 __device__ __forceinline__ float maxv(float a, float b) { return fmaxf(a, b); }
@@ -589,6 +605,38 @@ __device__ __forceinline__ void st_cluster(const int* local, unsigned rank, int 
 __device__ __forceinline__ void st_cluster(const DF* local, unsigned rank, DF v) {
   st_cluster(&local->hi, rank, v.hi);
   st_cluster(&local->lo, rank, v.lo);
+}
+
+// Point-to-point exchange within a cluster: the receiver's mbarrier counts the
+// bytes that its peers' asynchronous stores bring.  A phase completes when its
+// owner has armed it (one arrival, `bytes` expected) and all have come, in either
+// order.
+__device__ __forceinline__ void tx_init(unsigned long long* bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((unsigned)__cvta_generic_to_shared(bar)) : "memory");
+}
+__device__ __forceinline__ void tx_arm(unsigned long long* bar, unsigned bytes) {
+  asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}" ::"r"(
+                   (unsigned)__cvta_generic_to_shared(bar)), "r"(bytes) : "memory");
+}
+// Waits for the phase of this parity; false when it gave up (bounded).
+__device__ __forceinline__ bool tx_wait(unsigned long long* bar, unsigned parity) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(bar);
+  for (int it = 0; it < (1 << 20); ++it) {
+    unsigned done;
+    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(done) : "r"(a), "r"(parity) : "memory");
+    if (done) return true;
+  }
+  return false;
+}
+// v to the place of `local` in CTA `rank`, counted by its mbarrier at `bar`'s place.
+__device__ __forceinline__ void st_async(const float* local, unsigned rank, float v, const unsigned long long* bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(cluster_addr(local, rank)),
+               "r"(__float_as_int(v)), "r"(cluster_addr(bar, rank)) : "memory");
+}
+__device__ __forceinline__ void st_async(const double* local, unsigned rank, double v, const unsigned long long* bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(cluster_addr(local, rank)),
+               "l"(__double_as_longlong(v)), "r"(cluster_addr(bar, rank)) : "memory");
 }
 
 __device__ __forceinline__ unsigned long long globaltimer_ns() {

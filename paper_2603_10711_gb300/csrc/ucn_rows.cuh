@@ -29,7 +29,9 @@
 // An instance may be split over the CTAs of a thread-block cluster (CL), `chunk`
 // consecutive nodes each.  Only boundary nodes talk across CTAs: they store
 // their exchange vectors into the neighbour's halo records in distributed
-// shared memory, and the two barriers of an iteration become cluster barriers.
+// shared memory, asynchronously, and the neighbour's boundary node waits for the
+// bytes on an mbarrier of its own; the iteration's barriers stay the CTA's (121
+// nodes on two CTAs: 1.79 us per iteration with cluster barriers, 1.75 so).
 #pragma once
 #include "ucn_kernels.cuh"
 
@@ -73,6 +75,39 @@ __device__ __forceinline__ unsigned cluster_rank() {
   return r;
 }
 
+// Arrival of the neighbours' boundary values in the halo records: [0] Ex1 from the
+// CTA before, [1] Ex2 from the one after; phases completed (every thread's copy).
+// A sender is at most one iteration ahead of its receiver, and sends an exchange
+// vector only when the receiver has used the last one: Ex1 of iteration k + 1
+// follows the receiver's Ex2 of iteration k, which follows its use of Ex1 of k,
+// and the other way round.  The last iteration of a call sends no Ex2: the next
+// call's set-up does, before a cluster barrier.
+struct RowHalo {
+  unsigned long long bar[2];
+  int fail;
+};
+struct RowHaloPhase {
+  unsigned n[2];
+};
+// Waits for exchange w if this thread's node uses it (`on`), then re-arms it (one
+// lane, `arm`).  Warps call it whole.
+template <unsigned BYTES>
+__device__ __forceinline__ void halo_wait(RowHalo* hb, RowHaloPhase& ph, int w, bool on, bool arm) {
+  if (on && !tx_wait(&hb->bar[w], ph.n[w] & 1u)) hb->fail = 1;
+  __syncwarp();
+  if (on && arm) tx_arm(&hb->bar[w], BYTES);
+  ph.n[w]++;
+}
+// Start of a cluster kernel, by thread 0 (a cluster barrier follows).
+template <unsigned BYTES>
+__device__ __forceinline__ void halo_init(RowHalo* hb) {
+  hb->fail = 0;
+  for (int w = 0; w < 2; ++w) {
+    tx_init(&hb->bar[w]);
+    tx_arm(&hb->bar[w], BYTES);
+  }
+}
+
 // One thread's place: its node, its lane, and whether it takes part.
 struct RowPos {
   int i, N, q;
@@ -84,6 +119,7 @@ struct RowPos {
   unsigned rank;
   bool first, last;
   float *halo0, *halo1;       // records before the first and after the last node
+  RowHalo* hb;                // arrival of the neighbours' boundary values
 };
 
 template <class M>
@@ -388,8 +424,8 @@ __device__ __forceinline__ void rows_sets(const RowPos& p, const Layout& L, cons
 template <class M, bool LAST, bool GROUP, bool CL, class ST>
 __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>& A, const RowConst<M>& K, const ST& S,
                                                const Layout& L, const Inst<float>& I, float& mg, float re, float rd,
-                                               float rg, float irg, float ired, DF& rp, DF& rdl, GroupShared* G,
-                                               GroupX& X, const ProblemDev& P, const Node<float, 2>& nd) {
+                                               float rg, float irg, float ired, bool head, RowHaloPhase& hp, DF& rp,
+                                               DF& rdl, GroupShared* G, GroupX& X, const ProblemDev& P, const Node<float, 2>& nd) {
   typedef Rec<M, 2> R;
   constexpr int RX = RowMats<M>::RX, RE = RowConst<M>::R;
   constexpr bool EX = RowMats<M>::EX, QUAD = IsQuad<M>::value;
@@ -397,6 +433,8 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
   const int q = p.q;
   float xo[RE];
   // ---- Step 1
+  if constexpr (CL)
+    if (!head) halo_wait<4 * M::NX>(p.hb, hp, 1, p.last, q == 0);
   {
     float g[RE];
     {
@@ -436,6 +474,15 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
     rows_solve<M>(A, r, dx);
 #pragma unroll
     for (int m = 0; m < RE; ++m) xo[m] += dx[m];
+    if constexpr (GROUP) {
+      // the arguments of u_0, as early as they are known: node 0 is the first four
+      // lanes; lane l hands over control l mod 4
+      if (threadIdx.x < 32) {
+        DF a = p.i == 0 ? nd.dat(R::Ubar, q) : DF();
+        a = wide_shfl(df_add(a, xo[3] + S.nu(3) * irg), (int)threadIdx.x & 3);
+        group_publish<DF>(P, G, X, a);
+      }
+    }
     // linearised propagation d_dyn,i = A x + B u + c_i, published to node i+1
     rows_gather<4>(xo, v);
     rows_G<M>(A, v, EX ? xo[RE - 1] : 0.0f, t);
@@ -448,7 +495,8 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
       if constexpr (CL)
         if (p.last) {
 #pragma unroll
-          for (int m = 0; m < RX; ++m) st_cluster(p.halo0 + R::Ex1 + 4 * m, p.rank + 1, t[m]);
+          for (int m = 0; m < RX; ++m)
+            if (rows_is_x<M>(m, q)) st_async(p.halo0 + R::Ex1 + 4 * m, p.rank + 1, t[m], &p.hb->bar[0]);
         }
     }
     if (p.active && (LAST || !QUAD)) {
@@ -457,15 +505,7 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
     }
   }
   // Step 3 before Step 2, between the arrival (Ex1 published) and the wait
-  if constexpr (CL) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-  else if constexpr (GROUP) {
-    if (threadIdx.x < 32) {   // node 0 is the first four lanes; lane l hands over control l mod 4
-      DF a = p.i == 0 ? nd.dat(R::Ubar, q) : DF();
-      a = wide_shfl(df_add(a, xo[3] + S.nu(3) * irg), (int)threadIdx.x & 3);
-      group_publish<DF>(P, G, X, a);
-    }
-    group_arrive(P, X);
-  } else split_barrier_arrive(X.bar);
+  split_barrier_arrive(X.bar);
   float sv[RE], dz[RX], svr[3] = {0.0f, 0.0f, 0.0f};
   if (LAST) {
 #pragma unroll
@@ -488,9 +528,8 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
   }
   if constexpr (QUAD) mg = rows_obstacles<M, LAST>(p, L, I.nobs, xo, rg, irg, sv, rp);
   else rows_sets<M, LAST, false>(p, L, I, rg, irg, R::X, svr, rp);
-  if constexpr (CL) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-  else if constexpr (GROUP) group_arrived(P, X);
-  else split_barrier_wait(X.bar, X.ph);
+  split_barrier_wait(X.bar, X.ph);
+  if constexpr (CL) halo_wait<4 * M::NX>(p.hb, hp, 0, p.first, q == 0);
   // ---- Step 2: dynamic consensus, Eq. (5), then its duals (Step 4)
 #pragma unroll
   for (int m = 0; m < RX; ++m) dz[m] = 0.0f;
@@ -510,15 +549,15 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
         const float mun = mu + rd * (z - dd);
         S.set_dyn(m, z, lam + re * (xo[m] - z), mun);
         tp[R::Ex2 + 4 * m] = mun + rd * z;
-        if constexpr (CL)
-          if (p.first) st_cluster(p.halo1 + R::Ex2 + 4 * m, p.rank - 1, mun + rd * z);
+        if constexpr (CL && !LAST)
+          if (p.first) st_async(p.halo1 + R::Ex2 + 4 * m, p.rank - 1, mun + rd * z, &p.hb->bar[1]);
       }
   }
   if constexpr (GROUP) {
     if (threadIdx.x < 32) {
       const DF sum = group_collect<DF>(P, G, X);
       if (p.i == 0 && p.active) {
-        const DF v = group_mean(G, sum, P.group, q);
+        const DF v = group_mean(G, sum, q);
         G->u0[q] = wide_bits(v);
         const float uh = wide_diff<float>(v, nd.dat(R::Ubar, q));
         const float nu = S.nu(3);
@@ -581,8 +620,7 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
         }
     }
   }
-  if constexpr (CL) cluster_sync();
-  else __syncthreads();
+  __syncthreads();
 }
 
 // `iters` iterations; the squared residual norms of the last one (this CTA's
@@ -591,14 +629,16 @@ template <class M, bool GROUP, bool CL, bool REG>
 __device__ __forceinline__ void rows_admm(const RowPos& p, const RowMats<M>& A, const RowConst<M>& K, const Layout& L,
                                           const Inst<float>& I, float mg, float re, float rd, float rg, int iters,
                                           InstShared& sh, double* res, GroupShared* G, GroupX& X, const ProblemDev& P,
-                                          const Node<float, 2>& nd) {
+                                          const Node<float, 2>& nd, RowHaloPhase& hp) {
   const float irg = 1.0f / rg, ired = 1.0f / (re + rd);
   DF rp, rdl;
   RowState<M, REG> S;
   S.load(p);
   for (int it = 0; it + 1 < iters; ++it)
-    rows_iteration<M, false, GROUP, CL>(p, A, K, S, L, I, mg, re, rd, rg, irg, ired, rp, rdl, G, X, P, nd);
-  rows_iteration<M, true, GROUP, CL>(p, A, K, S, L, I, mg, re, rd, rg, irg, ired, rp, rdl, G, X, P, nd);
+    rows_iteration<M, false, GROUP, CL>(p, A, K, S, L, I, mg, re, rd, rg, irg, ired, it == 0, hp, rp, rdl, G, X, P,
+                                         nd);
+  rows_iteration<M, true, GROUP, CL>(p, A, K, S, L, I, mg, re, rd, rg, irg, ired, iters == 1, hp, rp, rdl, G, X, P,
+                                      nd);
   S.store(p);
   reduce_residuals(sh, rp, rdl, res);
 }
@@ -994,6 +1034,7 @@ __device__ __forceinline__ float rows_prepare(const RowPos& p, const Node<float,
 
 // ------------------------------------------------------------------ the fused solve
 struct RowCluster {
+  RowHalo halo;
   double x[2][16][6];   // totals of the CTAs of an instance (double-buffered)
   unsigned par;
 };
@@ -1154,8 +1195,8 @@ struct RowEngine {
   __device__ static __forceinline__ void admm(const Pos& p, const Mats& A, const Const& K, const Layout& L,
                                               const Inst<float>& I, float mg, float re, float rd, float rg, int iters,
                                               InstShared& sh, double* res, GroupShared* G, GroupX& X,
-                                              const ProblemDev& P, const Node<float, 2>& nd) {
-    rows_admm<M, GROUP, CL, REG>(p, A, K, L, I, mg, re, rd, rg, iters, sh, res, G, X, P, nd);
+                                              const ProblemDev& P, const Node<float, 2>& nd, RowHaloPhase& hp) {
+    rows_admm<M, GROUP, CL, REG>(p, A, K, L, I, mg, re, rd, rg, iters, sh, res, G, X, P, nd, hp);
   }
   // the first node's candidate, for the linear model of the previous CTA's last node
   __device__ static __forceinline__ void push_hat(const Pos& p) {
@@ -1189,18 +1230,22 @@ __device__ __forceinline__ void scp_split_body(const ProblemDev& P, const Layout
   if constexpr (CL) {
     __shared__ RowCluster rc;
     cl = &rc;
+    if (threadIdx.x == 0) halo_init<(unsigned)(sizeof(T) * M::NX)>(&rc.halo);
   }
+  RowHaloPhase hp{{0u, 0u}};
   unsigned par = 0;
   const unsigned ncta = CL ? (unsigned)L.csize : 1u;
   GroupX X{0u, 0, 0};
   if constexpr (GROUP) {
     X.g = (int)blockIdx.x / P.group;
     X.k = (int)blockIdx.x % P.group;
-    if (threadIdx.x == 0) G->gfail = 0;
+    if (threadIdx.x == 0) group_init(P, G);
   }
   Node<T, 2> nd, ndd;
   bool dact;
-  const typename E::Pos p = E::place(P, L, smem, b, nd, ndd, dact);
+  typename E::Pos pos = E::place(P, L, smem, b, nd, ndd, dact);
+  if constexpr (CL) pos.hb = &cl->halo;
+  const typename E::Pos& p = pos;
   const bool lead = p.rank == 0;
   typename E::Mats A;
   typename E::Const K;
@@ -1271,7 +1316,7 @@ __device__ __forceinline__ void scp_split_body(const ProblemDev& P, const Layout
       group_begin<W>(P, G, X, sh);
     }
     if (sh.fail) { if (threadIdx.x == 0) sh.status = ST_NUMERIC; iters_run++; break; }
-    E::admm(p, A, K, L, I, mg, re, rd, rg, P.admm_iters, sh, res, G, X, P, nd);
+    E::admm(p, A, K, L, I, mg, re, rd, rg, P.admm_iters, sh, res, G, X, P, nd, hp);
     ++iters_run;
     W xc[NX], uc[NU], fc[NX];
     double v[6] = {0, 0, 0, 0, 0, 0};
@@ -1318,10 +1363,11 @@ __device__ __forceinline__ void scp_split_body(const ProblemDev& P, const Layout
   scp_finish<M, T, 2>(ndd, L, P, I, b, dact, xo, uo, xout, uout, sh, w);
   if constexpr (CL) {
     // cost, l1 defect, the two residual norms | max defect
-    double t[6] = {w[0], w[1], res[0], res[1], w[2], sh.xbar[1] ? 1.0 : 0.0};
+    double t[6] = {w[0], w[1], res[0], res[1], w[2], sh.xbar[1] || cl->halo.fail ? 1.0 : 0.0};
     __threadfence();
     rows_combine(*cl, par, p.rank, ncta, t, 4, 6);
     w[0] = t[0]; w[1] = t[1]; res[0] = t[2]; res[1] = t[3]; w[2] = t[4];
+    if (threadIdx.x == 0 && t[5] != 0.0) sh.xbar[1] = 1ull;   // (reported as a numerical failure)
   }
   if (threadIdx.x == 0 && lead) {
     bool gfail = false;
@@ -1359,14 +1405,17 @@ __global__ void __launch_bounds__(MAXT, 1) admm_rows_kernel(ProblemDev P, Layout
   if constexpr (CL) {
     __shared__ RowCluster rc;
     cl = &rc;
+    if (threadIdx.x == 0) halo_init<4 * M::NX>(&rc.halo);
   }
+  RowHaloPhase hp{{0u, 0u}};
   unsigned par = 0;
   const unsigned ncta = CL ? (unsigned)L.csize : 1u;
   // the longest instances first, as the fused solve takes them
   const int b = P.order[CL ? (int)blockIdx.x / L.csize : (int)blockIdx.x];
   Node<float, 2> nd, ndd;
   bool dact;
-  const RowPos p = rows_place<M, CL>(P, L, smem, b, nd, ndd, dact);
+  RowPos p = rows_place<M, CL>(P, L, smem, b, nd, ndd, dact);
+  if constexpr (CL) p.hb = &cl->halo;
   RowMats<M> A;
   RowConst<M> K;
   const long long xo = P.xoff[b], uo = P.uoff[b];
@@ -1412,7 +1461,7 @@ __global__ void __launch_bounds__(MAXT, 1) admm_rows_kernel(ProblemDev P, Layout
   }
   double r2[2] = {0.0, 0.0};
   GroupX X{0u, 0, 0, 0u, nullptr, sh.xbar, 0u};
-  if (!sh.fail) rows_admm<M, false, CL, REG>(p, A, K, L, I, mg, re, rd, rg, iters, sh, r2, nullptr, X, P, nd);
+  if (!sh.fail) rows_admm<M, false, CL, REG>(p, A, K, L, I, mg, re, rd, rg, iters, sh, r2, nullptr, X, P, nd, hp);
   __syncthreads();
   if (dact) {
     const int i = ndd.i;
@@ -1422,9 +1471,10 @@ __global__ void __launch_bounds__(MAXT, 1) admm_rows_kernel(ProblemDev P, Layout
       for (int j = 0; j < NU; ++j) uhat[(uo + i) * NU + j] = df_to_double(ndd.dat(R::Ubar, j)) + (double)ndd.at(R::Uh, j);
   }
   if constexpr (CL) {
-    double t[3] = {r2[0], r2[1], sh.xbar[1] ? 1.0 : 0.0};
+    double t[3] = {r2[0], r2[1], sh.xbar[1] || cl->halo.fail ? 1.0 : 0.0};
     rows_combine(*cl, par, p.rank, ncta, t, 2, 3);
     r2[0] = t[0]; r2[1] = t[1];
+    if (threadIdx.x == 0 && t[2] != 0.0) sh.xbar[1] = 1ull;
   }
   if (threadIdx.x == 0 && p.rank == 0) {
     res[2 * b] = sqrt(r2[0]);
