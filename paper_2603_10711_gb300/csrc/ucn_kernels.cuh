@@ -178,6 +178,15 @@ template <class M> struct IsQuad {
 // The 6-DOF Mars model: its own sets (glide slope on r, tilt on (qy, qz), body
 // rate ball, thrust ball and lower bound, gimbal cone on the body thrust).
 template <class M> struct IsMars14 { static constexpr bool value = std::is_same<M, Mars14>::value; };
+// The 3-DOF Mars sets on the FP32 path without branches in the ADMM loop: every
+// set is computed, and one that is off (or a control set at node N) is selected
+// away.  A uniform branch and a divergent early return cost this 8-warps-per-SM
+// kernel more (branch resolution, reconvergence) than the few instructions: 304
+// instances of 31 nodes, 1.60 -> 1.30 us per ADMM iteration.
+template <class M, class T> struct FlatSets {
+  static constexpr bool value = std::is_same<M, Mars7>::value && std::is_same<T, float>::value;
+};
+
 // Mirror slots of the 6-DOF model in the record (scalars s and nu_s; data).
 struct M14 {
   static constexpr int S_CONE = 0, S_BALL = 3, S_HALF = 6, S_TILT = 7, S_W = 9, S_GIM = 12, MS = 15;
@@ -281,6 +290,24 @@ __device__ __forceinline__ void acc_AA(T& acc, const MS& MT, int k, int r, int c
   else if (kr == 1) acc += MT.A(k, c);
   else if (kc == 1) acc += MT.A(k, r);
   else acc += MT.A(k, r) * MT.A(k, c);
+}
+
+// The matrices of a thread whose node has no control, where the ADMM loop does not
+// branch on that (FlatSets): zero A and B.
+template <class M, class T, class MS>
+__device__ __forceinline__ void zero_dynamics(const MS& MT, bool none) {
+  if constexpr (FlatSets<M, T>::value) {
+    if (none) {
+#pragma unroll
+      for (int r = 0; r < M::NX; ++r) {
+#pragma unroll
+        for (int c = 0; c < M::NX; ++c)
+          if (MS::akind(r, c) == 2) MT.A(r, c) = T(0);
+#pragma unroll
+        for (int c = 0; c < M::NU; ++c) MT.B(r, c) = T(0);
+      }
+    }
+  }
 }
 
 template <class M, class T, int AOS>
@@ -1008,6 +1035,13 @@ __device__ void node_setup(const Node<T, AOS>& nd, const Layout& L, const Proble
     }
   }
   }
+  if constexpr (FlatSets<M, T>::value) {   // the cone's and the ball's Gram terms are diagonal
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      if (I.cone) K.hd[k] += rg;
+      if (I.ball && !term) K.hd[NX + k] += rg;
+    }
+  }
   node_mirror_data<M, T, AOS>(nd, L, P, b, xb, ub);
 }
 
@@ -1100,7 +1134,7 @@ __device__ __forceinline__ bool node_factor(const Node<T, AOS>& nd, const MS& MT
           }
         } else {
           constexpr int RC = IsMars14<M>::value ? 1 : 0;
-          if (r >= RC && r < RC + 3 && r == c && I.cone) h += rg;
+          if (!FlatSets<M, T>::value && r >= RC && r < RC + 3 && r == c && I.cone) h += rg;
           if constexpr (IsMars14<M>::value) {
             if (r == c && I.tilt && (r == 9 || r == 10)) h += rg;
             if (r == c && I.wball && r >= 11 && r <= 13) h += rg;
@@ -1120,7 +1154,7 @@ __device__ __forceinline__ bool node_factor(const Node<T, AOS>& nd, const MS& MT
         if (!term) h += rd * acc;
         if constexpr (!IsQuad<M>::value) {
           if (rr < 3 && cc < 3 && !term) {
-            if (rr == cc && I.ball) h += rg;
+            if (!FlatSets<M, T>::value && rr == cc && I.ball) h += rg;
             if (I.half) h += rg * nd.at(L.oMd, rr) * nd.at(L.oMd, cc);
             if constexpr (IsMars14<M>::value) {
               if (rr == cc && I.gim) h += rg;
@@ -1214,11 +1248,13 @@ __device__ __forceinline__ void apply_H(const Node<T, AOS>& nd, const MS& MT, co
   for (int j = 0; j < NX; ++j) out[j] = K.hd[j] * xi[j];
   const bool coupled = nd.i < nd.N;   // node N: identity control block, no coupling
   if constexpr (n > NX) {
-   if (!coupled) {
+   // (flat: A and B are zero at node N)
+   if (!FlatSets<M, T>::value && !coupled) {
 #pragma unroll
     for (int j = 0; j < NU; ++j) out[NX + j] = K.hd[NX + j] * xi[NX + j];
    } else {
     T v[NX];
+    const T rdc = coupled ? rd : T(0);
 #pragma unroll
     for (int r = 0; r < NX; ++r) {
       T acc = T(0);
@@ -1226,7 +1262,7 @@ __device__ __forceinline__ void apply_H(const Node<T, AOS>& nd, const MS& MT, co
       for (int c = 0; c < NX; ++c) acc_A(acc, MT, r, c, xi[c]);
 #pragma unroll
       for (int c = 0; c < NU; ++c) acc += MT.B(r, c) * xi[NX + c];
-      v[r] = rd * acc;
+      v[r] = rdc * acc;
     }
 #pragma unroll
     for (int j = 0; j < NX; ++j) {
@@ -1250,6 +1286,14 @@ __device__ __forceinline__ void apply_H(const Node<T, AOS>& nd, const MS& MT, co
       const T y = rg * (n0 * xi[0] + n1 * xi[1] + n2 * xi[2]);
       out[0] += n0 * y; out[1] += n1 * y; out[2] += n2 * y;
     }
+  } else if constexpr (FlatSets<M, T>::value) {
+    // (cone and ball are on the diagonal K.hd)
+    const bool half = I.half && coupled;
+    const T n0 = nd.at(L.oMd, 0), n1 = nd.at(L.oMd, 1), n2 = nd.at(L.oMd, 2);
+    const T y = rg * (n0 * xi[NX] + n1 * xi[NX + 1] + n2 * xi[NX + 2]);
+    out[NX] += half ? n0 * y : T(0);
+    out[NX + 1] += half ? n1 * y : T(0);
+    out[NX + 2] += half ? n2 * y : T(0);
   } else {
     constexpr int RC = IsMars14<M>::value ? 1 : 0;
     if (I.cone) { out[RC] += rg * xi[RC]; out[RC + 1] += rg * xi[RC + 1]; out[RC + 2] += rg * xi[RC + 2]; }
@@ -1334,11 +1378,15 @@ __device__ __forceinline__ void node_rhs(const Node<T, AOS>& nd, const MS& MT, c
     g[j] = v;
   }
   if constexpr (n > NX) {
-   if (i < nd.N) {
+   if (FlatSets<M, T>::value || i < nd.N) {
     // w_i = mu_{i+1} + rho_dyn (z_{i+1} - c_i); node i+1 publishes mu + rho_dyn z
     T w[NX];
 #pragma unroll
-    for (int k = 0; k < NX; ++k) w[k] = nd.nb(Rec<M, AOS>::Ex2, k, i + 1) - rd * nd.at(Rec<M, AOS>::C, k);
+    for (int k = 0; k < NX; ++k) {
+      // (flat: node N reads its own record, and drops it)
+      w[k] = nd.nb(Rec<M, AOS>::Ex2, k, FlatSets<M, T>::value ? min(i + 1, nd.N) : i + 1) - rd * nd.at(Rec<M, AOS>::C, k);
+      if constexpr (FlatSets<M, T>::value) w[k] = i < nd.N ? w[k] : T(0);
+    }
 #pragma unroll
     for (int j = 0; j < NX; ++j) {
       T acc = T(0);
@@ -1351,7 +1399,7 @@ __device__ __forceinline__ void node_rhs(const Node<T, AOS>& nd, const MS& MT, c
       T acc = T(0);
 #pragma unroll
       for (int k = 0; k < NX; ++k) acc += MT.B(k, j) * w[k];
-      g[NX + j] = -K.q[NX + j] + acc + rg * nd.at(Rec<M, AOS>::Uh, j) - S.nuu(j);
+      g[NX + j] = -K.q[NX + j] + acc + rg * nd.at(Rec<M, AOS>::Uh, j) - S.nuu(j);   // (0 at node N)
     }
    } else {
 #pragma unroll
@@ -1364,6 +1412,16 @@ __device__ __forceinline__ void node_rhs(const Node<T, AOS>& nd, const MS& MT, c
       g[0] += obs_at(nd, L, j, 0) * a;
       g[1] += obs_at(nd, L, j, 1) * a;
       g[2] += obs_at(nd, L, j, 2) * a;
+    }
+  } else if constexpr (FlatSets<M, T>::value) {
+    const bool ctl = i < nd.N, ball = I.ball && ctl, half = I.half && ctl;
+    const T a = rg * nd.at(L.oS, 6) - nd.at(L.oNus, 6);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const T c = rg * nd.at(L.oS, k) - nd.at(L.oNus, k), b = rg * nd.at(L.oS, 3 + k) - nd.at(L.oNus, 3 + k);
+      const T h = nd.at(L.oMd, k) * a;
+      g[k] += I.cone ? c : T(0);
+      g[NX + k] += (ball ? b : T(0)) + (half ? h : T(0));
     }
   } else {
     constexpr int RC = IsMars14<M>::value ? 1 : 0;
@@ -1413,6 +1471,47 @@ __device__ __forceinline__ void node_mirrors(const Node<T, AOS>& nd, const Layou
         sv[0] += n0 * ds; sv[1] += n1 * ds; sv[2] += n2 * ds;
         acc_sq_diff(rp, y, s);
       }
+    }
+  } else if constexpr (FlatSets<M, T>::value && n > NX) {
+    const bool ctl = nd.i < nd.N, ball = I.ball && ctl, half = I.half && ctl;
+    const T z = reseed ? T(0) : irg;
+    T xb[3], ub[3], vc[3], vb[3], nc[3], nb[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      xb[k] = nd.at(L.oMd, 4 + k); ub[k] = nd.at(L.oMd, 7 + k);
+      nc[k] = nd.at(L.oNus, k); nb[k] = nd.at(L.oNus, 3 + k);
+      vc[k] = xb[k] + xi[k] + nc[k] * z;
+      vb[k] = ub[k] + xi[NX + k] + nb[k] * z;
+    }
+    proj_cone3s(vc, I.tau, I.ca, I.sa);
+    proj_ball3s(vb, I.tmax);
+    const T n0 = nd.at(L.oMd, 0), n1 = nd.at(L.oMd, 1), n2 = nd.at(L.oMd, 2), bd = nd.at(L.oMd, 3);
+    const T y = n0 * xi[NX] + n1 * xi[NX + 1] + n2 * xi[NX + 2], nh = nd.at(L.oNus, 6);
+    const T sh = maxv(bd, y + nh * z);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const T sc = vc[k] - xb[k], sb = vb[k] - ub[k];
+      if (want_res) {
+        if (I.cone) { sv[k] += rg * (sc - nd.at(L.oS, k)); acc_sq_diff(rp, xi[k], sc); }
+        if (ball) { sv[NX + k] += rg * (sb - nd.at(L.oS, 3 + k)); acc_sq_diff(rp, xi[NX + k], sb); }
+      }
+      if (I.cone) {
+        nd.at(L.oS, k) = sc;
+        if (!reseed) nd.at(L.oNus, k) = nc[k] + rg * (xi[k] - sc);
+      }
+      if (ball) {
+        nd.at(L.oS, 3 + k) = sb;
+        if (!reseed) nd.at(L.oNus, 3 + k) = nb[k] + rg * (xi[NX + k] - sb);
+      }
+    }
+    if (half) {
+      if (want_res) {
+        const T ds = rg * (sh - nd.at(L.oS, 6));
+        sv[NX] += n0 * ds; sv[NX + 1] += n1 * ds; sv[NX + 2] += n2 * ds;
+        acc_sq_diff(rp, y, sh);
+      }
+      nd.at(L.oS, 6) = sh;
+      if (!reseed) nd.at(L.oNus, 6) = nh + rg * (y - sh);
     }
   } else {
     T xb[3], ub[3];
@@ -1978,6 +2077,7 @@ __global__ void __launch_bounds__(MAX_THREADS) admm_kernel(ProblemDev P, Layout 
   init_mats<M, T, AOS>(MT, nd, L);
   const int i = nd.i, N = nd.N;
   const bool active = i <= N;
+  zero_dynamics<M, T>(MT, i == N);
   const long long xo = P.xoff[b], uo = P.uoff[b];
   if (threadIdx.x == 0) { sh.fail = 0; split_barrier_init(sh.xbar, blockDim.x); }
   stage_params<M>(sh, P, b);
@@ -2366,6 +2466,7 @@ __device__ __forceinline__ void scp_body(const ProblemDev& P, const Layout& L, c
   typedef typename Node<T, AOS>::W W;
   const int i = nd.i, N = nd.N;
   const bool active = i <= N;
+  zero_dynamics<M, T>(MT, i == N);
   const long long xo = P.xoff[b], uo = P.uoff[b];
   const Step3<T> hs = step_of<T>(P.dt[b]);   // the RK4 step in T, once per launch
   const unsigned long long t0 = globaltimer_ns();
@@ -2484,9 +2585,10 @@ __global__ void __launch_bounds__(MAX_THREADS) scp_kernel(ProblemDev P, Layout L
 }
 
 // The same solve for CTAs of up to 128 threads, three resident per SM (168
-// registers; the ADMM state in the node records).  Each CTA runs ~1.45x longer
-// than in scp_kernel, so three per SM solve ~3% more instances per unit time;
-// the launcher uses it for the first round of a batch (see launch_scp_v).
+// registers; the ADMM state in the node records).  Each CTA runs 1.62x longer
+// than in scp_kernel, so three per SM solve no more instances per unit time (1.5x
+// the CTAs); the launcher uses it for the first round of a batch where that
+// leaves a fuller last round (see scp3_split).
 constexpr int SCP3_MAX_THREADS = 128;
 template <class M, class T, bool SMEM, bool REFINE>
 __global__ void __launch_bounds__(SCP3_MAX_THREADS, 3) scp_kernel_3(ProblemDev P, Layout L, const double* x0,

@@ -52,15 +52,16 @@ cudaError_t Scp3Variant<M, T, SMEM, R>::launch(const LaunchCfg& c, const Problem
 }
 
 // Time of one CTA of scp_kernel_3 (three per SM) over one of scp_kernel (two
-// per SM), measured on the Mars batch (6.78 vs 4.66 ms per instance, GB300).
-constexpr double SCP3_TIME_RATIO = 1.45;
+// per SM), measured on the Mars batch (a round of 456 against one of 304, 20
+// iterations: 2.66 and 1.65 ms, GB300).
+constexpr double SCP3_TIME_RATIO = 1.62;
 
 // How many of a launch's CTAs (taken in the launch's order) run as
 // scp_kernel_3 before the rest run as scp_kernel: the split with the shortest
 // modelled time, rounds(k3 on b3 per SM) x SCP3_TIME_RATIO + rounds(rest on b2
 // per SM).  Whole CTAs are resident in rounds, so a batch that is not a whole
 // number of rounds leaves SMs idle in its last one; one round of three CTAs per
-// SM followed by rounds of two fills 1024 CTAs on 152 SMs in 3.4 round-times
+// SM followed by rounds of two fills 1024 CTAs on 152 SMs in 3.6 round-times
 // instead of 4.  0 when the variant keeps no more CTAs resident.
 inline int scp3_split(int B, int sms, int b2, int b3) {
   if (b3 <= b2 || b2 < 1 || sms < 1) return 0;
