@@ -155,11 +155,11 @@ static Layout rows_layout_of(int nodes, int max_obs, int csize, int lanes) {
   return L;
 }
 
-// The fewest CTAs whose nodes fit their threads: a CTA of 61 nodes takes 1.25 us
-// per ADMM iteration, one of 91 (384 threads, 168 registers) 1.79 us, and 121
-// nodes as a cluster of two 1.75 us (GB300, 20 obstacles) -- a split costs two
-// cluster barriers per iteration, half a microsecond, so it is made only where
-// one CTA cannot hold the instance.
+// The fewest CTAs whose nodes fit their threads: a CTA of 61 nodes takes 1.14 us
+// per ADMM iteration, one of 91 (384 threads, 168 registers) 1.93 us with two
+// CTAs' worth of instances per SM, and 121 nodes as a cluster of two 1.70 us
+// (GB300, 20 obstacles) -- a split occupies twice the SMs for less than twice the
+// speed, so it is made only where one CTA cannot hold the instance.
 //
 // FP64: the fan kernel for batches of at most one instance per SM -- 32 lanes per
 // node and 16 CTAs for one or two instances, 16 lanes and eight CTAs while the

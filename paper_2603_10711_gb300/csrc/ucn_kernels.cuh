@@ -111,7 +111,9 @@ struct Rec<M, 2> {
   static constexpr int NX = M::NX, NU = M::NU, NN = NX + NU, PX = pad4(NX), PN = pad4(NN);
   static constexpr int C = 0, Z = PX, Lam = 2 * PX, Mu = 3 * PX, Ex1 = 4 * PX, Ex2 = 5 * PX;
   static constexpr int X = 6 * PX, U = X + NX, Xh = X + PN, Uh = Xh + NX, Nux = Xh + PN, Nuu = Nux + NX;
-  static constexpr int Xlo = Nux + PN, Ulo = Xlo + NX, Xhi = Xlo + PN, Uhi = Xhi + NX, Ga = Xhi + PN;
+  static constexpr int Xlo = Nux + PN, Ulo = Xlo + NX, Xhi = Xlo + PN, Uhi = Xhi + NX;
+  // constants of the rows (cost gradient, diagonal of H, obstacles' Gram rows)
+  static constexpr int Kq = Xhi + PN, Khd = Kq + PN, Gr = Khd + PN, Ga = Gr + (NX == 14 ? 0 : 16);
   static constexpr int END = Ga + (NX == 14 ? PN : 0);
   static constexpr int Xbar = 0, Ubar = NX, Xc = NX + NU, DEND = 2 * NX + NU;
 };
@@ -182,7 +184,7 @@ template <class M> struct IsMars14 { static constexpr bool value = std::is_same<
 // set is computed, and one that is off (or a control set at node N) is selected
 // away.  A uniform branch and a divergent early return cost this 8-warps-per-SM
 // kernel more (branch resolution, reconvergence) than the few instructions: 304
-// instances of 31 nodes, 1.60 -> 1.30 us per ADMM iteration.
+// instances of 101 nodes, 1.60 -> 1.30 us per ADMM iteration.
 template <class M, class T> struct FlatSets {
   static constexpr bool value = std::is_same<M, Mars7>::value && std::is_same<T, float>::value;
 };

@@ -18,13 +18,13 @@
 // summed once per SCP iteration.
 //
 // Measured on GB300 (fused solves, before -> with this kernel): 1023 quadrotors
-// of 40..120 nodes, 10 x 200 iterations, 207 -> 64.9 ms; one of 50 nodes 8.57 ->
-// 3.39 ms; 1000 6-DOF landers of 30 nodes, 40 x 100, 122 -> 38.3 ms; 256
-// quaternion quadrotors of 50 nodes, 20 x 100, 27.3 -> 8.08 ms; the ADMM call
-// on 511 quadrotors, 100 iterations, 8.15 -> 1.49 ms.  The error against FP64
+// of 40..120 nodes, 10 x 200 iterations, 207 -> 36.6 ms; one of 50 nodes 8.57 ->
+// 2.55 ms; 1000 6-DOF landers of 30 nodes, 40 x 100, 122 -> 35 ms; 256
+// quaternion quadrotors of 50 nodes, 20 x 100, 27.3 -> 7.4 ms; the ADMM call
+// on 511 quadrotors, 100 iterations, 8.15 -> 1.07 ms.  The error against FP64
 // is as before (3e-7, 4e-7, 1.1e-6, 4e-7, 1e-6).  What bounds it: latency at 8
-// warps per SM -- issue slots 20% used; stalls at the two barriers of an
-// iteration, instruction fetch and fixed-latency dependencies.
+// warps per SM -- issue slots 45% used in the ADMM loop; stalls at the two
+// barriers of an iteration, instruction fetch and fixed-latency dependencies.
 //
 // An instance may be split over the CTAs of a thread-block cluster (CL), `chunk`
 // consecutive nodes each.  Only boundary nodes talk across CTAs: they store
@@ -148,6 +148,7 @@ template <class M, bool REG>
 struct RowState;
 template <class M>
 struct RowState<M, true> {
+  static constexpr bool reg = true;
   typedef Rec<M, 2> R;
   static constexpr int RX = RowMats<M>::RX, RE = RowConst<M>::R;
   mutable float hv[RE], nv[RE], lv[RE], uv[RE], zv[RX], lamv[RX], muv[RX], cv[RX];
@@ -186,6 +187,7 @@ struct RowState<M, true> {
 };
 template <class M>
 struct RowState<M, false> {
+  static constexpr bool reg = false;
   typedef Rec<M, 2> R;
   static constexpr int RX = RowMats<M>::RX, RE = RowConst<M>::R;
   float* tp;
@@ -432,6 +434,11 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
   float* tp = p.tp;
   const int q = p.q;
   float xo[RE];
+  // the constants of the lane's rows: registers, or the record where those are short
+  auto at = [&](int field, int m) { return tp[field + (m < 4 ? 4 * m : 16 - q)]; };
+  auto kq = [&](int m) { return ST::reg ? K.kq[m] : at(R::Kq, m); };
+  auto khd = [&](int m) { return ST::reg ? K.khd[m] : at(R::Khd, m); };
+  auto gram = [&](int s) { return ST::reg ? K.gram[s] : tp[R::Gr + 4 * s]; };
   // ---- Step 1
   if constexpr (CL)
     if (!head) halo_wait<4 * M::NX>(p.hb, hp, 1, p.last, q == 0);
@@ -445,7 +452,7 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
     }
 #pragma unroll
     for (int m = 0; m < RE; ++m) {
-      float v = rg * S.hat(m) - S.nu(m) - K.kq[m];
+      float v = rg * S.hat(m) - S.nu(m) - kq(m);
       if (m < RX && rows_is_x<M>(m, q)) v += re * S.z(m) - S.lam(m);   // (both 0 at node 0)
       if constexpr (!QUAD) v += tp[R::Ga + (m < 4 ? 4 * m : 16 - q)];
       g[m] += v;
@@ -462,9 +469,9 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
     for (int m = 0; m < RX; ++m) t[m] *= rd;
     rows_GT<M>(A, t, r);
 #pragma unroll
-    for (int m = 0; m < RE; ++m) r[m] = g[m] - (K.khd[m] * xo[m] + r[m]);
+    for (int m = 0; m < RE; ++m) r[m] = g[m] - (khd(m) * xo[m] + r[m]);
     if constexpr (QUAD) {
-      r[0] -= (K.gram[0] * v[0][0].x + K.gram[1] * v[0][0].y) + (K.gram[2] * v[0][1].x + K.gram[3] * v[0][1].y);
+      r[0] -= (gram(0) * v[0][0].x + gram(1) * v[0][0].y) + (gram(2) * v[0][1].x + gram(3) * v[0][1].y);
     } else {
       const float y = rg * (rows_sum(K.nrow * xo[3]) + K.nx * xo[RE - 1]);
       r[3] -= K.nrow * y;
@@ -772,6 +779,8 @@ __device__ __forceinline__ void rows_setup(const RowPos& p, const Node<float, 2>
     if (p.active) {
       p.tp[R::Xlo + (m < 4 ? 4 * m : 16 - p.q)] = lo;
       p.tp[R::Xhi + (m < 4 ? 4 * m : 16 - p.q)] = hi;
+      p.tp[R::Kq + (m < 4 ? 4 * m : 16 - p.q)] = kq;
+      p.tp[R::Khd + (m < 4 ? 4 * m : 16 - p.q)] = khd;
     }
   }
 }
@@ -815,7 +824,10 @@ __device__ __forceinline__ float rows_obstacle_setup(const RowPos& p, const Node
   const float r0 = sel4(G[0], G[1], G[2], 0.0f, p.q), r1 = sel4(G[1], G[3], G[4], 0.0f, p.q),
               r2 = sel4(G[2], G[4], G[5], 0.0f, p.q);
 #pragma unroll
-  for (int s = 0; s < 4; ++s) K.gram[s] = sel4(r0, r1, r2, 0.0f, p.q ^ s);
+  for (int s = 0; s < 4; ++s) {
+    K.gram[s] = sel4(r0, r1, r2, 0.0f, p.q ^ s);
+    if (p.active) p.tp[R::Gr + 4 * s] = K.gram[s];
+  }
   return sel4(a0, a1, a2, 0.0f, p.q);
 }
 
