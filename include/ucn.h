@@ -174,6 +174,8 @@ void ucn_problem_destroy(ucn_problem* prob);
  * of 0..batch-1; NULL = instance order).  The default, set by
  * ucn_problem_create, is largest estimated work first, so that the long solves
  * of an uneven batch start in the first wave.  Results do not depend on it.
+ * (Where a batch is launched in parts of one CTA shape, see ucn_scp_solve, the
+ * order holds within each part.)
  * Synchronous (copies the permutation).  Errors: UCN_EINVAL, UCN_ECUDA. */
 ucn_status ucn_problem_set_order(ucn_problem* prob, const int* order);
 

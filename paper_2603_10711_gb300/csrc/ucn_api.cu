@@ -8,6 +8,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "ucn_internal.h"
@@ -231,6 +232,7 @@ struct ucn_problem {
   std::vector<int> horizon;
   cudaStream_t aux[MAX_ROW_PARTS - 1] = {};
   cudaEvent_t fork = nullptr, join[MAX_ROW_PARTS - 1] = {};
+  std::mutex parts_mu;   // one call's fork and joins at a time (the events are re-recorded by the next)
   unsigned char* warm_ones;   // batch flags, all 1: every instance starts from the given state
 };
 
@@ -640,12 +642,28 @@ static LaunchCfg cfg_of(ucn_problem* p, void* stream, bool admm = false) {
 // the caller's stream, the others on the problem's own, forked from it and
 // joined to it by events (so that a capture of the caller's stream holds them),
 // so that a part's CTAs fill the SMs that an earlier part's last ones leave.
+// While another stream's capture holds the problem's streams (they stay in it
+// until it ends), the parts run one after another on the caller's.
+static unsigned long long capture_of(cudaStream_t s) {   // id of the capture that holds s; 0: none
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamGetCaptureInfo(s, &st, &id) != cudaSuccess || st == cudaStreamCaptureStatusNone) return 0;
+  return id;
+}
+
 extern "C++" {
 template <class F>
 static cudaError_t launch_parts(ucn_problem* p, LaunchCfg c, bool admm, F launch) {
   if (!rows_on(p, admm) || p->parts.size() == 1) return launch(c);
+  std::lock_guard<std::mutex> lk(p->parts_mu);
   cudaStream_t s = c.stream;
-  cudaError_t e = cudaEventRecord(p->fork, s);
+  bool alone = false;
+  const unsigned long long mine = capture_of(s);
+  for (size_t k = 1; k < p->parts.size(); ++k) {
+    const unsigned long long held = capture_of(p->aux[k - 1]);
+    alone |= held != 0 && held != mine;
+  }
+  cudaError_t e = alone ? cudaSuccess : cudaEventRecord(p->fork, s);
   const ProblemDev base = *(const ProblemDev*)c.P;
   for (size_t k = 0; k < p->parts.size() && e == cudaSuccess; ++k) {
     const ucn_problem::RowsPart& q = p->parts[k];
@@ -653,12 +671,12 @@ static cudaError_t launch_parts(ucn_problem* p, LaunchCfg c, bool admm, F launch
     P.order = base.order + q.first;
     c.P = &P;
     c.L = &q.L; c.smem_bytes = q.L.bytes; c.blocks = q.count;
-    if (k > 0) {
+    if (k > 0 && !alone) {
       c.stream = p->aux[k - 1];
       e = cudaStreamWaitEvent(c.stream, p->fork, 0);
     }
     if (e == cudaSuccess) e = launch(c);
-    if (k > 0) {   // joined whatever the launch said: the caller's stream never runs ahead
+    if (k > 0 && !alone) {   // joined whatever the launch said: the caller's stream never runs ahead
       cudaError_t j = cudaEventRecord(p->join[k - 1], c.stream);
       if (j == cudaSuccess) j = cudaStreamWaitEvent(s, p->join[k - 1], 0);
       if (e == cudaSuccess) e = j;

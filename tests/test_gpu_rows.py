@@ -56,6 +56,31 @@ def test_uneven_batch_over_a_cluster():
     check(quad((3, 120), (0, 30), B=7))
 
 
+def test_uneven_batch_while_a_capture_holds_its_streams():
+    # the parts' streams belong to the capture until it ends: a solve on another
+    # stream meanwhile runs them on its own, with the same bits
+    s = ucn.Solver(quad((20, 120), (0, 9), B=9), precision=ucn.UCN_PREC_FP32_REFINE)
+    x0, u0 = s.tensor(s.prob.xguess), s.tensor(s.prob.uguess)
+    s.scp_solve(x0, u0)
+    torch.cuda.synchronize()
+    ref = s.x_out.clone()
+    s.x_out.zero_()
+    other, held, graph = torch.cuda.Stream(), torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(held):
+        graph.capture_begin(capture_error_mode="relaxed")
+        s.scp_solve(x0, u0, stream=held)
+        s.scp_solve(x0, u0, stream=other)
+        graph.capture_end()
+    torch.cuda.synchronize()
+    assert torch.equal(s.x_out, ref)
+    s.x_out.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(s.x_out, ref)
+    s.close()
+
+
 @pytest.mark.parametrize("N", [1, 30, 63, 64, 127, 128, 200])
 def test_quaternion_quadrotor_horizons(N):
     check(W.quat_study(2, seed=5, N=N, tf=0.12 * N, settings=dict(SHORT)))
