@@ -666,11 +666,14 @@ __device__ __forceinline__ void scp_lanes_body(const ProblemDev& P, const Layout
   if constexpr (GROUP) group_finish(P);
 }
 
-// CTAs of up to 512 threads; the compiler chooses the registers (128 at most).
+// CTAs of up to 512 threads: 128 registers with the records in shared memory, 64
+// with FP64 records in global memory, where two CTAs per SM hide each other's
+// loads (FP64, 2 x 200 iterations: 2048 quadrotors of 40..120 nodes 204 -> 188 ms,
+// 608 of them 59.8 -> 58.5).
 template <class M, class T, bool SMEM, bool REFINE, bool GROUP, int TPN>
-__global__ void __launch_bounds__(LANES_MAX_THREADS, 1) scp_kernel_lanes(ProblemDev P, Layout L, const double* x0,
-                                                                      const double* u0, double* xout, double* uout,
-                                                                      ucn_scp_stats* stats, int* status_out) {
+__global__ void __launch_bounds__(LANES_MAX_THREADS, !SMEM && sizeof(T) == 8 ? 2 : 1)
+    scp_kernel_lanes(ProblemDev P, Layout L, const double* x0, const double* u0, double* xout, double* uout,
+                     ucn_scp_stats* stats, int* status_out) {
   scp_lanes_body<M, T, SMEM, REFINE, GROUP, TPN>(P, L, x0, u0, xout, uout, stats, status_out, cta_instance<GROUP>(P));
 }
 
