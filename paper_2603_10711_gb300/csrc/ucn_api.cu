@@ -162,13 +162,37 @@ static Layout rows_layout_of(int nodes, int max_obs, int csize, int lanes) {
 // (GB300, 20 obstacles) -- a split occupies twice the SMs for less than twice the
 // speed, so it is made only where one CTA cannot hold the instance.
 //
-// FP64: the fan kernel for batches of at most one instance per SM -- 32 lanes per
-// node and 16 CTAs for one or two instances, 16 lanes and eight CTAs while the
-// SMs have room for them, else 8 lanes and 16 nodes per CTA.  More instances fill
-// the SMs' FP64 pipes with one CTA each, and four lanes per node do less work:
-// us per ADMM iteration, fan / lane kernel (GB300): one instance of 51 nodes 3.9
-// / 15.1, 40 of 31 nodes 7.2 / 11.1, 152 of 26 nodes 10.2 / 11.1, but 304 of
-// them 19.8 / 16.4 and 608 of 41 nodes 68 / 48.
+// FP64: the fan kernel for batches of at most one instance per SM (where
+// fan_pays) -- 32 lanes per node and 16 CTAs for one or two instances, 16 lanes
+// and eight CTAs while the SMs have room for them, else 8 lanes and 16 nodes per
+// CTA.  More instances fill the SMs' FP64 pipes with one CTA each, and four lanes
+// per node do less work: us per ADMM iteration, fan / lane kernel (GB300): one
+// instance of 51 nodes 3.9 / 15.1, 40 of 31 nodes 7.2 / 11.1, 152 of 26 nodes
+// 10.2 / 11.1, but 304 of them 19.8 / 16.4 and 608 of 41 nodes 68 / 48.
+// Whether the fan kernel beats one CTA per instance on an FP64 batch of at most
+// one instance per SM (`horizon` null: all of `nodes` nodes).  It spreads the
+// batch's nodes over all SMs, where the lane kernel waits for its longest
+// instance, but pays 1.36 times as much per node (a CTA less than three quarters
+// full as much as one of 12 nodes); up to 32 nodes the lane kernel is bound by
+// latency.  ms of 2 x 100 iterations, fan / lane kernel (GB300): 152 instances of
+// 31 nodes 2.73 / 3.29, of 41 5.88 / 3.57, of 101 12.6 / 8.4; 100 of 41 4.25 /
+// 3.57, of 61 5.25 / 6.10, of 101 7.92 / 8.34; 152 of 41..121 10.5 / 11.1.
+bool fan_pays(const int* horizon, int batch, int nodes) {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return false;
+  if (batch > sms) return false;
+  if (nodes <= 32) return true;
+  double work = 0.0;
+  for (int b = 0; b < batch; ++b) {
+    const int n = horizon ? horizon[b] + 1 : nodes;
+    int csize = 1;
+    while (csize < 8 && (n + csize - 1) / csize > 16) csize *= 2;
+    work += std::max(n, 12 * csize);
+  }
+  return 1.36 * work <= (double)sms * nodes;
+}
+
 bool rows_layout(int model, int precision, int nodes, int max_obs, int group, int tpn, int batch, int optin, Layout* out) {
   if (precision != UCN_PREC_FP32_REFINE) {
     if (model != UCN_MODEL_QUAD12 || tpn != 4 || group > 1) return false;
@@ -269,6 +293,7 @@ void rows_parts(ucn_problem* p, std::vector<int>& order) {
   p->parts.clear();
   const int tpn = default_tpn(p->model, p->Nmax + 1, p->precision);
   Layout L;
+  if (p->precision == UCN_PREC_FP64 && !fan_pays(p->horizon.data(), p->batch, p->Nmax + 1)) return;
   if (!rows_layout(p->model, p->precision, p->Nmax + 1, p->max_obs, p->group, tpn, p->batch, p->optin, &L)) return;
   if (p->group > 1) {
     p->parts.push_back({L, 0, p->batch});

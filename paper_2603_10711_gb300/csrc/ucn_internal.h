@@ -32,6 +32,9 @@ Layout make_layout(int model, int nodes, int max_obs, int tsize, bool reg_mats, 
 // FP64: the fan kernel's (ucn_fan.cuh) for the 12-state quadrotor at its default
 // threads per node, without scenario groups; `batch` instances share the device.
 bool rows_layout(int model, int precision, int nodes, int max_obs, int group, int tpn, int batch, int optin, Layout* out);
+// Whether the fan kernel is the faster one for an FP64 batch (its nodes, or each
+// instance's horizon).
+bool fan_pays(const int* horizon, int batch, int nodes);
 
 // Everything one kernel launch needs besides its buffers.
 struct LaunchCfg {

@@ -81,3 +81,9 @@ def test_uneven_batch_and_the_batch_beyond():
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     check(sms, (3, 60), (0, 12))
     check(sms + 1, (3, 30), (0, 6))
+
+
+# both sides of the rule that chooses between the fan and the lane kernel
+@pytest.mark.parametrize("B,N", [(152, 31), (152, 32), (100, 40), (100, 60), (128, (20, 60)), (130, (60, 70))])
+def test_batches_around_the_choice_of_kernel(B, N):
+    check(B, N, 2)
