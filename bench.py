@@ -438,15 +438,21 @@ def run_serving(args):
     # the same streams through the device-resident request loop: one persistent kernel
     # per server whose CTAs claim each request as it is submitted (no pump launches).
     # The loops run at the same time, so each holds a share of the device: server i
-    # needs c_i = rate_i x t_i CTAs to keep up (t_i: its mean device time per solve,
-    # measured in the pump sweep's first stream) and c_i / cap_i of the device (cap_i:
-    # its CTAs that fit at once), so c_i = cap_i x s_i with s_i proportional to
-    # n_i t_i / cap_i, 90% of the device in all
+    # needs c_i = rate_i x t_i CTAs to keep up (t_i: its mean device time per solve in
+    # the loop, measured on a first stream with equal shares; n_i: its requests) and
+    # c_i / cap_i of the device (cap_i: its CTAs that fit at once), so c_i = cap_i x s_i
+    # with s_i proportional to n_i t_i / cap_i, 90% of the device in all
     sv = servers(ucn.UCN_PREC_FP32_REFINE, 512)
-    busy = sweep[0]["solve_ms_by_server"]
     caps = {k: srv.loop_capacity() for k, srv in sv.items()}
     name = serving.server_name
-    need = {k: (busy[name(k)][0] * busy[name(k)][1] / caps[k] if name(k) in busy else 0.0) for k in sv}
+    for k, srv in sv.items():
+        srv.loop_start(ctas=max(1, int(0.9 * caps[k] / len(sv))), idle_s=2.0)
+    busy = serving.run_stream(W.serving_stream(400, rate=rates[0], seed=5), sv, route=route)["solve_ms_by_server"]
+    for s in sv.values():
+        s.loop_stop()
+    count = sweep[0]["solve_ms_by_server"]
+    need = {k: (count[name(k)][0] * busy[name(k)][1] / caps[k] if name(k) in busy and name(k) in count else 0.0)
+            for k in sv}
     total = sum(need.values())
     loop_ctas = {}
     for k, srv in sv.items():
