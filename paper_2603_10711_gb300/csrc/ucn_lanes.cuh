@@ -8,8 +8,9 @@
 // warps per scheduler and is latency-bound.  The per-SCP-iteration work
 // (assembly and factorisation, the wide rollout, acceptance) maps one thread
 // to one node again; the Jacobian directions are split over the lanes.
-// Serves the FP64 solves of more than one instance per SM, FP64 scenario groups
-// and the request loop; the others have the row and the fan kernel.
+// Serves the FP64 batches of more than one instance per SM or that fan_pays turns
+// down, FP64 scenario groups and the request loop; the others have the row and the
+// fan kernel.
 #pragma once
 #include "ucn_kernels.cuh"
 
