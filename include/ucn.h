@@ -236,8 +236,8 @@ ucn_status ucn_state_export(ucn_problem* prob, double* state_d, void* stream);
  * instance by persistent kernel launches that each run whole solves: per SCP
  * iteration the RK4 linearisation, assembly + factorisation, admm_iters ADMM
  * iterations, and the rollout / defect / trust-region acceptance test, all on
- * the device, one CTA per instance (or, FP32 and 16- or 17-row models beyond
- * 96 or 64 nodes, a thread-block cluster of two or four).  One launch; FP32
+ * the device, one CTA per instance (or, FP32 quadrotors beyond 96 nodes, 64 for
+ * the quaternion one, a thread-block cluster of two or four).  One launch; FP32
  * batches of those models whose instances need different CTA shapes take one
  * launch per shape, side by side on streams of the problem forked from and
  * joined to `stream`; for batches of the 3-DOF Mars

@@ -123,17 +123,15 @@ Layout make_layout(int model, int nodes, int max_obs, int tsize, bool reg_mats, 
   return L;
 }
 
-template <class M>
+template <class M>   // a quadrotor
 static Layout rows_layout_of(int nodes, int max_obs, int csize, int lanes) {
   typedef Rec<M, 2> R;
   Layout L;
   std::memset(&L, 0, sizeof(L));
-  const bool quad = IsQuad<M>::value;
-  const int mo = std::max(max_obs, 1);
-  L.MS = quad ? mo : M14::MS;
-  L.MB = quad ? max_obs : 6;
+  L.MS = std::max(max_obs, 1);
+  L.MB = max_obs;
   const int ms = pad4(L.MS);
-  L.MD = quad ? 4 * ms : pad4(M14::MD);
+  L.MD = 4 * ms;
   L.oS = R::END;
   L.oNus = L.oS + ms;
   L.oMd = L.oNus + ms;
@@ -214,14 +212,12 @@ bool rows_layout(int model, int precision, int nodes, int max_obs, int group, in
     return false;
   }
   const bool quad12 = model == UCN_MODEL_QUAD12;
-  if (quad12 ? tpn != 4 : (tpn != 1 || (model != UCN_MODEL_QUAT13 && model != UCN_MODEL_MARS14))) return false;
+  if (quad12 ? tpn != 4 : (tpn != 1 || model != UCN_MODEL_QUAT13)) return false;
   const long long fixed = (long long)sizeof(InstShared) + sizeof(RowCluster) + (group > 1 ? (long long)sizeof(GroupShared) : 0) + 64;
   for (int csize = 1; csize <= (group > 1 ? 1 : 4); csize *= 2) {
     const int cap = (csize == 1 && quad12 ? ROWS_WIDE_THREADS : ROWS_THREADS) / 4;
     if ((nodes + csize - 1) / csize > cap) continue;
-    const Layout L = quad12 ? rows_layout_of<Quad12>(nodes, max_obs, csize, 4)
-                     : model == UCN_MODEL_QUAT13 ? rows_layout_of<Quat13>(nodes, max_obs, csize, 4)
-                                                 : rows_layout_of<Mars14>(nodes, max_obs, csize, 4);
+    const Layout L = quad12 ? rows_layout_of<Quad12>(nodes, max_obs, csize, 4) : rows_layout_of<Quat13>(nodes, max_obs, csize, 4);
     if (L.bytes + fixed > optin) continue;
     *out = L;
     return true;

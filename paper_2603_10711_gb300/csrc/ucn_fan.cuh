@@ -529,10 +529,9 @@ struct FanEngine {
       }
     }
   }
-  __device__ static __forceinline__ double prepare(const Pos& p, const Node<double, 2>& nd, const Node<double, 2>&, bool,
-                                                   const Layout& L, const ProblemDev& P, const Inst<double>& I, int b,
-                                                   double rad, double re, double rd, double rg, Mats& A, Const& K,
-                                                   InstShared& sh) {
+  __device__ static __forceinline__ double prepare(const Pos& p, const Node<double, 2>& nd, const Layout& L,
+                                                   const ProblemDev& P, const Inst<double>& I, int b, double rad,
+                                                   double re, double rd, double rg, Mats& A, Const& K, InstShared& sh) {
     return fan_prepare<F, CL>(p, nd, L, P, I, b, rad, re, rd, rg, A, K, sh);
   }
   __device__ static __forceinline__ void admm(const Pos& p, const Mats& A, const Const& K, const Layout& L,

@@ -25,9 +25,8 @@ int fault_alloc_at();
 Layout make_layout(int model, int nodes, int max_obs, int tsize, bool reg_mats, int tpn);
 
 // The row kernel's layout (ucn_rows.cuh) of an instance of `nodes` nodes, for the
-// problems it serves: FP32, a 16- or 17-row model at its default threads per
-// node (12-state quadrotor 4, the others 1), 96 nodes per CTA (64 for the
-// others) and up to four CTAs per instance (one for scenario groups), within
+// problems it serves: FP32, a quadrotor at its default threads per node
+// (12-state 4, quaternion 1), 96 nodes per CTA (64 for the quaternion one) and up to four CTAs per instance (one for scenario groups), within
 // the device's shared memory per CTA.  False where it does not.
 // FP64: the fan kernel's (ucn_fan.cuh) for the 12-state quadrotor at its default
 // threads per node, without scenario groups; `batch` instances share the device.

@@ -103,8 +103,7 @@ struct Rec {
 // the record starts at a multiple of four, so that lane q of a node finds its
 // row 4 m + q at a compile-time distance from its own base, and the arrays over
 // the whole of xi = (x, u) are contiguous (U = X + NX and so on): row e of xi
-// is element e of all of them.  Ga (models with vector sets): the mirror sets'
-// part of the Step-1 right-hand side.
+// is element e of all of them.
 __host__ __device__ constexpr int pad4(int n) { return (n + 3) / 4 * 4; }
 template <class M>
 struct Rec<M, 2> {
@@ -113,8 +112,7 @@ struct Rec<M, 2> {
   static constexpr int X = 6 * PX, U = X + NX, Xh = X + PN, Uh = Xh + NX, Nux = Xh + PN, Nuu = Nux + NX;
   static constexpr int Xlo = Nux + PN, Ulo = Xlo + NX, Xhi = Xlo + PN, Uhi = Xhi + NX;
   // constants of the rows (cost gradient, diagonal of H, obstacles' Gram rows)
-  static constexpr int Kq = Xhi + PN, Khd = Kq + PN, Gr = Khd + PN, Ga = Gr + (NX == 14 ? 0 : 16);
-  static constexpr int END = Ga + (NX == 14 ? PN : 0);
+  static constexpr int Kq = Xhi + PN, Khd = Kq + PN, Gr = Khd + PN, END = Gr + 16;
   static constexpr int Xbar = 0, Ubar = NX, Xc = NX + NU, DEND = 2 * NX + NU;
 };
 
@@ -338,6 +336,8 @@ struct Inst {
   bool gim, tilt, wball;    // Mars 6-DOF: gimbal cone, tilt ball, body-rate ball
   T tg, cg, sg, rtilt, wmax;
   bool run_cost, term_quad; // nonzero running weights / terminal quadratic weights
+  T prm[8];                 // model constants in T (Jacobian passes of the 6-DOF lander: read from shared
+                            // memory they round differently, see rk4h)
 };
 
 // Obstacles of instance b, clamped to [0, max_obs]: ucn_problem_create checks
@@ -383,6 +383,8 @@ __device__ __forceinline__ Inst<T> make_inst(const ProblemDev& P, int b) {
   I.half = f & 1u; I.ball = f & 2u; I.cone = f & 4u;
   I.gim = f & 8u; I.tilt = f & 16u; I.wball = f & 32u;
   I.run_cost = f & 64u; I.term_quad = f & 128u;
+  if constexpr (IsMars14<M>::value)
+    for (int k = 0; k < 8; ++k) I.prm[k] = (T)P.params[b * 8 + k];
   return I;
 }
 
@@ -2509,7 +2511,7 @@ __device__ __forceinline__ void scp_body(const ProblemDev& P, const Layout& L, c
     const T re = rho_of<T>(sh, 0), rd = rho_of<T>(sh, 1), rg = rho_of<T>(sh, 2);
     const T radius = radius_of<T>(sh);
     if (active) {
-      if (i < N) node_jacobians<M, T, AOS>(nd, MT, prm_of<T>(sh), hs);
+      if (i < N) node_jacobians<M, T, AOS>(nd, MT, IsMars14<M>::value ? I.prm : prm_of<T>(sh), hs);
       node_setup<M, T, AOS>(nd, L, P, I, b, radius, sh.tmask, re, rg, K);
       const bool ok = node_factor<M, T, AOS, NN>(nd, MT, L, I, K, rd, rg);
       if (!ok) atomicOr(&sh.fail, 1);

@@ -204,8 +204,8 @@ cudaError_t launch_scpp_v(const LaunchCfg& c, const double* x0, const double* u0
 }
 
 // The row kernel (ucn_rows.cuh), one kernel per function, each in its own
-// translation unit (declared here, defined by UCN_DEFINE_ROWS_*).  The 17-row
-// models' FP32 solves run on nothing else (four CTAs of 64 nodes hold the
+// translation unit (declared here, defined by UCN_DEFINE_ROWS_*).  The quaternion
+// quadrotor's FP32 solves run on nothing else (four CTAs of 64 nodes hold the
 // longest horizon); the 12-state quadrotor's do on four threads per node (128
 // nodes at most), and keep the one-thread kernel beyond and on request.
 template <class M, class T>

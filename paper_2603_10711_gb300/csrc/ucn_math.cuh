@@ -207,22 +207,20 @@ constexpr int PRM = 16;
 // body rates), 4 rotor thrusts in a "+" layout.
 // prm: m, Jx, Jy, Jz, arm, km (yaw moment per unit thrust), drag, g | 1/m, 1/Jx,
 // 1/Jy, 1/Jz, drag/m, (Jz-Jy)/Jx, (Jx-Jz)/Jy, (Jy-Jx)/Jz.
-__host__ __device__ inline double rigid_param(const double* p, int k, int m, int jx) {
-  const double Jx = p[jx], Jy = p[jx + 1], Jz = p[jx + 2];
-  switch (k) {
-    case 8: return 1.0 / p[m];
-    case 9: return 1.0 / Jx;
-    case 10: return 1.0 / Jy;
-    case 11: return 1.0 / Jz;
-    case 13: return (Jz - Jy) / Jx;
-    case 14: return (Jx - Jz) / Jy;
-    default: return (Jy - Jx) / Jz;
-  }
-}
 struct Quad12 {
   static constexpr int NX = 12, NU = 4;
   __host__ __device__ static double derived(const double* p, int k) {
-    return k == 12 ? p[6] / p[0] : rigid_param(p, k, 0, 1);
+    const double m = p[0], Jx = p[1], Jy = p[2], Jz = p[3];
+    switch (k) {
+      case 8: return 1.0 / m;
+      case 9: return 1.0 / Jx;
+      case 10: return 1.0 / Jy;
+      case 11: return 1.0 / Jz;
+      case 12: return p[6] / m;
+      case 13: return (Jz - Jy) / Jx;
+      case 14: return (Jx - Jz) / Jy;
+      default: return (Jy - Jx) / Jz;
+    }
   }
   template <class S> struct Held { S Fm, ax, ay, az; };
   template <class S, class P>
@@ -342,46 +340,38 @@ struct Mars7 {
 // (Up-East-North), velocity, quaternion body-to-world scalar first, body rates;
 // control = thrust in the body frame (body x = thrust axis).  prm: alpha (mass
 // flow per unit thrust), g (along -Up), Jx, Jy, Jz, l (the thrust acts at
-// -l e_x in the body) | l/Jy at 10, l/Jz at 11, the inertia quotients at 13..15.
-// Non-dimensional units.
+// -l e_x in the body).  Non-dimensional units.  No Held: rk4h takes its stages as
+// they stand here.
 struct Mars14 {
   static constexpr int NX = 14, NU = 3;
-  __host__ __device__ static double derived(const double* p, int k) {
-    return k == 10 ? p[5] / p[3] : k == 11 ? p[5] / p[4] : k >= 13 ? rigid_param(p, k, 0, 2) : 0.0;
-  }
-  template <class S> struct Held { S u0, u1, u2, mdot, ay, az; };
+  __host__ __device__ static double derived(const double*, int) { return 0.0; }
   template <class S, class P>
-  __device__ static __forceinline__ Held<S> hold(const P* prm, const S* u) {
+  __device__ static void f(const P* prm, const S* x, const S* u, S* xd) {
     typedef typename BaseOf<S>::type R;
-    const S Tn = sqrt_(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-    return {u[0], u[1], u[2], -((R)prm[0] * Tn), (R)prm[10] * u[2], (R)prm[11] * u[1]};
-  }
-  template <class S, class P>
-  __device__ static __forceinline__ void f(const P* prm, const S* x, const Held<S>& H, S* xd) {
-    typedef typename BaseOf<S>::type R;
-    const R g = (R)prm[1];
+    const R alpha = (R)prm[0], g = (R)prm[1], Jx = (R)prm[2], Jy = (R)prm[3], Jz = (R)prm[4], l = (R)prm[5];
     const S qw = x[7], qx = x[8], qy = x[9], qz = x[10];
     const S wx = x[11], wy = x[12], wz = x[13];
+    const S Tn = sqrt_(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
     const S im = R(1) / x[0];
     // rotation body -> world (quadratic form), applied to the body thrust
     const S c00 = qw * qw + qx * qx - qy * qy - qz * qz, c01 = R(2) * (qx * qy - qw * qz), c02 = R(2) * (qx * qz + qw * qy);
     const S c10 = R(2) * (qx * qy + qw * qz), c11 = qw * qw - qx * qx + qy * qy - qz * qz, c12 = R(2) * (qy * qz - qw * qx);
     const S c20 = R(2) * (qx * qz - qw * qy), c21 = R(2) * (qy * qz + qw * qx), c22 = qw * qw - qx * qx - qy * qy + qz * qz;
-    xd[0] = H.mdot;
+    xd[0] = -(alpha * Tn);
     xd[1] = x[4];
     xd[2] = x[5];
     xd[3] = x[6];
-    xd[4] = (c00 * H.u0 + c01 * H.u1 + c02 * H.u2) * im - g;
-    xd[5] = (c10 * H.u0 + c11 * H.u1 + c12 * H.u2) * im;
-    xd[6] = (c20 * H.u0 + c21 * H.u1 + c22 * H.u2) * im;
+    xd[4] = (c00 * u[0] + c01 * u[1] + c02 * u[2]) * im - g;
+    xd[5] = (c10 * u[0] + c11 * u[1] + c12 * u[2]) * im;
+    xd[6] = (c20 * u[0] + c21 * u[1] + c22 * u[2]) * im;
     xd[7] = R(0.5) * (-(qx * wx) - qy * wy - qz * wz);
     xd[8] = R(0.5) * (qw * wx + qy * wz - qz * wy);
     xd[9] = R(0.5) * (qw * wy - qx * wz + qz * wx);
     xd[10] = R(0.5) * (qw * wz + qx * wy - qy * wx);
     // J w' = r_T x T - w x (J w), r_T = (-l, 0, 0): r_T x T = (0, l T_z, -l T_y)
-    xd[11] = -((R)prm[13] * (wy * wz));
-    xd[12] = H.ay - (R)prm[14] * (wz * wx);
-    xd[13] = -H.az - (R)prm[15] * (wx * wy);
+    xd[11] = (-((Jz - Jy) * wy * wz)) / Jx;
+    xd[12] = (l * u[2] - (Jx - Jz) * wz * wx) / Jy;
+    xd[13] = (-(l * u[1]) - (Jy - Jx) * wx * wy) / Jz;
   }
 };
 
@@ -400,11 +390,26 @@ __device__ __forceinline__ DF fma_(DF a, DF b, DF c) { return df_fma(a, b, c); }
 // loop: unrolled, a step of the larger models is 30 to 180 KB of code that runs
 // once per SCP iteration, and the instruction fetch is what it waits for.  The
 // 3-DOF Mars model's step is small outside double-float; rolled, its kernels
-// spill in the ADMM loop.
+// spill in the ADMM loop.  The 6-DOF lander's stays straight-line with quotients
+// and held terms in every stage: its FP32 solves meet decisions that a last bit
+// turns (one batch of 1000 in sixteen: up to 5e-5 normwise), so their results are
+// only as constant as this rounding.
 template <class M, class S, class P, class R>
 __device__ __forceinline__ void rk4h(const P* prm, R h, R hh, R h6, const S* x, const S* u, S* xn) {
   constexpr int NX = M::NX;
   S k[NX], t[NX], acc[NX];
+  if constexpr (std::is_same<M, Mars14>::value) {
+    M::f(prm, x, u, k);
+#pragma unroll
+    for (int j = 0; j < NX; ++j) { acc[j] = k[j]; t[j] = fma_(x[j], hh, k[j]); }
+    M::f(prm, t, u, k);
+#pragma unroll
+    for (int j = 0; j < NX; ++j) { acc[j] = fma_(acc[j], R(2), k[j]); t[j] = fma_(x[j], hh, k[j]); }
+    M::f(prm, t, u, k);
+#pragma unroll
+    for (int j = 0; j < NX; ++j) { acc[j] = fma_(acc[j], R(2), k[j]); t[j] = fma_(x[j], h, k[j]); }
+    M::f(prm, t, u, k);
+  } else {
   const typename M::template Held<S> H = M::template hold<S, P>(prm, u);
 #pragma unroll
   for (int j = 0; j < NX; ++j) t[j] = x[j];
@@ -422,6 +427,7 @@ __device__ __forceinline__ void rk4h(const P* prm, R h, R hh, R h6, const S* x, 
     }
 #pragma unroll
     for (int j = 0; j < NX; ++j) t[j] = fma_(x[j], w, k[j]);
+  }
   }
 #pragma unroll
   for (int j = 0; j < NX; ++j) xn[j] = fma_(x[j], h6, acc[j] + k[j]);

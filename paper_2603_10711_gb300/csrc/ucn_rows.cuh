@@ -1,6 +1,6 @@
-// Row kernel of the FP32 path for the 16- and 17-row models (12-state and
-// quaternion quadrotors, 6-DOF lander): four lanes of a warp share a time node
-// and keep its matrices in registers for a whole ADMM call.
+// Row kernel of the FP32 path for the quadrotors (12-state, 16 rows; quaternion,
+// 17 rows): four lanes of a warp share a time node and keep its matrices in
+// registers for a whole ADMM call.
 //
 // Lane q owns the rows e = q, q + 4, q + 8, q + 12 of xi = (x, u); a 17th row is
 // carried by all four lanes alike.  It holds its rows of G = [A B] and of H^-1
@@ -19,8 +19,7 @@
 //
 // Measured on GB300 (fused solves, before -> with this kernel): 1023 quadrotors
 // of 40..120 nodes, 10 x 200 iterations, 207 -> 36.6 ms; one of 50 nodes 8.57 ->
-// 2.55 ms; 1000 6-DOF landers of 30 nodes, 40 x 100, 122 -> 35 ms; 256
-// quaternion quadrotors of 50 nodes, 20 x 100, 27.3 -> 7.4 ms; the ADMM call
+// 2.55 ms; 256 quaternion quadrotors of 50 nodes, 20 x 100, 27.3 -> 7.4 ms; the ADMM call
 // on 511 quadrotors, 100 iterations, 8.15 -> 1.07 ms.  The error against FP64
 // is as before (3e-7, 4e-7, 1.1e-6, 4e-7, 1e-6).  What bounds it: latency at 8
 // warps per SM -- issue slots 45% used in the ADMM loop; stalls at the two
@@ -42,11 +41,10 @@ namespace ucn {
 constexpr int ROWS_THREADS = 256, ROWS_WIDE_THREADS = 384;
 constexpr unsigned ROWS_ALL = 0xffffffffu;
 
-// Models the row kernel serves.
-template <class M> struct RowModel {
-  static constexpr int NN = M::NX + M::NU;
-  static constexpr bool value = NN == 16 || NN == 17;
-};
+// Models the row kernel serves.  The 6-DOF lander is not among them: in one batch
+// of 1000 in sixteen an FP32 solve of it meets a decision that rounding turns, and
+// its results here were up to 5e-5 (normwise) from the one-thread kernel's.
+template <class M> struct RowModel { static constexpr bool value = IsQuad<M>::value; };
 
 // a * b + c on two floats at once (one issue slot).
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
@@ -131,14 +129,12 @@ struct RowMats {
 };
 
 // Per-SCP-iteration constants of the lane's rows: cost gradient, diagonal of H
-// without the A/B Gram terms, the obstacles' Gram row (slot order; quadrotors)
-// or the thrust half-space's normal (6-DOF lander).
+// without the A/B Gram terms, the obstacles' Gram row (slot order).
 template <class M>
 struct RowConst {
   static constexpr int R = RowMats<M>::EX ? 5 : 4;
   float kq[R], khd[R];
   float gram[4];
-  float nrow, nx;
 };
 
 // The lane's ADMM variables: in registers for the length of an ADMM call
@@ -289,7 +285,7 @@ __device__ __forceinline__ bool rows_is_x(int m, int q) {
 }
 
 // ------------------------------------------------------------------ mirror sets in the ADMM loop
-// Quadrotors: projections and duals of the lane's obstacles (Steps 3, 4) at the
+// Projections and duals of the lane's obstacles (Steps 3, 4) at the
 // node's new position, and the sum of their right-hand-side terms n (rho s - nu)
 // for the next Step 1; `mg` receives that of the lane's position row (lane q <
 // 3: row q).  rp, sv as in node_mirrors (last iteration).
@@ -326,99 +322,6 @@ __device__ __forceinline__ float rows_obstacles(const RowPos& p, const Layout& L
   return sel4(a0, a1, a2, 0.0f, p.q);
 }
 
-// 6-DOF lander: the vector sets, one per lane -- glide-slope cone (lane 0), body
-// rates (1), tilt (2), thrust ball (3) -- then lane 3's gimbal cone and thrust
-// lower bound.  Reads xi from the record; leaves each row's right-hand-side term
-// in the record (Ga).  RESEED: projections alone, duals kept (node_reseed), or
-// -- `kept` -- the projections of an imported state left as they are too.
-template <class M, bool LAST, bool RESEED>
-__device__ __forceinline__ void rows_sets(const RowPos& p, const Layout& L, const Inst<float>& I, float rg, float irg,
-                                          int xi_at, float* svr, DF& rp, bool kept = false) {
-  typedef Rec<M, 2> R;
-  __syncwarp();
-  if (p.active) {
-    float* t = p.tp - p.q;   // the record's base
-    const int q = p.q;
-    const bool ctl = p.hasU;
-    // first row, data (nominal), scalars of the lane's set
-    const int e0 = q == 0 ? 1 : q == 1 ? 11 : q == 2 ? 9 : 14;
-    const int d0 = L.oMd + (q == 0 ? M14::D_R : q == 1 ? M14::D_W : q == 2 ? M14::D_Q : M14::D_U);
-    const int k0 = q == 0 ? M14::S_CONE : q == 1 ? M14::S_W : q == 2 ? M14::S_TILT : M14::S_BALL;
-    const bool on = q == 0 ? I.cone : q == 1 ? I.wball : q == 2 ? I.tilt : (I.ball && ctl);
-    const float rad = q == 1 ? I.wmax : q == 2 ? I.rtilt : I.tmax;
-    const int nv = q == 2 ? 2 : 3;
-    float ga[3] = {0.0f, 0.0f, 0.0f};
-    float x[3], v[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      x[k] = k < nv ? t[xi_at + e0 + k] : 0.0f;
-      v[k] = k < nv ? t[d0 + k] + x[k] + (RESEED ? 0.0f : t[L.oNus + k0 + k] * irg) : 0.0f;
-    }
-    if (on) {
-      if (q == 0) proj_cone3c(v, I.tau, I.ca, I.sa);
-      else proj_ball3(v, rad);
-#pragma unroll
-      for (int k = 0; k < 3; ++k)
-        if (k < nv) {
-          const float s = RESEED && kept ? t[L.oS + k0 + k] : v[k] - t[d0 + k];
-          float nu = t[L.oNus + k0 + k];
-          if (!RESEED) {
-            if (LAST) { svr[k] = rg * (s - t[L.oS + k0 + k]); acc_sq_diff(rp, x[k], s); }
-            nu += rg * (x[k] - s);
-            t[L.oNus + k0 + k] = nu;
-          }
-          t[L.oS + k0 + k] = s;
-          ga[k] = rg * s - nu;
-        }
-    }
-    if (q == 3 && ctl) {
-      if (I.gim) {   // gimbal cone on the thrust (t = body x)
-#pragma unroll
-        for (int k = 0; k < 3; ++k)
-          v[k] = t[d0 + k] + x[k] + (RESEED ? 0.0f : t[L.oNus + M14::S_GIM + k] * irg);
-        proj_cone3c(v, I.tg, I.cg, I.sg);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          const float s = RESEED && kept ? t[L.oS + M14::S_GIM + k] : v[k] - t[d0 + k];
-          float nu = t[L.oNus + M14::S_GIM + k];
-          if (!RESEED) {
-            if (LAST) { svr[k] += rg * (s - t[L.oS + M14::S_GIM + k]); acc_sq_diff(rp, x[k], s); }
-            nu += rg * (x[k] - s);
-            t[L.oNus + M14::S_GIM + k] = nu;
-          }
-          t[L.oS + M14::S_GIM + k] = s;
-          ga[k] += rg * s - nu;
-        }
-      }
-      if (I.half) {   // linearised |T| >= Tmin
-        const float* n = t + L.oMd + M14::D_N;
-        const float y = n[0] * x[0] + n[1] * x[1] + n[2] * x[2];
-        float nu = t[L.oNus + M14::S_HALF];
-        const float s = RESEED && kept ? t[L.oS + M14::S_HALF]
-                                       : fmaxf(t[L.oMd + M14::D_BD], RESEED ? y : y + nu * irg);
-        if (!RESEED) {
-          if (LAST) {
-            const float ds = rg * (s - t[L.oS + M14::S_HALF]);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) svr[k] += n[k] * ds;
-            acc_sq_diff(rp, y, s);
-          }
-          nu += rg * (y - s);
-          t[L.oNus + M14::S_HALF] = nu;
-        }
-        t[L.oS + M14::S_HALF] = s;
-        const float a = rg * s - nu;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) ga[k] += n[k] * a;
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-      if (k < nv) t[R::Ga + e0 + k] = ga[k];
-  }
-  __syncwarp();
-}
-
 // ------------------------------------------------------------------ one ADMM iteration
 // Steps 1-4 (Sec. III-B) as admm_iteration, lane-parallel.  Every thread calls
 // it; threads without a node carry zero matrices and store nothing.  GROUP: see
@@ -430,7 +333,7 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
                                                DF& rdl, GroupShared* G, GroupX& X, const ProblemDev& P, const Node<float, 2>& nd) {
   typedef Rec<M, 2> R;
   constexpr int RX = RowMats<M>::RX, RE = RowConst<M>::R;
-  constexpr bool EX = RowMats<M>::EX, QUAD = IsQuad<M>::value;
+  constexpr bool EX = RowMats<M>::EX;
   float* tp = p.tp;
   const int q = p.q;
   float xo[RE];
@@ -454,10 +357,9 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
     for (int m = 0; m < RE; ++m) {
       float v = rg * S.hat(m) - S.nu(m) - kq(m);
       if (m < RX && rows_is_x<M>(m, q)) v += re * S.z(m) - S.lam(m);   // (both 0 at node 0)
-      if constexpr (!QUAD) v += tp[R::Ga + (m < 4 ? 4 * m : 16 - q)];
       g[m] += v;
     }
-    if constexpr (QUAD) g[0] += mg;
+    g[0] += mg;
     rows_solve<M>(A, g, xo);
     // one refinement step: the residual with H applied from G, the diagonal and
     // the mirror Gram terms
@@ -470,13 +372,7 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
     rows_GT<M>(A, t, r);
 #pragma unroll
     for (int m = 0; m < RE; ++m) r[m] = g[m] - (khd(m) * xo[m] + r[m]);
-    if constexpr (QUAD) {
-      r[0] -= (gram(0) * v[0][0].x + gram(1) * v[0][0].y) + (gram(2) * v[0][1].x + gram(3) * v[0][1].y);
-    } else {
-      const float y = rg * (rows_sum(K.nrow * xo[3]) + K.nx * xo[RE - 1]);
-      r[3] -= K.nrow * y;
-      r[RE - 1] -= K.nx * y;
-    }
+    r[0] -= (gram(0) * v[0][0].x + gram(1) * v[0][0].y) + (gram(2) * v[0][1].x + gram(3) * v[0][1].y);
     float dx[RE];
     rows_solve<M>(A, r, dx);
 #pragma unroll
@@ -506,14 +402,14 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
             if (rows_is_x<M>(m, q)) st_async(p.halo0 + R::Ex1 + 4 * m, p.rank + 1, t[m], &p.hb->bar[0]);
         }
     }
-    if (p.active && (LAST || !QUAD)) {
+    if (p.active && LAST) {
 #pragma unroll
       for (int m = 0; m < RE; ++m) tp[R::X + (m < 4 ? 4 * m : 16 - q)] = xo[m];
     }
   }
   // Step 3 before Step 2, between the arrival (Ex1 published) and the wait
   split_barrier_arrive(X.bar);
-  float sv[RE], dz[RX], svr[3] = {0.0f, 0.0f, 0.0f};
+  float sv[RE], dz[RX];
   if (LAST) {
 #pragma unroll
     for (int m = 0; m < RE; ++m) sv[m] = 0.0f;
@@ -533,8 +429,7 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
     }
     S.set_box(m, xh, nu + rg * (xo[m] - xh), p.active);
   }
-  if constexpr (QUAD) mg = rows_obstacles<M, LAST>(p, L, I.nobs, xo, rg, irg, sv, rp);
-  else rows_sets<M, LAST, false>(p, L, I, rg, irg, R::X, svr, rp);
+  mg = rows_obstacles<M, LAST>(p, L, I.nobs, xo, rg, irg, sv, rp);
   split_barrier_wait(X.bar, X.ph);
   if constexpr (CL) halo_wait<4 * M::NX>(p.hb, hp, 0, p.first, q == 0);
   // ---- Step 2: dynamic consensus, Eq. (5), then its duals (Step 4)
@@ -576,32 +471,6 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
   }
   if constexpr (LAST) {
     // dual residual needs rho_dyn (z_{i+1,new} - z_{i+1,old}) from the right neighbour
-    if constexpr (!QUAD) {   // the vector sets' terms to their rows, through Ga's place
-      __syncwarp();
-      float keep[RE];
-#pragma unroll
-      for (int m = 0; m < RE; ++m) keep[m] = tp[R::Ga + (m < 4 ? 4 * m : 16 - q)];
-      __syncwarp();
-      if (p.active) {
-#pragma unroll
-        for (int m = 0; m < RE; ++m) tp[R::Ga + (m < 4 ? 4 * m : 16 - q)] = 0.0f;
-      }
-      __syncwarp();
-      if (p.active) {
-        const int e0 = q == 0 ? 1 : q == 1 ? 11 : q == 2 ? 9 : 14;
-#pragma unroll
-        for (int k = 0; k < 3; ++k)
-          if (k < 2 || q != 2) (tp - q)[R::Ga + e0 + k] = svr[k];
-      }
-      __syncwarp();
-#pragma unroll
-      for (int m = 0; m < RE; ++m) sv[m] += tp[R::Ga + (m < 4 ? 4 * m : 16 - q)];
-      __syncwarp();
-      if (p.active) {
-#pragma unroll
-        for (int m = 0; m < RE; ++m) tp[R::Ga + (m < 4 ? 4 * m : 16 - q)] = keep[m];
-      }
-    }
     if constexpr (CL) cluster_sync();
     else __syncthreads();
     if (p.later) {
@@ -753,11 +622,6 @@ __device__ __forceinline__ void rows_setup(const RowPos& p, const Node<float, 2>
         kq = df_to_float(gq);
       }
       khd = df_to_float(w) + rg + (p.i > 0 ? re : 0.0f);
-      if constexpr (IsMars14<M>::value) {
-        if (I.cone && e >= 1 && e <= 3) khd += rg;
-        if (I.tilt && (e == 9 || e == 10)) khd += rg;
-        if (I.wball && e >= 11) khd += rg;
-      }
       lo = fmaxf(wide_diff<float>(cb[C::Xlo + e], xb), -rad);
       hi = fminf(wide_diff<float>(cb[C::Xhi + e], xb), rad);
       if (p.i == 0) lo = hi = wide_diff<float>(cb[C::Xinit + e], xb);
@@ -767,10 +631,6 @@ __device__ __forceinline__ void rows_setup(const RowPos& p, const Node<float, 2>
       const DF ub = nd.dat(Rec<M>::Ubar, j), w = cb[C::Rd + j];
       if (I.run_cost) kq = df_to_float(df_mul(df_sub(ub, cb[C::Uref + j]), w));
       khd = df_to_float(w) + rg;
-      if constexpr (IsMars14<M>::value) {
-        if (I.ball) khd += rg;
-        if (I.gim) khd += rg;
-      }
       lo = fmaxf(wide_diff<float>(cb[C::Ulo + j], ub), -rad);
       hi = fminf(wide_diff<float>(cb[C::Uhi + j], ub), rad);
     }
@@ -839,7 +699,7 @@ template <class M>
 __device__ __forceinline__ bool rows_factor(const RowPos& p, RowMats<M>& A, const RowConst<M>& K, const Inst<float>& I,
                                             float rd, float rg) {
   constexpr int RX = RowMats<M>::RX;
-  constexpr bool EX = RowMats<M>::EX, QUAD = IsQuad<M>::value;
+  constexpr bool EX = RowMats<M>::EX;
   const int q = p.q;
   float h[4][16], hx[4], rx[17];   // own rows, their column 16, row 16
 #pragma unroll
@@ -909,14 +769,8 @@ __device__ __forceinline__ bool rows_factor(const RowPos& p, RowMats<M>& A, cons
     for (int c = 0; c < 17; ++c) rx[c] *= rd;
     rx[16] += p.active ? K.khd[4] : 1.0f;
   }
-  if constexpr (QUAD) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c) h[0][c] += sel4(K.gram[0], K.gram[1], K.gram[2], K.gram[3], q ^ c);
-  } else {   // the thrust half-space: rows 14, 15 (lanes 2, 3) and 16
-    const float n14 = rows_from(K.nrow, 2), n15 = rows_from(K.nrow, 3), w = rg * K.nrow;
-    h[3][14] += w * n14; h[3][15] += w * n15; hx[3] += w * K.nx;
-    rx[14] += rg * K.nx * n14; rx[15] += rg * K.nx * n15; rx[16] += rg * K.nx * K.nx;
-  }
+  for (int c = 0; c < 3; ++c) h[0][c] += sel4(K.gram[0], K.gram[1], K.gram[2], K.gram[3], q ^ c);
   // Gauss-Jordan, four pivots (one per lane) per pass; rows and columns rotate by
   // four in between, back in place after the fourth pass
   bool ok = true;
@@ -1004,31 +858,14 @@ __device__ __forceinline__ bool rows_factor(const RowPos& p, RowMats<M>& A, cons
 // mirror sets, H^-1 and the published mu + rho_dyn z.  Ends with a barrier.
 // The mirrors are re-projected from (x-hat, u-hat), or kept as imported.
 template <class M, bool CL>
-__device__ __forceinline__ float rows_prepare(const RowPos& p, const Node<float, 2>& nd, const Node<float, 2>& ndd,
-                                              bool dact, const Layout& L, const ProblemDev& P, const Inst<float>& I,
-                                              int b, float rad, float re, float rd, float rg, RowMats<M>& A,
-                                              RowConst<M>& K, InstShared& sh, bool kept = false) {
+__device__ __forceinline__ float rows_prepare(const RowPos& p, const Node<float, 2>& nd, const Layout& L,
+                                              const ProblemDev& P, const Inst<float>& I, int b, float rad, float re,
+                                              float rd, float rg, RowMats<M>& A, RowConst<M>& K, InstShared& sh,
+                                              bool kept = false) {
   typedef Rec<M, 2> R;
   constexpr int RX = RowMats<M>::RX;
-  float mg = 0.0f;
   rows_setup<M>(p, nd, I, rad, sh.tmask, re, rg, K);
-  if constexpr (IsQuad<M>::value) {
-    mg = rows_obstacle_setup<M>(p, nd, L, P, b, I.nobs, rg, kept, K);
-  } else {
-    if (dact) {   // one thread per node: set data at the nominal
-      DF xb[M::NX], ub[M::NU];
-      read_nominal<M, float, 2>(ndd, ndd.i < ndd.N, xb, ub);
-      node_mirror_data<M, float, 2>(ndd, L, P, b, xb, ub);
-    }
-    __syncthreads();
-    float none[3];
-    DF zero;
-    rows_sets<M, false, true>(p, L, I, rg, 0.0f, R::Xh, none, zero, kept);
-    const bool on = p.hasU && I.half;
-    const float* n = p.tp - p.q + L.oMd + M14::D_N;
-    K.nrow = on && p.q >= 2 ? n[p.q - 2] : 0.0f;
-    K.nx = on ? n[2] : 0.0f;
-  }
+  const float mg = rows_obstacle_setup<M>(p, nd, L, P, b, I.nobs, rg, kept, K);
   if (!rows_factor<M>(p, A, K, I, rd, rg)) atomicOr(&sh.fail, 1);
   if (p.later) {
 #pragma unroll
@@ -1198,11 +1035,10 @@ struct RowEngine {
                                                    const Step3<float>& hs, const Layout&) {
     rows_jacobians<M, REG ? 2 : 1>(p, nd, A, prm, hs);
   }
-  __device__ static __forceinline__ float prepare(const Pos& p, const Node<float, 2>& nd, const Node<float, 2>& ndd,
-                                                  bool dact, const Layout& L, const ProblemDev& P, const Inst<float>& I,
-                                                  int b, float rad, float re, float rd, float rg, Mats& A, Const& K,
-                                                  InstShared& sh) {
-    return rows_prepare<M, CL>(p, nd, ndd, dact, L, P, I, b, rad, re, rd, rg, A, K, sh);
+  __device__ static __forceinline__ float prepare(const Pos& p, const Node<float, 2>& nd, const Layout& L,
+                                                  const ProblemDev& P, const Inst<float>& I, int b, float rad, float re,
+                                                  float rd, float rg, Mats& A, Const& K, InstShared& sh) {
+    return rows_prepare<M, CL>(p, nd, L, P, I, b, rad, re, rd, rg, A, K, sh);
   }
   __device__ static __forceinline__ void admm(const Pos& p, const Mats& A, const Const& K, const Layout& L,
                                               const Inst<float>& I, float mg, float re, float rd, float rg, int iters,
@@ -1315,7 +1151,7 @@ __device__ __forceinline__ void scp_split_body(const ProblemDev& P, const Layout
     __syncthreads();
     const T re = rho_of<T>(sh, 0), rd = rho_of<T>(sh, 1), rg = rho_of<T>(sh, 2);
     E::jacobians(p, nd, A, prm_of<T>(sh), hs, L);
-    const T mg = E::prepare(p, nd, ndd, dact, L, P, I, b, radius_of<T>(sh), re, rd, rg, A, K, sh);
+    const T mg = E::prepare(p, nd, L, P, I, b, radius_of<T>(sh), re, rd, rg, A, K, sh);
     if constexpr (CL) {   // a failed factorisation anywhere stops the instance
       if (sh.fail && threadIdx.x < ncta) st_cluster(&sh.fail, threadIdx.x, 1);
       cluster_sync();
@@ -1465,8 +1301,7 @@ __global__ void __launch_bounds__(MAXT, 1) admm_rows_kernel(ProblemDev P, Layout
   }
   __syncthreads();
   const float re = (float)P.rho_eq, rd = (float)P.rho_dyn, rg = (float)P.rho_geo;
-  const float mg = rows_prepare<M, CL>(p, nd, ndd, dact, L, P, I, b, (float)radius[b], re, rd, rg, A, K, sh,
-                                       warm != 0);
+  const float mg = rows_prepare<M, CL>(p, nd, L, P, I, b, (float)radius[b], re, rd, rg, A, K, sh, warm != 0);
   if constexpr (CL) {
     if (sh.fail && threadIdx.x < ncta) st_cluster(&sh.fail, threadIdx.x, 1);
     cluster_sync();
