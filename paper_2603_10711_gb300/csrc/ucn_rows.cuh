@@ -1274,7 +1274,10 @@ __global__ void __launch_bounds__(MAXT, 1) admm_rows_kernel(ProblemDev P, Layout
   stage_params<M>(sh, P, b);
   stage_consts<M, float, 2>(ndd, P, b);
   if (dact) load_nominal<M, float, 2>(ndd, L, xbar, ubar, xo, uo);
-  __syncthreads();
+  // a cluster's CTAs have all started and cleared their records before the first
+  // store into one of them (rows_prepare's halo)
+  if constexpr (CL) cluster_sync();
+  else __syncthreads();
   rows_load_G<M>(p, A, Ag, Bg, uo + p.i);
   if (p.hasU) {
     // deviation affine term c_i = A xbar_i + B ubar_i + d_i - xbar_{i+1} in FP64 (once per call)
