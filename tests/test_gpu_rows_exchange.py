@@ -36,7 +36,7 @@ def admm(prob, x, u, lin, iters):
 
 # instances over clusters of two (and four) CTAs, more than the device holds at a
 # time: the CTAs of a cluster start while others still run
-@pytest.mark.parametrize("make", [lambda: W.quad_box(400, seed=21, N_range=(97, 127), obs_range=(2, 6)),
+@pytest.mark.parametrize("make", [lambda: W.quad_box(400, seed=21, N_range=(110, 110), obs_range=(2, 6)),
                                   lambda: W.quat_study(400, seed=22, N=70, tf=8.4),
                                   lambda: W.quat_study(200, seed=23, N=200, tf=24.0)])
 def test_admm_over_a_cluster_is_the_same_in_a_full_device_as_alone(make):
