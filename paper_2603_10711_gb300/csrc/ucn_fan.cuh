@@ -219,15 +219,22 @@ __device__ __forceinline__ void fan_iteration(const FanPos& p, const FanMats<F>&
   }
   split_barrier_arrive(X.bar);
   // ---- Step 3 (before Step 2: see admm_iteration) and Step 4 for nu_x, nu_u
-  double sv[RW], dz[RW];
+  // (F = 32: both lanes of a row read its variables before either stores them)
+  double sv[RW], dz[RW], nus[RW], old[RW];
+#pragma unroll
+  for (int m = 0; m < RW; ++m) {
+    nus[m] = t[R::Nux + q + F * m];
+    old[m] = LAST ? t[R::Xh + q + F * m] : 0.0;
+  }
+  if constexpr (F == 32) __syncwarp();
 #pragma unroll
   for (int m = 0; m < RW; ++m) {
     const int e = q + F * m;
     sv[m] = dz[m] = 0.0;
-    const double nu = t[R::Nux + e];
+    const double nu = nus[m];
     const double xh = clampv(xo[m] + nu * irg, t[R::Xlo + e], t[R::Xhi + e]);
     if (LAST) {
-      sv[m] = rg * (xh - t[R::Xh + e]);
+      sv[m] = rg * (xh - old[m]);
       if (p.active && p.owner) acc_sq_diff(rp, xo[m], xh);
     }
     if (p.active) {
@@ -239,15 +246,24 @@ __device__ __forceinline__ void fan_iteration(const FanPos& p, const FanMats<F>&
   split_barrier_wait(X.bar, X.ph);
   if constexpr (CL) halo_wait<8 * NX>(p.hb, hp, 0, p.first, p.lane == 0);
   // ---- Step 2: dynamic consensus, Eq. (5), then its duals (Step 4)
-  if (p.later) {
+  if (p.later) {   // (F = 32: a warp is one node, and takes the branch whole)
+    double lams[RW], mus[RW];
+#pragma unroll
+    for (int m = 0; m < RW; ++m) {
+      const int e = q + F * m < NX ? q + F * m : 0;
+      lams[m] = t[R::Lam + e];
+      mus[m] = t[R::Mu + e];
+      if (LAST) old[m] = t[R::Z + e];
+    }
+    if constexpr (F == 32) __syncwarp();
 #pragma unroll
     for (int m = 0; m < RW; ++m) {
       const int e = q + F * m;
       if (e < NX) {
-        const double dd = t[R::Ex1 + e - p.NS], lam = t[R::Lam + e], mu = t[R::Mu + e];
+        const double dd = t[R::Ex1 + e - p.NS], lam = lams[m], mu = mus[m];
         const double z = (re * xo[m] + lam + rd * dd - mu) * ired;
         if (LAST) {
-          dz[m] = z - t[R::Z + e];
+          dz[m] = z - old[m];
           sv[m] += re * dz[m];
           if (p.owner) {
             acc_sq_diff(rp, xo[m], z);

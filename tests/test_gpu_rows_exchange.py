@@ -49,3 +49,28 @@ def test_admm_over_a_cluster_is_the_same_in_a_full_device_as_alone(make):
         np.testing.assert_array_equal(one[0], xh[xo:xo + N + 1])
         np.testing.assert_array_equal(one[1], uh[uo:uo + N])
         np.testing.assert_array_equal(one[2][0], res[b])
+
+
+def solve(s):
+    x, u = s.scp_solve()
+    torch.cuda.synchronize()
+    return x.cpu().numpy().copy(), u.cpu().numpy().copy(), s.stats_host().copy()
+
+
+def same(a, b):
+    np.testing.assert_array_equal(a[0], b[0])
+    np.testing.assert_array_equal(a[1], b[1])
+    for f in ("primal_res", "dual_res", "merit", "accept_mask"):
+        np.testing.assert_array_equal(a[2][f], b[2][f])
+
+
+# 32 lanes per node: two lanes share a row of every node, on one CTA boundary and on many
+@pytest.mark.parametrize("N", [4, 50, 127])
+@pytest.mark.parametrize("iters", [1, 40])
+def test_fan_solves_repeat_their_bits(N, iters):
+    prob = W.quad_box(2, seed=24, N_range=(N, N), obs_range=(3, 5), settings=dict(scp_iters=3, admm_iters=iters, stop=0))
+    s = ucn.Solver(prob, precision=ucn.UCN_PREC_FP64)
+    first = solve(s)
+    for _ in range(10):
+        same(solve(s), first)
+    s.close()
