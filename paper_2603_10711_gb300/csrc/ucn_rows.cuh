@@ -415,9 +415,16 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
     for (int m = 0; m < RE; ++m) sv[m] = 0.0f;
   }
   // ---- Step 3: projections onto the boxes (Eq. (7)) and Step 4 for nu_x, nu_u
+  // (row 16 lies in the record for all four lanes: each reads it before any stores it)
+  float nu16 = 0.0f, hat16 = 0.0f;
+  if constexpr (EX) {
+    nu16 = S.nu(RE - 1);
+    hat16 = S.hat(RE - 1);
+    __syncwarp();
+  }
 #pragma unroll
   for (int m = 0; m < RE; ++m) {
-    const float nu = S.nu(m), arg = xo[m] + nu * irg;
+    const float nu = m < 4 ? S.nu(m) : nu16, arg = xo[m] + nu * irg;
     if constexpr (GROUP) {
       if (m == 3 && p.i == 0) continue;   // the consensus sets it
     }
@@ -425,7 +432,7 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
     if (LAST) {
       // row 16 counts once; a control row at node N is zero throughout
       if (p.active && (m < 4 || q == 0)) acc_sq_diff(rp, xo[m], xh);
-      sv[m] += rg * (xh - S.hat(m));
+      sv[m] += rg * (xh - (m < 4 ? S.hat(m) : hat16));
     }
     S.set_box(m, xh, nu + rg * (xo[m] - xh), p.active);
   }

@@ -74,3 +74,15 @@ def test_fan_solves_repeat_their_bits(N, iters):
     for _ in range(10):
         same(solve(s), first)
     s.close()
+
+
+# the 17th row, carried by all four lanes of a node; one CTA and a cluster
+@pytest.mark.parametrize("N", [1, 50, 70])
+@pytest.mark.parametrize("iters", [1, 40])
+def test_quaternion_solves_repeat_their_bits(N, iters):
+    prob = W.quat_study(40, seed=25, N=N, tf=0.12 * N, settings=dict(scp_iters=3, admm_iters=iters, stop=0))
+    s = ucn.Solver(prob, precision=ucn.UCN_PREC_FP32_REFINE)
+    first = solve(s)
+    for _ in range(10):
+        same(solve(s), first)
+    s.close()
