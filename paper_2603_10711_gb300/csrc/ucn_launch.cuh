@@ -333,7 +333,7 @@ cudaError_t launch_scp_t(const LaunchCfg& c, const double* x0, const double* u0,
 }
 
 // The group kernels of the lane layout, one per register class (each in its
-// own translation unit: defined there).
+// own translation unit: defined there; FP32: of LANES_MAX_THREADS alone).
 template <class M, class T, bool R>
 using ScpKernelPtr = void (*)(ProblemDev, Layout, const double*, const double*, double*, double*, ucn_scp_stats*, int*);
 template <class M, class T, bool R, int MAXT>
@@ -374,11 +374,14 @@ cudaError_t launch_scp_group_t(const LaunchCfg& c, const double* x0, const doubl
   ScpKernelPtr<M, T, R> k = scp_kernel<M, T, true, R, true>;
   cudaError_t e = cudaSuccess;
   if (c.tpn == 4) {
-    // four threads per node: FP32 records that fit the lane layout fit the row kernel's
+    // four threads per node, FP32: the row kernel, whose records are the smaller ones,
+    // up to its 96 nodes; beyond (with at most one obstacle 99 still fit) the lane kernel
     if constexpr (std::is_same<T, float>::value) {
-      if (L.csize != 1) return cudaErrorInvalidConfiguration;
-      e = rows_pick(c, threads, rows_scp_kernel<M, true, false, ROWS_THREADS>(),
-                    rows_scp_kernel<M, true, false, ROWS_WIDE_THREADS>(), &k);
+      if (L.csize == 1)
+        e = rows_pick(c, threads, rows_scp_kernel<M, true, false, ROWS_THREADS>(),
+                      rows_scp_kernel<M, true, false, ROWS_WIDE_THREADS>(), &k);
+      else
+        k = scp_group_lanes<M, T, R, LANES_MAX_THREADS>();
     } else {
       e = pick_group_lanes<M, T, R>(c, threads, &k);
     }
