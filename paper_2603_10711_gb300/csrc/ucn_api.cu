@@ -244,11 +244,14 @@ struct ucn_problem {
   int tpn;               // threads per node of the fused solve
   int last_launches = 0; // kernel launches of the last fused solve
   int optin;             // shared memory per CTA the device allows
-  // The row kernel serves this problem at its default threads per node, in parts
-  // of the CTA order: instances of the same CTA shape (see rows_parts), each part
-  // a launch of its own layout, the second and later ones on streams of their own.
+  // The row kernel serves this problem at its default threads per node, in parts:
+  // instances of the same CTA shape (see rows_parts), each part a launch of its own
+  // layout, the second and later ones on streams of their own.  Both stand from
+  // create on; order_d holds the CTA order and, with more than one part, the same
+  // order part by part after it.
   struct RowsPart { Layout L; int first, count; };
   std::vector<RowsPart> parts;
+  std::vector<int> part_of;   // of each instance
   std::vector<int> horizon;
   cudaStream_t aux[MAX_ROW_PARTS - 1] = {};
   cudaEvent_t fork = nullptr, join[MAX_ROW_PARTS - 1] = {};
@@ -280,17 +283,17 @@ cudaStream_t as_stream(void* s) { return (cudaStream_t)s; }
 
 // The row kernel's parts of a batch: its instances by the CTA shape their own
 // length needs -- one CTA of 64 nodes, of 96 (12-state quadrotor), clusters of
-// two, of four -- longest first, the given order kept within each.  One layout
+// two, of four -- longest first.  One layout
 // for the longest would give every instance the largest shape: 1023 quadrotors
 // of 40..120 nodes took 57.9 ms as clusters of two throughout, 36.9 ms in parts
 // (64 nodes: 1.14 us per ADMM iteration on one SM; 91: 2.0; 121: 1.6 on two).
 // At most MAX_ROW_PARTS: shorter shapes join the next longer one beyond that.
-void rows_parts(ucn_problem* p, std::vector<int>& order) {
-  p->parts.clear();
+void rows_parts(ucn_problem* p) {
   const int tpn = default_tpn(p->model, p->Nmax + 1, p->precision);
   Layout L;
   if (p->precision == UCN_PREC_FP64 && !fan_pays(p->horizon.data(), p->batch, p->Nmax + 1)) return;
   if (!rows_layout(p->model, p->precision, p->Nmax + 1, p->max_obs, p->group, tpn, p->batch, p->optin, &L)) return;
+  p->part_of.assign(p->batch, 0);
   if (p->group > 1) {
     p->parts.push_back({L, 0, p->batch});
     return;
@@ -311,16 +314,24 @@ void rows_parts(ucn_problem* p, std::vector<int>& order) {
     for (int& v : s) v = std::max(v, all[MAX_ROW_PARTS - 1]);
     all.resize(MAX_ROW_PARTS);
   }
-  std::vector<int> out;
-  for (int v : all) {
-    const int first = (int)out.size();
-    int nodes = 0;
-    for (int b : order)
-      if (s[b] == v) { out.push_back(b); nodes = std::max(nodes, p->horizon[b] + 1); }
+  int first = 0;
+  for (size_t k = 0; k < all.size(); ++k) {
+    int nodes = 0, count = 0;
+    for (int b = 0; b < p->batch; ++b)
+      if (s[b] == all[k]) { p->part_of[b] = (int)k; nodes = std::max(nodes, p->horizon[b] + 1); ++count; }
     rows_layout(p->model, p->precision, nodes, p->max_obs, 1, tpn, p->batch, p->optin, &L);
-    p->parts.push_back({L, first, (int)out.size() - first});
+    p->parts.push_back({L, first, count});
+    first += count;
   }
-  order = out;
+}
+
+// What order_d holds for a CTA order: the order, and again part by part.
+std::vector<int> order_of(const ucn_problem* p, std::vector<int> order) {
+  if (p->parts.size() > 1)
+    for (size_t k = 0; k < p->parts.size(); ++k)
+      for (int i = 0; i < p->batch; ++i)
+        if (p->part_of[order[i]] == (int)k) order.push_back(order[i]);
+  return order;
 }
 
 }  // namespace
@@ -483,9 +494,10 @@ ucn_status ucn_problem_create(const ucn_problem_desc* d, ucn_problem** out) {
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return w[x] > w[y]; });
   }
   p->horizon.assign(d->horizon, d->horizon + B);
-  rows_parts(p, order);
+  rows_parts(p);
+  order = order_of(p, order);
   int* ord = nullptr;
-  COPY(ord, order.data(), B);
+  COPY(ord, order.data(), order.size());
   const std::vector<double> fac = rho_schedule(d->rho_final, d->rho_geo, d->scp_iters);
   double* facd = nullptr;
   COPY(facd, fac.data(), fac.size());
@@ -607,8 +619,8 @@ ucn_status ucn_problem_set_order(ucn_problem* p, const int* order) {
   } else {
     for (int b = 0; b < p->batch; ++b) o[b] = b;
   }
-  rows_parts(p, o);
-  const cudaError_t e = cudaMemcpy(p->order_d, o.data(), sizeof(int) * p->batch, cudaMemcpyHostToDevice);
+  o = order_of(p, o);
+  const cudaError_t e = cudaMemcpy(p->order_d, o.data(), sizeof(int) * o.size(), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return fail(UCN_ECUDA, "order copy: %s", cudaGetErrorString(e));
   return UCN_OK;
 }
@@ -689,7 +701,7 @@ static cudaError_t launch_parts(ucn_problem* p, LaunchCfg c, bool admm, F launch
   for (size_t k = 0; k < p->parts.size() && e == cudaSuccess; ++k) {
     const ucn_problem::RowsPart& q = p->parts[k];
     ProblemDev P = base;
-    P.order = base.order + q.first;
+    P.order = p->order_d + p->batch + q.first;
     c.P = &P;
     c.L = &q.L; c.smem_bytes = q.L.bytes; c.blocks = q.count;
     if (k > 0 && !alone) {
