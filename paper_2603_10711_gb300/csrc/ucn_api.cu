@@ -576,7 +576,10 @@ ucn_status ucn_problem_create(const ucn_problem_desc* d, ucn_problem** out) {
     P.gflag = (unsigned*)gf;
   }
   P.ws = nullptr;
-  if (!p->smem) {
+  // (the quaternion quadrotor's FP32 solves and ADMM calls run on the row kernel
+  // alone, whose records are in shared memory at every size)
+  const bool rows_only = d->precision == UCN_PREC_FP32_REFINE && d->model == UCN_MODEL_QUAT13 && !p->parts.empty();
+  if (!p->smem && !rows_only) {
     char* ws = nullptr;
     ++na;
     if (fa > 0 && na == fa) { ucn_problem_destroy(p); return fail(UCN_ENOMEM, "injected allocation failure (UCN_FAULT_ALLOC=%d)", fa); }
