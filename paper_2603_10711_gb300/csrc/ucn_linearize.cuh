@@ -104,7 +104,8 @@ __global__ void __launch_bounds__(128) linearize_kernel(ProblemDev P, const int*
       }
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      acc[F::R + k] -= x[F::R + k] + drv * x[F::V + k];
+      acc[F::R + k] -= x[F::R + k];
+      acc[F::R + k] -= drv * x[F::V + k];
       acc[F::V + k] -= dvv * x[F::V + k];
     }
   }

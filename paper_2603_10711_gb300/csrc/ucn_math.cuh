@@ -27,8 +27,20 @@ template <class T> __device__ __forceinline__ Dual<T> operator+(Dual<T> a, Dual<
 template <class T> __device__ __forceinline__ Dual<T> operator-(Dual<T> a, Dual<T> b) { return {a.v - b.v, a.d - b.d}; }
 template <class T> __device__ __forceinline__ Dual<T> operator-(Dual<T> a) { return {-a.v, -a.d}; }
 template <class T> __device__ __forceinline__ Dual<T> operator*(Dual<T> a, Dual<T> b) { return {a.v * b.v, a.d * b.v + a.v * b.d}; }
+// a / b from b's correctly rounded reciprocal r: a r corrected by its exact residue
+// is the correctly rounded quotient (Markstein 1990), at three instructions instead
+// of a division's chain.
+__device__ __forceinline__ double quot_(double a, double b, double r) {
+  const double q = a * r;
+  return fma(fma(-q, b, a), r, q);
+}
+__device__ __forceinline__ float quot_(float a, float b, float r) {
+  const float q = a * r;
+  return fmaf(fmaf(-q, b, a), r, q);
+}
+__device__ __forceinline__ DF quot_(DF a, DF, DF r) { return df_mul(a, r); }
 // Duals divide through one reciprocal (the Jacobian passes' latency is the chain
-// of divisions), correctly rounded in FP32.
+// of divisions): FP32 by products with it, FP64 by correctly rounded quotients.
 __device__ __forceinline__ Dual<float> operator/(Dual<float> a, Dual<float> b) {
   const float r = __frcp_rn(b.v), q = a.v * r;
   return {q, (a.d - q * b.d) * r};
@@ -38,9 +50,10 @@ __device__ __forceinline__ Dual<float> operator/(float a, Dual<float> b) {
   return {q, -q * b.d * r};
 }
 template <class T> __device__ __forceinline__ Dual<T> operator/(Dual<T> a, Dual<T> b) {
-  const T r = T(1) / b.v, q = a.v * r;
-  return {q, (a.d - q * b.d) * r};
+  const T r = T(1) / b.v, q = quot_(a.v, b.v, r);
+  return {q, quot_(a.d - q * b.d, b.v, r)};
 }
+template <class T> __device__ __forceinline__ Dual<T> quot_(Dual<T> a, T b, T r) { return {quot_(a.v, b, r), quot_(a.d, b, r)}; }
 template <class T> __device__ __forceinline__ Dual<T> operator+(Dual<T> a, T b) { return {a.v + b, a.d}; }
 template <class T> __device__ __forceinline__ Dual<T> operator+(T b, Dual<T> a) { return {a.v + b, a.d}; }
 template <class T> __device__ __forceinline__ Dual<T> operator-(Dual<T> a, T b) { return {a.v - b, a.d}; }
@@ -49,8 +62,8 @@ template <class T> __device__ __forceinline__ Dual<T> operator*(Dual<T> a, T b) 
 template <class T> __device__ __forceinline__ Dual<T> operator*(T b, Dual<T> a) { return {a.v * b, a.d * b}; }
 template <class T> __device__ __forceinline__ Dual<T> operator/(Dual<T> a, T b) { return {a.v / b, a.d / b}; }
 template <class T> __device__ __forceinline__ Dual<T> operator/(T a, Dual<T> b) {
-  const T r = T(1) / b.v, q = a * r;
-  return {q, -q * b.d * r};
+  const T r = T(1) / b.v, q = quot_(a, b.v, r);
+  return {q, quot_(-q * b.d, b.v, r)};
 }
 
 // K tangent directions on one value (the Jacobian passes of the FP32 path): the
@@ -136,18 +149,25 @@ template <class T> __device__ __forceinline__ Dual<T> sqrt_(Dual<T> a) {
 template <int K> __device__ __forceinline__ DualN<double, K> operator/(DualN<double, K> a, DualN<double, K> b) {
   const double rr = 1.0 / b.v;
   DualN<double, K> r;
-  r.v = a.v * rr;
+  r.v = quot_(a.v, b.v, rr);
 #pragma unroll
-  for (int q = 0; q < K; ++q) r.d[q] = (a.d[q] - r.v * b.d[q]) * rr;
+  for (int q = 0; q < K; ++q) r.d[q] = quot_(a.d[q] - r.v * b.d[q], b.v, rr);
   return r;
 }
 template <int K> __device__ __forceinline__ DualN<double, K> operator/(double a, DualN<double, K> b) {
   const double rr = 1.0 / b.v;
   DualN<double, K> r;
-  r.v = a * rr;
+  r.v = quot_(a, b.v, rr);
 #pragma unroll
-  for (int q = 0; q < K; ++q) r.d[q] = -r.v * b.d[q] * rr;
+  for (int q = 0; q < K; ++q) r.d[q] = quot_(-r.v * b.d[q], b.v, rr);
   return r;
+}
+template <class T, int K> __device__ __forceinline__ DualN<T, K> quot_(DualN<T, K> a, T b, T r) {
+  DualN<T, K> c;
+  c.v = quot_(a.v, b, r);
+#pragma unroll
+  for (int q = 0; q < K; ++q) c.d[q] = quot_(a.d[q], b, r);
+  return c;
 }
 template <int K> __device__ __forceinline__ DualN<float, K> operator/(DualN<float, K> a, DualN<float, K> b) {
   const float rr = __frcp_rn(b.v);
@@ -228,10 +248,10 @@ struct Quad12 {
     typedef typename BaseOf<S>::type R;
     const R arm = (R)prm[4], km = (R)prm[5];
     Held<S> H;
-    H.Fm = (u[0] + u[1] + u[2] + u[3]) * (R)prm[8];
-    H.ax = (arm * (R)prm[9]) * (u[1] - u[3]);
-    H.ay = (arm * (R)prm[10]) * (u[2] - u[0]);
-    H.az = (km * (R)prm[11]) * (u[0] - u[1] + u[2] - u[3]);
+    H.Fm = quot_(u[0] + u[1] + u[2] + u[3], (R)prm[0], (R)prm[8]);
+    H.ax = quot_(arm * (u[1] - u[3]), (R)prm[1], (R)prm[9]);
+    H.ay = quot_(arm * (u[2] - u[0]), (R)prm[2], (R)prm[10]);
+    H.az = quot_(km * (u[0] - u[1] + u[2] - u[3]), (R)prm[3], (R)prm[11]);
     return H;
   }
   template <class S, class P>
@@ -274,10 +294,10 @@ struct Quat13 {
   __device__ static __forceinline__ Held<S> hold(const P* prm, const S* u) {
     typedef typename BaseOf<S>::type R;
     Held<S> H;
-    H.Tm = u[0] * (R)prm[8];
-    H.ax = u[1] * (R)prm[9];
-    H.ay = u[2] * (R)prm[10];
-    H.az = u[3] * (R)prm[11];
+    H.Tm = quot_(u[0], (R)prm[0], (R)prm[8]);
+    H.ax = quot_(u[1], (R)prm[1], (R)prm[9]);
+    H.ay = quot_(u[2], (R)prm[2], (R)prm[10]);
+    H.az = quot_(u[3], (R)prm[3], (R)prm[11]);
     return H;
   }
   template <class S, class P>
