@@ -106,53 +106,13 @@ __device__ __forceinline__ DF df_sqrt(DF a) {
   return df_quick_two_sum(s, __fdiv_rn(r.hi, __fmul_rn(2.0f, s)));
 }
 
-// sin a and cos a.  Range reduction by multiples of pi/2 held in three floats
-// (Cody and Waite 1980), their products with k error-free; then the Taylor
-// series of both on |r| <= pi/4, terms whose float rounding is below 2^-50 of
-// the result in float, the others in double-float.  Beyond 2^15 (or for a NaN
-// or an infinity) through FP64.  About 250 FP32 instructions; sin and cos in
-// FP64 took ~70 on a pipe of 1/64 the rate.
-__device__ __noinline__ inline void df_sincos_fp64(DF a, DF& s, DF& c) {
+// sin a and cos a through FP64 (to double-float's last bit: a series in double-float
+// arithmetic is faster and 1.2 to 1.8 times as far off, 7 times at worst).
+__device__ __noinline__ inline void df_sincos(DF a, DF& s, DF& c) {
   double sd, cd;
   sincos(df_to_double(a), &sd, &cd);
   s = df_from(sd);
   c = df_from(cd);
-}
-__device__ __noinline__ inline void df_sincos(DF a, DF& so, DF& co) {
-  if (!(fabsf(a.hi) < 32768.0f)) {
-    df_sincos_fp64(a, so, co);
-    return;
-  }
-  // pi/2 = P0 + P1 + P2 to ~2^-76
-  constexpr double HPI = 1.57079632679489661923, HPI_LO = 6.12323399573676588e-17;
-  constexpr float P0 = (float)HPI, P1 = (float)(HPI - (double)P0), P2 = (float)((HPI - (double)P0 - (double)P1) + HPI_LO);
-  const float k = rintf(__fmul_rn(a.hi, 0.636619772367581343f));
-  DF r = df_sub(a, df_two_prod(k, P0));
-  r = df_sub(r, df_two_prod(k, P1));
-  r = df_add(r, __fmul_rn(-k, P2));
-  const DF z = df_mul(r, r);
-  const float zf = z.hi;
-  // sin r = r + r z (S1 + z (S2 + ...)), S_n = (-1)^n / (2n+1)!
-  float p = __fmaf_rn(zf, -1.0f / 1307674368000.0f, 1.0f / 6227020800.0f);
-  p = __fmaf_rn(zf, p, -1.0f / 39916800.0f);
-  DF h = df_add(DF(1.0 / 362880.0), __fmul_rn(zf, p));
-  h = df_fma(DF(-1.0 / 5040.0), z, h);
-  h = df_fma(DF(1.0 / 120.0), z, h);
-  h = df_fma(DF(-1.0 / 6.0), z, h);
-  const DF s = df_fma(r, df_mul(r, z), h);
-  // cos r = 1 + z (C1 + z (C2 + ...)), C_n = (-1)^n / (2n)!
-  p = __fmaf_rn(zf, 1.0f / 20922789888000.0f, -1.0f / 87178291200.0f);
-  p = __fmaf_rn(zf, p, 1.0f / 479001600.0f);
-  h = df_add(DF(-1.0 / 3628800.0), __fmul_rn(zf, p));
-  h = df_fma(DF(1.0 / 40320.0), z, h);
-  h = df_fma(DF(-1.0 / 720.0), z, h);
-  h = df_fma(DF(1.0 / 24.0), z, h);
-  h = df_fma(DF(-0.5), z, h);
-  const DF c = df_fma(DF(1.0), z, h);
-  const int q = (int)k & 3;
-  const DF sv = (q & 1) ? c : s, cv = (q & 1) ? s : c;
-  so = (q & 2) ? df_neg(sv) : sv;
-  co = ((q + 1) & 2) ? df_neg(cv) : cv;
 }
 
 __device__ __forceinline__ DF operator+(DF a, DF b) { return df_add(a, b); }
