@@ -553,7 +553,7 @@ struct FanEngine {
   __device__ static __forceinline__ void admm(const Pos& p, const Mats& A, const Const& K, const Layout& L,
                                               const Inst<double>& I, double mg, double re, double rd, double rg,
                                               int iters, InstShared& sh, double* res, GroupShared*, GroupX& X,
-                                              const ProblemDev&, const Node<double, 2>&, RowHaloPhase& hp) {
+                                              const ProblemDev&, RowHaloPhase& hp) {
     const double irg = 1.0 / rg, ired = 1.0 / (re + rd);
     double rp = 0.0, rdl = 0.0;
     for (int it = 0; it + 1 < iters; ++it)

@@ -426,10 +426,11 @@ template <> __device__ __forceinline__ const float* prm_of<float>(const InstShar
 // Per-CTA state of a scenario group's exchanges (one CTA per scenario).
 struct GroupShared {
   double mine[2][16];   // this CTA's contribution to the current exchange (double-buffered)
-  double inv;           // 1 / K (wide type)
+  double count, inv;    // K, 1 / K
+  double ub[4];         // this scenario's nominal u_0
   double box[8];        // the scenarios' common box of u_0: max lower, -(min upper), absolute
   unsigned long long bar[2];   // one cluster per group: arrival of the peers' arguments, by parity
-  double u0[4];         // the consensus u-hat_0 of the latest iteration, absolute (wide type)
+  double u0[4];         // the consensus u-hat_0 of the latest iteration, absolute
   int gfail;            // sticky: a wait for another scenario of the group gave up
 };
 
@@ -438,8 +439,8 @@ struct GroupX {
   unsigned epoch;       // exchanges done
   int g, k;             // group index, scenario index within the group
   unsigned pub;         // consensus exchanges done within one cluster
-  // one cluster per group: the scenarios' Step-3 arguments of u_0 (in the wide
-  // type's 8 bytes), pushed by their CTAs, [2][16][4] double-buffered -- in
+  // one cluster per group: the scenarios' Step-3 arguments of u_0, absolute,
+  // pushed by their CTAs, [2][16][4] double-buffered -- in
   // InstShared::red, which no reduction uses during an ADMM call (cluster
   // barriers lie between a CTA's last reduction and its peers' next push)
   double* in;
@@ -604,70 +605,50 @@ __device__ __forceinline__ void group_init(const ProblemDev& P, GroupShared* G) 
 // publishes its scenario's Step-3 arguments as soon as Step 1 is done (lane l
 // holds that of control l mod 4), and collects the group's sums after Step 2:
 // the exchange has Steps 2 and 3 to travel.  The boxes are constant over an
-// ADMM call and are intersected before it (GroupShared::box).  Values are of the
-// wide type W -- double-float on the FP32 path, whose sum of a 64-scenario group
-// is FP32 work: as FP64 all-reduce of twelve values (sums and both bounds) the
-// exchange took 9 us per iteration of a 16-scenario group, the iteration itself
-// 1.6 us.  Every CTA of a group gets the same bits: one order of summation, of
-// an addition that commutes.
+// ADMM call and are intersected before it (GroupShared::box).  Sums, mean and box
+// are FP64 in both precisions; an all-reduce of twelve FP64 values (sums and both
+// bounds) in their place took 9 us per iteration of a 16-scenario group, the
+// iteration itself 1.6 us.  Every CTA of a group gets the same bits: one order of
+// summation, of an addition that commutes.
 //
 // One cluster per group: each CTA stores its values into all its peers' shared
 // memory, which count the bytes on an mbarrier that warp 0 waits on -- no barrier
 // across the cluster (with a cluster barrier per iteration 16 groups of 16 took
 // 6.04 us per iteration, so 5.37; 64 groups 15.1, so 13.6).  Several:
 // through its global slot and counter, as group_allreduce_flat.
-__device__ __forceinline__ double wide_shfl_xor(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
-__device__ __forceinline__ DF wide_shfl_xor(DF a, int o) {
-  return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
-}
-__device__ __forceinline__ double wide_shfl(double a, int l) { return __shfl_sync(0xffffffffu, a, l); }
-__device__ __forceinline__ DF wide_shfl(DF a, int l) {
-  return {__shfl_sync(0xffffffffu, a.hi, l), __shfl_sync(0xffffffffu, a.lo, l)};
-}
-__device__ __forceinline__ double wide_bits(double a) { return a; }
-__device__ __forceinline__ double wide_bits(DF a) { return __hiloint2double(__float_as_int(a.lo), __float_as_int(a.hi)); }
-template <class W> __device__ __forceinline__ W wide_of_bits(double a);
-template <> __device__ __forceinline__ double wide_of_bits<double>(double a) { return a; }
-template <> __device__ __forceinline__ DF wide_of_bits<DF>(double a) {
-  return {__int_as_float(__double2loint(a)), __int_as_float(__double2hiint(a))};
-}
-template <class W>
-__device__ __forceinline__ void group_publish(const ProblemDev& P, GroupShared* G, const GroupX& X, W v) {
+__device__ __forceinline__ void group_publish(const ProblemDev& P, GroupShared* G, const GroupX& X, double v) {
   const int lane = threadIdx.x, j = lane & 3;
-  const double bits = wide_bits(v);
   if (P.gclusters <= 1) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int r = (lane >> 2) + 8 * h;
-      if (r < P.group) st_async(X.in + ((X.pub & 1) * 16 + X.k) * 4 + j, (unsigned)r, bits, &G->bar[X.pub & 1]);
+      if (r < P.group) st_async(X.in + ((X.pub & 1) * 16 + X.k) * 4 + j, (unsigned)r, v, &G->bar[X.pub & 1]);
     }
   } else {
     double* slot = P.gx + (((long long)X.g * P.group + X.k) * 2 + (X.epoch & 1)) * 16;
     if (lane < 4) {
-      __stcg(slot + j, bits);
+      __stcg(slot + j, v);
       __threadfence();
     }
     __syncwarp();
     if (lane == 0) st_release_gpu(&P.gflag[(long long)X.g * P.group + X.k], X.epoch + 1);
   }
 }
-template <class W>
-__device__ __forceinline__ W group_collect(const ProblemDev& P, GroupShared* G, const GroupX& X) {
+__device__ __forceinline__ double group_collect(const ProblemDev& P, GroupShared* G, const GroupX& X) {
   const int lane = threadIdx.x, j = lane & 3, K = P.group;
-  W a = W();
   if (P.gclusters <= 1) {
     const double* in = X.in + (X.pub & 1) * 64;
     if (!G->gfail && !tx_wait(&G->bar[X.pub & 1], (X.pub >> 1) & 1)) G->gfail = 1;
     __syncwarp();
     if (lane == 0) tx_arm(&G->bar[X.pub & 1], (unsigned)K * 32u);   // the exchange after next
-    if ((lane >> 2) < K) a = wide_of_bits<W>(in[4 * (lane >> 2) + j]);
-    if ((lane >> 2) + 8 < K) a = a + wide_of_bits<W>(in[4 * (lane >> 2) + 32 + j]);
+    double a = (lane >> 2) < K ? in[4 * (lane >> 2) + j] : 0.0;
+    if ((lane >> 2) + 8 < K) a += in[4 * (lane >> 2) + 32 + j];
 #pragma unroll
-    for (int o = 4; o <= 16; o <<= 1) a = a + wide_shfl_xor(a, o);
+    for (int o = 4; o <= 16; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
     return a;
   }
   const long long base = (long long)X.g * K;
-  W s[4] = {W(), W(), W(), W()};
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
   for (int r = lane; r < K; r += 32) {
     if (!group_wait(P, G, &P.gflag[base + r], X.epoch + 1)) continue;
     const double* src = P.gx + ((base + r) * 2 + (X.epoch & 1)) * 16;
@@ -675,13 +656,13 @@ __device__ __forceinline__ W group_collect(const ProblemDev& P, GroupShared* G, 
 #pragma unroll
     for (int i = 0; i < 4; ++i) v[i] = __ldcg(src + i);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) s[i] = s[i] + wide_of_bits<W>(v[i]);
+    for (int i = 0; i < 4; ++i) s[i] += v[i];
   }
 #pragma unroll
   for (int o = 16; o >= 1; o >>= 1)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) s[i] = s[i] + wide_shfl_xor(s[i], o);
-  const W lo = (j & 1) ? s[1] : s[0], hi = (j & 1) ? s[3] : s[2];
+    for (int i = 0; i < 4; ++i) s[i] += __shfl_xor_sync(0xffffffffu, s[i], o);
+  const double lo = (j & 1) ? s[1] : s[0], hi = (j & 1) ? s[3] : s[2];
   return (j & 2) ? hi : lo;
 }
 // Both are done (every thread's sequence state).
@@ -689,41 +670,31 @@ __device__ __forceinline__ void group_advance(const ProblemDev& P, GroupX& X) {
   if (P.gclusters <= 1) X.pub++;
   else X.epoch++;
 }
-// The average of the K arguments of control j, clamped to the common box.
+// The average of the K arguments of control j, clamped to the common box (the bits
+// of the division sum / K: an infinite sum stays one).
 __device__ __forceinline__ double group_mean(const GroupShared* G, double sum, int j) {
-  return fmin(fmax(sum * G->inv, G->box[j]), -G->box[4 + j]);
-}
-__device__ __forceinline__ bool df_less(DF a, DF b) { return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo); }
-__device__ __forceinline__ DF group_mean(const GroupShared* G, DF sum, int j) {
-  DF v = df_mul(sum, wide_of_bits<DF>(G->inv));
-  const DF lo = wide_of_bits<DF>(G->box[j]), hi = wide_of_bits<DF>(G->box[4 + j]);
-  if (df_less(v, lo)) v = lo;
-  if (df_less(hi, v)) v = hi;
-  return v;
+  const bool finite = (__double2hiint(sum) & 0x7ff00000) != 0x7ff00000;
+  const double v = finite ? quot_(sum, G->count, G->inv) : sum;
+  return fmin(fmax(v, G->box[j]), -G->box[4 + j]);
 }
 // The common box of u_0 and whether any scenario's factorisation failed, before
-// an ADMM call; lo, hi: absolute, this scenario's, by the thread(s) of node 0
-// for the controls j they hold (put in G->mine beforehand, entries 1 + j and 5 + j).
-template <class W>
-__device__ __forceinline__ void group_box_put(GroupShared* G, const GroupX& X, int j, W lo, W hi) {
+// an ADMM call; ub, lo, hi: this scenario's nominal and box of control j, by the
+// thread of node 0 that holds it (in G->mine beforehand, entries 1 + j and 5 + j).
+__device__ __forceinline__ void group_box_put(GroupShared* G, const GroupX& X, int j, double ub, double lo, double hi) {
   double* m = G->mine[X.epoch & 1];
-  m[1 + j] = wide_to_double(lo);
-  m[5 + j] = -wide_to_double(hi);
+  G->ub[j] = ub;
+  m[1 + j] = ub + lo;
+  m[5 + j] = -(ub + hi);
 }
-template <class W>
 __device__ __forceinline__ void group_begin(const ProblemDev& P, GroupShared* G, GroupX& X, InstShared& sh) {
   if (threadIdx.x == 0) G->mine[X.epoch & 1][0] = (double)sh.fail;
   double a[9];
   group_allreduce<9>(P, G, X, 0, a);
   if (threadIdx.x == 0) {
     sh.fail = a[0] != 0.0;
-    G->inv = wide_bits(wide_from_double<W>(1.0 / (double)P.group));
-    for (int j = 0; j < 4; ++j) {
-      const double hi = -a[5 + j];
-      G->box[j] = wide_bits(wide_from_double<W>(a[1 + j]));
-      // (the FP64 form keeps the negated bound, as it was exchanged)
-      G->box[4 + j] = std::is_same<W, double>::value ? a[5 + j] : wide_bits(wide_from_double<W>(hi));
-    }
+    G->count = (double)P.group;
+    G->inv = 1.0 / (double)P.group;
+    for (int j = 0; j < 8; ++j) G->box[j] = a[1 + j];
   }
   __syncthreads();
 }
@@ -1699,16 +1670,15 @@ __device__ __forceinline__ void admm_iteration(const Node<T, AOS>& nd, const MS&
     // projects instead of idling at a barrier.
     if constexpr (GROUP) {
       if (threadIdx.x < 32) {   // node 0 is lane 0; lane l hands over control l mod 4
-        typedef typename Node<T, AOS>::W W;
-        W own = W();
+        double own = 0.0;
 #pragma unroll
         for (int j = 0; j < NU; ++j) {
-          W v = W();
-          if (i == 0) v = wide_add(nd.dat(Rec<M, AOS>::Ubar, j), x[NX + j] + S.nuu(j) * irg);
-          v = wide_shfl(v, 0);
+          double v = 0.0;
+          if (i == 0) v = G->ub[j] + (double)(x[NX + j] + S.nuu(j) * irg);
+          v = __shfl_sync(0xffffffffu, v, 0);
           if (((int)threadIdx.x & 3) == j) own = v;
         }
-        group_publish<W>(P, G, X, own);
+        group_publish(P, G, X, own);
       }
     }
     split_barrier_arrive(X.bar);
@@ -1764,20 +1734,19 @@ __device__ __forceinline__ void admm_iteration(const Node<T, AOS>& nd, const MS&
       }
     }
     if constexpr (GROUP) {
-      typedef typename Node<T, AOS>::W W;
-      W tot[NU];
+      double tot[NU];
       if (threadIdx.x < 32) {
-        const W sum = group_collect<W>(P, G, X);
+        const double sum = group_collect(P, G, X);
 #pragma unroll
-        for (int j = 0; j < NU; ++j) tot[j] = wide_shfl(sum, j);
+        for (int j = 0; j < NU; ++j) tot[j] = __shfl_sync(0xffffffffu, sum, j);
       }
       group_advance(P, X);
       if (active && i == 0 && i < N) {
 #pragma unroll
         for (int j = 0; j < NU; ++j) {
-          const W v = group_mean(G, tot[j], j);
-          G->u0[j] = wide_bits(v);
-          const T uh = wide_diff<T>(v, nd.dat(Rec<M, AOS>::Ubar, j));
+          const double v = group_mean(G, tot[j], j);
+          G->u0[j] = v;
+          const T uh = (T)(v - G->ub[j]);
           const T nuu = S.nuu(j);
           if (last) { sv[NX + j] += rg * (uh - nd.at(Rec<M, AOS>::Uh, j)); acc_sq_diff(rp, x[NX + j], uh); }
           nd.at(Rec<M, AOS>::Uh, j) = uh;
@@ -2275,7 +2244,7 @@ __device__ void scp_candidate(const Node<T, AOS>& nd, const MS& MT, const Proble
     if constexpr (GROUP) {
       // the shared first control exactly (bitwise equal across the group)
       if (i == 0)
-        for (int j = 0; j < NU; ++j) uc[j] = wide_of_bits<W>(G->u0[j]);
+        for (int j = 0; j < NU; ++j) uc[j] = wide_from_double<W>(G->u0[j]);
     }
   }
   __syncthreads();
@@ -2523,9 +2492,9 @@ __device__ __forceinline__ void scp_body(const ProblemDev& P, const Layout& L, c
       // a failed factorisation in any scenario stops the whole group
       if (i == 0)
         for (int j = 0; j < NU; ++j)
-          group_box_put<W>(G, X, j, wide_add(nd.dat(Rec<M, AOS>::Ubar, j), nd.at(Rec<M, AOS>::Ulo, j)),
-                           wide_add(nd.dat(Rec<M, AOS>::Ubar, j), nd.at(Rec<M, AOS>::Uhi, j)));
-      group_begin<W>(P, G, X, sh);
+          group_box_put(G, X, j, wide_to_double(nd.dat(Rec<M, AOS>::Ubar, j)), nd.at(Rec<M, AOS>::Ulo, j),
+                        nd.at(Rec<M, AOS>::Uhi, j));
+      group_begin(P, G, X, sh);
     }
     if (sh.fail) { if (threadIdx.x == 0) sh.status = ST_NUMERIC; iters_run++; break; }
     admm_iterations<M, T, AOS, REFINE, GROUP, REGS>(nd, MT, L, I, K, active, re, rd, rg, P.admm_iters, sh, res, G, X, P);

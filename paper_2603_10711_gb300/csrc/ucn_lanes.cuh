@@ -352,11 +352,9 @@ __device__ __forceinline__ void admm_iteration_lanes(const Node<T, AOS>& nd, con
   // neighbour's Ex1
   if constexpr (GROUP) {
     if (threadIdx.x < 32) {   // node 0 is the first four lanes; lane l hands over control l mod 4
-      typedef typename Node<T, AOS>::W W;
-      W a = i == 0 ? nd.dat(Rec<M>::Ubar, q) : W();
       const T nuu = i == 0 ? nd.at(Rec<M>::Nuu, q) : T(0);
-      a = wide_shfl(wide_add(a, xo[RX] + nuu * irg), (int)threadIdx.x & 3);
-      group_publish<W>(P, G, X, a);
+      const double a = G->ub[q] + (double)(xo[RX] + nuu * irg);
+      group_publish(P, G, X, __shfl_sync(WARP_ALL, a, (int)threadIdx.x & 3));
     }
   }
   split_barrier_arrive(X.bar);
@@ -434,13 +432,12 @@ __device__ __forceinline__ void admm_iteration_lanes(const Node<T, AOS>& nd, con
     }
   }
   if constexpr (GROUP) {
-    typedef typename Node<T, AOS>::W W;
     if (threadIdx.x < 32) {
-      const W sum = group_collect<W>(P, G, X);
+      const double sum = group_collect(P, G, X);
       if (active && i == 0 && i < N) {
-        const W v = group_mean(G, sum, q);
-        G->u0[q] = wide_bits(v);
-        const T uh = wide_diff<T>(v, nd.dat(Rec<M>::Ubar, q));
+        const double v = group_mean(G, sum, q);
+        G->u0[q] = v;
+        const T uh = (T)(v - G->ub[q]);
         const T nuu = nd.at(Rec<M>::Nuu, q);
         if (LAST) {
           sv[RX] += rg * (uh - nd.at(Rec<M>::Uh, q));
@@ -617,9 +614,8 @@ __device__ __forceinline__ void scp_lanes_body(const ProblemDev& P, const Layout
     H.load(MT, q, active);
     if constexpr (GROUP) {
       if (i == 0 && active)
-        group_box_put<W>(G, X, q, wide_add(nd.dat(Rec<M>::Ubar, q), nd.at(Rec<M>::Ulo, q)),
-                         wide_add(nd.dat(Rec<M>::Ubar, q), nd.at(Rec<M>::Uhi, q)));
-      group_begin<W>(P, G, X, sh);
+        group_box_put(G, X, q, wide_to_double(nd.dat(Rec<M>::Ubar, q)), nd.at(Rec<M>::Ulo, q), nd.at(Rec<M>::Uhi, q));
+      group_begin(P, G, X, sh);
     }
     if (sh.fail) { if (threadIdx.x == 0) sh.status = ST_NUMERIC; iters_run++; break; }
     admm_iterations_lanes<M, T, AOS, REFINE, GROUP, TPN>(nd, MT, H, L, I, kq, khd, active, q, re, rd, rg, P.admm_iters,

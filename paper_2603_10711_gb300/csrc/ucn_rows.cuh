@@ -330,7 +330,7 @@ template <class M, bool LAST, bool GROUP, bool CL, class ST>
 __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>& A, const RowConst<M>& K, const ST& S,
                                                const Layout& L, const Inst<float>& I, float& mg, float re, float rd,
                                                float rg, float irg, float ired, bool head, RowHaloPhase& hp, DF& rp,
-                                               DF& rdl, GroupShared* G, GroupX& X, const ProblemDev& P, const Node<float, 2>& nd) {
+                                               DF& rdl, GroupShared* G, GroupX& X, const ProblemDev& P) {
   typedef Rec<M, 2> R;
   constexpr int RX = RowMats<M>::RX, RE = RowConst<M>::R;
   constexpr bool EX = RowMats<M>::EX;
@@ -381,9 +381,8 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
       // the arguments of u_0, as early as they are known: node 0 is the first four
       // lanes; lane l hands over control l mod 4
       if (threadIdx.x < 32) {
-        DF a = p.i == 0 ? nd.dat(R::Ubar, q) : DF();
-        a = wide_shfl(df_add(a, xo[3] + S.nu(3) * irg), (int)threadIdx.x & 3);
-        group_publish<DF>(P, G, X, a);
+        const double a = G->ub[q] + (double)(xo[3] + S.nu(3) * irg);
+        group_publish(P, G, X, __shfl_sync(ROWS_ALL, a, (int)threadIdx.x & 3));
       }
     }
     // linearised propagation d_dyn,i = A x + B u + c_i, published to node i+1
@@ -464,11 +463,11 @@ __device__ __forceinline__ void rows_iteration(const RowPos& p, const RowMats<M>
   }
   if constexpr (GROUP) {
     if (threadIdx.x < 32) {
-      const DF sum = group_collect<DF>(P, G, X);
+      const double sum = group_collect(P, G, X);
       if (p.i == 0 && p.active) {
-        const DF v = group_mean(G, sum, q);
-        G->u0[q] = wide_bits(v);
-        const float uh = wide_diff<float>(v, nd.dat(R::Ubar, q));
+        const double v = group_mean(G, sum, q);
+        G->u0[q] = v;
+        const float uh = (float)(v - G->ub[q]);
         const float nu = S.nu(3);
         if (LAST) { sv[3] += rg * (uh - S.hat(3)); acc_sq_diff(rp, xo[3], uh); }
         S.set_box(3, uh, nu + rg * (xo[3] - uh), true);
@@ -512,16 +511,14 @@ template <class M, bool GROUP, bool CL, bool REG>
 __device__ __forceinline__ void rows_admm(const RowPos& p, const RowMats<M>& A, const RowConst<M>& K, const Layout& L,
                                           const Inst<float>& I, float mg, float re, float rd, float rg, int iters,
                                           InstShared& sh, double* res, GroupShared* G, GroupX& X, const ProblemDev& P,
-                                          const Node<float, 2>& nd, RowHaloPhase& hp) {
+                                          RowHaloPhase& hp) {
   const float irg = 1.0f / rg, ired = 1.0f / (re + rd);
   DF rp, rdl;
   RowState<M, REG> S;
   S.load(p);
   for (int it = 0; it + 1 < iters; ++it)
-    rows_iteration<M, false, GROUP, CL>(p, A, K, S, L, I, mg, re, rd, rg, irg, ired, it == 0, hp, rp, rdl, G, X, P,
-                                         nd);
-  rows_iteration<M, true, GROUP, CL>(p, A, K, S, L, I, mg, re, rd, rg, irg, ired, iters == 1, hp, rp, rdl, G, X, P,
-                                      nd);
+    rows_iteration<M, false, GROUP, CL>(p, A, K, S, L, I, mg, re, rd, rg, irg, ired, it == 0, hp, rp, rdl, G, X, P);
+  rows_iteration<M, true, GROUP, CL>(p, A, K, S, L, I, mg, re, rd, rg, irg, ired, iters == 1, hp, rp, rdl, G, X, P);
   S.store(p);
   reduce_residuals(sh, rp, rdl, res);
 }
@@ -990,7 +987,7 @@ __device__ __forceinline__ void split_candidate(const typename E::Pos& p, const 
     for (int j = 0; j < NU; ++j) uc[j] = i < N ? wide_add(nd.dat(R::Ubar, j), nd.at(R::Uh, j)) : W();
     if constexpr (E::GROUP) {
       if (i == 0)
-        for (int j = 0; j < NU; ++j) uc[j] = wide_of_bits<W>(G->u0[j]);
+        for (int j = 0; j < NU; ++j) uc[j] = wide_from_double<W>(G->u0[j]);
     }
   }
   if constexpr (E::CL) {
@@ -1050,8 +1047,8 @@ struct RowEngine {
   __device__ static __forceinline__ void admm(const Pos& p, const Mats& A, const Const& K, const Layout& L,
                                               const Inst<float>& I, float mg, float re, float rd, float rg, int iters,
                                               InstShared& sh, double* res, GroupShared* G, GroupX& X,
-                                              const ProblemDev& P, const Node<float, 2>& nd, RowHaloPhase& hp) {
-    rows_admm<M, GROUP, CL, REG>(p, A, K, L, I, mg, re, rd, rg, iters, sh, res, G, X, P, nd, hp);
+                                              const ProblemDev& P, RowHaloPhase& hp) {
+    rows_admm<M, GROUP, CL, REG>(p, A, K, L, I, mg, re, rd, rg, iters, sh, res, G, X, P, hp);
   }
   // the first node's candidate, for the linear model of the previous CTA's last node
   __device__ static __forceinline__ void push_hat(const Pos& p) {
@@ -1165,13 +1162,13 @@ __device__ __forceinline__ void scp_split_body(const ProblemDev& P, const Layout
     }
     if constexpr (GROUP) {
       if (p.i == 0 && p.active) {
-        const W ub = nd.dat(Rec<M, 2>::Ubar, p.q);
-        group_box_put<W>(G, X, p.q, wide_add(ub, p.tp[Rec<M, 2>::Xlo + 12]), wide_add(ub, p.tp[Rec<M, 2>::Xhi + 12]));
+        group_box_put(G, X, p.q, wide_to_double(nd.dat(Rec<M, 2>::Ubar, p.q)), p.tp[Rec<M, 2>::Xlo + 12],
+                      p.tp[Rec<M, 2>::Xhi + 12]);
       }
-      group_begin<W>(P, G, X, sh);
+      group_begin(P, G, X, sh);
     }
     if (sh.fail) { if (threadIdx.x == 0) sh.status = ST_NUMERIC; iters_run++; break; }
-    E::admm(p, A, K, L, I, mg, re, rd, rg, P.admm_iters, sh, res, G, X, P, nd, hp);
+    E::admm(p, A, K, L, I, mg, re, rd, rg, P.admm_iters, sh, res, G, X, P, hp);
     ++iters_run;
     W xc[NX], uc[NU], fc[NX];
     double v[6] = {0, 0, 0, 0, 0, 0};
@@ -1318,7 +1315,7 @@ __global__ void __launch_bounds__(MAXT, 1) admm_rows_kernel(ProblemDev P, Layout
   }
   double r2[2] = {0.0, 0.0};
   GroupX X{0u, 0, 0, 0u, nullptr, sh.xbar, 0u};
-  if (!sh.fail) rows_admm<M, false, CL, REG>(p, A, K, L, I, mg, re, rd, rg, iters, sh, r2, nullptr, X, P, nd, hp);
+  if (!sh.fail) rows_admm<M, false, CL, REG>(p, A, K, L, I, mg, re, rd, rg, iters, sh, r2, nullptr, X, P, hp);
   __syncthreads();
   if (dact) {
     const int i = ndd.i;
