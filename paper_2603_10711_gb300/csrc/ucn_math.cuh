@@ -410,7 +410,9 @@ __device__ __forceinline__ DF fma_(DF a, DF b, DF c) { return df_fma(a, b, c); }
 // loop: unrolled, a step of the larger models is 30 to 180 KB of code that runs
 // once per SCP iteration, and the instruction fetch is what it waits for.  The
 // 3-DOF Mars model's step is small outside double-float; rolled, its kernels
-// spill in the ADMM loop.  The 6-DOF lander's stays straight-line with quotients
+// spill in the ADMM loop.  The quaternion quadrotor's in FP64 waits for the FP64
+// pipe instead, and a loop's frame costs its one-thread kernel more (152 of 50
+// nodes, 4 x 100 iterations: 22.72 ms rolled, 22.16 straight).  The 6-DOF lander's stays straight-line with quotients
 // and held terms in every stage: its FP32 solves meet decisions that a last bit
 // turns (one batch of 1000 in sixteen: up to 5e-5 normwise), so their results are
 // only as constant as this rounding.
@@ -433,7 +435,7 @@ __device__ __forceinline__ void rk4h(const P* prm, R h, R hh, R h6, const S* x, 
   const typename M::template Held<S> H = M::template hold<S, P>(prm, u);
 #pragma unroll
   for (int j = 0; j < NX; ++j) t[j] = x[j];
-#pragma unroll (M::NX == 7 && !std::is_same<S, DF>::value ? 4 : 1)
+#pragma unroll ((M::NX == 7 && !std::is_same<S, DF>::value) || (M::NX == 13 && std::is_same<R, double>::value) ? 4 : 1)
   for (int s = 0; s < 4; ++s) {
     M::template f<S, P>(prm, t, H, k);
     if (s == 3) break;
