@@ -154,6 +154,48 @@ static Layout rows_layout_of(int nodes, int max_obs, int csize, int lanes) {
   return L;
 }
 
+// CTAs of the fan kernel at 8 lanes per node (16 nodes each) for `nodes` nodes.
+static int fan_ctas(int nodes) {
+  int csize = 1;
+  while (csize < 8 && (nodes + csize - 1) / csize > 16) csize *= 2;
+  return csize;
+}
+
+// Whether the fan kernel beats one CTA per instance (the lane kernel) on an FP64
+// batch of at most one instance per SM (`horizon` null: all of `nodes` nodes).
+// Batches that take more than 8 lanes per node, and of up to 32 nodes, always;
+// else by the times of both, in ms per 200 ADMM iterations at 10 obstacles (GB300):
+//   lane kernel   2.0 + 0.039 a node of its longest instance with the records in
+//                 shared memory, 2.75 + 0.052 in global memory; 1.25% an obstacle
+//   fan kernel    0.67 a warp of a CTA and round of resident CTAs, 0.4% an obstacle.
+//                 1.84 CTAs per SM are resident (560 clusters of four or eight run
+//                 as two rounds, 608 do not); an uneven batch's rounds overlap.
+// Measured, fan / lane: 60 instances of 41 nodes 2.18 / 3.57, 76 of them 3.75 /
+// 3.56; 140 of 64 5.29 / 5.71, 152 of them 6.82 / 5.77; 100 of 101 7.90 / 8.36, 110
+// of them 9.37 / 8.37; 120 of 41..121 7.88 / 9.31, 152 of them 10.35 / 9.35, with 30
+// obstacles 10.94 / 11.62.
+bool fan_pays(const int* horizon, int batch, int nodes, int max_obs, int optin) {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return false;
+  if (batch > sms) return false;
+  if ((long long)batch * 8 <= sms || nodes <= 32) return true;
+  long long ctas = 0;
+  int shortest = nodes;
+  for (int b = 0; b < batch; ++b) {
+    const int n = horizon ? horizon[b] + 1 : nodes;
+    ctas += fan_ctas(n);
+    shortest = std::min(shortest, n);
+  }
+  double rounds = std::max(1.0, (double)ctas / (1.84 * sms));
+  if (5 * shortest >= 4 * nodes) rounds = std::ceil(rounds);
+  const int chunk = (nodes + fan_ctas(nodes) - 1) / fan_ctas(nodes);
+  const double fan = rounds * 0.67 * ((8 * chunk + 31) / 32) * (0.96 + 0.004 * max_obs);
+  const bool shared = make_layout(UCN_MODEL_QUAD12, nodes, max_obs, 8, false, 4).bytes + (long long)sizeof(InstShared) + 64 <= optin;
+  const double lane = (shared ? 2.0 + 0.039 * nodes : 2.75 + 0.052 * nodes) * (0.875 + 0.0125 * max_obs);
+  return fan < lane;
+}
+
 // The fewest CTAs whose nodes fit their threads: a CTA of 61 nodes takes 1.14 us
 // per ADMM iteration, one of 91 (384 threads, 168 registers) 1.93 us with two
 // CTAs' worth of instances per SM, and 121 nodes as a cluster of two 1.70 us
@@ -167,30 +209,6 @@ static Layout rows_layout_of(int nodes, int max_obs, int csize, int lanes) {
 // per node do less work: us per ADMM iteration, fan / lane kernel (GB300): one
 // instance of 51 nodes 3.9 / 15.1, 40 of 31 nodes 7.2 / 11.1, 152 of 26 nodes
 // 10.2 / 11.1, but 304 of them 19.8 / 16.4 and 608 of 41 nodes 68 / 48.
-// Whether the fan kernel beats one CTA per instance on an FP64 batch of at most
-// one instance per SM (`horizon` null: all of `nodes` nodes).  It spreads the
-// batch's nodes over all SMs, where the lane kernel waits for its longest
-// instance, but pays 1.36 times as much per node (a CTA less than three quarters
-// full as much as one of 12 nodes); up to 32 nodes the lane kernel is bound by
-// latency.  ms of 2 x 100 iterations, fan / lane kernel (GB300): 152 instances of
-// 31 nodes 2.73 / 3.29, of 41 5.88 / 3.57, of 101 12.6 / 8.4; 100 of 41 4.25 /
-// 3.57, of 61 5.25 / 6.10, of 101 7.92 / 8.34; 152 of 41..121 10.5 / 11.1.
-bool fan_pays(const int* horizon, int batch, int nodes) {
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return false;
-  if (batch > sms) return false;
-  if (nodes <= 32) return true;
-  double work = 0.0;
-  for (int b = 0; b < batch; ++b) {
-    const int n = horizon ? horizon[b] + 1 : nodes;
-    int csize = 1;
-    while (csize < 8 && (n + csize - 1) / csize > 16) csize *= 2;
-    work += std::max(n, 12 * csize);
-  }
-  return 1.36 * work <= (double)sms * nodes;
-}
-
 bool rows_layout(int model, int precision, int nodes, int max_obs, int group, int tpn, int batch, int optin, Layout* out) {
   if (precision != UCN_PREC_FP32_REFINE) {
     if (model != UCN_MODEL_QUAD12 || tpn != 4 || group > 1) return false;
@@ -291,7 +309,7 @@ cudaStream_t as_stream(void* s) { return (cudaStream_t)s; }
 void rows_parts(ucn_problem* p) {
   const int tpn = default_tpn(p->model, p->Nmax + 1, p->precision);
   Layout L;
-  if (p->precision == UCN_PREC_FP64 && !fan_pays(p->horizon.data(), p->batch, p->Nmax + 1)) return;
+  if (p->precision == UCN_PREC_FP64 && !fan_pays(p->horizon.data(), p->batch, p->Nmax + 1, p->max_obs, p->optin)) return;
   if (!rows_layout(p->model, p->precision, p->Nmax + 1, p->max_obs, p->group, tpn, p->batch, p->optin, &L)) return;
   p->part_of.assign(p->batch, 0);
   if (p->group > 1) {

@@ -26,14 +26,15 @@ Layout make_layout(int model, int nodes, int max_obs, int tsize, bool reg_mats, 
 
 // The row kernel's layout (ucn_rows.cuh) of an instance of `nodes` nodes, for the
 // problems it serves: FP32, a quadrotor at its default threads per node
-// (12-state 4, quaternion 1), 96 nodes per CTA (64 for the quaternion one) and up to four CTAs per instance (one for scenario groups), within
-// the device's shared memory per CTA.  False where it does not.
+// (12-state 4, quaternion 1), 96 nodes per CTA (64 for the quaternion one) and up
+// to four CTAs per instance (one for scenario groups), within the device's shared
+// memory per CTA.  False where it does not.
 // FP64: the fan kernel's (ucn_fan.cuh) for the 12-state quadrotor at its default
 // threads per node, without scenario groups; `batch` instances share the device.
 bool rows_layout(int model, int precision, int nodes, int max_obs, int group, int tpn, int batch, int optin, Layout* out);
 // Whether the fan kernel is the faster one for an FP64 batch (its nodes, or each
 // instance's horizon).
-bool fan_pays(const int* horizon, int batch, int nodes);
+bool fan_pays(const int* horizon, int batch, int nodes, int max_obs, int optin);
 
 // Everything one kernel launch needs besides its buffers.
 struct LaunchCfg {

@@ -371,7 +371,7 @@ ucn_status ucn_serve_create(const ucn_serve_config* c, ucn_server** out) {
     s->L = make_layout(c->model, s->Nmax + 1, s->max_obs, tsize, false, s->tpn);
   }
   s->smem_bytes = s->smem ? s->L.bytes : 0;
-  s->rows = (c->precision != UCN_PREC_FP64 || fan_pays(nullptr, S, s->Nmax + 1)) &&
+  s->rows = (c->precision != UCN_PREC_FP64 || fan_pays(nullptr, S, s->Nmax + 1, s->max_obs, optin)) &&
             rows_layout(c->model, c->precision, s->Nmax + 1, s->max_obs, 1, s->tpn, S, optin, &s->Lr);
   s->threads = (s->Nmax + 1 + 31) / 32 * 32;
   s->R = c->kept > 0 ? c->kept : 2 * S;
