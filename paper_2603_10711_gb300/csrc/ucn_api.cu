@@ -168,8 +168,8 @@ static int fan_ctas(int nodes) {
 //   lane kernel   2.0 + 0.039 a node of its longest instance with the records in
 //                 shared memory, 2.75 + 0.052 in global memory; 1.25% an obstacle
 //   fan kernel    0.67 a warp of a CTA and round of resident CTAs, 0.4% an obstacle.
-//                 1.84 CTAs per SM are resident (560 clusters of four or eight run
-//                 as two rounds, 608 do not); an uneven batch's rounds overlap.
+//                 1.85 CTAs per SM are resident (560 in clusters of four or eight
+//                 run as two rounds, 608 do not); an uneven batch's rounds overlap.
 // Measured, fan / lane: 60 instances of 41 nodes 2.18 / 3.57, 76 of them 3.75 /
 // 3.56; 140 of 64 5.29 / 5.71, 152 of them 6.82 / 5.77; 100 of 101 7.90 / 8.36, 110
 // of them 9.37 / 8.37; 120 of 41..121 7.88 / 9.31, 152 of them 10.35 / 9.35, with 30
@@ -181,16 +181,16 @@ bool fan_pays(const int* horizon, int batch, int nodes, int max_obs, int optin) 
   if (batch > sms) return false;
   if ((long long)batch * 8 <= sms || nodes <= 32) return true;
   long long ctas = 0;
-  int shortest = nodes;
+  int shortest = nodes, warps = 1;
   for (int b = 0; b < batch; ++b) {
-    const int n = horizon ? horizon[b] + 1 : nodes;
-    ctas += fan_ctas(n);
+    const int n = horizon ? horizon[b] + 1 : nodes, c = fan_ctas(n);
+    ctas += c;
     shortest = std::min(shortest, n);
+    warps = std::max(warps, (8 * ((n + c - 1) / c) + 31) / 32);
   }
-  double rounds = std::max(1.0, (double)ctas / (1.84 * sms));
+  double rounds = std::max(1.0, (double)ctas / (1.85 * sms));
   if (5 * shortest >= 4 * nodes) rounds = std::ceil(rounds);
-  const int chunk = (nodes + fan_ctas(nodes) - 1) / fan_ctas(nodes);
-  const double fan = rounds * 0.67 * ((8 * chunk + 31) / 32) * (0.96 + 0.004 * max_obs);
+  const double fan = rounds * 0.67 * warps * (0.96 + 0.004 * max_obs);
   const bool shared = make_layout(UCN_MODEL_QUAD12, nodes, max_obs, 8, false, 4).bytes + (long long)sizeof(InstShared) + 64 <= optin;
   const double lane = (shared ? 2.0 + 0.039 * nodes : 2.75 + 0.052 * nodes) * (0.875 + 0.0125 * max_obs);
   return fan < lane;
