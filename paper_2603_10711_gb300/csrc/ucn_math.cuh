@@ -214,10 +214,10 @@ template <class T, int K> __device__ __forceinline__ void sincos_(DualN<T, K> a,
 
 // ------------------------------------------------------------------ models
 // A model's constants as the dynamics read them: PRM values, the problem's
-// eight (model_params) and quotients of them, formed once per instance in FP64
-// (derived_param) and rounded to the arithmetic's type -- a division costs ~25
-// dependent FP64 instructions, or ~40 FP32 ones in double-float, and the RK4
-// map evaluated nine of them at every stage of every tangent.
+// eight (model_params) and reciprocals and differences of them, formed once per
+// instance in FP64 (derived_param) and rounded to the arithmetic's type -- a
+// division costs ~25 dependent FP64 instructions, or ~40 FP32 ones in double-float,
+// and the RK4 map has nine of them at every stage of every tangent.
 constexpr int PRM = 16;
 
 // What an RK4 step holds constant: the control enters through a few combined
@@ -226,7 +226,9 @@ constexpr int PRM = 16;
 // Quadrotor, 12 states (position, velocity, ZYX Euler angles phi/theta/psi,
 // body rates), 4 rotor thrusts in a "+" layout.
 // prm: m, Jx, Jy, Jz, arm, km (yaw moment per unit thrust), drag, g | 1/m, 1/Jx,
-// 1/Jy, 1/Jz, drag/m, (Jz-Jy)/Jx, (Jx-Jz)/Jy, (Jy-Jx)/Jz.
+// 1/Jy, 1/Jz, drag/m, Jz-Jy, Jx-Jz, Jy-Jx.  The quotients by m and J are taken at
+// every stage: one rounding of a held quotient would be the same in all four, and
+// add up where four of their own average out.
 struct Quad12 {
   static constexpr int NX = 12, NU = 4;
   __host__ __device__ static double derived(const double* p, int k) {
@@ -237,27 +239,27 @@ struct Quad12 {
       case 10: return 1.0 / Jy;
       case 11: return 1.0 / Jz;
       case 12: return p[6] / m;
-      case 13: return (Jz - Jy) / Jx;
-      case 14: return (Jx - Jz) / Jy;
-      default: return (Jy - Jx) / Jz;
+      case 13: return Jz - Jy;
+      case 14: return Jx - Jz;
+      default: return Jy - Jx;
     }
   }
-  template <class S> struct Held { S Fm, ax, ay, az; };
+  template <class S> struct Held { S F, tx, ty, tz; };
   template <class S, class P>
   __device__ static __forceinline__ Held<S> hold(const P* prm, const S* u) {
     typedef typename BaseOf<S>::type R;
     const R arm = (R)prm[4], km = (R)prm[5];
     Held<S> H;
-    H.Fm = quot_(u[0] + u[1] + u[2] + u[3], (R)prm[0], (R)prm[8]);
-    H.ax = quot_(arm * (u[1] - u[3]), (R)prm[1], (R)prm[9]);
-    H.ay = quot_(arm * (u[2] - u[0]), (R)prm[2], (R)prm[10]);
-    H.az = quot_(km * (u[0] - u[1] + u[2] - u[3]), (R)prm[3], (R)prm[11]);
+    H.F = u[0] + u[1] + u[2] + u[3];
+    H.tx = arm * (u[1] - u[3]);
+    H.ty = arm * (u[2] - u[0]);
+    H.tz = km * (u[0] - u[1] + u[2] - u[3]);
     return H;
   }
   template <class S, class P>
   __device__ static __forceinline__ void f(const P* prm, const S* x, const Held<S>& H, S* xd) {
     typedef typename BaseOf<S>::type R;
-    const R g = (R)prm[7], cdm = (R)prm[12];
+    const R m = (R)prm[0], rm = (R)prm[8], g = (R)prm[7], cdm = (R)prm[12];
     S sph, cph, sth, cth, sps, cps;
     sincos_(x[6], sph, cph);
     sincos_(x[7], sth, cth);
@@ -267,9 +269,9 @@ struct Quad12 {
     xd[0] = x[3];
     xd[1] = x[4];
     xd[2] = x[5];
-    xd[3] = (cs * cps + sph * sps) * H.Fm - cdm * x[3];
-    xd[4] = (cs * sps - sph * cps) * H.Fm - cdm * x[4];
-    xd[5] = (cph * cth) * H.Fm - g - cdm * x[5];
+    xd[3] = quot_((cs * cps + sph * sps) * H.F, m, rm) - cdm * x[3];
+    xd[4] = quot_((cs * sps - sph * cps) * H.F, m, rm) - cdm * x[4];
+    xd[5] = quot_((cph * cth) * H.F, m, rm) - g - cdm * x[5];
     const S wx = x[9], wy = x[10], wz = x[11];
     // Euler-angle rates from body rates (ZYX kinematics)
     const S w = (sph * wy + cph * wz) / cth;
@@ -277,9 +279,9 @@ struct Quad12 {
     xd[7] = cph * wy - sph * wz;
     xd[8] = w;
     // rigid-body rotation: J w' = tau - w x (J w)
-    xd[9] = H.ax - (R)prm[13] * (wy * wz);
-    xd[10] = H.ay - (R)prm[14] * (wz * wx);
-    xd[11] = H.az - (R)prm[15] * (wx * wy);
+    xd[9] = quot_(H.tx - (R)prm[13] * wy * wz, (R)prm[1], (R)prm[9]);
+    xd[10] = quot_(H.ty - (R)prm[14] * wz * wx, (R)prm[2], (R)prm[10]);
+    xd[11] = quot_(H.tz - (R)prm[15] * wx * wy, (R)prm[3], (R)prm[11]);
   }
 };
 
@@ -289,15 +291,15 @@ struct Quad12 {
 struct Quat13 {
   static constexpr int NX = 13, NU = 4;
   __host__ __device__ static double derived(const double* p, int k) { return Quad12::derived(p, k); }
-  template <class S> struct Held { S Tm, ax, ay, az; };
+  template <class S> struct Held { S Tm, tx, ty, tz; };
   template <class S, class P>
   __device__ static __forceinline__ Held<S> hold(const P* prm, const S* u) {
     typedef typename BaseOf<S>::type R;
     Held<S> H;
     H.Tm = quot_(u[0], (R)prm[0], (R)prm[8]);
-    H.ax = quot_(u[1], (R)prm[1], (R)prm[9]);
-    H.ay = quot_(u[2], (R)prm[2], (R)prm[10]);
-    H.az = quot_(u[3], (R)prm[3], (R)prm[11]);
+    H.tx = u[1];
+    H.ty = u[2];
+    H.tz = u[3];
     return H;
   }
   template <class S, class P>
@@ -321,9 +323,9 @@ struct Quat13 {
     xd[7] = R(0.5) * (qw * wx + qy * wz - qz * wy);
     xd[8] = R(0.5) * (qw * wy - qx * wz + qz * wx);
     xd[9] = R(0.5) * (qw * wz + qx * wy - qy * wx);
-    xd[10] = H.ax - (R)prm[13] * (wy * wz);
-    xd[11] = H.ay - (R)prm[14] * (wz * wx);
-    xd[12] = H.az - (R)prm[15] * (wx * wy);
+    xd[10] = quot_(H.tx - (R)prm[13] * wy * wz, (R)prm[1], (R)prm[9]);
+    xd[11] = quot_(H.ty - (R)prm[14] * wz * wx, (R)prm[2], (R)prm[10]);
+    xd[12] = quot_(H.tz - (R)prm[15] * wx * wy, (R)prm[3], (R)prm[11]);
   }
 };
 
@@ -412,10 +414,10 @@ __device__ __forceinline__ DF fma_(DF a, DF b, DF c) { return df_fma(a, b, c); }
 // 3-DOF Mars model's step is small outside double-float; rolled, its kernels
 // spill in the ADMM loop.  The quaternion quadrotor's in FP64 waits for the FP64
 // pipe instead, and a loop's frame costs its one-thread kernel more (152 of 50
-// nodes, 4 x 100 iterations: 22.72 ms rolled, 22.16 straight).  The 6-DOF lander's stays straight-line with quotients
-// and held terms in every stage: its FP32 solves meet decisions that a last bit
-// turns (one batch of 1000 in sixteen: up to 5e-5 normwise), so their results are
-// only as constant as this rounding.
+// nodes, 4 x 100 iterations: 22.72 ms rolled, 22.16 straight).  The 6-DOF
+// lander's stays straight-line with quotients and held terms in every stage: its
+// FP32 solves meet decisions that a last bit turns (one batch of 1000 in sixteen:
+// up to 5e-5 normwise), so their results are only as constant as this rounding.
 template <class M, class S, class P, class R>
 __device__ __forceinline__ void rk4h(const P* prm, R h, R hh, R h6, const S* x, const S* u, S* xn) {
   constexpr int NX = M::NX;
