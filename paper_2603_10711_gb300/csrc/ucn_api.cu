@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -39,6 +40,15 @@ long long round_up(long long v, long long m) { return (v + m - 1) / m * m; }
 namespace ucn {
 
 void set_error_message(const char* msg) { snprintf(g_err, sizeof(g_err), "%s", msg); }
+
+static std::atomic<int> loops_on[64];
+void loop_count(int device, int by) {
+  if (device >= 0 && device < 64) loops_on[device].fetch_add(by);
+}
+bool loop_on_device() {
+  int dev = 0;
+  return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 && loops_on[dev].load() > 0;
+}
 
 int fault_alloc_at() {
   const char* e = std::getenv("UCN_FAULT_ALLOC");
@@ -674,9 +684,11 @@ long long ucn_total_x(const ucn_problem* p) { return p ? p->total_x : -1; }
 long long ucn_total_u(const ucn_problem* p) { return p ? p->total_u : -1; }
 long long ucn_state_size(const ucn_problem* p) { return p ? p->state_size : -1; }
 
-// Whether the fused solve (or the ADMM call: FP32) runs the row or fan kernel.
+// Whether the fused solve (or the ADMM call: FP32) runs the row or fan kernel:
+// asked once per call, the launch goes by the layout it is given.
 static bool rows_on(const ucn_problem* p, bool admm) {
-  return !p->parts.empty() && !(admm && p->precision == UCN_PREC_FP64) && p->tpn == default_tpn(p->model, p->Nmax + 1, p->precision);
+  if (p->parts.empty() || p->tpn != default_tpn(p->model, p->Nmax + 1, p->precision)) return false;
+  return p->precision != UCN_PREC_FP64 || !(admm || loop_on_device());
 }
 
 static LaunchCfg cfg_of(ucn_problem* p, void* stream, bool admm = false) {
@@ -707,8 +719,8 @@ static unsigned long long capture_of(cudaStream_t s) {   // id of the capture th
 
 extern "C++" {
 template <class F>
-static cudaError_t launch_parts(ucn_problem* p, LaunchCfg c, bool admm, F launch) {
-  if (!rows_on(p, admm) || p->parts.size() == 1) return launch(c);
+static cudaError_t launch_parts(ucn_problem* p, LaunchCfg c, F launch) {
+  if (((const Layout*)c.L)->csize == 0 || p->parts.size() == 1) return launch(c);
   std::lock_guard<std::mutex> lk(p->parts_mu);
   cudaStream_t s = c.stream;
   bool alone = false;
@@ -761,7 +773,7 @@ ucn_status ucn_admm_solve(ucn_problem* p, const double* xbar_d, const double* ub
   if (p->group > 1) return fail(UCN_EINVAL, "the scenario consensus runs inside ucn_scp_solve only");
   const LaunchCfg c = cfg_of(p, stream, true);
   auto fn = launchers_for(p->model, p->precision).admm;
-  const cudaError_t e = launch_parts(p, c, true, [&](const LaunchCfg& k) {
+  const cudaError_t e = launch_parts(p, c, [&](const LaunchCfg& k) {
     return fn(k, xbar_d, ubar_d, A_d, B_d, d_d, radius_d, iters, warm ? 1 : 0, xhat_d, uhat_d, res_d, status_d);
   });
   if (e != cudaSuccess) return fail(UCN_ECUDA, "admm launch: %s", cudaGetErrorString(e));
@@ -796,7 +808,7 @@ ucn_status ucn_scp_solve(ucn_problem* p, const double* x0_d, const double* u0_d,
     return UCN_OK;
   }
   auto fn = launchers_for(p->model, p->precision).scp;
-  const cudaError_t e = launch_parts(p, c, false, [&](const LaunchCfg& k) {
+  const cudaError_t e = launch_parts(p, c, [&](const LaunchCfg& k) {
     return fn(k, x0_d, u0_d, x_out_d, u_out_d, stats_d, status_d);
   });
   if (e != cudaSuccess) return fail(UCN_ECUDA, "scp launch: %s", cudaGetErrorString(e));
@@ -819,7 +831,7 @@ ucn_status ucn_scp_solve_warm(ucn_problem* p, const double* x0_d, const double* 
   LaunchCfg c = cfg_of(p, stream);
   c.P = &Pw;
   auto fn = launchers_for(p->model, p->precision).scp;
-  const cudaError_t e = launch_parts(p, c, false, [&](const LaunchCfg& k) {
+  const cudaError_t e = launch_parts(p, c, [&](const LaunchCfg& k) {
     return fn(k, x0_d, u0_d, x_out_d, u_out_d, stats_d, status_d);
   });
   if (e != cudaSuccess) return fail(UCN_ECUDA, "scp launch: %s", cudaGetErrorString(e));

@@ -36,6 +36,14 @@ bool rows_layout(int model, int precision, int nodes, int max_obs, int group, in
 // instance's horizon).
 bool fan_pays(const int* horizon, int batch, int nodes, int max_obs, int optin);
 
+// Request loops that are on, by device (ucn_serve_loop_start .. _stop): their CTAs
+// stay on their SMs, and the fan kernel's clusters of up to 16 CTAs, which need their
+// SMs free at one time, would wait for a loop's end where a single CTA finds a place
+// (a loop of 100 CTAs with 1.5 s idle time: one FP64 quadrotor 1301 ms instead of 5).
+// While a loop is on, FP64 solves run as one CTA per instance, on the lane kernel.
+void loop_count(int device, int by);
+bool loop_on_device();   // the current device
+
 // Everything one kernel launch needs besides its buffers.
 struct LaunchCfg {
   const void* P;        // ProblemDev*

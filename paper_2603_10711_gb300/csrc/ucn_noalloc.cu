@@ -212,7 +212,7 @@ extern "C" ucn_status ucn_scp_solve_noalloc(const ucn_problem_desc* d, const dou
   c.threads = (int)((Nmax + 1 + 31) / 32 * 32); c.blocks = B; c.stream = st; c.group = 1;
   c.nodes = Nmax + 1; c.tpn = tpn;
   Layout Lr;
-  if ((d->precision != UCN_PREC_FP64 || fan_pays(nullptr, B, Nmax + 1, max_obs, optin)) &&   // (one shape for all: that of the longest)
+  if ((d->precision != UCN_PREC_FP64 || (fan_pays(nullptr, B, Nmax + 1, max_obs, optin) && !loop_on_device())) &&   // (one shape for all: that of the longest)
       rows_layout(d->model, d->precision, Nmax + 1, max_obs, 1, tpn, B, optin, &Lr)) { c.L = &Lr; c.smem_bytes = Lr.bytes; }
   auto fn = launchers_for(d->model, d->precision).scp;
   e = fn(c, x0_d, u0_d, x_out_d, u_out_d, stats_d, status_d);

@@ -128,6 +128,7 @@ struct ucn_server {
   cudaStream_t loop_stream = nullptr;
   cudaEvent_t loop_done = nullptr;
   bool loop_on = false;         // submit publishes to the loop (ucn_serve_loop_start .. _stop)
+  int loop_dev = 0;             // the device it was started on
   bool loop_live = false;       // a loop launch has been made and not seen to end
   int loop_ctas = 0;            // CTAs asked for (0: every CTA that can be resident)
   unsigned long long loop_idle_ns = 0;
@@ -326,6 +327,7 @@ void ucn_serve_destroy(ucn_server* s) {
   if (!s) return;
   if (s->lstop_h) __atomic_store_n(s->lstop_h, 1u, __ATOMIC_RELEASE);   // a running loop ends
   cudaDeviceSynchronize();
+  if (s->loop_on) loop_count(s->loop_dev, -1);
   if (s->loop_stream) cudaStreamDestroy(s->loop_stream);
   if (s->loop_done) cudaEventDestroy(s->loop_done);
   for (cudaStream_t st : s->streams) cudaStreamDestroy(st);
@@ -602,7 +604,7 @@ ucn_status ucn_serve_pump(ucn_server* s, int* launched) {
     c.P = &P; c.L = &s->L; c.smem = s->smem; c.smem_bytes = s->smem_bytes;
     c.threads = s->threads; c.blocks = n; c.stream = st; c.group = 1;
     c.nodes = s->cfg.max_horizon + 1; c.tpn = s->tpn;
-    if (s->rows) { c.L = &s->Lr; c.smem = true; c.smem_bytes = s->Lr.bytes; }
+    if (s->rows && !(s->cfg.precision == UCN_PREC_FP64 && loop_on_device())) { c.L = &s->Lr; c.smem = true; c.smem_bytes = s->Lr.bytes; }
     auto fn = launchers_for(s->cfg.model, s->cfg.precision).scp;
     e = fn(c, s->D.x0, s->D.u0, s->D.xo, s->D.uo, s->D.stats, s->status_d);
   }
@@ -722,6 +724,8 @@ ucn_status ucn_serve_loop_start(ucn_server* s, int ctas, double idle_s) {
   s->loop_error = cudaSuccess;
   __atomic_store_n(s->lstop_h, 0u, __ATOMIC_RELEASE);
   s->loop_on = true;
+  cudaGetDevice(&s->loop_dev);
+  loop_count(s->loop_dev, 1);
   // requests admitted and not pumped go to the loop, oldest first
   std::vector<std::pair<unsigned long long, int>> adm;
   for (int k = 0; k < s->S; ++k)
@@ -746,6 +750,7 @@ ucn_status ucn_serve_loop_stop(ucn_server* s) {
   if (e == cudaSuccess) e = s->loop_error;
   __atomic_store_n(s->lstop_h, 0u, __ATOMIC_RELEASE);
   s->loop_on = false;
+  loop_count(s->loop_dev, -1);
   if (e != cudaSuccess) return sfail(UCN_ECUDA, "request loop failed: %s", cudaGetErrorString(e));
   // every published request has been delivered: the ring entries it wrote are complete
   for (int r = 0; r < s->R; ++r)
