@@ -631,6 +631,11 @@ ucn_status ucn_problem_create(const ucn_problem_desc* d, ucn_problem** out) {
       return fail(UCN_ECUDA, "streams of the batch's parts: %s", cudaGetErrorString(e));
     }
   }
+  if (d->precision == UCN_PREC_FP64 && !p->parts.empty()) {
+    LaunchCfg c = {};
+    c.P = &p->dev; c.L = &p->L; c.smem = p->smem; c.smem_bytes = p->smem_bytes; c.nodes = Nmax + 1;
+    if (quad64_load_lanes(c) != cudaSuccess) cudaGetLastError();
+  }
   *out = p;
   return UCN_OK;
 }

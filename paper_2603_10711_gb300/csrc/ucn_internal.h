@@ -60,6 +60,11 @@ struct LaunchCfg {
   int* launched = nullptr;   // out (when not NULL): kernel launches the fused solve made
 };
 
+// FP64 12-state quadrotors that the fan kernel serves: loads the lane kernel, which
+// takes their solves while a request loop is on -- by then too late: a kernel's
+// first use waits for the loop.
+cudaError_t quad64_load_lanes(const LaunchCfg& c);
+
 // Threads per node the fused solve uses by default for a model, node count and
 // precision (records in shared memory; 1 otherwise for the 3-DOF Mars model).
 int default_tpn(int model, int nodes, int precision);

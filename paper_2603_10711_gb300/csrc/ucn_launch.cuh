@@ -185,6 +185,19 @@ cudaError_t launch_scpl_v(const LaunchCfg& c, const double* x0, const double* u0
               : Narrow::launch(c, threads, x0, u0, xo, uo, st, status);
 }
 
+// Loads the lane kernel that a launch would take, without launching it (a kernel's
+// first use loads it, and waits for whatever runs on the device).
+template <class M, class T, bool SMEM, bool R>
+cudaError_t load_scpl_v(const LaunchCfg& c) {
+  using Wide = LanesVariant<M, T, SMEM, R, LANES_WIDE_THREADS>;
+  using Narrow = LanesVariant<M, T, SMEM, R, LANES_MAX_THREADS>;
+  const int threads = (4 * c.nodes + 31) / 32 * 32;
+  bool wide = false;
+  int n = 0;
+  const cudaError_t e = lanes_prefer_wide<Wide, Narrow>(c, threads, &wide);
+  return e == cudaSuccess ? Narrow::occupancy(c, threads, &n) : e;
+}
+
 // The pair kernel (2 threads per node; 3-DOF Mars, FP32, records in shared memory).
 template <class M, bool R>
 cudaError_t launch_scpp_v(const LaunchCfg& c, const double* x0, const double* u0, double* xo, double* uo,

@@ -211,6 +211,7 @@ extern "C" ucn_status ucn_scp_solve_noalloc(const ucn_problem_desc* d, const dou
   c.P = &P; c.L = &L; c.smem = true; c.smem_bytes = L.bytes;
   c.threads = (int)((Nmax + 1 + 31) / 32 * 32); c.blocks = B; c.stream = st; c.group = 1;
   c.nodes = Nmax + 1; c.tpn = tpn;
+  if (d->precision == UCN_PREC_FP64 && d->model == UCN_MODEL_QUAD12 && tpn == 4 && quad64_load_lanes(c) != cudaSuccess) cudaGetLastError();
   Layout Lr;
   if ((d->precision != UCN_PREC_FP64 || (fan_pays(nullptr, B, Nmax + 1, max_obs, optin) && !loop_on_device())) &&   // (one shape for all: that of the longest)
       rows_layout(d->model, d->precision, Nmax + 1, max_obs, 1, tpn, B, optin, &Lr)) { c.L = &Lr; c.smem_bytes = Lr.bytes; }

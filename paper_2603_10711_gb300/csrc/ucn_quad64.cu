@@ -9,3 +9,8 @@ UCN_EXTERN_SCPL(Quad12, double, false, false, ucn::LANES_WIDE_THREADS)
 UCN_EXTERN_ADMM(Quad12, double, true, false)
 UCN_EXTERN_ADMM(Quad12, double, false, false)
 UCN_DEFINE_LAUNCHERS(quad64, Quad12, double, false)
+namespace ucn {
+cudaError_t quad64_load_lanes(const LaunchCfg& c) {
+  return c.smem ? load_scpl_v<Quad12, double, true, false>(c) : load_scpl_v<Quad12, double, false, false>(c);
+}
+}  // namespace ucn

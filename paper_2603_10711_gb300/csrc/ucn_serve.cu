@@ -375,6 +375,11 @@ ucn_status ucn_serve_create(const ucn_serve_config* c, ucn_server** out) {
   s->smem_bytes = s->smem ? s->L.bytes : 0;
   s->rows = (c->precision != UCN_PREC_FP64 || fan_pays(nullptr, S, s->Nmax + 1, s->max_obs, optin)) &&
             rows_layout(c->model, c->precision, s->Nmax + 1, s->max_obs, 1, s->tpn, S, optin, &s->Lr);
+  if (s->rows && c->precision == UCN_PREC_FP64) {
+    LaunchCfg k = {};
+    k.L = &s->L; k.smem = s->smem; k.smem_bytes = s->smem_bytes; k.nodes = s->Nmax + 1;
+    if (quad64_load_lanes(k) != cudaSuccess) cudaGetLastError();
+  }
   s->threads = (s->Nmax + 1 + 31) / 32 * 32;
   s->R = c->kept > 0 ? c->kept : 2 * S;
   s->rl = rec_layout(NX, NU, MO, (int)Xn, (int)Un);
