@@ -189,10 +189,10 @@ ucn_status ucn_problem_set_lanes(ucn_problem* prob, int lanes_per_node);
 int ucn_problem_lanes(const ucn_problem* prob);
 
 /* Kernel launches made by the last ucn_scp_solve / ucn_scp_solve_warm /
- * ucn_admm_solve call on this problem: 1; 2 when the fused
- * solve ran a first round on its three-CTAs-per-SM variant; up to 3 for an
- * uneven FP32 batch, one per CTA shape (see ucn_scp_solve); 0 before the first call, -1 for NULL.  (Not in the paper;
- * for launch accounting.) */
+ * ucn_admm_solve call on this problem: 1; 2 when the fused solve ran a first
+ * round on its three-CTAs-per-SM variant; up to 3 for an uneven quadrotor batch,
+ * one per CTA shape (see ucn_scp_solve); 0 before the first call, -1 for NULL.
+ * (Not in the paper; for launch accounting.) */
 int ucn_problem_last_launches(const ucn_problem* prob);
 
 /* Number of elements of the packed state / trajectory buffers. */
@@ -236,14 +236,16 @@ ucn_status ucn_state_export(ucn_problem* prob, double* state_d, void* stream);
  * instance by persistent kernel launches that each run whole solves: per SCP
  * iteration the RK4 linearisation, assembly + factorisation, admm_iters ADMM
  * iterations, and the rollout / defect / trust-region acceptance test, all on
- * the device, one CTA per instance (or, FP32 quadrotors beyond 96 nodes, 64 for
- * the quaternion one, a thread-block cluster of two or four).  One launch; FP32
- * batches of those models whose instances need different CTA shapes take one
- * launch per shape, side by side on streams of the problem forked from and
- * joined to `stream`; for batches of the 3-DOF Mars
- * model in FP32 that are not a whole number of resident rounds, a first launch
- * runs one round on a three-CTAs-per-SM variant of the same kernel and a second
- * the rest (same results per instance).  In: initial guesses x0_d, u0_d.  Out:
+ * the device, one CTA per instance, or a thread-block cluster: of two or four
+ * for FP32 quadrotors beyond 96 nodes (64 for the quaternion one), of up to 16
+ * for FP64 12-state quadrotors in batches of at most one instance per SM, where
+ * that is the faster form and no request loop is on (ucn_serve_loop_start).  One
+ * launch; batches of those kinds whose instances need different CTA shapes take
+ * one launch per shape, at most three, side by side on streams of the problem
+ * forked from and joined to `stream`; for batches of the 3-DOF Mars model in FP32
+ * that are not a whole number of resident rounds, a first launch runs one round on
+ * a three-CTAs-per-SM variant of the same kernel and a second the rest (same
+ * results per instance).  In: initial guesses x0_d, u0_d.  Out:
  * x_out_d, u_out_d (the last accepted trajectory), stats_d [batch], status_d
  * [batch] (== stats.status).  An instance whose data or guesses hold a NaN (or an
  * infinity outside the bounds and set parameters) ends UCN_ENUMERIC after its
@@ -437,10 +439,12 @@ int ucn_serve_free_slots(ucn_server* srv);
  * publishes each admitted request at once -- its record into mapped host
  * memory, the slot into a queue, then the queue head -- and a CTA of the
  * running kernel that is free claims it (in submission order), copies its data
- * into the slot, runs the same fused SCP solve as a pump launch (Secs. III-A,
- * III-B: the same kernel body on the same slot layout), keeps its result in the
- * ring and delivers it to host memory; there is no pump and no launch per
- * request.  Requests admitted and not pumped when the loop starts go to it
+ * into the slot, runs the fused SCP solve (Secs. III-A, III-B) on the lane or
+ * one-thread kernel -- pump launches of FP32 quadrotors take the row kernel, which
+ * is several times faster --, keeps its result in the ring and delivers it to host
+ * memory; there is no pump and no launch per request.  The loop's CTAs stay on
+ * their SMs: while a loop is on, FP64 quadrotor solves on its device run as one CTA
+ * per instance (results agree to rounding).  Requests admitted and not pumped when the loop starts go to it
  * first.  Every wait of the kernel is bounded: once no request has been
  * published to the server for `idle_s` seconds (0 < idle_s <= 60) its CTAs
  * end (each CTA's idle clock restarts whenever a request is published, so the

@@ -1,5 +1,5 @@
-// Kernel instantiations: 13-state quaternion quadrotor, FP32 path with refinement.  The fused
-// solve with global-memory records and the stand-alone ADMM compile in their
-// own units (ucn_quat32_*.cu).
+// Kernel instantiations: 13-state quaternion quadrotor, FP32 path with refinement:
+// the linearisation; solves and ADMM calls run on the row kernel, in its own units
+// (ucn_quat32_rows*.cu).
 #include "ucn_launch.cuh"
 UCN_DEFINE_LAUNCHERS(quat32, Quat13, float, true)
