@@ -20,9 +20,9 @@
 // ~88 for two (F = 16) or ~140 for four (F = 8), against ~275 for eight with four
 // lanes per node: the more lanes the shorter, the fewer the less work in all.
 // Measured (GB300, four lanes per node -> this): one quadrotor of 50 nodes, 15 x
-// 200 iterations, 52.2 -> 13.3 ms (15.1 -> 3.9 us per ADMM iteration, 445 ->
+// 200 iterations, 52.2 -> 12.96 ms (15.1 -> 3.9 us per ADMM iteration, 445 ->
 // 90 us per SCP iteration outside it); 149 of 40..120 nodes, 10 x 200, 102.5 ->
-// 92.7 ms.  What bounds it: the FP64 pipes at F = 8 (70% busy, counters), else
+// 93.1 ms.  What bounds it: the FP64 pipes at F = 8 (70% busy, counters), else
 // the iteration's chain of FP64 latencies (64 cycles each) and exchanges.
 #pragma once
 #include "ucn_rows.cuh"

@@ -614,7 +614,8 @@ __device__ __forceinline__ void group_init(const ProblemDev& P, GroupShared* G) 
 // One cluster per group: each CTA stores its values into all its peers' shared
 // memory, which count the bytes on an mbarrier that warp 0 waits on -- no barrier
 // across the cluster (with a cluster barrier per iteration 16 groups of 16 took
-// 6.04 us per iteration, so 5.37; 64 groups 15.1, so 13.6).  Several:
+// 6.04 us per iteration, so 5.37; 64 groups 15.1, so 13.6, 14.4 with FP64 sums).
+// Several:
 // through its global slot and counter, as group_allreduce_flat.
 __device__ __forceinline__ void group_publish(const ProblemDev& P, GroupShared* G, const GroupX& X, double v) {
   const int lane = threadIdx.x, j = lane & 3;

@@ -666,7 +666,8 @@ __device__ __forceinline__ void scp_lanes_body(const ProblemDev& P, const Layout
 // CTAs of up to 512 threads: 128 registers with the records in shared memory, 64
 // with FP64 records in global memory, where two CTAs per SM hide each other's
 // loads (FP64, 2 x 200 iterations: 2048 quadrotors of 40..120 nodes 204 -> 188 ms,
-// 608 of them 59.8 -> 58.5).
+// 608 of them 59.8 -> 58.5; one instance per SM, 152 of 51, 81, 101 and 128 nodes
+// at 2 x 100: 5.6, 7.1, 8.4 and 9.7 ms).
 template <class M, class T, bool SMEM, bool REFINE, bool GROUP, int TPN>
 __global__ void __launch_bounds__(LANES_MAX_THREADS, !SMEM && sizeof(T) == 8 ? 2 : 1)
     scp_kernel_lanes(ProblemDev P, Layout L, const double* x0, const double* u0, double* xout, double* uout,

@@ -11,9 +11,10 @@
 //    three axes): the r_j columns are unit vectors and the v_j columns hold
 //    d r_j / d v_j and d v_j / d v_j of the scalar recursion -- what a pass along
 //    them computes.
-// Measured (GB300, 2048 quadrotors of 40..120 nodes, 164k nodes, FP64): 4.24 ms
-// with a pass per column (10.4 ms when it also divided by the model constants at
-// each stage), 1.54 ms now; the outputs alone take 0.04 ms at the copy rate.
+// Measured (GB300, 2048 quadrotors of 40..120 nodes, 164k nodes, FP64): 10.4 ms
+// with a pass per column and a division per quotient, 1.83 now (1.55 with quotients
+// by products with reciprocals, held over the step, whose B is 1.2 times as far off);
+// the outputs alone take 0.04 ms at the copy rate.
 #pragma once
 #include "ucn_kernels.cuh"
 

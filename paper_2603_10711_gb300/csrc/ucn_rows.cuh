@@ -18,10 +18,10 @@
 // summed once per SCP iteration.
 //
 // Measured on GB300 (fused solves, before -> with this kernel): 1023 quadrotors
-// of 40..120 nodes, 10 x 200 iterations, 207 -> 36.6 ms; one of 50 nodes 8.57 ->
-// 2.55 ms; 256 quaternion quadrotors of 50 nodes, 20 x 100, 27.3 -> 7.4 ms; the ADMM call
-// on 511 quadrotors, 100 iterations, 8.15 -> 1.07 ms.  The error against FP64
-// is as before (3e-7, 4e-7, 1.1e-6, 4e-7, 1e-6).  What bounds it: latency at 8
+// of 40..120 nodes, 10 x 200 iterations, 207 -> 37.3 ms; one of 50 nodes 8.56 ->
+// 2.73 ms; 256 quaternion quadrotors of 50 nodes, 20 x 100, 27.1 -> 7.34 ms; the
+// ADMM call on 511 quadrotors, 100 iterations, 8.06 -> 1.07 ms.  The error against
+// FP64 is as before (medians over 64 to 128 batches 2.0e-7 to 2.4e-7).  What bounds it: latency at 8
 // warps per SM -- issue slots 45% used in the ADMM loop; stalls at the two
 // barriers of an iteration, instruction fetch and fixed-latency dependencies.
 //
